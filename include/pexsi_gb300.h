@@ -69,7 +69,11 @@ typedef struct pexsi_opts {
   int32_t leaf_cols;       /* nested-dissection leaf size in columns (default 96)    */
   int32_t amalgamate;      /* 1: relaxed supernode amalgamation (default), 0: off    */
   int32_t max_batch;       /* poles / shifts per device batch, 0 = automatic         */
-  int32_t split_slices;    /* 0: FP64 GEMMs (default). 2..6: the supernode GEMMs
+  int32_t split_slices;    /* 0: FP64 products (default): exact integer products of
+                              58-bit operands in residues modulo 15 numbers on the
+                              tcgen05 tensor cores, accurate to 2^-59 of the
+                              operands' row norms, or FP64 multiply-adds where the
+                              budget leaves no room for their scratch. 2..6: the supernode GEMMs
                               (panel solve L = W D^-1, Schur update F -= L W^T,
                               Takahashi step Y[S,P] = -Y[S,S] L[S,P] and Y[P,P] =
                               D^-1 - L[S,P]^T Y[S,P]; real ones of the inertia
@@ -80,7 +84,7 @@ typedef struct pexsi_opts {
                               Requires panel = 64; other values are INVALID_ARG. */
   int64_t hbm_budget;      /* bytes of device workspace the batch may use, 0 = auto  */
   int64_t wait_ns;         /* bound, in ns of wall time, of every wait of one role of
-                              a split-precision kernel on another (an mbarrier phase
+                              a tensor-core kernel on another (an mbarrier phase
                               of a copy, of the MMAs, of a TMEM drain); 0 = 1 s. A
                               wait that runs out stops the launch cleanly (every
                               role returns, TMEM is freed, later launches of the
@@ -178,7 +182,7 @@ int pexsi_pole_table(double beta, double delta_e, int32_t n_poles, double mu,
  * output may be NULL. S == NULL means S = I (H's diagonal positions). The
  * call is synchronous. On error the outputs are undefined.
  * Errors: INVALID_ARG, NOMEM, CUDA, BREAKDOWN (info->breakdown_front),
- * TIMEOUT (split-precision path only: a bounded device-side wait ran out). */
+ * TIMEOUT (a bounded device-side wait of a tensor-core kernel ran out). */
 int pexsi_dm(pexsi_plan* plan, const double* H, const double* S, double mu, double beta,
              int32_t n_poles, double delta_e, double* dm, double* edm, double* fdm,
              pexsi_dm_info* info);

@@ -20,8 +20,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -ffp-contract=off: host arithmetic (the ordering's Lanczos runs) must give
 # bit-identical results on x86-64 and aarch64 hosts
 COMMON = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off", "-lineinfo", "-I" + os.path.join(HERE, "..", "include")]
-SOURCES = ["symbolic.cpp", "poles.cpp", "kernels.cu", "ozaki.cu", "engine.cu", "server.cu", "mu.cu", "spectral.cu", "noalloc.cu"]
-HEADERS = ["symbolic.hpp", "kernels.cuh", "plan.hpp"]
+SOURCES = ["symbolic.cpp", "poles.cpp", "kernels.cu", "ozaki.cu", "rns.cu", "engine.cu", "server.cu", "mu.cu", "spectral.cu", "noalloc.cu"]
+HEADERS = ["symbolic.hpp", "kernels.cuh", "tensor_core.cuh", "rns.cuh", "plan.hpp"]
 
 
 def nvcc() -> str:

@@ -76,15 +76,39 @@ int64_t kpart_stride(const pexsi_plan* p) {
   return p->oz_slices > 0 ? 0 : p->part_stride / (int64_t(p->b) * p->b) * kMaxKsplit * kTile * p->b;
 }
 
-int64_t bytes_per_pole(const pexsi_plan* p) {
-  return (2 * p->sym.front_elems + p->part_stride + kpart_stride(p)) * int64_t(sizeof(double2)) +
+int64_t bytes_per_pole(const pexsi_plan* p, bool rns) {
+  return (2 * p->sym.front_elems + p->part_stride + (rns ? 0 : kpart_stride(p))) * int64_t(sizeof(double2)) +
          2 * p->sym.n * int64_t(p->b) * int64_t(sizeof(double)) +
          std::max(p->ozA_stride, 2 * p->ozA_stride_r) + std::max(p->ozB_stride, 2 * p->ozB_stride_r) +
          8 * (p->exA_stride + p->exB_stride) + 4 * p->ymax_stride;
 }
 
 int64_t bytes_fixed(const pexsi_plan* p) {
-  return 9 * p->sym.nnz * int64_t(sizeof(double)) + 4 * p->trace_blocks * 8 + 4096;
+  return 9 * p->sym.nnz * int64_t(sizeof(double)) + 4 * p->trace_blocks * 8 + 4096 +
+         (p->oz_slices > 0 ? 0 : 2 * p->sym.nnz + 4 * p->sym.n);
+}
+
+void rns_scratch(const pexsi_plan* p, int batch, int64_t most, int64_t& planes, int64_t& out) {
+  planes = out = 0;
+  if (p->oz_slices > 0) return;
+  int64_t least, want;
+  rns_scratch_range(p, batch, least, want);
+  planes = std::max(least, std::min(want, most));
+  out = rns_out_bytes(p, batch);
+}
+
+int fit_batch(const pexsi_plan* p, int64_t budget, int most, int64_t& planes, int64_t& out) {
+  const int64_t room = budget - bytes_fixed(p);
+  if (p->oz_slices == 0) {
+    rns_scratch(p, most, kRnsPlaneBytes, planes, out);
+    const int64_t nb = (room - planes - out) / bytes_per_pole(p, true);
+    if (nb >= 1) return int(std::min<int64_t>(nb, most));
+    rns_scratch(p, 1, 0, planes, out);
+    if (room - planes - out >= bytes_per_pole(p, true)) return 1;
+  }
+  planes = out = 0;
+  const int64_t nb = room / std::max<int64_t>(bytes_per_pole(p, false), 1);
+  return int(std::max<int64_t>(0, std::min<int64_t>(nb, most)));
 }
 
 namespace {
@@ -110,7 +134,8 @@ void wsalloc(T** ptr, size_t bytes, Workspace& ws, const char* what) {
 }
 }  // namespace
 
-void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, cudaStream_t stream, bool async) {
+void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, int64_t rns_planes, int64_t rns_out,
+                     cudaStream_t stream, bool async) {
   ws.async = async;
   ws.stream = stream;
   ws.batch = batch;
@@ -119,7 +144,7 @@ void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, cudaStream_t
   wsalloc(&ws.F, sizeof(double2) * pool * batch, ws, "alloc(F)");
   wsalloc(&ws.Y, sizeof(double2) * pool * batch, ws, "alloc(Y)");
   wsalloc(&ws.part, sizeof(double2) * size_t(p->part_stride) * batch, ws, "alloc(partials)");
-  if (kpart_stride(p) > 0)
+  if (rns_planes == 0 && kpart_stride(p) > 0)
     wsalloc(&ws.kpart, sizeof(double2) * size_t(kpart_stride(p)) * batch, ws, "alloc(split-K partials)");
   wsalloc(&ws.H, sizeof(double) * nnz, ws, "alloc(H)");
   wsalloc(&ws.S, sizeof(double) * nnz, ws, "alloc(S)");
@@ -133,13 +158,22 @@ void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, cudaStream_t
   wsalloc(&ws.neg, sizeof(int) * kMaxBatch, ws, "alloc(status)");
   wsalloc(&ws.partials, sizeof(double) * 4 * p->trace_blocks, ws, "alloc(trace)");
   wsalloc(&ws.trace3, sizeof(double) * 4, ws, "alloc(trace)");
+  wsalloc(&ws.ozfail, 2 * sizeof(int), ws, "alloc(status)");
+  if (rns_planes > 0) {
+    wsalloc(&ws.rns.planes, size_t(rns_planes), ws, "alloc(residue planes)");
+    wsalloc(&ws.rns.out, size_t(rns_out), ws, "alloc(residue tiles)");
+    wsalloc(&ws.g, sizeof(int32_t) * size_t(p->sym.n), ws, "alloc(scaling)");
+    wsalloc(&ws.gs, sizeof(int16_t) * nnz, ws, "alloc(scaling)");
+    ws.rns.plane_bytes = rns_planes;
+    ws.rns.out_bytes = rns_out;
+    ws.rns.wait_ns = p->wait_ns;
+  }
   if (p->oz_slices > 0) {
     // complex poles use `batch` members, the real inertia shifts up to 2 batch
     wsalloc(&ws.ozA, size_t(std::max(p->ozA_stride, 2 * p->ozA_stride_r)) * batch, ws, "alloc(split A)");
     wsalloc(&ws.ozB, size_t(std::max(p->ozB_stride, 2 * p->ozB_stride_r)) * batch, ws, "alloc(split B)");
     wsalloc(&ws.exA, sizeof(int) * size_t(p->exA_stride) * 2 * batch, ws, "alloc(split exponents)");
     wsalloc(&ws.exB, sizeof(int) * size_t(p->exB_stride) * 2 * batch, ws, "alloc(split exponents)");
-    wsalloc(&ws.ozfail, 2 * sizeof(int), ws, "alloc(status)");
     wsalloc(&ws.ymax, sizeof(uint32_t) * size_t(p->ymax_stride) * batch, ws, "alloc(split row maxima)");
   }
   if (!ws.ev0) ck(cudaEventCreate(&ws.ev0), "cudaEventCreate");
@@ -151,7 +185,7 @@ void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, cudaStream_t
 void workspace_free(Workspace& ws) {
   void* ptrs[] = {ws.F,  ws.Y,        ws.part,  ws.H,    ws.S,   ws.out, ws.brk, ws.minpiv, ws.neg,
                   ws.partials, ws.trace3, ws.ainv, ws.ozA, ws.ozB, ws.exA, ws.exB, ws.ozfail, ws.ymax, ws.kpart,
-                  ws.dsave};
+                  ws.dsave, ws.rns.planes, ws.rns.out, ws.g, ws.gs};
   for (void* q : ptrs) {
     if (!q) continue;
     if (ws.async) cudaFreeAsync(q, ws.stream);
@@ -277,6 +311,16 @@ void factor_batch(const pexsi_plan* p, Workspace& ws, T* F, const BatchShifts& s
                            lv.ea_total[k], sh, st);
       pf.end(a, P_EXTEND, st, 0.0, nb * lv.ea_elems[k] * es);
     }
+    if (ws.rns.planes) {
+      RnsScratch sc = ws.rns;
+      sc.fail = ws.ozfail + (count ? 1 : 0);
+      for (int p0 = 0; p0 < lv.max_s; p0 += rns_block(b)) {
+        int nact = 0;
+        while (nact < int(lv.s.size()) && lv.s[nact] > p0) ++nact;
+        rns_factor_block<T>(sc, F, reinterpret_cast<T*>(ws.Y), fr, dfr, lv.s.data(), lv.m.data(), nact, p0, b, sh, status, count, pf, st);
+      }
+      continue;
+    }
     for (int p0 = 0; p0 < lv.max_s; p0 += b) {
       PanelGeom g = panel_geom(lv, p0, b);
       PanelWork w = pf.on ? panel_work(lv, p0, b, es, fl) : PanelWork();
@@ -389,6 +433,16 @@ void selinv_batch(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh, Pro
       a = pf.begin(st);
       launch_oz_rowmax_init(ws.Y, fr, dfr, int(lv.fronts.size()), max_m, split_scratch(p, ws, false), sh.nb, st);
       pf.end(a, P_SLICE, st, 0.0, nb * lv.gather_bytes);
+    }
+    if (ws.rns.planes) {
+      RnsScratch sc = ws.rns;
+      sc.fail = ws.ozfail;
+      for (int p0 = (lv.max_s - 1) / rns_block(b) * rns_block(b); p0 >= 0; p0 -= rns_block(b)) {
+        int nact = 0;
+        while (nact < int(lv.s.size()) && lv.s[nact] > p0) ++nact;
+        rns_selinv_block(sc, ws.Y, ws.F, fr, dfr, lv.s.data(), lv.m.data(), nact, p0, b, sh.nb, pf, st);
+      }
+      continue;
     }
     int last = ((lv.max_s - 1) / b) * b;
     for (int p0 = last; p0 >= 0; p0 -= b) {
@@ -516,12 +570,21 @@ void factor_selinv(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh, Pr
   ck(cudaGraphLaunch(g.exec, ws.stream), "cudaGraphLaunch");
 }
 
+// The scaling exponents of the values H and S (plans and workspaces with
+// residue products; wide: 1 real, 2 complex values).
+void set_scales(const pexsi_plan* p, Workspace& ws, const double* dH, const double* dS, int wide = 1, size_t q = 0) {
+  if (!ws.gs) return;
+  const int64_t e0 = p->sys_entry_off[q], ne = p->sys_entry_off[q + 1] - e0;
+  launch_rns_scales(dH, dS, wide, p->d_diag, p->sys_col_off[q], p->sys_col_off[q + 1] - p->sys_col_off[q], p->d_row,
+                    p->d_col, e0, ne, ws.g, ws.gs, ws.stream);
+}
+
 void run_complex_batch(const pexsi_plan* p, Workspace& ws, const double* dH, const double* dS, const BatchShifts& sh,
                        Profiler& pf) {
   const int64_t pool = p->sym.front_elems;
   ck(cudaMemsetAsync(ws.F, 0, sizeof(double2) * size_t(pool) * sh.nb, ws.stream), "memset(F)");
   cudaEvent_t a = pf.begin(ws.stream);
-  launch_assemble<double2>(ws.F, dH, dS, p->d_asm_src, p->d_asm_pos, p->nlow, pool, sh, ws.stream);
+  launch_assemble<double2>(ws.F, dH, dS, p->d_asm_src, p->d_asm_pos, p->nlow, pool, sh, ws.gs, ws.stream);
   pf.end(a, P_ASSEMBLE, ws.stream, 0.0, double(p->nlow) * (32.0 + 16.0 * sh.nb));
   factor_selinv(p, ws, sh, pf);
 }
@@ -545,6 +608,7 @@ int dm_range(const pexsi_plan* p, Workspace& ws, Profiler* prof, const double* d
   // them (info != NULL) reports a breakdown or a timed-out wait of any batch
   // of the chain.
   if (!accumulate) reset_status(ws, 0);
+  set_scales(p, ws, dH, S);
   bool first = true;
   for (int b0 = begin; b0 < end; b0 += ws.batch) {
     int nb = std::min(ws.batch, end - b0);
@@ -559,7 +623,7 @@ int dm_range(const pexsi_plan* p, Workspace& ws, Profiler* prof, const double* d
     int overwrite = (first && !accumulate) ? 1 : 0;
     cudaEvent_t a = pf.begin(st);
     launch_pole_sum(ws.Y, p->sym.front_elems, p->d_entry_pos, p->sym.nnz, sh, overwrite, d_dm, d_edm, d_fdm, d_ddm,
-                    st);
+                    ws.gs, st);
     int nout = 1 + (d_dm ? 1 : 0) + (d_edm ? 1 : 0) + (d_fdm ? 1 : 0);
     pf.end(a, P_POLESUM, st, 6.0 * nout * nb * double(p->sym.nnz),
            double(p->sym.nnz) * (8.0 + 16.0 * nb + 8.0 * nout * (overwrite ? 1 : 2)));
@@ -590,7 +654,7 @@ int dm_range(const pexsi_plan* p, Workspace& ws, Profiler* prof, const double* d
   info->gemm_flops = (p->flops.factor_gemm + p->flops.selinv_gemm) * (end - begin);
   info->n_poles = end - begin;
   info->breakdown_front = brk == INT_MAX ? -1 : brk;
-  if (split_failed(ws, 0, err, "split-precision GEMM")) return PEXSI_ERR_TIMEOUT;
+  if (split_failed(ws, 0, err, "tensor-core GEMM")) return PEXSI_ERR_TIMEOUT;
   if (brk != INT_MAX) {
     *err = "zero or tiny pivot in front " + std::to_string(brk);
     return PEXSI_ERR_BREAKDOWN;
@@ -611,6 +675,7 @@ int inertia_range(const pexsi_plan* p, Workspace& ws, Profiler* prof, const doub
   std::vector<std::complex<double>> z(n_shifts);
   for (int t = 0; t < n_shifts; ++t) z[t] = {shifts[t], 0.0};
   int brk_all = INT_MAX;
+  set_scales(p, ws, dH, S);  // a congruence: the counts are the same
   for (int b0 = 0; b0 < n_shifts; b0 += cap) {
     int nb = std::min(cap, n_shifts - b0);
     BatchShifts sh = make_shifts(z, nullptr, nullptr, nullptr, b0, nb);
@@ -618,7 +683,7 @@ int inertia_range(const pexsi_plan* p, Workspace& ws, Profiler* prof, const doub
     ck(cudaMemsetAsync(ws.neg, 0, sizeof(int) * kMaxBatch, st), "status");
     ck(cudaMemsetAsync(F, 0, sizeof(double) * size_t(pool) * nb, st), "memset(F)");
     cudaEvent_t a = pf.begin(st);
-    launch_assemble<double>(F, dH, S, p->d_asm_src, p->d_asm_pos, p->nlow, pool, sh, st);
+    launch_assemble<double>(F, dH, S, p->d_asm_src, p->d_asm_pos, p->nlow, pool, sh, ws.gs, st);
     pf.end(a, P_ASSEMBLE, st, 0.0, double(p->nlow) * (32.0 + 8.0 * nb));
     factor_batch<double>(p, ws, F, sh, true, pf);
     int neg[kMaxBatch];
@@ -628,7 +693,7 @@ int inertia_range(const pexsi_plan* p, Workspace& ws, Profiler* prof, const doub
     ck(cudaStreamSynchronize(st), "sync");
     for (int t = 0; t < nb; ++t) counts[b0 + t] = neg[t];
     brk_all = std::min(brk_all, brk);
-    if (split_failed(ws, 1, err, "split-precision GEMM (inertia)")) return PEXSI_ERR_TIMEOUT;
+    if (split_failed(ws, 1, err, "tensor-core GEMM (inertia)")) return PEXSI_ERR_TIMEOUT;
   }
   if (brk_all != INT_MAX) {
     *err = "zero or tiny pivot in front " + std::to_string(brk_all);
@@ -642,13 +707,14 @@ int selinv_one(const pexsi_plan* p, Workspace& ws, const double* dH, const doubl
   std::vector<std::complex<double>> z{{z_re, z_im}};
   BatchShifts sh = make_shifts(z, nullptr, nullptr, nullptr, 0, 1);
   reset_status(ws, 0);
+  set_scales(p, ws, dH, dS ? dS : p->d_ident);
   run_complex_batch(p, ws, dH, dS ? dS : p->d_ident, sh, g_off);
-  launch_extract(ws.Y, p->d_entry_pos, p->sym.nnz, d_ainv, ws.stream);
+  launch_extract(ws.Y, p->d_entry_pos, p->sym.nnz, d_ainv, ws.gs, ws.stream);
   ck(cudaGetLastError(), "extract");
   int brk = INT_MAX;
   ck(cudaMemcpyAsync(&brk, ws.brk, sizeof(int), cudaMemcpyDeviceToHost, ws.stream), "status");
   ck(cudaStreamSynchronize(ws.stream), "sync");
-  if (split_failed(ws, 0, err, "split-precision GEMM")) return PEXSI_ERR_TIMEOUT;
+  if (split_failed(ws, 0, err, "tensor-core GEMM")) return PEXSI_ERR_TIMEOUT;
   if (brk != INT_MAX) {
     *err = "zero or tiny pivot in front " + std::to_string(brk);
     return PEXSI_ERR_BREAKDOWN;
@@ -852,7 +918,7 @@ int selinv_one_herm(const pexsi_plan* p, Workspace& ws, const double2* dH, const
   BatchShifts sh = make_shifts(z, nullptr, nullptr, nullptr, 0, 1);
   reset_status(ws, 0);
   run_gen_batch(p, ws, dH, dS ? dS : p->d_ident_c, sh, false, true, g_off);
-  launch_extract(ws.Y, p->d_pos_full, p->sym.nnz, d_ainv, ws.stream);
+  launch_extract(ws.Y, p->d_pos_full, p->sym.nnz, d_ainv, nullptr, ws.stream);
   ck(cudaGetLastError(), "extract");
   int brk = INT_MAX;
   ck(cudaMemcpyAsync(&brk, ws.brk, sizeof(int), cudaMemcpyDeviceToHost, ws.stream), "status");
@@ -941,6 +1007,7 @@ int dm_range_group(const pexsi_plan* p, Workspace& ws, Profiler* prof, int wave,
   wave = std::max(1, std::min(wave > 0 ? wave : ws.batch, ws.batch));
   if (info) ck(cudaEventRecord(ws.ev0, st), "event");
   if (!accumulate) reset_status(ws, 0);
+  for (int q = 0; q < nsys; ++q) set_scales(p, ws, dH[q], dS[q] ? dS[q] : p->d_ident + p->sys_entry_off[q], 1, q);
   bool first = true;
   for (int b0 = begin; b0 < end; b0 += wave) {
     const int nb = std::min(wave, end - b0);
@@ -951,7 +1018,8 @@ int dm_range_group(const pexsi_plan* p, Workspace& ws, Profiler* prof, int wave,
       const int64_t a0 = p->sys_asm_off[q], na = p->sys_asm_off[q + 1] - a0;
       const double* S = dS[q] ? dS[q] : p->d_ident + p->sys_entry_off[q];
       cudaEvent_t a = pf.begin(st);
-      launch_assemble<double2>(ws.F, dH[q], S, p->d_asm_src + a0, p->d_asm_pos + a0, na, pool, sh[q], st);
+      launch_assemble<double2>(ws.F, dH[q], S, p->d_asm_src + a0, p->d_asm_pos + a0, na, pool, sh[q],
+                               ws.gs ? ws.gs + p->sys_entry_off[q] : nullptr, st);
       pf.end(a, P_ASSEMBLE, st, 0.0, double(na) * (32.0 + 16.0 * nb));
     }
     factor_selinv(p, ws, sh[0], pf);
@@ -960,7 +1028,7 @@ int dm_range_group(const pexsi_plan* p, Workspace& ws, Profiler* prof, int wave,
       const int64_t e0 = p->sys_entry_off[q], ne = p->sys_entry_off[q + 1] - e0;
       cudaEvent_t a = pf.begin(st);
       launch_pole_sum(ws.Y, pool, p->d_entry_pos + e0, ne, sh[q], overwrite, d_dm[q], d_edm[q], d_fdm[q],
-                      ws.out + 3 * nnz_all + e0, st);
+                      ws.out + 3 * nnz_all + e0, ws.gs ? ws.gs + e0 : nullptr, st);
       pf.end(a, P_POLESUM, st, 24.0 * nb * double(ne), double(ne) * (8.0 + 16.0 * nb + 32.0 * (overwrite ? 1 : 2)));
     }
     first = false;
@@ -993,7 +1061,7 @@ int dm_range_group(const pexsi_plan* p, Workspace& ws, Profiler* prof, int wave,
     in.n_poles = end - begin;
     in.breakdown_front = bsys == q ? brk - f_off[q] : -1;
   }
-  if (split_failed(ws, 0, err, "split-precision GEMM")) return PEXSI_ERR_TIMEOUT;
+  if (split_failed(ws, 0, err, "tensor-core GEMM")) return PEXSI_ERR_TIMEOUT;
   if (brk != INT_MAX) {
     *err = "zero or tiny pivot in front " + std::to_string(brk - f_off[bsys]) + " of system " + std::to_string(bsys);
     return PEXSI_ERR_BREAKDOWN;
@@ -1012,7 +1080,7 @@ void free_plan_device(pexsi_plan* p) {
                   p->d_entry_pos, p->d_level_fronts, p->d_ea, p->d_tile_pref, p->d_part_off, p->d_ident,
                   p->d_ozA_off, p->d_ozB_off, p->d_exA_off, p->d_exB_off, p->d_ozA_off_r, p->d_ozB_off_r,
                   p->d_ymax_off, p->d_pos_full, p->d_pos_t, p->d_ident_c, p->d_hH, p->d_hS, p->d_hout,
-                  p->d_col0, p->d_bk_slots};
+                  p->d_col0, p->d_bk_slots, p->d_diag, p->d_row, p->d_col};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   cudaStream_t st = p->ws.stream;
@@ -1170,11 +1238,11 @@ int ensure_workspace(pexsi_plan* p) {
   size_t free_b = 0, total_b = 0;
   ck(cudaMemGetInfo(&free_b, &total_b), "cudaMemGetInfo");
   int64_t budget = p->opts.hbm_budget > 0 ? p->opts.hbm_budget : int64_t(0.6 * double(free_b));
-  int64_t nb = (budget - bytes_fixed(p)) / std::max<int64_t>(bytes_per_pole(p), 1);
-  if (p->opts.max_batch > 0) nb = std::min<int64_t>(nb, p->opts.max_batch);
-  nb = std::min<int64_t>(nb, kMaxBatch);
+  int64_t planes, out;
+  const int most = p->opts.max_batch > 0 ? std::min(p->opts.max_batch, kMaxBatch) : kMaxBatch;
+  const int nb = fit_batch(p, budget, most, planes, out);
   if (nb < 1) return fail(p, PEXSI_ERR_NOMEM, "device workspace for one pole exceeds the HBM budget");
-  workspace_alloc(p, p->ws, int(nb), p->ws.stream, false);
+  workspace_alloc(p, p->ws, nb, planes, out, p->ws.stream, false);
   return PEXSI_OK;
 }
 
@@ -1209,6 +1277,7 @@ int upload_plan(pexsi_plan* p) {
   ck(cudaSetDevice(p->opts.device), "cudaSetDevice");
   ck(configure_kernels(p->b), "cudaFuncSetAttribute");
   if (p->oz_slices > 0) ck(oz_configure(p->oz_slices), "cudaFuncSetAttribute(split)");
+  else ck(rns_configure(), "cudaFuncSetAttribute(residues)");
   const Symbolic& S = p->sym;
   std::vector<int32_t> hs(S.nsuper), hm(S.nsuper);
   for (int32_t K = 0; K < S.nsuper; ++K) { hs[K] = S.s(K); hm[K] = S.m(K); }
@@ -1282,6 +1351,14 @@ int upload_plan(pexsi_plan* p) {
     std::vector<double> ident(S.nnz, 0.0);  // S = I on the pattern
     for (int64_t e : p->diag_entries) ident[e] = 1.0;
     p->d_ident = dev_upload(ident);
+  }
+  if (p->sys_col_off.empty()) p->sys_col_off = {0, S.n};
+  if (p->oz_slices == 0) {
+    std::vector<int32_t> col(S.nnz);
+    for (int64_t c = 0; c < S.n; ++c) std::fill(col.begin() + p->col_start[c], col.begin() + p->col_start[c + 1], int32_t(c));
+    p->d_diag = dev_upload(p->diag_entries);
+    p->d_row = dev_upload(p->entry_row);
+    p->d_col = dev_upload(col);
   }
   ck(cudaStreamCreateWithFlags(&p->ws.stream, cudaStreamNonBlocking), "cudaStreamCreate");
   return PEXSI_OK;
@@ -1447,6 +1524,8 @@ int pexsi_setup(int64_t n, const int64_t* colptr, const int32_t* rowind, const i
     for (int64_t j = 0; j < n; ++j)
       for (int64_t e = colptr[j]; e < colptr[j + 1]; ++e)
         if (rowind[e] == j) p->diag_entries.push_back(e);
+    p->entry_row.assign(rowind, rowind + colptr[n]);
+    p->col_start.assign(colptr, colptr + n + 1);
     if (p->opts.device < 0) {  // host-only plan: symbolic analysis only
       *out = p;
       return PEXSI_OK;
@@ -1829,12 +1908,18 @@ int pexsi_group_create(const pexsi_plan* const* plans, int32_t n_plans, const pe
     p->sym = merge_symbolic(parts);
     p->flops = count_flops(p->sym, p->b);
     p->sys_entry_off.assign(1, 0);
+    p->sys_col_off.assign(1, 0);
     g->f_off.assign(1, 0);
     for (int q = 0; q < n_plans; ++q) {
       for (int64_t e : plans[q]->diag_entries) p->diag_entries.push_back(e + p->sys_entry_off.back());
+      for (int32_t r : plans[q]->entry_row) p->entry_row.push_back(r + int32_t(p->sys_col_off.back()));
+      for (int64_t c = 0; c < plans[q]->sym.n; ++c)
+        p->col_start.push_back(plans[q]->col_start[c] + p->sys_entry_off.back());
+      p->sys_col_off.push_back(p->sys_col_off.back() + plans[q]->sym.n);
       p->sys_entry_off.push_back(p->sys_entry_off.back() + plans[q]->sym.nnz);
       g->f_off.push_back(g->f_off.back() + plans[q]->sym.nsuper);
     }
+    p->col_start.push_back(p->sys_entry_off.back());
     rc = upload_plan(p);
     if (rc == PEXSI_OK) rc = ensure_workspace(p);
     if (rc) {

@@ -303,13 +303,20 @@ __device__ __forceinline__ void zero_acc(T (&acc)[4][4]) {
 }
 
 // ------------------------------------------------------------ assembly
+// 2^-g of entry e of a plan whose rows and columns are scaled (gs: sum of the
+// two exponents per CSC entry; NULL: no scaling), |g| <= 1022.
+__device__ __forceinline__ double entry_scale(const int16_t* __restrict__ gs, int64_t e) {
+  return gs ? __hiloint2double((1023 - int(gs[e])) << 20, 0) : 1.0;
+}
+
 template <typename T>
 __global__ void k_assemble(T* __restrict__ F, const double* __restrict__ H, const double* __restrict__ S,
                            const int64_t* __restrict__ src, const int64_t* __restrict__ pos, int64_t nlow,
-                           int64_t pool, BatchShifts sh) {
+                           int64_t pool, BatchShifts sh, const int16_t* __restrict__ gs) {
   for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < nlow; t += int64_t(gridDim.x) * blockDim.x) {
     int64_t e = src[t], p = pos[t];
-    double h = H[e], s = S[e];
+    const double sc = entry_scale(gs, e);
+    double h = H[e] * sc, s = S[e] * sc;
     for (int b = 0; b < sh.nb; ++b) F[b * pool + p] = make_shift<T>(h, s, sh, b);
   }
 }
@@ -1176,7 +1183,8 @@ __global__ void k_selinv_diag_reduce(double2* __restrict__ Y, const double2* __r
 // ------------------------------------------------------------ pole sum
 __global__ void k_pole_sum(const double2* __restrict__ Y, int64_t pool, const int64_t* __restrict__ entry_pos,
                            int64_t nnz, BatchShifts sh, int overwrite, double* __restrict__ dm,
-                           double* __restrict__ edm, double* __restrict__ fdm, double* __restrict__ ddm) {
+                           double* __restrict__ edm, double* __restrict__ fdm, double* __restrict__ ddm,
+                           const int16_t* __restrict__ gs) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t p = entry_pos[e];
     double a = 0.0, ae = 0.0, af = 0.0, ad = 0.0;
@@ -1188,6 +1196,11 @@ __global__ void k_pole_sum(const double2* __restrict__ Y, int64_t pool, const in
       af = fma(sh.wf_re[b], v.y, fma(sh.wf_im[b], v.x, af));
       ad = fma(sh.wd_re[b], v.y, fma(sh.wd_im[b], v.x, ad));
     }
+    const double sc = entry_scale(gs, e);
+    a *= sc;
+    ae *= sc;
+    af *= sc;
+    ad *= sc;
     if (dm) dm[e] = overwrite ? a : dm[e] + a;
     if (edm) edm[e] = overwrite ? ae : edm[e] + ae;
     if (fdm) fdm[e] = overwrite ? af : fdm[e] + af;
@@ -1238,15 +1251,15 @@ __global__ void k_pole_sum_herm(const double2* __restrict__ Y, int64_t pool, con
 }
 
 __global__ void k_extract(const double2* __restrict__ Y, const int64_t* __restrict__ entry_pos, int64_t nnz,
-                          double2* __restrict__ out) {
+                          double2* __restrict__ out, const int16_t* __restrict__ gs) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x)
-    out[e] = Y[entry_pos[e]];
+    out[e] = scalev(Y[entry_pos[e]], entry_scale(gs, e));
 }
 
 __global__ void k_scaled_imag(const double2* __restrict__ Y, const int64_t* __restrict__ entry_pos, int64_t nnz,
-                              double scale, double* __restrict__ out) {
+                              double scale, double* __restrict__ out, const int16_t* __restrict__ gs) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x)
-    out[e] = scale * Y[entry_pos[e]].y;
+    out[e] = scale * (Y[entry_pos[e]].y * entry_scale(gs, e));
 }
 
 __global__ void k_trace_partial(const double* dm, const double* edm, const double* fdm, const double* ddm,
@@ -1291,8 +1304,8 @@ inline int grid_for(int64_t n, int threads) {
 // ------------------------------------------------------------ launchers
 template <typename T>
 void launch_assemble(T* F, const double* H, const double* S, const int64_t* src, const int64_t* pos, int64_t nlow,
-                     int64_t pool, const BatchShifts& sh, cudaStream_t st) {
-  k_assemble<T><<<grid_for(nlow, 256), 256, 0, st>>>(F, H, S, src, pos, nlow, pool, sh);
+                     int64_t pool, const BatchShifts& sh, const int16_t* gs, cudaStream_t st) {
+  k_assemble<T><<<grid_for(nlow, 256), 256, 0, st>>>(F, H, S, src, pos, nlow, pool, sh, gs);
 }
 
 template <typename T>
@@ -1408,17 +1421,19 @@ void launch_selinv_diag_reduce(double2* Y, const double2* F, const double2* part
 }
 
 void launch_pole_sum(const double2* Y, int64_t pool, const int64_t* entry_pos, int64_t nnz, const BatchShifts& sh,
-                     int overwrite, double* dm, double* edm, double* fdm, double* ddm, cudaStream_t st) {
-  k_pole_sum<<<grid_for(nnz, 256), 256, 0, st>>>(Y, pool, entry_pos, nnz, sh, overwrite, dm, edm, fdm, ddm);
+                     int overwrite, double* dm, double* edm, double* fdm, double* ddm, const int16_t* gs,
+                     cudaStream_t st) {
+  k_pole_sum<<<grid_for(nnz, 256), 256, 0, st>>>(Y, pool, entry_pos, nnz, sh, overwrite, dm, edm, fdm, ddm, gs);
 }
 
-void launch_extract(const double2* Y, const int64_t* entry_pos, int64_t nnz, double2* out, cudaStream_t st) {
-  k_extract<<<grid_for(nnz, 256), 256, 0, st>>>(Y, entry_pos, nnz, out);
+void launch_extract(const double2* Y, const int64_t* entry_pos, int64_t nnz, double2* out, const int16_t* gs,
+                    cudaStream_t st) {
+  k_extract<<<grid_for(nnz, 256), 256, 0, st>>>(Y, entry_pos, nnz, out, gs);
 }
 
 void launch_scaled_imag(const double2* Y, const int64_t* entry_pos, int64_t nnz, double scale, double* out,
-                        cudaStream_t st) {
-  k_scaled_imag<<<grid_for(nnz, 256), 256, 0, st>>>(Y, entry_pos, nnz, scale, out);
+                        const int16_t* gs, cudaStream_t st) {
+  k_scaled_imag<<<grid_for(nnz, 256), 256, 0, st>>>(Y, entry_pos, nnz, scale, out, gs);
 }
 
 void launch_traces(const double* dm, const double* edm, const double* fdm, const double* ddm, const double* S,
@@ -1540,7 +1555,7 @@ template void launch_bk_count_all<double2>(const int32_t*, int, const DevFronts&
 
 #define PEXSI_INSTANTIATE(T)                                                                                        \
   template void launch_assemble<T>(T*, const double*, const double*, const int64_t*, const int64_t*, int64_t,    \
-                                   int64_t, const BatchShifts&, cudaStream_t);                                   \
+                                   int64_t, const BatchShifts&, const int16_t*, cudaStream_t);                   \
   template void launch_extend_add<T>(T*, const DevFronts&, const int32_t*, int, const int32_t*, int64_t,        \
                                      const BatchShifts&, cudaStream_t);                                           \
   template void launch_diag_inv<T>(T*, const DevFronts&, const int32_t*, int, int, int, const BatchShifts&,      \

@@ -75,9 +75,11 @@ struct OzScratch {
 };
 
 // ---- launchers (T = double for real inertia, double2 for complex poles) ----
+// gs (per CSC entry, NULL: none): A is assembled as D A D with D = 2^-g per row,
+// and Y is read out as D Y D, 2^-gs[e] per entry (see launch_rns_scales).
 template <typename T>
 void launch_assemble(T* F, const double* H, const double* S, const int64_t* src, const int64_t* pos, int64_t nlow,
-                     int64_t pool, const BatchShifts& sh, cudaStream_t st);
+                     int64_t pool, const BatchShifts& sh, const int16_t* gs, cudaStream_t st);
 
 template <typename T>
 void launch_extend_add(T* F, const DevFronts& fr, const int32_t* children, int nchild, const int32_t* pref,
@@ -113,13 +115,15 @@ void launch_selinv_diag_reduce(double2* Y, const double2* F, const double2* part
                                int b, const BatchShifts& sh, cudaStream_t st);
 
 void launch_pole_sum(const double2* Y, int64_t pool, const int64_t* entry_pos, int64_t nnz, const BatchShifts& sh,
-                     int overwrite, double* dm, double* edm, double* fdm, double* ddm, cudaStream_t st);
+                     int overwrite, double* dm, double* edm, double* fdm, double* ddm, const int16_t* gs,
+                     cudaStream_t st);
 
-void launch_extract(const double2* Y, const int64_t* entry_pos, int64_t nnz, double2* out, cudaStream_t st);
+void launch_extract(const double2* Y, const int64_t* entry_pos, int64_t nnz, double2* out, const int16_t* gs,
+                    cudaStream_t st);
 
 // out[e] = scale * Im Y[entry_pos[e]] (the LDOS matrix from one selected inverse).
 void launch_scaled_imag(const double2* Y, const int64_t* entry_pos, int64_t nnz, double scale, double* out,
-                        cudaStream_t st);
+                        const int16_t* gs, cudaStream_t st);
 
 // Split-precision Takahashi step Y[S,P] = -Y[S,S] L[S,P] and its mirror, with
 // A = Y[S,S] sliced on the fly inside the GEMM: prep = true computes the row

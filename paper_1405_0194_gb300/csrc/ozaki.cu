@@ -60,6 +60,7 @@
 #include <cuda_bf16.h>
 
 #include "kernels.cuh"
+#include "tensor_core.cuh"
 
 namespace pexsi {
 namespace {
@@ -75,112 +76,6 @@ constexpr int kSlotsB = 2;    // B ring: all S slices of one K tile per slot
 constexpr int kEpiWarps = 8;  // two per TMEM lane quarter, 32 columns each
 constexpr int kGemmThreads = (kEpiWarps + 2) * 32;  // + producer warp + MMA warp
 constexpr int kNanExp = 0x7FFF;                     // exponent marker of a row holding Inf or NaN
-constexpr uint64_t kWaitNs = 1000000000ull;         // 1 s per wait
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// Shared-memory matrix descriptor, no swizzle, K-major: LBO = 128 B between
-// core matrices along K, SBO = 512 B between 8-row groups, version 1.
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  return uint64_t((saddr & 0x3FFFF) >> 4) | (uint64_t(128 >> 4) << 16) | (uint64_t(512 >> 4) << 32) |
-         (uint64_t(1) << 46);
-}
-
-// The same for 16-deep K tiles: SBO = 256 B.
-__device__ __forceinline__ uint64_t sdesc16(uint32_t saddr) {
-  return uint64_t((saddr & 0x3FFFF) >> 4) | (uint64_t(128 >> 4) << 16) | (uint64_t(256 >> 4) << 32) |
-         (uint64_t(1) << 46);
-}
-
-// Instruction descriptor, kind::f16: D f32, A and B bf16, both K-major,
-// M = 128, N = 64 g; optionally B negated.
-__host__ __device__ constexpr uint32_t idesc(int g, bool negate_b) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (negate_b ? (1u << 14) : 0u) | (uint32_t(64 * g >> 3) << 17) |
-         (uint32_t(128 >> 4) << 24);
-}
-
-__device__ __forceinline__ bool bar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Bounded wait (budget_ns of wall time, the plan's wait bound) for the
-// completion of the barrier phase of the given parity; gives up early once
-// another role has recorded a failure.
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, const volatile int* fail, uint64_t budget_ns) {
-  if (bar_try(bar, parity)) return true;
-  const uint64_t t0 = global_ns();
-  for (uint32_t it = 1;; ++it) {
-    if (bar_try(bar, parity)) return true;
-    if (*fail) return false;
-    if ((it & 255u) == 0 && global_ns() - t0 > budget_ns) return false;
-  }
-}
-
-// Bounded wait that ignores failures (draining own copies / MMAs in flight):
-// always the full second, whatever the plan's wait bound, since what it
-// waits for was issued and completes on its own.
-__device__ __forceinline__ bool bar_wait_all(uint32_t bar, uint32_t parity) {
-  if (bar_try(bar, parity)) return true;
-  const uint64_t t0 = global_ns();
-  for (uint32_t it = 1;; ++it) {
-    if (bar_try(bar, parity)) return true;
-    if ((it & 255u) == 0 && global_ns() - t0 > kWaitNs) return false;
-  }
-}
-
-__device__ __forceinline__ void bar_init(uint32_t bar, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-
-__device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void bar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-
-__device__ __forceinline__ void mma(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t id, uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-          tmem_d),
-      "l"(a), "l"(b), "r"(id), "r"(accumulate));
-}
-
-// Arrives on `bar` once every tcgen05.mma this thread issued so far is done.
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// Descriptor d moved by off 16-byte units: the start address field is the
-// low 14 bits and shared-memory addresses stay below 2^18, so the low word
-// takes the add without a carry.
-__device__ __forceinline__ uint64_t desc_off(uint64_t d, uint32_t off) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(uint32_t(d) + off), "r"(uint32_t(d >> 32)));
-  return r;
-}
-
 // Products of one slice of A with the B slices T0 + 1 .. T0 + G of a K tile
 // (KSTEPS steps of 16): the G slices of Br (and of Bi) are consecutive 64-row
 // blocks of BLK bytes, and the accumulators of their diagonals consecutive
@@ -230,34 +125,6 @@ __device__ __forceinline__ void mma_slice(int c, uint32_t acc, uint64_t a1, uint
       mma_group<CPLX, KSTEPS, BLK, 0, 1>(acc, a1, a2, br, bi, first);
       break;
   }
-}
-
-// 32 lanes x 8 consecutive TMEM columns, without the wait: tcgen05.wait::ld
-// before any register is read.
-__device__ __forceinline__ void tmem_ld8_nw(uint32_t addr, uint32_t (&v)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-               : "r"(addr));
-}
-
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// 32 lanes x 16 consecutive TMEM columns, without the wait.
-__device__ __forceinline__ void tmem_ld16_nw(uint32_t addr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(addr));
-}
-
-__device__ __forceinline__ void tmem_st16(uint32_t addr, const uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
-          addr),
-      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
-      "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
-      : "memory");
 }
 
 // w_c += v_c 2^sh on the 64-bit integers w_c = (w[2c + 1], w[2c]), c < 8,
@@ -324,18 +191,6 @@ __device__ __forceinline__ void acc_add_diags8(uint32_t (&w)[16], const uint32_t
     w[2 * c] = uint32_t(a64);
     w[2 * c + 1] = uint32_t(a64 >> 32);
   }
-}
-
-__device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t* v) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
-      "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-        "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(addr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;");
 }
 
 // The integer X nearest to x 2^(7 S - e) (|x| < 2^e, so |X| <= 2^(7 S)),
@@ -670,13 +525,6 @@ __global__ void __launch_bounds__(256) k_oz_slice_real(double* __restrict__ F, D
     uint8_t* p = rowbase + int64_t(o >> 2) * S * slice + (o & 3) * 128;
     with_slices(S, [&](auto SC) { store_slices_r<decltype(SC)::value>(Y, p, slice); });
   }
-}
-
-// Where a wait ran out: site (1..8) + 16 * (K tile mod 16), below 256; the
-// launch reports 1 + (mode << 28) + (this << 20) + CTA index, mode 1-3 for the
-// short-K GEMM (its MODE), 0 for the Takahashi / Y[P,P] kernel.
-__device__ __forceinline__ void record_fail(int* s_fail, int site, int kt) {
-  atomicCAS(s_fail, 0, site + 16 * (kt & 15));
 }
 
 // ---------------------------------------------------------------- GEMM (short K)

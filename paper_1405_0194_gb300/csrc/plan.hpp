@@ -13,6 +13,7 @@
 
 #include "../../include/pexsi_gb300.h"
 #include "kernels.cuh"
+#include "rns.cuh"
 #include "symbolic.hpp"
 
 namespace pexsi {
@@ -104,6 +105,9 @@ struct Workspace {
   uint8_t *ozA = nullptr, *ozB = nullptr;  // split-precision slice tiles
   int *exA = nullptr, *exB = nullptr, *ozfail = nullptr;
   uint32_t* ymax = nullptr;  // split path: row maxima of Y per pole
+  RnsScratch rns;            // FP64 path: scratch of the residue products (no planes: DFMA kernels)
+  int32_t* g = nullptr;      // its power-of-two scaling: exponent per row, and per CSC entry of the current H and S
+  int16_t* gs = nullptr;
   cudaStream_t stream = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // captured level schedules (factorisation + selected inversion of nb
@@ -163,10 +167,14 @@ struct pexsi_plan {
   int32_t *d_col0 = nullptr, *d_bk_slots = nullptr;  // first column per front; (front, p0) of every panel
   int32_t n_bk_slots = 0;
   std::vector<int64_t> diag_entries;  // CSC entries on the diagonal
+  std::vector<int32_t> entry_row;     // row of every CSC entry, and the column bounds, both of this plan's matrix
+  std::vector<int64_t> col_start;
+  int64_t* d_diag = nullptr;          // FP64 plans: the diagonal entry of every column, the row and column of every entry
+  int32_t *d_row = nullptr, *d_col = nullptr;
   // A plan that merges several systems (pexsi_group): the first CSC entry of
   // each system among the concatenated entries (nsys + 1), and each system's
-  // range of the assembly list; {0, nnz} and {0, nlow} for a single system.
-  std::vector<int64_t> sys_entry_off, sys_asm_off;
+  // range of the assembly list and its columns; {0, nnz}, {0, nlow} and {0, n} for a single system.
+  std::vector<int64_t> sys_entry_off, sys_asm_off, sys_col_off;
   double2 *d_ident_c = nullptr, *d_hH = nullptr, *d_hS = nullptr, *d_hout = nullptr;
 
   pexsi::DevFronts fronts() const {
@@ -184,13 +192,36 @@ struct pexsi_plan {
 
 namespace pexsi {
 
-// Bytes of workspace one pole adds (F and Y fronts + partials).
-int64_t bytes_per_pole(const pexsi_plan* p);
+// Bytes of workspace one pole adds (F and Y fronts + partials); rns: with the
+// residue products' scratch, which replaces the DFMA kernels' split-K partials.
+int64_t bytes_per_pole(const pexsi_plan* p, bool rns);
 // Fixed bytes of a workspace (staging + status + trace scratch).
 int64_t bytes_fixed(const pexsi_plan* p);
 
-// Allocates ws for `batch` poles on `stream` (cudaMallocAsync when async).
-void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, cudaStream_t stream, bool async);
+// Residue scratch of FP64 plans (rns.cu): planes for `batch` poles, at most
+// `most` bytes unless the largest front needs more, and the output tiles; both
+// 0 for split-precision plans.
+void rns_scratch(const pexsi_plan* p, int batch, int64_t most, int64_t& planes, int64_t& out);
+void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& want);
+int64_t rns_out_bytes(const pexsi_plan* p, int batch);
+constexpr int64_t kRnsPlaneBytes = int64_t(2) << 30;  // default of `most`
+
+// The largest batch (at most `most`) whose workspace fits the budget, with
+// residue scratch where that fits too (planes, out; 0 without); 0: none fits.
+int fit_batch(const pexsi_plan* p, int64_t budget, int most, int64_t& planes, int64_t& out);
+
+template <typename T>
+void rns_factor_block(const RnsScratch& sc, T* F, T* Y, const DevFronts& fr, const int32_t* dfr, const int32_t* s,
+                      const int32_t* m, int nact, int p0, int b, const BatchShifts& sh, DevStatus status, bool count,
+                      Profiler& pf, cudaStream_t st);
+void rns_selinv_block(const RnsScratch& sc, double2* Y, double2* F, const DevFronts& fr, const int32_t* dfr,
+                      const int32_t* s, const int32_t* m, int nact, int p0, int b, int nb, Profiler& pf,
+                      cudaStream_t st);
+
+// Allocates ws for `batch` poles on `stream` (cudaMallocAsync when async),
+// with residue scratch of the given sizes (0: none).
+void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, int64_t rns_planes, int64_t rns_out,
+                     cudaStream_t stream, bool async);
 void workspace_free(Workspace& ws);
 
 // Poles [begin, end) of the P-pole table into d_dm/d_edm/d_fdm (device, any

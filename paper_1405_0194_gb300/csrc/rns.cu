@@ -1,0 +1,1199 @@
+// FP64 supernode products on the tcgen05 tensor cores in a residue number
+// system (the Chinese-remainder form of the Ozaki scheme: Ozaki, Uchino and
+// Imamura 2025), FP64 in and out.
+//
+// Why: an SM issues 2 FP64 multiply-adds per clock (1.26 TFLOP/s on the chip,
+// DMMA no faster), its bf16 tensor cores 4096. Each operand row is scaled by a
+// power of two above its 2-norm and rounded to integers of 58 bits; the
+// integers' residues modulo 15 pairwise coprime moduli p <= 256 are exact in
+// bf16 (|r| <= 128), so the product modulo every p is one bf16 GEMM whose FP32
+// accumulators hold exact integers (2 x 480 products of at most 2^14 stay
+// below 2^24), and the 15 residues give the exact integer product (below
+// 2^116, half the product of the moduli is 2^116.4) by the remainder theorem.
+// The only errors are the rounding of the operands (2^-59 of the row norms,
+// against the 2^-53 of each FP64 multiply-add) and of the result. A complex
+// product costs 15 x 4 bf16 multiply-adds per complex multiply-add, against
+// 45 x 4 for bf16 slices of the same accuracy (9 slices of 7 bits).
+//
+// Three kernels per product C = A B^T of rows of A (the N operand of the MMA:
+// rows of the front) and rows of B (the M operand: panel columns):
+//   k_rns_conv   row norms, integers and residues of an operand (HBM bound:
+//                16 B read, 60 B written per complex entry)
+//   k_rns_gemm   one bf16 GEMM per modulus, residues of C as bytes (tensor
+//                bound)
+//   k_rns_recon  the integers of C, their FP64 values and the update of F or Y
+//                (integer pipe bound: about 130 operations per real entry)
+//
+// The fronts are eliminated in blocks of kRnsBlock = 256 columns (against the
+// panels of the DFMA path): the 256 x 256 diagonal block B is inverted by
+// symmetric sweeps over its panels (k_diag_inv per panel, the rest as residue
+// products), L[S,B] = W[S,B] B^-1 and F[S,S] -= L W^T are one product of K = 256
+// each, and Y[S,B] = -Y[S,S] L[S,B] converts Y[S,S] once per 256 columns.
+#include <algorithm>
+#include <cstdint>
+#include <utility>
+#include <vector>
+
+#include "plan.hpp"
+#include "rns.cuh"
+#include "tensor_core.cuh"
+
+namespace pexsi {
+namespace {
+
+// ------------------------------------------------------------ moduli
+typedef unsigned __int128 u128;
+typedef __int128 i128;
+
+// Pairwise coprime, largest first. 255 is left out: the FP32 quotient by it may
+// round the other way for accumulators near 2^24, and the residue 128 would not
+// fit its byte (256 has an exact reciprocal, and 128 = -128 modulo it).
+__host__ __device__ constexpr int modulus(int l) {
+  constexpr int t[kRnsModuli] = {256, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+  return t[l];
+}
+__host__ __device__ constexpr u128 mod_product() {
+  u128 p = 1;
+  for (int l = 0; l < kRnsModuli; ++l) p *= u128(modulus(l));
+  return p;
+}
+// P / p_l, and its inverse modulo p_l (folded into one operand's residues)
+__host__ __device__ constexpr u128 cofactor(int l) { return mod_product() / u128(modulus(l)); }
+__host__ __device__ constexpr int cofactor_inv(int l) {
+  const int p = modulus(l), c = int(cofactor(l) % u128(p));
+  for (int x = 1; x < p; ++x)
+    if (c * x % p == 1) return x;
+  return 0;
+}
+// residue of 2^(15 j) (times the inverse of the cofactor) in [-p/2, p/2]
+__host__ __device__ constexpr int piece_coef(int l, int j, bool scaled) {
+  const int p = modulus(l);
+  long long r = 1;
+  for (int q = 0; q < 15 * j; ++q) r = r * 2 % p;
+  if (scaled) r = r * cofactor_inv(l) % p;
+  return int(r > p / 2 ? r - p : r);
+}
+// limbs of the cofactors: 20 bits (sums of 15 byte multiples stay below 2^32), then 32, 32 and the rest
+__host__ __device__ constexpr uint32_t limb(u128 v, int j) {
+  return j == 0 ? uint32_t(v & 0xFFFFF) : j == 1 ? uint32_t(v >> 20) : j == 2 ? uint32_t(v >> 52) : uint32_t(v >> 84);
+}
+// The residues are stored as r + 128: minus 128 times the sum of the cofactors' limbs.
+__host__ __device__ constexpr long long limb_bias(int j) {
+  long long s = 0;
+  for (int l = 0; l < kRnsModuli; ++l) s += limb(cofactor(l), j);
+  return -128 * s;
+}
+
+constexpr int kBeta = 58;       // bits of the scaled integers
+constexpr int kNanRow = 0x7FFF; // exponent marker of a row holding Inf or NaN
+constexpr int kK = 32;          // K per staged tile
+constexpr int kPlane = kRnsTile * kK * 2;  // bytes of a 128 x 32 residue tile
+constexpr int kChunkTiles = 15;            // 480 of K: 2 x 480 x 2^14 + 2^7 < 2^24
+constexpr int kStages = 6;
+constexpr int kEpi = 8;                    // epilogue warps: 4 lane quarters x (re, im)
+constexpr int kThreads = (kEpi + 2) * 32;
+static_assert(mod_product() >> 117 == 1, "the bound on the integer products needs 2^117 <= P < 2^118");
+static_assert(2 * kChunkTiles * kK * 128 * 128 + 128 < (1 << 24), "the FP32 accumulators stay exact");
+
+// ------------------------------------------------------------ jobs
+// Products (rows of N x rows of M, contraction K) of one block of panels
+// [p0, p0 + bw), bw = min(rns_block, s - p0), S = the mp rows below it:
+enum Mode {
+  kSweepT,  // T = V D^-1: V = B[:,p] of the diagonal block B, D^-1 = its inverted panel block
+  kSweepU,  // B[R,R] -= T V^T, R = the block's rows outside the panel p
+  kResid,   // R = I - B X, X = the swept inverse, B = the block as it was (kept in Y, which takes R)
+  kRefine,  // X += X R
+  kPanel,   // L[S,B] = W[S,B] B^-1
+  kSchur,   // F[S,S] -= L W^T (lower triangle)
+  kTak,     // Y[S,B] = -Y[S,S] L[S,B] and its mirror
+  kDiag     // Y[B,B] = B^-1 - L[S,B]^T Y[S,B]
+};
+// Operands of k_rns_conv.
+enum Operand { kOpV, kOpD, kOpT, kOpR, kOpW, kOpB, kOpL, kOpLt, kOpY, kOpYt };
+
+struct Job {
+  int mode, nf, np, pole0;   // nf fronts of the level's list, poles pole0 .. pole0 + np - 1
+  int p0, pc, b;             // block start, panel start inside the block (sweeps), panel width
+  int rt0;                   // first row tile of N (a front whose row tiles are taken in pieces)
+  int o0, on;                // output tiles of this launch
+  int kt;                    // K tiles of a slot
+  int64_t slot, n_base, m_base;
+  int pref_n[kRnsFronts + 1], pref_m[kRnsFronts + 1], pref_o[kRnsFronts + 1];
+};
+
+struct Dims {
+  int s, m, bw, q0, mp, pb;
+};
+
+__host__ __device__ __forceinline__ Dims dims_of(int s, int m, int p0, int pc, int b) {
+  Dims d;
+  d.s = s;
+  d.m = m;
+  const int blk = rns_block(b);
+  d.bw = s - p0 < blk ? s - p0 : blk;
+  d.q0 = p0 + d.bw;
+  d.mp = m - d.q0;
+  d.pb = d.bw - pc < b ? d.bw - pc : b;
+  return d;
+}
+
+__host__ __device__ __forceinline__ int tiles128(int n) { return n <= 0 ? 0 : (n + kRnsTile - 1) / kRnsTile; }
+
+// rows of N, rows of M, K of a product; sweeps skip blocks of one panel
+__host__ __device__ __forceinline__ void product_dims(int mode, const Dims& d, int b, int& rn, int& rm, int& k) {
+  switch (mode) {
+    case kSweepT: rn = d.bw > b && d.pb > 0 ? d.bw : 0; rm = rn ? d.pb : 0; k = d.pb; break;
+    case kSweepU: rn = rm = d.bw > b && d.pb > 0 ? d.bw : 0; k = d.pb; break;
+    case kResid: case kRefine: rn = rm = d.bw > b ? d.bw : 0; k = d.bw; break;
+    case kPanel: rn = d.mp; rm = d.mp > 0 ? d.bw : 0; k = d.bw; break;
+    case kSchur: rn = rm = d.mp; k = d.bw; break;
+    case kTak: rn = d.mp; rm = d.mp > 0 ? d.bw : 0; k = d.mp; break;
+    default: rn = rm = d.bw; k = d.mp; break;
+  }
+}
+
+__host__ __device__ __forceinline__ bool triangular(int mode) {
+  return mode == kSweepU || mode == kRefine || mode == kSchur || mode == kDiag;
+}
+
+// largest f with pref[f] <= t
+__device__ __forceinline__ int owner(const int* pref, int n, int t) {
+  int lo = 0, hi = n;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (pref[mid] <= t) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
+struct OutTile {
+  int pole, f, nt, mt;  // pole and front list index of the job, tile of N, tile of M
+};
+
+__device__ __forceinline__ OutTile out_tile(const Job& j, int o) {
+  OutTile t;
+  const int per = j.pref_o[j.nf];
+  t.pole = o / per;
+  const int x = o - t.pole * per;
+  t.f = owner(j.pref_o, j.nf, x);
+  const int y = x - j.pref_o[t.f];
+  if (triangular(j.mode)) {
+    int i = int((sqrtf(8.0f * float(y) + 1.0f) - 1.0f) * 0.5f);
+    while (i * (i + 1) / 2 > y) --i;
+    while ((i + 1) * (i + 2) / 2 <= y) ++i;
+    t.nt = i;
+    t.mt = y - i * (i + 1) / 2;
+  } else {
+    const int mtn = j.pref_m[t.f + 1] - j.pref_m[t.f];
+    t.nt = y / mtn;
+    t.mt = y - t.nt * mtn;
+  }
+  return t;
+}
+
+// ------------------------------------------------------------ conversion
+template <typename F, int... L>
+__device__ __forceinline__ void each_modulus(F&& f, std::integer_sequence<int, L...>) {
+  (f(std::integral_constant<int, L>{}), ...);
+}
+template <typename F>
+__device__ __forceinline__ void each_modulus(F&& f) {
+  each_modulus(f, std::make_integer_sequence<int, kRnsModuli>{});
+}
+
+// The integer nearest to x 2^(58 - e) (|x| < 2^e) as four floats: 15-bit
+// pieces from the low end, the top one signed (two's complement).
+__device__ __forceinline__ void pieces(double x, int e, float (&p)[4]) {
+  const uint32_t hi = uint32_t(__double2hiint(x)), lo = uint32_t(__double2loint(x));
+  const int E = int((hi >> 20) & 0x7FF);
+  const uint32_t mh = (hi & 0xFFFFFu) | (E ? 0x100000u : 0u);
+  const unsigned long long mant = (static_cast<unsigned long long>(mh) << 32) | lo;
+  const int n = 1022 + e - (E ? E : 1);  // >= 0
+  const unsigned long long t = n > 63 ? 0ull : (mant << 6) >> n;
+  long long X = static_cast<long long>((t + 1) >> 1);
+  if (int(hi) < 0) X = -X;
+  const uint32_t xl = uint32_t(X), xh = uint32_t(static_cast<unsigned long long>(X) >> 32);
+  p[0] = __uint_as_float(0x4B000000u | (xl & 0x7FFFu)) - 8388608.0f;
+  p[1] = __uint_as_float(0x4B000000u | ((xl >> 15) & 0x7FFFu)) - 8388608.0f;
+  p[2] = __uint_as_float(0x4B000000u | (__funnelshift_r(xl, xh, 30) & 0x7FFFu)) - 8388608.0f;
+  p[3] = __int_as_float(0x4B400000 + (int(xh) >> 13)) - 12582912.0f;
+}
+
+__device__ __forceinline__ uint32_t bf16x2(float a, float b) {
+  return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+
+// Residues of 8 consecutive k of one row: one 16-byte word per modulus. The
+// sum of pieces times coefficients is an exact integer below 2^24 in FP32, its
+// quotient by p is rounded by the add of 1.5 2^23, and the residue is exact.
+template <bool SCALED>
+__device__ __forceinline__ void store_residues(const float (&p)[8][4], uint8_t* dst, int64_t step) {
+  each_modulus([&](auto LC) {
+    constexpr int l = decltype(LC)::value;
+    constexpr float c0 = float(piece_coef(l, 0, SCALED)), c1 = float(piece_coef(l, 1, SCALED)),
+                    c2 = float(piece_coef(l, 2, SCALED)), c3 = float(piece_coef(l, 3, SCALED)), pm = float(modulus(l)),
+                    inv = 1.0f / float(modulus(l));
+    float r[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      float t = SCALED ? p[u][0] * c0 : p[u][0];
+      t = fmaf(p[u][1], c1, t);
+      t = fmaf(p[u][2], c2, t);
+      t = fmaf(p[u][3], c3, t);
+      const float q = fmaf(t, inv, 12582912.0f) - 12582912.0f;
+      r[u] = fmaf(q, -pm, t);
+    }
+    *reinterpret_cast<uint4*>(dst + l * step) =
+        make_uint4(bf16x2(r[0], r[1]), bf16x2(r[2], r[3]), bf16x2(r[4], r[5]), bf16x2(r[6], r[7]));
+  });
+}
+
+// |x| as a float, rounded down; 0 below the float range, garbage above it
+// (rows of such magnitude take the bound by their largest entry).
+__device__ __forceinline__ float abs_float(uint32_t hi, uint32_t lo) {
+  const uint32_t a = hi & 0x7FFFFFFFu;
+  return a < (897u << 20) ? 0.0f : __uint_as_float(((a - (896u << 20)) << 3) | (lo >> 29));
+}
+
+// Row exponent: 2^e above the 2-norm of the row, from the FP32 sum of squares
+// (2% margin for its rounding), or for magnitudes whose squares leave the FP32
+// range from the largest entry and the entry count.
+__device__ __forceinline__ int row_exponent(uint32_t mx, float sum, int count) {
+  if (mx >= 0x7FF00000u) return kNanRow;
+  if (mx == 0) return 0;
+  const int e = int(mx >> 20) - 1022;  // 2^e above the largest entry
+  if (e > 40 || e < -40) return e + (32 - __clz(count)) / 2 + 1;
+  const int e2 = int(__float_as_uint(sum * 1.02f) >> 23) - 126;  // 2^e2 above the sum
+  return (e2 + 1) >> 1;
+}
+
+// One operand (or two, the second by the blocks from nblk_a on) of a job into
+// its slots. A block of 256 threads takes 32 / OC groups of 8 rows: thread (row
+// r = tid % 8, octet o of OC) reads entries 8 o .. 8 o + 7 of its row, twice
+// when K > 8 OC (norm, then residues).
+template <typename T, int OC>
+__global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, const T* __restrict__ Y, DevFronts fr,
+                                                     const int32_t* __restrict__ fronts, const __grid_constant__ Job j,
+                                                     uint8_t* __restrict__ planes, int op_a, int nblk_a, int op_b) {
+  constexpr bool CPLX = sizeof(T) == 16;
+  constexpr int G = 32 / OC;  // row groups per block
+  const bool second = int(blockIdx.x) >= nblk_a;
+  const int op = second ? op_b : op_a;
+  const int blk = second ? int(blockIdx.x) - nblk_a : int(blockIdx.x);
+  const bool m_side = op == kOpD || op == kOpB || op == kOpLt;
+  const int* pref = m_side ? j.pref_m : j.pref_n;
+  const int per = pref[j.nf];
+  const int sub = threadIdx.x / (8 * OC);
+  const int grp = blk * G + sub;             // 8-row group in the launch
+  const int flat = grp >> 4;                 // slot
+  const bool in = flat < per * j.np;
+  __shared__ float s_sum[8][8];
+  __shared__ uint32_t s_max[8][8];
+  const int r = threadIdx.x & 7, o0 = (threadIdx.x / 8) % OC;
+  const int warp = threadIdx.x >> 5;
+  Dims d = {};
+  int rows = 0, K = 0, row = 0;
+  const T* src = nullptr;
+  int64_t sk = 0;
+  if (in) {
+    const int pole = flat / per, x = flat - pole * per, fi = owner(pref, j.nf, x);
+    const int f = fronts[fi];
+    d = dims_of(fr.s[f], fr.m[f], j.p0, j.pc, j.b);
+    const int rt = x - pref[fi] + (m_side ? 0 : j.rt0);
+    row = rt * kRnsTile + (grp & 15) * 8 + r;
+    const int64_t base = int64_t(j.pole0 + pole) * fr.pool + fr.off[f], m = d.m;
+    int64_t si = 1;
+    switch (op) {
+      case kOpV: case kOpT: src = F + base + j.p0 + m * (j.p0 + j.pc); rows = d.bw; K = d.pb; sk = m; break;
+      case kOpD: src = F + base + (j.p0 + j.pc) + m * (j.p0 + j.pc); rows = K = d.pb; si = m; sk = 1; break;
+      case kOpR: src = Y + base + j.p0 + m * j.p0; rows = K = d.bw; si = m; sk = 1; break;
+      case kOpW: case kOpL: src = F + base + d.q0 + m * j.p0; rows = d.mp; K = d.bw; sk = m; break;
+      case kOpB: src = F + base + j.p0 + m * j.p0; rows = K = d.bw; si = m; sk = 1; break;
+      case kOpLt: src = F + base + d.q0 + m * j.p0; rows = d.bw; K = d.mp; si = m; sk = 1; break;
+      case kOpY: src = Y + base + d.q0 + m * d.q0; rows = K = d.mp; si = m; sk = 1; break;
+      default: src = Y + base + d.q0 + m * j.p0; rows = d.bw; K = d.mp; si = m; sk = 1; break;  // kOpYt
+    }
+    src += si * row;
+  }
+  const bool row_in = in && row < rows;
+  auto load = [&](int o, double (&re)[8], double (&im)[8]) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = o * 8 + u;
+      re[u] = im[u] = 0.0;
+      if (row_in && k < K) {
+        if constexpr (CPLX) {
+          const double2 v = src[sk * k];
+          re[u] = v.x;
+          im[u] = v.y;
+        } else {
+          re[u] = src[sk * k];
+        }
+      }
+    }
+  };
+  double re[8], im[8];
+  float sum = 0.0f;
+  uint32_t mx = 0;
+  const int no = (K + 31) / 32 * 4;  // octets of the padded row
+  for (int o = o0; o < no; o += OC) {
+    load(o, re, im);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const uint32_t hr = uint32_t(__double2hiint(re[u])), hm = uint32_t(__double2hiint(im[u]));
+      mx = max(mx, max(hr & 0x7FFFFFFFu, hm & 0x7FFFFFFFu));
+      const float a = abs_float(hr, uint32_t(__double2loint(re[u])));
+      sum = fmaf(a, a, sum);
+      if (CPLX) {
+        const float c = abs_float(hm, uint32_t(__double2loint(im[u])));
+        sum = fmaf(c, c, sum);
+      }
+    }
+  }
+  // over the octets of a row: lanes 8 and 16 apart, then the group's OC / 4 warps
+#pragma unroll
+  for (int s = 8; s < 32; s <<= 1) {
+    sum += __shfl_xor_sync(0xFFFFFFFFu, sum, s);
+    mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, s));
+  }
+  if ((threadIdx.x & 31) < 8) {
+    s_sum[warp][r] = sum;
+    s_max[warp][r] = mx;
+  }
+  __syncthreads();
+  if (!row_in && (!in || (row & ~7) >= rows)) return;  // whole groups of rows past the operand
+  sum = 0.0f;
+  mx = 0;
+  const int w0 = sub * (OC / 4);
+#pragma unroll
+  for (int w = 0; w < OC / 4; ++w) {
+    sum += s_sum[w0 + w][r];
+    mx = max(mx, s_max[w0 + w][r]);
+  }
+  const int e = row_exponent(mx, sum, CPLX ? 2 * K : K);
+  uint8_t* slot = planes + (m_side ? j.m_base : j.n_base) + int64_t(flat) * j.slot;
+  if (o0 == 0) reinterpret_cast<int*>(slot + j.slot - kRnsTile * sizeof(int))[row & (kRnsTile - 1)] = e;
+  const bool scaled = op == kOpD || op == kOpT || op == kOpB || op == kOpL || op == kOpLt;
+  const int ex = e == kNanRow ? 4000 : e;  // a row with Inf or NaN gives zeros here and NaN in the results
+  const int64_t step = int64_t(j.kt) * (CPLX ? 2 : 1) * kPlane;
+  const bool again = no > OC;
+  for (int o = o0; o < no; o += OC) {
+    if (again) load(o, re, im);
+    uint8_t* dst = slot + int64_t(o >> 2) * ((CPLX ? 2 : 1) * kPlane) + ((row & (kRnsTile - 1)) >> 3) * 512 +
+                   (o & 3) * 128 + r * 16;
+#pragma unroll
+    for (int c = 0; c < (CPLX ? 2 : 1); ++c) {
+      float p[8][4];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) pieces(c ? im[u] : re[u], ex, p[u]);
+      if (scaled) store_residues<true>(p, dst + c * kPlane, step);
+      else store_residues<false>(p, dst + c * kPlane, step);
+    }
+  }
+}
+
+// ------------------------------------------------------------ GEMM
+__constant__ float c_mod[kRnsModuli] = {256, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+
+// Persistent: CTA x walks the (modulus, output tile) items x, x + gridDim.x,
+// ... (moduli outermost: the operand planes of one modulus stay in L2). Warp 8
+// streams K tiles of both operands (one bulk copy each, 6 stages of 32 KiB),
+// warp 9 issues the MMAs, warps 0-7 reduce the accumulators modulo p and store
+// them as bytes. Complex: accumulator columns 0-127 hold Re, 128-255 Im of the
+// tile (lane = row of M, column = row of N): Mr [Nr Ni] is one MMA of N = 256,
+// -Mi Ni and Mi Nr two of N = 128. The two accumulators (2 x 256 of 512 TMEM
+// columns) alternate between items, so that an item's reduction overlaps the
+// next one's MMAs. Items with K > 480 alternate them between chunks of 480: a
+// chunk's accumulator is reduced in place while the other one fills, and
+// carries its residue on.
+template <bool CPLX>
+__global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(DevFronts fr, const int32_t* __restrict__ fronts,
+                                                          const __grid_constant__ Job j,
+                                                          const uint8_t* __restrict__ planes, uint8_t* __restrict__ out,
+                                                          int* __restrict__ gfail, uint64_t wait_ns) {
+  constexpr int C = CPLX ? 2 : 1;
+  constexpr int kOp = C * kPlane;  // bytes of one operand's K tile
+  extern __shared__ __align__(128) uint8_t sm[];
+  __shared__ __align__(8) uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], mma_done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int s_fail, s_skip;
+  if (threadIdx.x == 0) s_skip = *static_cast<volatile int*>(gfail);
+  __syncthreads();
+  if (s_skip) return;  // an earlier CTA gave up: leave together
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* fail = &s_fail;
+  if (threadIdx.x == 0) {
+    s_fail = 0;
+    for (int i = 0; i < kStages; ++i) {
+      bar_init(smem_u32(&full[i]), 1);
+      bar_init(smem_u32(&empty[i]), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      bar_init(smem_u32(&acc_full[i]), 1);
+      bar_init(smem_u32(&acc_empty[i]), kEpi);
+    }
+    bar_init(smem_u32(&mma_done), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  if (warp == kEpi + 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = tmem_slot;
+  const int items = j.on * kRnsModuli;
+
+  // item -> modulus, output tile, K tiles (0: nothing to do)
+  auto decode = [&](int it, int& l, OutTile& t, int& rn, int& rm) -> int {
+    l = it / j.on;
+    t = out_tile(j, j.o0 + it - l * j.on);
+    const int f = fronts[t.f];
+    const Dims d = dims_of(fr.s[f], fr.m[f], j.p0, j.pc, j.b);
+    int k;
+    product_dims(j.mode, d, j.b, rn, rm, k);
+    return k <= 0 ? 0 : (k + kK - 1) / kK;
+  };
+
+  if (warp == kEpi) {
+    if (lane == 0) {  // ---- producer
+      int n = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; it < items && ok && !*fail; it += gridDim.x) {
+        int l, rn, rm;
+        OutTile t;
+        const int nkt = decode(it, l, t, rn, rm);
+        const int64_t lo = int64_t(l) * j.kt * kOp;
+        const uint8_t* gn = planes + j.n_base + (int64_t(t.pole) * j.pref_n[j.nf] + j.pref_n[t.f] + t.nt) * j.slot + lo;
+        const uint8_t* gm = planes + j.m_base + (int64_t(t.pole) * j.pref_m[j.nf] + j.pref_m[t.f] + t.mt) * j.slot + lo;
+        for (int kt = 0; kt < nkt; ++kt, ++n) {
+          const int st = n % kStages, u = n / kStages;
+          if (u > 0 && !bar_wait(smem_u32(&empty[st]), (u - 1) & 1, fail, wait_ns)) {
+            record_fail(&s_fail, 9, kt);
+            ok = false;
+            break;
+          }
+          bar_expect(smem_u32(&full[st]), 2 * kOp);
+          bulk_load(smem_u32(sm + st * 2 * kOp), gm + int64_t(kt) * kOp, kOp, smem_u32(&full[st]));
+          bulk_load(smem_u32(sm + st * 2 * kOp + kOp), gn + int64_t(kt) * kOp, kOp, smem_u32(&full[st]));
+        }
+      }
+      // every copy issued has landed before the CTA leaves (bounded)
+      for (int i = 0; i < kStages; ++i)
+        if (n > i && !bar_wait_all(smem_u32(&full[i]), ((n - 1 - i) / kStages) & 1)) record_fail(&s_fail, 3, i);
+    }
+  } else if (warp == kEpi + 1) {
+    if (lane == 0) {  // ---- MMA issuer
+      int n = 0, u = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+        int l, rn, rm;
+        OutTile t;
+        const int nkt = decode(it, l, t, rn, rm);
+        for (int k0 = 0; k0 < nkt && ok; k0 += kChunkTiles, ++u) {
+          const int buf = u & 1;
+          if (u > 1 && !bar_wait(smem_u32(&acc_empty[buf]), ((u >> 1) - 1) & 1, fail, wait_ns)) {
+            record_fail(&s_fail, 10, k0);
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const uint32_t acc = tmem + uint32_t(buf * 256);
+          const int k1 = min(nkt, k0 + kChunkTiles);
+          for (int kt = k0; kt < k1; ++kt, ++n) {
+            const int st = n % kStages;
+            if (!bar_wait(smem_u32(&full[st]), (n / kStages) & 1, fail, wait_ns)) {
+              record_fail(&s_fail, 11, kt);
+              ok = false;
+              break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint64_t mr = sdesc(smem_u32(sm + st * 2 * kOp)), mi = desc_off(mr, kPlane / 16),
+                           nr = desc_off(mr, kOp / 16), ni = desc_off(nr, kPlane / 16);
+#pragma unroll
+            for (int ks = 0; ks < 2; ++ks) {
+              // the third chunk on continues from the reduced residue
+              const uint32_t on = (kt > k0 || ks > 0 || k0 >= 2 * kChunkTiles) ? 1u : 0u;
+              mma(acc, desc_off(mr, ks * 16), desc_off(nr, ks * 16), idesc(CPLX ? 4 : 2, false), on);
+              if (CPLX) {
+                mma(acc, desc_off(mi, ks * 16), desc_off(ni, ks * 16), idesc(2, true), 1u);
+                mma(acc + 128u, desc_off(mi, ks * 16), desc_off(nr, ks * 16), idesc(2, false), 1u);
+              }
+            }
+            mma_commit(smem_u32(&empty[st]));
+          }
+          if (!ok) break;
+          mma_commit(smem_u32(&acc_full[buf]));
+        }
+      }
+      // every MMA issued has completed before TMEM is read for the last time or freed
+      mma_commit(smem_u32(&mma_done));
+      if (!bar_wait_all(smem_u32(&mma_done), 0)) record_fail(&s_fail, 7, 0);
+    }
+  } else {  // ---- reduction modulo p
+    const int q = warp & 3, h = warp >> 2;
+    const uint32_t lanes = uint32_t(q * 32) << 16;
+    // complex: half h reduces Re (columns 0-127) or Im; real: columns 64 h .. 64 h + 63
+    constexpr int NC = CPLX ? 128 : 64;
+    const uint32_t col0 = uint32_t(h * NC);
+    const int mrow = q * 32 + lane;
+    int u = 0;
+    bool ok = true;
+    auto wait_full = [&](int use) {
+      bool got = true;
+      if (lane == 0) got = bar_wait(smem_u32(&acc_full[use & 1]), (use >> 1) & 1, fail, wait_ns);
+      got = __shfl_sync(0xFFFFFFFFu, got, 0);
+      if (!got && lane == 0) record_fail(&s_fail, 12, use);
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      return got;
+    };
+    auto release = [&](int use) {
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      __syncwarp();
+      if (lane == 0) bar_arrive(smem_u32(&acc_empty[use & 1]));
+    };
+    for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      int l, rn, rm;
+      OutTile t;
+      const int nkt = decode(it, l, t, rn, rm), nch = (nkt + kChunkTiles - 1) / kChunkTiles;
+      if (nch == 0) continue;
+      const float p = c_mod[l], inv = 1.0f / p;
+      for (int c = 0; c + 2 < nch && ok; ++c, ++u) {  // chunks whose accumulator carries on: reduced in place
+        if (!(ok = wait_full(u))) break;
+        const uint32_t a = tmem + lanes + uint32_t((u & 1) * 256) + col0;
+#pragma unroll 1
+        for (int x = 0; x < NC; x += 16) {
+          uint32_t v[16];
+          tmem_ld16_nw(a + x, v);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float f = __uint_as_float(v[i]);
+            v[i] = __float_as_uint(fmaf(fmaf(f, inv, 12582912.0f) - 12582912.0f, -p, f));
+          }
+          tmem_st16(a + x, v);
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;");
+        release(u);
+      }
+      if (!ok) break;
+      const bool two = nch > 1;
+      if (two) {  // the last two chunks' accumulators are added here
+        if (!(ok = wait_full(u))) break;
+        ++u;
+      }
+      if (!(ok = wait_full(u))) break;
+      const uint32_t a = tmem + lanes + uint32_t((u & 1) * 256) + col0,
+                     a2 = tmem + lanes + uint32_t(((u & 1) ^ 1) * 256) + col0;
+      const int nn = min(kRnsTile, rn - (j.rt0 + t.nt) * kRnsTile);  // rows of N in the tile
+      const bool m_in = t.mt * kRnsTile + mrow < rm;
+      // (re, im) x 128 rows of M x 128 rows of N, one byte each
+      uint8_t* o = out + (int64_t(it - l * j.on) * kRnsModuli + l) * (C * kRnsTile * kRnsTile) +
+                   (CPLX ? h * kRnsTile * kRnsTile : 0) + mrow * kRnsTile + (CPLX ? 0 : h * NC);
+#pragma unroll 1
+      for (int x = 0; x < NC; x += 16) {
+        if ((CPLX ? 0 : h * NC) + x >= nn) break;
+        uint32_t v[16], w[16];
+        tmem_ld16_nw(a + x, v);
+        if (two) tmem_ld16_nw(a2 + x, w);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          float f = __uint_as_float(v[i]);
+          if (two) {
+            const float g = __uint_as_float(w[i]);
+            f += fmaf(fmaf(g, inv, 12582912.0f) - 12582912.0f, -p, g);
+          }
+          // r + 128 in the low byte (r = 128 of p = 256 wraps to its other representative)
+          v[i] = __float_as_uint(fmaf(fmaf(f, inv, 12582912.0f) - 12582912.0f, -p, f) + 12583040.0f);
+        }
+        uint4 b;
+        uint32_t* bw = &b.x;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          bw[i] = __byte_perm(__byte_perm(v[4 * i], v[4 * i + 1], 0x0040), __byte_perm(v[4 * i + 2], v[4 * i + 3], 0x0040),
+                              0x5410);
+        if (m_in) *reinterpret_cast<uint4*>(o + x) = b;
+      }
+      if (two) release(u - 1);
+      release(u);
+      ++u;
+    }
+  }
+  __syncthreads();
+  if (s_fail && threadIdx.x == 0)
+    atomicMax(gfail, 1 + (min(s_fail, 255) << 20) + min(int(blockIdx.x), (1 << 20) - 1));
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  if (warp == kEpi + 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+// ------------------------------------------------------------ reconstruction
+// v 2^sc of a 128-bit integer, from its 64 leading bits, rounded to nearest.
+__device__ __forceinline__ double i128_scaled(i128 v, int sc) {
+  if (v == 0) return 0.0;
+  const unsigned long long sign = v < 0 ? (1ull << 63) : 0ull;
+  const u128 a = v < 0 ? u128(-v) : u128(v);
+  unsigned long long hi = static_cast<unsigned long long>(a >> 64), lo = static_cast<unsigned long long>(a);
+  int lz;
+  if (hi == 0) {
+    lz = 64 + __clzll(static_cast<long long>(lo));
+    hi = lo;
+    lo = 0;
+  } else {
+    lz = __clzll(static_cast<long long>(hi));
+  }
+  const int s = lz & 63;
+  const unsigned long long top = s ? (hi << s) | (lo >> (64 - s)) : hi;
+  unsigned long long mant = top >> 11;
+  const unsigned long long rest = top & 0x7FFull;
+  if (rest > 0x400ull || (rest == 0x400ull && (mant & 1ull))) ++mant;
+  int E = 127 - lz + sc + 1023;
+  if (mant >> 53) {
+    mant >>= 1;
+    ++E;
+  }
+  if (E <= 0 || E >= 2047) return ldexp(sign ? -static_cast<double>(mant) : static_cast<double>(mant), E - 1075);
+  return __longlong_as_double(static_cast<long long>(sign | (static_cast<unsigned long long>(E) << 52) | (mant & 0xFFFFFFFFFFFFFull)));
+}
+
+// The integer of magnitude below P / 2 whose residues (plus 128) are byte
+// `b` of w: sum of u_l P / p_l less a multiple of P, exactly, in limbs.
+__device__ __forceinline__ double from_residues(const uint32_t (&w)[kRnsModuli], int b, int sc) {
+  uint32_t a0 = 0;
+  unsigned long long a1 = 0, a2 = 0, a3 = 0;
+  each_modulus([&](auto LC) {
+    constexpr int l = decltype(LC)::value;
+    constexpr uint32_t l0 = limb(cofactor(l), 0), l1 = limb(cofactor(l), 1), l2 = limb(cofactor(l), 2),
+                       l3 = limb(cofactor(l), 3);
+    const uint32_t u = (w[l] >> (8 * b)) & 255u;
+    a0 += u * l0;
+    a1 += static_cast<unsigned long long>(u) * l1;
+    a2 += static_cast<unsigned long long>(u) * l2;
+    a3 += static_cast<unsigned long long>(u) * l3;
+  });
+  constexpr u128 P = mod_product();
+  constexpr long long b0 = limb_bias(0), b1 = limb_bias(1), b2 = limb_bias(2), b3 = limb_bias(3);
+  const long long s0 = static_cast<long long>(a0) + b0, s1 = static_cast<long long>(a1) + b1,
+                  s2 = static_cast<long long>(a2) + b2, s3 = static_cast<long long>(a3) + b3;
+  // the multiple of P, from the leading limb alone: |value| <= 2^116 against P / 2 > 2^116.3, and what the
+  // lower limbs and the float rounding leave out is below 2^-9 of P
+  constexpr float pinv = float(1.0 / (double(P >> 60) * double(1ull << 60)) * 19342813113834066795298816.0);  // 2^84 / P
+  const int k = __float2int_rn(__int2float_rn(static_cast<int>(s3 >> 8)) * (256.0f * pinv));
+  const i128 v = i128(s0) + (i128(s1) << 20) + (i128(s2) << 52) + (i128(s3) << 84) - i128(k) * i128(P);
+  return i128_scaled(v, sc);
+}
+
+__device__ __forceinline__ double nan_of() { return __longlong_as_double(0x7FF8000000000000LL); }
+__device__ __forceinline__ double sub(double a, double b) { return a - b; }
+__device__ __forceinline__ double2 sub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double neg(double a) { return -a; }
+__device__ __forceinline__ double2 neg(double2 a) { return make_double2(-a.x, -a.y); }
+__device__ __forceinline__ double one_of(double) { return 1.0; }
+__device__ __forceinline__ double2 one_of(double2) { return make_double2(1.0, 0.0); }
+__device__ __forceinline__ double half_sum(double a, double b) { return 0.5 * (a + b); }
+__device__ __forceinline__ double2 half_sum(double2 a, double2 b) {
+  return make_double2(0.5 * (a.x + b.x), 0.5 * (a.y + b.y));
+}
+
+// One block per output tile and 16 of its rows of M (front columns): a warp
+// takes 2 of them, a lane 4 consecutive rows of N (front rows, contiguous in
+// memory).
+template <typename T>
+__global__ void __launch_bounds__(256) k_rns_recon(T* __restrict__ F, T* __restrict__ Y, DevFronts fr,
+                                                   const int32_t* __restrict__ fronts, const __grid_constant__ Job j,
+                                                   const uint8_t* __restrict__ planes, const uint8_t* __restrict__ out) {
+  constexpr bool CPLX = sizeof(T) == 16;
+  constexpr int C = CPLX ? 2 : 1;
+  const OutTile t = out_tile(j, j.o0 + int(blockIdx.x));
+  const int f = fronts[t.f];
+  const Dims d = dims_of(fr.s[f], fr.m[f], j.p0, j.pc, j.b);
+  int rn, rm, K;
+  product_dims(j.mode, d, j.b, rn, rm, K);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n0 = (j.rt0 + t.nt) * kRnsTile + lane * 4;
+  const int64_t base = int64_t(j.pole0 + t.pole) * fr.pool + fr.off[f], m = d.m;
+  const int tail = kRnsTile * int(sizeof(int));
+  const int* en = reinterpret_cast<const int*>(planes + j.n_base +
+                                               (int64_t(t.pole) * j.pref_n[j.nf] + j.pref_n[t.f] + t.nt + 1) * j.slot - tail);
+  const int* em = reinterpret_cast<const int*>(planes + j.m_base +
+                                               (int64_t(t.pole) * j.pref_m[j.nf] + j.pref_m[t.f] + t.mt + 1) * j.slot - tail);
+  const bool last = j.pc + d.pb == d.bw;
+#pragma unroll 1
+  for (int x = 0; x < 2; ++x) {
+    const int mr = int(blockIdx.y) * 16 + warp * 2 + x, c = t.mt * kRnsTile + mr;
+    if (c >= rm || n0 >= rn) continue;
+    if (triangular(j.mode) && n0 + 3 < c) continue;
+    T v[4];
+    if (K > 0) {
+      const int eb = em[mr];
+      int ea[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) ea[i] = n0 + i < rn ? en[lane * 4 + i] : 0;
+#pragma unroll
+      for (int part = 0; part < C; ++part) {
+        uint32_t w[kRnsModuli];
+        const uint8_t* src = out + int64_t(blockIdx.x) * kRnsModuli * (C * kRnsTile * kRnsTile) +
+                             part * kRnsTile * kRnsTile + mr * kRnsTile + lane * 4;
+#pragma unroll
+        for (int l = 0; l < kRnsModuli; ++l)
+          w[l] = *reinterpret_cast<const uint32_t*>(src + int64_t(l) * (C * kRnsTile * kRnsTile));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          double r = from_residues(w, i, ea[i] + eb - 2 * kBeta);
+          if (ea[i] == kNanRow || eb == kNanRow) r = nan_of();
+          if constexpr (CPLX) {
+            if (part) v[i].y = r;
+            else v[i].x = r;
+          } else {
+            v[i] = r;
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = T{};
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = n0 + i;
+      if (r >= rn) break;
+      switch (j.mode) {
+        case kSweepT: {  // column c of the panel; the block holds minus the inverse until the last panel's sweep
+          T* col = F + base + m * (j.p0 + j.pc + c) + j.p0;
+          if (r >= j.pc && r < j.pc + d.pb) {
+            if (!last) col[r] = neg(col[r]);
+          } else {
+            const T val = last ? neg(v[i]) : v[i];
+            col[r] = val;
+            F[base + m * (j.p0 + r) + j.p0 + j.pc + c] = val;
+          }
+          break;
+        }
+        case kSweepU: {
+          if (r < c || (r >= j.pc && r < j.pc + d.pb) || (c >= j.pc && c < j.pc + d.pb)) break;
+          T* e = F + base + m * (j.p0 + c) + j.p0 + r;
+          // the last sweep's T is already negated, and so is its result
+          const T val = last ? neg(sub(*e, neg(v[i]))) : sub(*e, v[i]);
+          *e = val;
+          F[base + m * (j.p0 + r) + j.p0 + c] = val;
+          break;
+        }
+        case kResid: {
+          T x = neg(v[i]);
+          if (r == c) x = sub(one_of(x), v[i]);
+          Y[base + m * (j.p0 + c) + j.p0 + r] = x;
+          break;
+        }
+        case kRefine: {
+          if (r < c) break;
+          T* e = F + base + m * (j.p0 + c) + j.p0 + r;
+          const T val = sub(*e, neg(v[i]));
+          *e = val;
+          F[base + m * (j.p0 + r) + j.p0 + c] = val;
+          break;
+        }
+        case kPanel: F[base + m * (j.p0 + c) + d.q0 + r] = v[i]; break;
+        case kSchur:
+          if (r >= c) {
+            T* e = F + base + m * (d.q0 + c) + d.q0 + r;
+            *e = sub(*e, v[i]);
+          }
+          break;
+        case kTak: {
+          const T val = neg(v[i]);
+          Y[base + m * (j.p0 + c) + d.q0 + r] = val;
+          Y[base + m * (d.q0 + r) + j.p0 + c] = val;
+          break;
+        }
+        default: {  // kDiag
+          if (r < c) break;
+          const T a = F[base + m * (j.p0 + c) + j.p0 + r], b = F[base + m * (j.p0 + r) + j.p0 + c];
+          const T val = sub(half_sum(a, b), v[i]);
+          Y[base + m * (j.p0 + c) + j.p0 + r] = val;
+          Y[base + m * (j.p0 + r) + j.p0 + c] = val;
+          break;
+        }
+      }
+    }
+  }
+}
+
+// Diagonal blocks of more than one panel before their inversion, both
+// triangles, into Y (free during the factorisation). One block of threads per
+// 16 columns, front and pole.
+template <typename T>
+__global__ void __launch_bounds__(256) k_rns_save(const T* __restrict__ F, T* __restrict__ Y, DevFronts fr,
+                                                  const int32_t* __restrict__ fronts, int p0, int b) {
+  const int f = fronts[blockIdx.y];
+  const Dims d = dims_of(fr.s[f], fr.m[f], p0, 0, b);
+  if (d.bw <= b) return;
+  const int64_t base = int64_t(blockIdx.z) * fr.pool + fr.off[f] + p0 + int64_t(d.m) * p0;
+  for (int c = blockIdx.x * 16; c < min(d.bw, int(blockIdx.x) * 16 + 16); ++c)
+    for (int r = threadIdx.x; r < d.bw; r += 256) {
+      const int hi = max(r, c), lo = min(r, c);
+      Y[base + int64_t(d.m) * c + r] = F[base + int64_t(d.m) * lo + hi];
+    }
+}
+
+// ------------------------------------------------------------ scaling
+__global__ void k_rns_row_scale(const double* __restrict__ H, const double* __restrict__ S, int wide,
+                                const int64_t* __restrict__ diag, int64_t c0, int64_t n, int64_t e0,
+                                int32_t* __restrict__ g) {
+  for (int64_t c = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; c < n; c += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t e = (diag[c0 + c] - e0) * wide;
+    const double a = fmax(fabs(H[e]), fabs(S[e]));
+    const int E = int((__double2hiint(a) >> 20) & 0x7FF);
+    // zero, subnormal and non-finite diagonals stay unscaled
+    g[c0 + c] = E == 0 || E == 0x7FF ? 0 : max(-500, min(500, (E - 1023) >> 1));
+  }
+}
+
+__global__ void k_rns_entry_scale(const int32_t* __restrict__ row, const int32_t* __restrict__ col, int64_t e0,
+                                  int64_t nnz, const int32_t* __restrict__ g, int16_t* __restrict__ gs) {
+  for (int64_t e = e0 + blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < e0 + nnz;
+       e += int64_t(gridDim.x) * blockDim.x)
+    gs[e] = int16_t(g[row[e]] + g[col[e]]);
+}
+
+// ------------------------------------------------------------ host schedule
+int sms() {
+  static int n = 0;
+  if (!n) {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    n = v > 0 ? v : 152;
+  }
+  return n;
+}
+
+// Fronts [f0, f0 + nf) of a level's list for the poles [pole0, pole0 + np), or
+// row tiles [rt0, rt0 + rtn) of the one front's N operand (rtn = 0: all).
+struct Piece {
+  int f0, nf, pole0, np, rt0, rtn;
+};
+
+struct Slots {
+  int fixed, n;  // operand slots of a front: fixed ones, and those of N row tiles that may be taken in pieces
+  int k;         // contraction length: the slot size
+};
+
+// The pieces of a launch sequence that fit the scratch, in order. A front whose
+// fixed slots alone do not fit cannot occur (rns_min_bytes).
+template <typename Fn>
+std::vector<Piece> pieces_of(int nact, int nb, int64_t cap, bool cplx, Fn slots) {
+  std::vector<Piece> out;
+  for (int f0 = 0; f0 < nact;) {
+    int nf = 0, k = 0;
+    int64_t sum = 0;
+    while (f0 + nf < nact && nf < kRnsFronts) {
+      const Slots q = slots(f0 + nf);
+      const int kk = std::max(k, q.k);
+      if (nf > 0 && (sum + q.fixed + q.n) * rns_slot_bytes(kk, cplx) > cap) break;
+      sum += q.fixed + q.n;
+      k = kk;
+      ++nf;
+    }
+    const int64_t fit = cap / rns_slot_bytes(k, cplx);
+    if (sum > fit) {  // one front, in pieces of its row tiles
+      const Slots q = slots(f0);
+      const int step = int(std::max<int64_t>(1, fit - q.fixed));
+      for (int pole = 0; pole < nb; ++pole)
+        for (int r = 0; r < q.n; r += step) out.push_back({f0, 1, pole, 1, r, std::min(step, q.n - r)});
+    } else if (sum > 0) {
+      const int np = int(std::min<int64_t>(nb, fit / sum));
+      for (int pole = 0; pole < nb; pole += np) out.push_back({f0, nf, pole, std::min(np, nb - pole), 0, 0});
+    } else {
+      out.push_back({f0, nf, 0, nb, 0, 0});
+    }
+    f0 += nf;
+  }
+  return out;
+}
+
+template <typename T>
+struct Runner {
+  static constexpr bool CPLX = sizeof(T) == 16;
+  const RnsScratch& sc;
+  DevFronts fr;
+  T *F, *Y;
+  const int32_t* fronts;  // device list of the level
+  const int32_t *s, *m;   // the same on the host
+  int b;
+  cudaStream_t st;
+
+  // Tile counts of a product over a piece; returns the output tiles.
+  int job(Job& j, Mode mode, const Piece& q, int p0, int pc, int kt) const {
+    j.mode = mode;
+    j.nf = q.nf;
+    j.np = q.np;
+    j.pole0 = q.pole0;
+    j.p0 = p0;
+    j.pc = pc;
+    j.b = b;
+    j.rt0 = mode == kTak ? q.rt0 : 0;
+    j.kt = kt;
+    j.slot = rns_slot_bytes(32 * kt, CPLX);
+    j.pref_n[0] = j.pref_m[0] = j.pref_o[0] = 0;
+    for (int f = 0; f < q.nf; ++f) {
+      int rn, rm, k;
+      product_dims(mode, dims_of(s[q.f0 + f], m[q.f0 + f], p0, pc, b), b, rn, rm, k);
+      const int tn = q.rtn > 0 && mode == kTak ? q.rtn : tiles128(rn), tm = tiles128(rm);
+      j.pref_n[f + 1] = j.pref_n[f] + (k > 0 ? tn : 0);  // K = 0 (Y[B,B] of a front without rows below): no operands
+      j.pref_m[f + 1] = j.pref_m[f] + (k > 0 ? tm : 0);
+      j.pref_o[f + 1] = j.pref_o[f] + (triangular(mode) ? tn * (tn + 1) / 2 : tn * tm);
+    }
+    return j.pref_o[q.nf] * q.np;
+  }
+  int n_slots(const Job& j) const { return j.pref_n[j.nf] * j.np; }
+  int m_slots(const Job& j) const { return j.pref_m[j.nf] * j.np; }
+
+  static bool m_side(Operand op) { return op == kOpD || op == kOpB || op == kOpLt; }
+
+  void conv(const Job& j, const Piece& q, Operand a) const { conv2(j, q, a, a, false); }
+  void conv(const Job& j, const Piece& q, Operand a, Operand c) const { conv2(j, q, a, c, true); }
+  void conv2(const Job& j, const Piece& q, Operand a, Operand c, bool both) const {
+    const int oc = j.kt <= 2 ? 8 : 32, g = 32 / oc;
+    auto blocks = [&](Operand op) { return ((m_side(op) ? m_slots(j) : n_slots(j)) * 16 + g - 1) / g; };
+    const int na = blocks(a), n = na + (both ? blocks(c) : 0);
+    if (n <= 0) return;
+    if (oc == 8) k_rns_conv<T, 8><<<n, 256, 0, st>>>(F, Y, fr, fronts + q.f0, j, sc.planes, a, na, c);
+    else k_rns_conv<T, 32><<<n, 256, 0, st>>>(F, Y, fr, fronts + q.f0, j, sc.planes, a, na, c);
+  }
+
+  // The product and its reconstruction, in pieces of the output scratch.
+  void product(Job& j, const Piece& q, int tiles) const {
+    const int cap = int(std::min<int64_t>(sc.out_bytes / (int64_t(kRnsOutTile) * (CPLX ? 2 : 1)), 1 << 20));
+    for (int o = 0; o < tiles; o += cap) {
+      j.o0 = o;
+      j.on = std::min(cap, tiles - o);
+      k_rns_gemm<CPLX><<<std::min(sms(), j.on * kRnsModuli), kThreads, kStages * 2 * (CPLX ? 2 : 1) * kPlane, st>>>(
+          fr, fronts + q.f0, j, sc.planes, sc.out, sc.fail, sc.wait_ns);
+      k_rns_recon<T><<<dim3(j.on, kRnsTile / 16), 256, 0, st>>>(F, Y, fr, fronts + q.f0, j, sc.planes, sc.out);
+    }
+  }
+};
+
+constexpr int kNewton = 1;  // Newton steps on the inverse of a diagonal block
+
+// Slots of the launch sequences of one front.
+Slots sweep_slots(const Dims& d, int b) {
+  if (d.bw <= b) return {0, 0, 32};
+  return {2 * tiles128(d.bw) + 1, 0, b};
+}
+Slots refine_slots(const Dims& d, int b) { return {d.bw > b ? 3 * tiles128(d.bw) : 0, 0, d.bw}; }
+Slots schur_slots(const Dims& d) { return {d.mp > 0 ? 2 * tiles128(d.mp) + tiles128(d.bw) : 0, 0, d.bw}; }
+Slots tak_slots(const Dims& d) {
+  const int tm = tiles128(d.bw), tn = tiles128(d.mp);
+  return {d.mp > 0 ? tm : 0, d.mp > 0 ? std::max(tn, tm) : 0, d.mp};
+}
+
+}  // namespace
+
+void launch_rns_scales(const double* H, const double* S, int wide, const int64_t* diag, int64_t c0, int64_t n,
+                       const int32_t* row, const int32_t* col, int64_t e0, int64_t nnz, int32_t* g, int16_t* gs,
+                       cudaStream_t st) {
+  auto grid = [](int64_t k) { return int(std::min<int64_t>((k + 255) / 256, 152 * 8)); };
+  k_rns_row_scale<<<grid(n), 256, 0, st>>>(H, S, wide, diag, c0, n, e0, g);
+  k_rns_entry_scale<<<grid(nnz), 256, 0, st>>>(row, col, e0, nnz, g, gs);
+}
+
+cudaError_t rns_configure() {
+  cudaError_t e = cudaFuncSetAttribute(k_rns_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStages * 4 * kPlane);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_rns_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStages * 2 * kPlane);
+  return e;
+}
+
+// Scratch bytes below which some front's operands do not fit (a front's Y[S,S]
+// is taken in pieces of at least its panel operand's tiles), and what lets
+// every level run in one piece; both with room for the output tiles.
+void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& want) {
+  least = want = 0;
+  for (const Level& lv : p->levels) {
+    int64_t lw = 0, tw = 0, sw = 0;
+    int ks = 32, kt = 32;
+    for (size_t t = 0; t < lv.s.size(); ++t) {
+      const Dims d = dims_of(lv.s[t], lv.m[t], 0, 0, p->b);
+      const Slots a = sweep_slots(d, p->b), c = schur_slots(d), y = tak_slots(d), e = refine_slots(d, p->b);
+      const int64_t one = std::max({a.fixed * rns_slot_bytes(a.k, true), e.fixed * rns_slot_bytes(e.k, true), c.fixed * rns_slot_bytes(c.k, true),
+                                    2 * y.fixed * rns_slot_bytes(y.k, true)});
+      least = std::max(least, one);
+      sw += a.fixed;
+      lw += c.fixed;
+      tw += y.fixed + y.n;
+      ks = std::max(ks, c.k);
+      kt = std::max(kt, y.k);
+    }
+    want = std::max({want, sw * batch * rns_slot_bytes(p->b, true), lw * batch * rns_slot_bytes(ks, true),
+                     tw * batch * rns_slot_bytes(kt, true)});
+  }
+  least += rns_slot_bytes(32, true);
+  want = std::max(want, least);
+}
+
+int64_t rns_out_bytes(const pexsi_plan* p, int batch) {
+  int64_t tiles = 1;
+  for (const Level& lv : p->levels) {
+    int64_t t = 0;
+    for (size_t f = 0; f < lv.s.size(); ++f) {
+      const int64_t n = tiles128(lv.m[f]);
+      t += std::max<int64_t>(3, n * (n + 1) / 2);
+    }
+    tiles = std::max(tiles, t * batch);
+  }
+  return std::min<int64_t>(tiles, kRnsOutTiles) * kRnsOutTile * 2;
+}
+
+// Eliminates the block of columns [p0, p0 + 256) of the level's fronts (the
+// first nact, those with s > p0): inverts the diagonal block, L[S,B] and the
+// update of F[S,S].
+template <typename T>
+void rns_factor_block(const RnsScratch& sc, T* F, T* Y, const DevFronts& fr, const int32_t* dfr, const int32_t* s,
+                      const int32_t* m, int nact, int p0, int b, const BatchShifts& sh, DevStatus status, bool count,
+                      Profiler& pf, cudaStream_t st) {
+  Runner<T> r{sc, fr, F, Y, dfr, s, m, b, st};
+  constexpr bool CPLX = sizeof(T) == 16;
+  const int bw = std::min(rns_block(b), s[0] - p0);  // the widest front's block
+  if (bw > b) k_rns_save<T><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b);
+  for (int pc = 0; pc < bw; pc += b) {
+    int n = 0;
+    while (n < nact && s[n] > p0 + pc) ++n;
+    cudaEvent_t a = pf.begin(st);
+    launch_diag_inv<T>(F, fr, dfr, n, p0 + pc, b, sh, status, count, st);
+    pf.end(a, P_DIAG, st, 0.0, 0.0);
+    if (bw <= b) continue;
+    a = pf.begin(st);
+    auto slots = [&](int f) { return sweep_slots(dims_of(s[f], m[f], p0, pc, b), b); };
+    int kernels = 0;
+    for (const Piece& q : pieces_of(n, sh.nb, sc.plane_bytes, CPLX, slots)) {
+      const int kt = (b + kK - 1) / kK;
+      Job t, u;
+      const int to = r.job(t, kSweepT, q, p0, pc, kt), uo = r.job(u, kSweepU, q, p0, pc, kt);
+      if (to == 0) continue;
+      t.n_base = u.m_base = 0;  // V, T, D
+      u.n_base = int64_t(r.n_slots(t)) * t.slot;
+      t.m_base = 2 * u.n_base;
+      r.conv(t, q, kOpV, kOpD);
+      r.product(t, q, to);
+      r.conv(u, q, kOpT);
+      r.product(u, q, uo);
+      kernels += 6;
+    }
+    pf.end(a, P_PANEL, st, 0.0, 0.0, kernels);
+  }
+  // One Newton step X += X (I - B X) on the swept inverse: a panel block that is
+  // nearly singular within a well conditioned B leaves large intermediate
+  // inverses, whose rounding the sweeps keep; the residual product is accurate
+  // to 2^-59 of the norms, so the step brings X to FP64 accuracy of B^-1.
+  if (bw > b) {
+    cudaEvent_t a = pf.begin(st);
+    int kernels = 0;
+    auto rslots = [&](int f) { return refine_slots(dims_of(s[f], m[f], p0, 0, b), b); };
+    for (const Piece& q : pieces_of(nact, sh.nb, sc.plane_bytes, CPLX, rslots)) {
+      const int kt = (std::min(rns_block(b), s[q.f0] - p0) + kK - 1) / kK;
+      Job t, u;
+      const int to = r.job(t, kResid, q, p0, 0, kt), uo = r.job(u, kRefine, q, p0, 0, kt);
+      if (to == 0) continue;
+      t.n_base = 0;  // B, X, R
+      t.m_base = u.n_base = int64_t(r.n_slots(t)) * t.slot;
+      u.m_base = 2 * t.m_base;
+      Job c = t;
+      c.n_base = u.m_base;
+      for (int step = 0; step < kNewton; ++step) {
+        if (step == 0) r.conv(t, q, kOpR, kOpB);
+        else r.conv(t, q, kOpB);
+        r.product(t, q, to);
+        r.conv(c, q, kOpR);
+        r.product(u, q, uo);
+      }
+      kernels += 6 * kNewton;
+    }
+    pf.end(a, P_PANEL, st, 0.0, 0.0, kernels);
+  }
+  auto slots = [&](int f) { return schur_slots(dims_of(s[f], m[f], p0, 0, b)); };
+  for (const Piece& q : pieces_of(nact, sh.nb, sc.plane_bytes, CPLX, slots)) {
+    const int kt = (std::min(rns_block(b), s[q.f0] - p0) + kK - 1) / kK;
+    Job l, u;
+    const int lo = r.job(l, kPanel, q, p0, 0, kt), uo = r.job(u, kSchur, q, p0, 0, kt);
+    if (lo == 0) continue;
+    l.n_base = 0;
+    u.n_base = int64_t(r.n_slots(l)) * l.slot;
+    l.m_base = 2 * u.n_base;  // W, L, B^-1
+    u.m_base = 0;
+    double fl = 0, sfl = 0;
+    if (pf.on)
+      for (int f = q.f0; f < q.f0 + q.nf; ++f) {
+        const Dims d = dims_of(s[f], m[f], p0, 0, b);
+        const double fma_fl = CPLX ? 8.0 : 2.0;
+        fl += fma_fl * q.np * d.mp * double(d.bw) * d.bw;
+        sfl += fma_fl * q.np * (double(d.mp) * (d.mp + 1) / 2) * d.bw;
+      }
+    cudaEvent_t a = pf.begin(st);
+    r.conv(l, q, kOpW, kOpB);
+    pf.end(a, P_SLICE, st, 0.0, 0.0);
+    a = pf.begin(st);
+    r.product(l, q, lo);
+    pf.end(a, P_PANEL, st, fl, 0.0, 2, fl * kRnsModuli);
+    a = pf.begin(st);
+    r.conv(u, q, kOpL);
+    pf.end(a, P_SLICE, st, 0.0, 0.0);
+    a = pf.begin(st);
+    r.product(u, q, uo);
+    pf.end(a, P_SCHUR, st, sfl, 0.0, 2, sfl * kRnsModuli);
+  }
+}
+
+// Y[S,B], its mirror and Y[B,B] of the block at p0 of the level's first nact fronts.
+void rns_selinv_block(const RnsScratch& sc, double2* Y, double2* F, const DevFronts& fr, const int32_t* dfr,
+                      const int32_t* s, const int32_t* m, int nact, int p0, int b, int nb, Profiler& pf,
+                      cudaStream_t st) {
+  Runner<double2> r{sc, fr, F, Y, dfr, s, m, b, st};
+  auto slots = [&](int f) { return tak_slots(dims_of(s[f], m[f], p0, 0, b)); };
+  for (const Piece& q : pieces_of(nact, nb, sc.plane_bytes, true, slots)) {
+    int k = 32;
+    double fl = 0;
+    for (int f = q.f0; f < q.f0 + q.nf; ++f) {
+      const Dims d = dims_of(s[f], m[f], p0, 0, b);
+      k = std::max(k, d.mp);
+      fl += 8.0 * q.np * double(d.bw) * d.mp * (q.rtn > 0 ? double(q.rtn) * kRnsTile : d.mp);
+    }
+    const int kt = (k + kK - 1) / kK;
+    Job t, g;
+    const int to = r.job(t, kTak, q, p0, 0, kt), go = r.job(g, kDiag, q, p0, 0, kt);
+    const bool more = q.rtn > 0, first = !more || q.rt0 == 0;
+    // the front's last piece also takes Y[B,B]
+    const bool last = !more || q.rt0 + q.rtn >= tiles128(dims_of(s[q.f0], m[q.f0], p0, 0, b).mp);
+    t.m_base = g.m_base = 0;
+    t.n_base = g.n_base = int64_t(r.m_slots(t)) * t.slot;
+    if (to > 0) {
+      cudaEvent_t a = pf.begin(st);
+      if (first) r.conv(t, q, kOpLt, kOpY);
+      else r.conv(t, q, kOpY);
+      pf.end(a, P_SLICE, st, 0.0, 0.0);
+      a = pf.begin(st);
+      r.product(t, q, to);
+      pf.end(a, P_OFFDIAG, st, fl, 0.0, 2, fl * kRnsModuli);
+    }
+    if (last) {
+      cudaEvent_t a = pf.begin(st);
+      if (to > 0) r.conv(g, q, kOpYt);
+      r.product(g, q, go);
+      pf.end(a, P_DPART, st, 0.0, 0.0, 3);
+    }
+  }
+}
+
+template void rns_factor_block<double>(const RnsScratch&, double*, double*, const DevFronts&, const int32_t*, const int32_t*,
+                                       const int32_t*, int, int, int, const BatchShifts&, DevStatus, bool, Profiler&,
+                                       cudaStream_t);
+template void rns_factor_block<double2>(const RnsScratch&, double2*, double2*, const DevFronts&, const int32_t*, const int32_t*,
+                                        const int32_t*, int, int, int, const BatchShifts&, DevStatus, bool, Profiler&,
+                                        cudaStream_t);
+
+}  // namespace pexsi

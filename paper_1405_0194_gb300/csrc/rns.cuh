@@ -1,0 +1,53 @@
+// FP64 supernode products on the tensor cores in a residue number system
+// (rns.cu): device kernels' job description and the host-side schedule of one
+// block of panels.
+#pragma once
+
+#include <cstdint>
+
+#include "kernels.cuh"
+
+namespace pexsi {
+
+constexpr int kRnsModuli = 15;   // product of the moduli 2^117.8
+constexpr int kRnsBlock = 256;   // most columns eliminated together (a block of panels)
+constexpr int kRnsFronts = 128;  // fronts per launch (tile prefix sums travel as kernel arguments)
+constexpr int kRnsTile = 128;    // rows of an operand tile, edge of an output tile
+constexpr int kRnsOutTile = kRnsTile * kRnsTile * kRnsModuli;  // residue bytes of a real output tile
+
+// Columns of a block: whole panels of width b.
+__host__ __device__ inline int rns_block(int b) { return kRnsBlock / b * b; }
+
+// Scratch of the residue path: operand planes (slots of one 128-row tile each)
+// and residue output tiles, both reused by every launch.
+struct RnsScratch {
+  uint8_t* planes = nullptr;
+  int64_t plane_bytes = 0;
+  uint8_t* out = nullptr;
+  int64_t out_bytes = 0;
+  int* fail = nullptr;
+  uint64_t wait_ns = 0;
+};
+
+// Bytes of one operand slot: 128 rows x K (rounded up to 32) bf16 residues of
+// every modulus (re and im planes for complex operands), and the row exponents.
+inline int64_t rns_slot_bytes(int k, bool cplx) {
+  return int64_t((k + 31) / 32) * 8192 * (cplx ? 2 : 1) * kRnsModuli + kRnsTile * int64_t(sizeof(int));
+}
+
+constexpr int kRnsOutTiles = 160;  // most output tiles of a launch: 79 MB of residues, which stay in L2
+
+cudaError_t rns_configure();
+
+// Exponents of the symmetric scaling D A D, D = 2^-g, that brings the diagonal
+// of A = H - z S near 1: the residue products round each operand row relative
+// to its norm, so rows and columns of one size are the premise of their FP64
+// accuracy (a power of two is exact, and FP64 multiply-adds do not see it).
+// For columns [c0, c0 + n) with the values of one system (HS components wide:
+// 1 real, 2 complex): g[c] from max(|H_cc|, |S_cc|), then gs[e] = g[row] + g[col]
+// of its entries [e0, e0 + nnz); diag, row and col are the plan's.
+void launch_rns_scales(const double* H, const double* S, int wide, const int64_t* diag, int64_t c0, int64_t n,
+                       const int32_t* row, const int32_t* col, int64_t e0, int64_t nnz, int32_t* g, int16_t* gs,
+                       cudaStream_t st);
+
+}  // namespace pexsi

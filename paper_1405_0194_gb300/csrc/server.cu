@@ -39,7 +39,7 @@ struct Request {
   pexsi_request req{};
   std::vector<double> H, S, shifts;
   int batch = 1;
-  int64_t footprint = 0;
+  int64_t footprint = 0, rns_planes = 0, rns_out = 0;
   enum State { QUEUED, RUNNING, DONE } state = QUEUED;
   std::atomic<bool> cancel{false};
   int bypassed = 0;  // times a later request was admitted before this one
@@ -88,7 +88,7 @@ int execute(Request& r, cudaStream_t st, std::string* err) {
   ws.use_graphs = false;  // a request's workspace lives for one request
   int rc = PEXSI_OK;
   try {
-    pexsi::workspace_alloc(p, ws, r.batch, st, true);
+    pexsi::workspace_alloc(p, ws, r.batch, r.rns_planes, r.rns_out, st, true);
     ck(cudaMemcpyAsync(ws.H, r.H.data(), sizeof(double) * nnz, cudaMemcpyHostToDevice, st), "H2D(H)");
     const double* dS = nullptr;
     if (!r.S.empty()) {
@@ -255,10 +255,10 @@ int pexsi_server_submit(pexsi_server* s, const pexsi_request* req, int64_t* tick
   }
   // batch: the server's, shrunk until one request fits the whole budget
   int batch = std::max(1, std::min(s->opts.batch, std::max(req->n_poles, (req->n_shifts + 1) / 2)));
-  while (batch > 1 && pexsi::bytes_fixed(p) + batch * pexsi::bytes_per_pole(p) > s->budget) --batch;
+  batch = pexsi::fit_batch(p, s->budget, batch, r->rns_planes, r->rns_out);
+  if (batch < 1) return PEXSI_ERR_NOMEM;
   r->batch = batch;
-  r->footprint = pexsi::bytes_fixed(p) + batch * pexsi::bytes_per_pole(p);
-  if (r->footprint > s->budget) return PEXSI_ERR_NOMEM;
+  r->footprint = pexsi::bytes_fixed(p) + batch * pexsi::bytes_per_pole(p, r->rns_planes > 0) + r->rns_planes + r->rns_out;
   r->res.batch = batch;
   r->res.footprint_bytes = r->footprint;
   r->res.breakdown_front = -1;

@@ -1,0 +1,122 @@
+"""The FP64 products in residues (csrc/rns.cu) at the sizes where their tiling
+can go wrong, against dense inverses: fronts around the 64-wide panels, the
+128-row tiles, the 256-wide blocks and the 480-deep accumulator chunks, rows of
+very different scale, non-finite input, and a memory budget that leaves no room
+for their scratch."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import nao_synth as ns  # noqa: E402
+import paper_1405_0194_gb300 as px  # noqa: E402
+from oracle import dense  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_1405_0194_gb300 import build
+    build.build()
+
+
+def _full(n, seed):
+    """A dense symmetric pair on the full pattern (one front of n columns), S diagonally dominant."""
+    rng = np.random.default_rng(seed)
+    H = rng.standard_normal((n, n)) / np.sqrt(n)
+    S = 0.1 * rng.standard_normal((n, n)) / n
+    H, S = H + H.T, S + S.T
+    S[np.arange(n), np.arange(n)] = 1.0 + np.abs(S).sum(axis=0)
+    colptr = np.arange(0, n * n + 1, n, dtype=np.int64)
+    rowind = np.tile(np.arange(n, dtype=np.int32), n)
+    return colptr, rowind, H, S
+
+
+def _selinv(n, colptr, rowind, h, s, z, **opts):
+    plan = px.pexsi_setup(n, colptr, rowind, opts=px.pexsi_opts_default(max_batch=2, **opts))
+    try:
+        return px.pexsi_selinv(plan, h, s, z)
+    finally:
+        px.pexsi_plan_destroy(plan)
+
+
+# The error of an unpivoted block factorisation at |Im z| = 0.05 with entries of order one: about
+# n eps |G|^2 (|G| <= 1 / Im z / lambda_min(S) = 20) < 1e-10, relative to the largest entry.
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 127, 129, 192, 255, 256, 257, 320, 385, 511, 513, 768, 1000])
+def test_one_front(n):
+    colptr, rowind, H, S = _full(n, n)
+    z = 0.1 + 0.05j
+    got = _selinv(n, colptr, rowind, H.T.ravel(), S.T.ravel(), z).reshape(n, n).T
+    ref = np.linalg.inv(H - z * S)
+    assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+# several atoms of many orbitals in a row: fronts with rows below them, ragged in every size
+@pytest.mark.parametrize("norb,atoms", [(37, 9), (70, 9), (131, 7), (150, 6)])
+def test_fronts_with_update_sets(norb, atoms):
+    s = ns.make_chain(natoms=atoms, seed=norb, norb=norb)
+    z = 0.2 + 0.05j
+    ref = dense.selected_inverse(s.n, s.colptr, s.rowind, s.H, s.S, z)
+    got = _selinv(s.n, s.colptr, s.rowind, s.H, s.S, z, leaf_cols=2 * norb, amalgamate=0)
+    assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [64, 65, 200, 257, 600])
+def test_inertia_of_one_front(n):
+    colptr, rowind, H, S = _full(n, 3 * n)
+    shifts = np.array([-0.7, -0.05, 0.3, 1.1])
+    plan = px.pexsi_setup(n, colptr, rowind, opts=px.pexsi_opts_default(max_batch=2))
+    got = px.pexsi_inertia(plan, H.T.ravel(), S.T.ravel(), shifts)
+    px.pexsi_plan_destroy(plan)
+    ref = dense.inertia_counts(n, colptr, rowind, H.T.ravel(), S.T.ravel(), shifts)
+    assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("power", [300, -300, 90])
+def test_scaled_rows(power):
+    """Powers of two: a uniform factor, or one per row and column (D A D), only move exponents in FP64; the
+    residue scaling follows the rows, and the inverse has to as well."""
+    n = 300
+    colptr, rowind, H, S = _full(n, 7)
+    z = 0.1 + 0.05j
+    ref = np.linalg.inv(H - z * S)
+    d = np.full(n, 2.0 ** (power / 2)) if power != 90 else 2.0 ** np.random.default_rng(1).integers(-45, 46, n)
+    A = d[:, None] * d[None, :]
+    got = _selinv(n, colptr, rowind, (H * A).T.ravel(), (S * A).T.ravel(), z).reshape(n, n).T * A
+    assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+def test_non_finite_input_is_reported():
+    n = 300
+    colptr, rowind, H, S = _full(n, 9)
+    H[5, 5] = np.nan
+    with pytest.raises(px.PexsiError) as e:
+        _selinv(n, colptr, rowind, H.T.ravel(), S.T.ravel(), 0.1 + 0.05j)
+    assert e.value.code == -5
+
+
+def test_budget_without_room_for_the_scratch():
+    """The smallest budget that a plan accepts leaves no residue scratch; the DFMA kernels then give the same
+    inverse to rounding."""
+    n = 400
+    colptr, rowind, H, S = _full(n, 11)
+    z = 0.1 + 0.05j
+    h, s = H.T.ravel(), S.T.ravel()
+    lo, hi = 1 << 16, 1 << 30
+    while hi - lo > 1 << 16:
+        mid = (lo + hi) // 2
+        try:
+            small = _selinv(n, colptr, rowind, h, s, z, hbm_budget=mid)
+            hi = mid
+        except px.PexsiError as e:
+            assert e.code == -3
+            lo = mid
+    big = _selinv(n, colptr, rowind, h, s, z)
+    small = _selinv(n, colptr, rowind, h, s, z, hbm_budget=hi)
+    ref = np.linalg.inv(H - z * S).T.ravel()
+    assert np.abs(small - ref).max() <= 1e-10 * np.abs(ref).max()
+    assert np.abs(big - ref).max() <= 1e-10 * np.abs(ref).max()
+    assert not np.array_equal(big, small)  # two different kernels ran
