@@ -325,7 +325,7 @@ void factor_batch(const pexsi_plan* p, Workspace& ws, T* F, const BatchShifts& s
       PanelGeom g = panel_geom(lv, p0, b);
       PanelWork w = pf.on ? panel_work(lv, p0, b, es, fl) : PanelWork();
       cudaEvent_t a = pf.begin(st);
-      launch_diag_inv<T>(F, fr, dfr, g.nact, p0, b, sh, status, count, st);
+      launch_diag_inv<T>(F, fr, dfr, g.nact, p0, b, sh, status, st);
       pf.end(a, P_DIAG, st, nb * w.diag_fl, nb * w.diag_by);
       a = pf.begin(st);
       const int S = p->oz_slices;
@@ -754,7 +754,7 @@ void factor_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
       PanelGeom g = panel_geom(lv, p0, b);
       PanelWork w = pf.on ? panel_work(lv, p0, b, 16.0, 8.0) : PanelWork();
       cudaEvent_t a = pf.begin(st);
-      launch_diag_inv_gen(ws.F, fr, dfr, g.nact, p0, b, sh, status, count, st);
+      launch_diag_inv_gen(ws.F, fr, dfr, g.nact, p0, b, sh, status, st);
       pf.end(a, P_DIAG, st, nb * w.diag_fl, nb * w.diag_by);
       a = pf.begin(st);
       launch_panel_solve_gen(ws.F, fr, dfr, g.nact, g.row_tiles, p0, b, sh, st, false);

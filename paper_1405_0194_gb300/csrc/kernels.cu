@@ -22,6 +22,8 @@
 //   Y[P,P]  = D^{-1} - L[S,P]^T Y[S,P]
 #include <cfloat>
 #include <climits>
+#include <cstddef>
+#include <utility>
 
 #include <cooperative_groups.h>
 
@@ -68,8 +70,22 @@ __device__ __forceinline__ double absv(double2 a) { return hypot(a.x, a.y); }
 // diagonal entry, unpivoted (far outside the scale of H - zS here; a zero or
 // relatively tiny pivot still reports a breakdown through the pivot ratio).
 __device__ __forceinline__ float pivmag(double a) { return fabsf(__double2float_rn(a)); }
-__device__ __forceinline__ float pivmag(double2 a) {
-  return fabsf(__double2float_rn(a.x)) + fabsf(__double2float_rn(a.y));
+__device__ __forceinline__ float pivmag(double2 a) { return pivmag(a.x) + pivmag(a.y); }
+// The same without FP64 conversions (each holds its SM partition's FP64 unit for
+// 64 cycles) for zero and the normal float range: |a| rounded to nearest even.
+__device__ __forceinline__ bool quick_mag(double a, float& mag) {
+  const uint32_t hi = uint32_t(__double2hiint(a)) & 0x7FFFFFFFu, lo = uint32_t(__double2loint(a));
+  const uint32_t t = ((hi - (896u << 20)) << 3) | (lo >> 29);
+  const uint32_t up = t + (((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (t & 1u)) >> 29);
+  const bool zero = (hi | lo) == 0u;
+  mag = __uint_as_float(zero ? 0u : up);
+  return zero || hi - (897u << 20) < (254u << 20);
+}
+__device__ __forceinline__ bool quick_mag(double2 a, float& mag) {
+  float x, y;
+  const bool p = quick_mag(a.x, x), q = quick_mag(a.y, y);
+  mag = x + y;
+  return p && q;
 }
 __device__ __forceinline__ double mag1(double a) { return fabs(a); }
 __device__ __forceinline__ double mag1(double2 a) { return fabs(a.x) + fabs(a.y); }
@@ -80,9 +96,13 @@ __device__ __forceinline__ double mag1(double2 a) { return fabs(a.x) + fabs(a.y)
 // three divisions of Smith's method.
 __device__ __forceinline__ double recip_piv(double a) { return __drcp_rn(a); }
 __device__ __forceinline__ double2 recip_piv(double2 a) {
-  const double m = fmax(fabs(a.x), fabs(a.y));
-  const int e = min(((__double2hiint(m) >> 20) & 0x7FF) - 1023, 1022);  // exponent of m (subnormal: -1023)
-  const double sc = __hiloint2double((1023 - e) << 20, 0);             // 2^-e
+  // exponent of max(|x|, |y|) (subnormal: -1023), from the high words: FP64 operations are slow to return
+  const int e = min((max(__double2hiint(a.x) & 0x7FFFFFFF, __double2hiint(a.y) & 0x7FFFFFFF) >> 20) - 1023, 1022);
+  if (e > -400 && e < 400) {  // the squares stay in range: the same bits without the scaling
+    const double r = __drcp_rn(fma(a.x, a.x, a.y * a.y));
+    return make_double2(a.x * r, -(a.y * r));
+  }
+  const double sc = __hiloint2double((1023 - e) << 20, 0);  // 2^-e
   const double x = a.x * sc, y = a.y * sc;
   const double r = __drcp_rn(fma(x, x, y * y));
   return make_double2(x * r * sc, -(y * r) * sc);
@@ -359,10 +379,8 @@ __global__ void k_extend_add(T* __restrict__ F, DevFronts fr, const int32_t* __r
 }
 
 // ------------------------------------------------------------ diagonal blocks
-// Inverse of the (complex-)symmetric panel block D by Gauss-Jordan with
-// partial (row) pivoting, written back as the full block; for real symmetric
-// D (inertia) also the number of negative eigenvalues, from a Bunch-Kaufman
-// symmetric-pivoted LDL^T of D (Sylvester's law, Sec. II.C).
+// Negative eigenvalues of a panel block of an inertia shift, from a
+// Bunch-Kaufman symmetric-pivoted LDL^T of D (Sylvester's law, Sec. II.C).
 template <typename T>
 __device__ void bk_count(T* Bm, int n, int ld, int* out_neg, bool* singular);
 
@@ -586,13 +604,291 @@ __device__ void bk_count<double>(double* Bm, int n, int ld, int* out_neg, bool* 
   __syncthreads();
 }
 
-// Threads of a block inversion (8 warps; 16 measured slower: the FP64 pipe
-// of each SM is the bound, not the latency of its multiply-adds).
+// ------------------------------------------------------------ block inverses
+// Inverse of a panel block D (bb x bb, bb <= 64) by in-place Gauss-Jordan with
+// partial (row) pivoting, written back as the full block. Two forms with the
+// same operations on every entry, so with the same bits:
+//
+// k_diag_inv_one, one CTA per inversion, for launches that fill the chip: bound
+// by the FP64 units (bb^3 complex multiply-adds; 1216 of 48 x 48 in 1075 us, 84%
+// of that bound).
+//
+// k_diag_inv_cluster, a cluster of C = 8 CTAs per inversion: CTA r owns columns
+// [r W, (r + 1) W), W = ceil(bb / C), in the registers of its update threads
+// (thread (row i, group g) holds the columns g, g + ng, ... of row i).
+// What bounds it: bb dependent pivot steps, each a chain of some 15 dependent
+// FP64 operations, a search and two hops between CTAs, and the FP64 units: an
+// FP64 instruction of a warp holds its SM partition's unit for 64 cycles (a
+// step's update of 64 x 64 complex entries is 8192 cycles on one SM, 1024 on
+// eight). So the steps are pipelined: at step k the holders of column k + 1
+// update it first, send it to every CTA (st.async) and hand it to their CTA's
+// search warp, which finds the pivot row and then takes the pivot's reciprocal
+// while every CTA exchanges the two rows and the update threads finish the
+// other columns of step k. Every step has buffers and barriers of its own (64
+// columns of 1 KiB), so no CTA waits for another one to have read. Measured, one
+// 64 x 64 inverse on 8 SMs: complex 118 us, real 79 us, against 191 and 170 us
+// for search, reciprocal, publication, cluster barrier, swap, scaling and update
+// one after the other on blocks in shared memory.
+//
+// Warps: 6 update warps on three of the four SM partitions (warps 0-2, 4-6), the
+// search warp alone on the fourth (warp 3; warp 7 only takes part in the CTA
+// barriers), whose chain of steps the updates would hold up: 118 us against 124.
+//
+// Clusters up to 99 inversions of a launch, one CTA each from 100 (48 x 48
+// complex, us): 40: 116 against 217; 80: 209 / 216; 160: 389 / 295. Clusters of 2
+// and 4 lie between the two.
+constexpr int kDiagCtas = 8;
+constexpr int kDiagUpdate = 192;
 constexpr int kDiagThreads = 256;
+constexpr int kDiagClusterMost = 99;
+constexpr unsigned long long kDiagWaitNs = 1000000000ull;
+
+template <typename T>
+struct DiagStep {  // what a pivot step needs besides the column, sent by the column's owner
+  T inv;           // reciprocal of the pivot (0 once a pivot was zero or not finite)
+  double best;     // |Re| + |Im| of the pivot
+  long long bad;   // whether this or an earlier pivot was zero or not finite
+  long long row;   // the pivot's row
+  long long pad;
+};
+
+template <typename T>
+constexpr size_t diag_smem() {
+  return 64 * (64 * sizeof(T) + sizeof(DiagStep<T>) + 3 * sizeof(uint64_t)) + 64 * sizeof(T) +
+         4 * (64 / kDiagCtas + 1) * sizeof(T);
+}
+
+// Bounded wait for phase 0 of a barrier; false after a second (the block is
+// then reported as broken down, and the kernel runs on without waiting).
+__device__ __forceinline__ bool diag_wait(uint32_t bar) {
+  unsigned long long t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, "
+        "p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar)
+        : "memory");
+    if (ok) return true;
+    if ((it & 63u) == 63u) {
+      unsigned long long t;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > kDiagWaitNs) return false;
+    }
+  }
+}
+
+// v to shared address a of CTA `rank`, its bytes counted by that CTA's barrier.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void send(uint32_t a, double v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(a),
+               "l"(__double_as_longlong(v)), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void send(uint32_t a, double2 v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(a),
+               "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "r"(bar)
+               : "memory");
+}
+
+template <typename T, bool GEN>
+__global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restrict__ F, DevFronts fr,
+                                                                      const int32_t* __restrict__ fronts, int p0, int b,
+                                                                      DevStatus st) {
+  namespace cg = cooperative_groups;
+  constexpr int C = kDiagCtas, NU = kDiagUpdate;
+  constexpr int E = (64 / C + NU / 64 - 1) / (NU / 64);  // columns of a thread, at most
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* s_col = reinterpret_cast<T*>(smem_raw);                              // [64][64]: column of each step
+  DiagStep<T>* s_step = reinterpret_cast<DiagStep<T>*>(s_col + 64 * 64);  // [64]
+  T* s_stage = reinterpret_cast<T*>(s_step + 64);                         // [64]: next column, for the search warp
+  T* s_raw = s_stage + 64;                                                // [2][W + 1]: pivot row, unscaled
+  T* s_row = s_raw + 2 * (64 / C + 1);                                    // [2][W + 1]: row k before the swap
+  uint64_t* s_full = reinterpret_cast<uint64_t*>(s_row + 2 * (64 / C + 1));  // [64]: column and pivot row are here
+  uint64_t* s_inv = s_full + 64;                                             // [64]: the reciprocal is here
+  uint64_t* s_ready = s_inv + 64;                                            // [64]: the next column is staged
+  __shared__ double s_lmax, s_maxes[C];
+  __shared__ T s_scaled[64 / C];
+  const int f = fronts[blockIdx.x / C];
+  const int r = int(cg::this_cluster().block_rank());
+  const int pb = blockIdx.y;
+  const int s = fr.s[f], m = fr.m[f];
+  if (p0 >= s) return;  // the same for every CTA of the cluster
+  const int bb = min(b, s - p0);
+  const int W = (bb + C - 1) / C;
+  const int c0 = r * W, nc = max(0, min(bb, c0 + W) - c0);
+  const int ng = NU / bb;  // >= NU / 64 groups, so at most E columns each
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = tid >> 5;
+  const bool searcher = warp == 3;
+  const bool updater = !searcher && warp != 7;
+  const int ut = warp > 3 ? tid - 32 : tid;  // update thread
+  const int g = ut / bb, i = ut - g * bb;
+  const bool holds = updater && g < ng;
+  T* Fd = F + int64_t(pb) * fr.pool + fr.off[f] + p0 + int64_t(m) * p0;
+  const uint32_t full0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_full));
+  const uint32_t inv0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_inv));
+  const uint32_t ready0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_ready));
+  const uint32_t col0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_col));
+  const uint32_t step0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_step));
+  if (tid < 64) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8 * tid));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(inv0 + 8 * tid));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(ready0 + 8 * tid), "r"(bb));
+    asm volatile("fence.mbarrier_init.release.cluster;");
+    // the bytes each step brings: the column and the pivot row; the reciprocal, its size and the flag
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full0 + 8 * tid),
+                 "r"(int(bb * sizeof(T)) + 8)
+                 : "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(inv0 + 8 * tid), "r"(int(sizeof(T)) + 16)
+                 : "memory");
+  }
+  if (tid == 0) s_lmax = 0.0;
+  __syncthreads();
+  // symmetric fronts hold the lower triangle; LDU fronts (GEN) both
+  T a[E];
+  double lmax = 0.0;
+  T* save = st.dsave ? reinterpret_cast<T*>(st.dsave) + int64_t(pb) * st.dsave_stride + int64_t(st.col0[f] + p0) * b
+                     : nullptr;  // inertia shifts: the block before inversion, counted later
+#pragma unroll
+  for (int q = 0; q < E; ++q) {
+    const int jl = g + ng * q, j = c0 + jl;
+    a[q] = zero_of(T());
+    if (holds && jl < nc) {
+      a[q] = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
+      lmax = fmax(lmax, mag1(a[q]));
+      if (save) save[i * b + j] = a[q];
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+  if (lane == 0) atomicMax(reinterpret_cast<unsigned long long*>(&s_lmax), __double_as_longlong(lmax));
+  __syncthreads();
+  cg::this_cluster().sync();  // every CTA runs and its barriers are set before any remote access
+  if (tid == 0) *cg::this_cluster().map_shared_rank(&s_maxes[r], 0) = s_lmax;  // block max, gathered in CTA 0
+  bool lost = false;  // a wait ran out
+  // the holder of row i of column k hands it on: to its search warp and to every CTA
+  auto hand_on = [&](int k, T v) {
+    s_stage[i] = v;
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ready0 + 8 * k) : "memory");
+#pragma unroll
+    for (int q = 0; q < C; ++q)
+      send(cluster_addr(col0 + uint32_t((k * 64 + i) * sizeof(T)), q), v, cluster_addr(full0 + 8 * k, q));
+  };
+  if (r == 0 && holds && g == 0) hand_on(0, a[0]);
+
+  if (searcher) {
+    for (int k = c0; k < c0 + nc; ++k) {
+      if (!diag_wait(ready0 + 8 * k)) lost = true;
+      // the first row from k on of the largest magnitude, as a serial scan finds it; NaN counts as below all
+      const T v0 = lane >= k && lane < bb ? s_stage[lane] : zero_of(T());
+      const T v1 = lane + 32 >= k && lane + 32 < bb ? s_stage[lane + 32] : zero_of(T());
+      float m0, m1;
+      const bool quick = quick_mag(v0, m0) & quick_mag(v1, m1);
+      if (!__all_sync(0xffffffffu, quick)) {
+        m0 = pivmag(v0);
+        m1 = pivmag(v1);
+      }
+      const uint32_t key[2] = {lane >= k && lane < bb && m0 >= 0.0f ? __float_as_uint(m0) + 1u : 0u,
+                               lane + 32 >= k && lane + 32 < bb && m1 >= 0.0f ? __float_as_uint(m1) + 1u : 0u};
+      const uint32_t top = __reduce_max_sync(0xffffffffu, max(key[0], key[1]));
+      const uint32_t low = __ballot_sync(0xffffffffu, key[0] == top), high = __ballot_sync(0xffffffffu, key[1] == top);
+      const int row = top == 0u ? k : low ? __ffs(low) - 1 : 31 + __ffs(high);
+      if (lane < C)
+        send(cluster_addr(step0 + uint32_t(k * sizeof(DiagStep<T>) + offsetof(DiagStep<T>, row)), lane),
+             __longlong_as_double(row), cluster_addr(full0 + 8 * k, lane));
+      const T piv = s_stage[row];
+      const T rec = recip_piv(piv);
+      const double best = mag1(piv);
+      if (k > 0 && !diag_wait(inv0 + 8 * (k - 1))) lost = true;  // long here: column k was updated with it
+      const bool bad = (k > 0 && s_step[k - 1].bad) || !(best > 0.0) || !isfinite(best);
+      if (lane < C) {
+        const uint32_t d = cluster_addr(step0 + uint32_t(k * sizeof(DiagStep<T>)), lane), bar = cluster_addr(inv0 + 8 * k, lane);
+        send(d + uint32_t(offsetof(DiagStep<T>, inv)), bad ? zero_of(T()) : rec, bar);
+        send(d + uint32_t(offsetof(DiagStep<T>, best)), best, bar);
+        send(d + uint32_t(offsetof(DiagStep<T>, bad)), __longlong_as_double(bad ? 1 : 0), bar);
+      }
+    }
+  } else if (updater) {
+    for (int k = 0; k < bb; ++k) {
+      if (!diag_wait(full0 + 8 * k)) lost = true;
+      const int row = int(s_step[k].row), par = (k & 1) * (64 / C + 1);
+      const T fac = s_col[k * 64 + (i == row ? k : i)];
+      if (holds && (i == row || i == k)) {
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+          const int jl = g + ng * q;
+          if (jl < nc) {
+            if (i == row) s_raw[par + jl] = a[q];
+            if (i == k) s_row[par + jl] = a[q];
+          }
+        }
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(NU) : "memory");
+      if (!diag_wait(inv0 + 8 * k)) lost = true;
+      const T inv = s_step[k].inv;
+      // row k is scaled by the reciprocal; column k keeps the multipliers' negatives over the pivot
+      auto update = [&](T old, int jl, T rk) {
+        const T x = i == row ? s_row[par + jl] : old;
+        return i == k ? rk : fmsv(c0 + jl == k ? zero_of(T()) : x, fac, rk);
+      };
+      const int next = k + 1 - c0;  // the next pivot column, if it is one of this CTA's
+      if (holds && next >= 0 && next < nc && next % ng == g) {
+        const T rk = mulv(s_raw[par + next], inv);
+#pragma unroll
+        for (int q = 0; q < E; ++q)
+          if (g + ng * q == next) {
+            a[q] = update(a[q], next, rk);
+            hand_on(k + 1, a[q]);
+          }
+      }
+      // the other columns: the row is scaled once, by as few warps as hold its columns
+      if (ut < nc) s_scaled[ut] = c0 + ut == k ? inv : mulv(s_raw[par + ut], inv);
+      asm volatile("bar.sync 1, %0;" ::"n"(NU) : "memory");
+      if (holds) {
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+          const int jl = g + ng * q;
+          if (jl < nc && jl != next) a[q] = update(a[q], jl, s_scaled[jl]);
+        }
+      }
+    }
+    // write back: the row interchanges are column interchanges of the inverse,
+    // undone in reverse order, applied to each column's destination index
+#pragma unroll
+    for (int q = 0; q < E; ++q) {
+      const int jl = g + ng * q;
+      if (holds && jl < nc) {
+        int pos = c0 + jl;
+        for (int k = bb - 1; k >= 0; --k) {
+          const int x = int(s_step[k].row);
+          if (pos == k) pos = x;
+          else if (pos == x) pos = k;
+        }
+        Fd[i + int64_t(m) * pos] = a[q];
+      }
+    }
+  }
+  if (lost) atomicMin(st.breakdown_front, f);
+  cg::this_cluster().sync();  // every remote write of the cluster is done before any CTA leaves
+  if (r == 0 && tid == 0) {
+    double mx = 0.0, pmin = DBL_MAX;
+    for (int q = 0; q < C; ++q) mx = fmax(mx, s_maxes[q]);
+    for (int k = 0; k < bb; ++k) pmin = fmin(pmin, s_step[k].best);
+    const double ratio = mx > 0 ? pmin / mx : 0.0;
+    atomicMin(st.min_pivot, (unsigned long long)__double_as_longlong(ratio));
+    if (s_step[bb - 1].bad || ratio < 1e-13) atomicMin(st.breakdown_front, f);
+  }
+}
 
 template <typename T, bool GEN = false>
-__global__ void __launch_bounds__(kDiagThreads) k_diag_inv(T* __restrict__ F, DevFronts fr, const int32_t* __restrict__ fronts, int p0, int b,
-                           DevStatus st, int count_inertia) {
+__global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFronts fr,
+                                                      const int32_t* __restrict__ fronts, int p0, int b, DevStatus st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* Aug = reinterpret_cast<T*>(smem_raw);  // bb x bb, row-major, stride b+1, inverted in place
   const int f = fronts[blockIdx.x];
@@ -612,7 +908,7 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_inv(T* __restrict__ F, De
   if (threadIdx.x == 0) { s_max = 0.0; s_pmin = DBL_MAX; s_bad = false; }
   __syncthreads();
   double lmax = 0.0;
-  for (int idx = threadIdx.x; idx < bb * bb; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < bb * bb; idx += 256) {
     int i = idx % bb, j = idx / bb;
     // symmetric fronts hold the lower triangle; LDU fronts (GEN) both
     T v = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
@@ -624,32 +920,12 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_inv(T* __restrict__ F, De
   if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned long long*>(&s_max), __double_as_longlong(lmax));
   __syncthreads();
 
-  if (count_inertia && st.dsave) {
-    // the block as it is before inversion, counted later (launch_bk_count_all)
+  if (st.dsave) {
+    // inertia shifts: the block as it is before inversion, counted later (launch_bk_count_all)
     T* save = reinterpret_cast<T*>(st.dsave) + int64_t(pb) * st.dsave_stride + int64_t(st.col0[f] + p0) * b;
-    for (int idx = threadIdx.x; idx < bb * bb; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < bb * bb; idx += 256) {
       const int i = idx / bb, j = idx % bb;
       save[i * b + j] = Aug[i * ld + j];
-    }
-  } else if (count_inertia) {
-    // Bunch-Kaufman count on a copy placed after the augmented matrix
-    // (real symmetric blocks, or Hermitian ones of an LDU front with a real shift)
-    if constexpr (sizeof(T) == sizeof(double) || GEN) {
-      T* Bm = Aug + bb * ld;
-      for (int idx = threadIdx.x; idx < bb * bb; idx += blockDim.x) {
-        int i = idx % bb, j = idx / bb;
-        Bm[i * b + j] = Aug[i * ld + j];
-      }
-      __syncthreads();
-      __shared__ int s_neg;
-      __shared__ bool s_sing;
-      if (threadIdx.x == 0) s_sing = false;
-      __syncthreads();
-      bk_count<T>(Bm, bb, b, &s_neg, &s_sing);
-      if (threadIdx.x == 0) {
-        atomicAdd(&st.neg_count[pb], s_neg);
-        if (s_sing) atomicMin(st.breakdown_front, f);
-      }
     }
   }
 
@@ -677,7 +953,7 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_inv(T* __restrict__ F, De
     const int pr = s_piv;
     if (threadIdx.x == 0) s_perm[k] = pr;
     if (pr != k)
-      for (int j = threadIdx.x; j < bb; j += blockDim.x) {
+      for (int j = threadIdx.x; j < bb; j += 256) {
         T t = Aug[k * ld + j]; Aug[k * ld + j] = Aug[pr * ld + j]; Aug[pr * ld + j] = t;
       }
     __syncthreads();
@@ -685,12 +961,12 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_inv(T* __restrict__ F, De
     // over the pivot, row k is scaled by the pivot's reciprocal (one thread
     // takes the reciprocal: the FP64 pipe of an SM does 2 multiply-adds per clock)
     if (threadIdx.x == 0) s_inv = s_bad ? zero_of(T()) : recip_piv(Aug[k * ld + k]);
-    for (int i = threadIdx.x; i < bb; i += blockDim.x) s_fac[i] = Aug[i * ld + k];
+    for (int i = threadIdx.x; i < bb; i += 256) s_fac[i] = Aug[i * ld + k];
     __syncthreads();
     const T inv = s_inv;
-    for (int j = threadIdx.x; j < bb; j += blockDim.x) Aug[k * ld + j] = (j == k) ? inv : mulv(Aug[k * ld + j], inv);
+    for (int j = threadIdx.x; j < bb; j += 256) Aug[k * ld + j] = (j == k) ? inv : mulv(Aug[k * ld + j], inv);
     __syncthreads();
-    for (int idx = threadIdx.x; idx < bb * bb; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < bb * bb; idx += 256) {
       const int i = idx / bb, j = idx % bb;
       if (i == k) continue;
       Aug[i * ld + j] = (j == k) ? fmsv(zero_of(T()), s_fac[i], inv) : fmsv(Aug[i * ld + j], s_fac[i], Aug[k * ld + j]);
@@ -701,12 +977,12 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_inv(T* __restrict__ F, De
   for (int k = bb - 1; k >= 0; --k) {
     const int pr = s_perm[k];
     if (pr != k)
-      for (int i = threadIdx.x; i < bb; i += blockDim.x) {
+      for (int i = threadIdx.x; i < bb; i += 256) {
         T t = Aug[i * ld + k]; Aug[i * ld + k] = Aug[i * ld + pr]; Aug[i * ld + pr] = t;
       }
     __syncthreads();
   }
-  for (int idx = threadIdx.x; idx < bb * bb; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < bb * bb; idx += 256) {
     int i = idx % bb, j = idx / bb;
     Fd[i + int64_t(m) * j] = Aug[i * ld + j];
   }
@@ -717,158 +993,9 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_inv(T* __restrict__ F, De
   }
 }
 
-// The same inversion of a complex panel block, split over a cluster of
-// kDiagCluster (2, 4 or 8) CTAs (one SM each): CTA r owns columns [r W, (r+1) W) of the
-// bb x bb block (W = ceil(bb / kDiagCluster)) in its shared memory. At pivot
-// step k the owner of column k searches it for the pivot, swaps rows k and
-// pr in its columns and writes the pivot row index, the reciprocal of the
-// pivot and the (swapped) column k into every CTA's shared memory
-// (distributed shared memory, double-buffered by step parity); after one
-// cluster barrier every CTA swaps, scales row k and updates its own columns.
-// The buffer written at step k + 2 is no longer read then: every CTA has
-// passed the barrier of step k + 1, after its update of step k. The final
-// column interchanges are applied when the columns are written back. One
-// inversion thus runs on kDiagCluster SMs' FP64 pipes instead of one.
-template <typename T, bool GEN, int kDiagCluster>
-__global__ void __launch_bounds__(kDiagThreads) k_diag_inv_cluster(T* __restrict__ F, DevFronts fr,
-                                                                   const int32_t* __restrict__ fronts, int p0, int b,
-                                                                   DevStatus st) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
-  __shared__ T A[64][64 / kDiagCluster + 1];  // this CTA's columns (row-major in i)
-  __shared__ T pub_fac[2][64];
-  __shared__ T pub_inv[2];
-  __shared__ T s_inv;
-  __shared__ int pub_piv[2];
-  __shared__ double pub_best[2];
-  __shared__ double s_maxes[kDiagCluster];
-  __shared__ int s_perm[64];
-  __shared__ double s_lmax;
-  const int f = fronts[blockIdx.x / kDiagCluster];
-  const int r = int(cluster.block_rank());
-  const int pb = blockIdx.y;
-  const int s = fr.s[f], m = fr.m[f];
-  if (p0 >= s) return;  // the same for every CTA of the cluster
-  const int bb = min(b, s - p0);
-  const int W = (bb + kDiagCluster - 1) / kDiagCluster;
-  const int c0 = r * W, nc = max(0, min(bb, c0 + W) - c0);
-  T* Fd = F + int64_t(pb) * fr.pool + fr.off[f] + p0 + int64_t(m) * p0;
-  if (threadIdx.x == 0) s_lmax = 0.0;
-  __syncthreads();
-  double lmax = 0.0;
-  for (int idx = threadIdx.x; idx < bb * nc; idx += blockDim.x) {
-    const int i = idx % bb, jl = idx / bb, j = c0 + jl;
-    const T v = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
-    A[i][jl] = v;
-    lmax = fmax(lmax, mag1(v));
-  }
-  if (st.dsave) {  // inertia shifts: this CTA's columns of the block before inversion, counted later
-    T* save = reinterpret_cast<T*>(st.dsave) + int64_t(pb) * st.dsave_stride + int64_t(st.col0[f] + p0) * b;
-    for (int idx = threadIdx.x; idx < bb * nc; idx += blockDim.x) {
-      const int i = idx % bb, jl = idx / bb;
-      save[i * b + c0 + jl] = A[i][jl];
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned long long*>(&s_lmax), __double_as_longlong(lmax));
-  __syncthreads();
-  cluster.sync();  // every CTA of the cluster runs before any distributed shared memory access
-  if (threadIdx.x == 0) *cluster.map_shared_rank(&s_maxes[r], 0) = s_lmax;  // block max, gathered in CTA 0
-  bool bad = false;
-  double pmin = DBL_MAX;
-  for (int k = 0; k < bb; ++k) {
-    const int par = k & 1, owner = k / W;
-    if (r == owner) {
-      const int lk = k - c0;
-      if (threadIdx.x < 32) {
-        float bestf = -1.0f;
-        int bi = k;
-        for (int i = k + threadIdx.x; i < bb; i += 32) {
-          const float a = pivmag(A[i][lk]);
-          if (a > bestf) { bestf = a; bi = i; }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          const float ob = __shfl_xor_sync(0xffffffffu, bestf, o);
-          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-          if (ob > bestf || (ob == bestf && oi < bi)) { bestf = ob; bi = oi; }
-        }
-        if (threadIdx.x == 0) {
-          pub_piv[par] = bi;
-          pub_best[par] = mag1(A[bi][lk]);
-        }
-      }
-      __syncthreads();
-      const int pr = pub_piv[par];
-      if (pr != k)
-        for (int jl = threadIdx.x; jl < nc; jl += blockDim.x) {
-          const T t = A[k][jl]; A[k][jl] = A[pr][jl]; A[pr][jl] = t;
-        }
-      __syncthreads();
-      const double best = pub_best[par];
-      const bool now_bad = bad || !(best > 0.0) || !isfinite(best);
-      // one thread takes the reciprocal (the FP64 pipe of an SM does 2 multiply-adds per clock)
-      if (threadIdx.x == 0) s_inv = now_bad ? zero_of(T()) : recip_piv(A[k][lk]);
-      __syncthreads();
-      const T inv = s_inv;
-      // publish into every CTA of the cluster, all (CTA, row) pairs at once
-      for (int idx = threadIdx.x; idx < kDiagCluster * bb; idx += blockDim.x) {
-        const int q = idx / bb, i = idx - q * bb;
-        *cluster.map_shared_rank(&pub_fac[par][i], q) = A[i][lk];
-      }
-      if (threadIdx.x < kDiagCluster) {
-        const int q = threadIdx.x;
-        *cluster.map_shared_rank(&pub_inv[par], q) = inv;
-        *cluster.map_shared_rank(&pub_piv[par], q) = pr;
-        *cluster.map_shared_rank(&pub_best[par], q) = best;
-      }
-    }
-    cluster.sync();
-    const int pr = pub_piv[par];
-    const double best = pub_best[par];
-    const T inv = pub_inv[par];
-    bad = bad || !(best > 0.0) || !isfinite(best);
-    pmin = fmin(pmin, best);
-    if (threadIdx.x == 0) s_perm[k] = pr;
-    if (r != owner && pr != k)
-      for (int jl = threadIdx.x; jl < nc; jl += blockDim.x) {
-        const T t = A[k][jl]; A[k][jl] = A[pr][jl]; A[pr][jl] = t;
-      }
-    __syncthreads();
-    // row k scaled by the pivot's reciprocal; column k keeps the multipliers' negatives over the pivot
-    for (int jl = threadIdx.x; jl < nc; jl += blockDim.x) A[k][jl] = (c0 + jl == k) ? inv : mulv(A[k][jl], inv);
-    __syncthreads();
-    const T* fac = pub_fac[par];
-    for (int idx = threadIdx.x; idx < bb * nc; idx += blockDim.x) {
-      const int i = idx / nc, jl = idx % nc;
-      if (i == k) continue;
-      A[i][jl] = (c0 + jl == k) ? fmsv(zero_of(T()), fac[i], inv) : fmsv(A[i][jl], fac[i], A[k][jl]);
-    }
-    __syncthreads();
-  }
-  // write back: the row interchanges are column interchanges of the inverse,
-  // undone in reverse order, applied to each column's destination index
-  for (int jl = 0; jl < nc; ++jl) {
-    int pos = c0 + jl;
-    for (int k = bb - 1; k >= 0; --k) {
-      const int q = s_perm[k];
-      if (pos == k) pos = q;
-      else if (pos == q) pos = k;
-    }
-    for (int i = threadIdx.x; i < bb; i += blockDim.x) Fd[i + int64_t(m) * pos] = A[i][jl];
-  }
-  cluster.sync();  // every remote write of the cluster is done before any CTA leaves
-  if (r == 0 && threadIdx.x == 0) {
-    double mx = 0.0;
-    for (int q = 0; q < kDiagCluster; ++q) mx = fmax(mx, s_maxes[q]);
-    const double ratio = mx > 0 ? pmin / mx : 0.0;
-    atomicMin(st.min_pivot, (unsigned long long)__double_as_longlong(ratio));
-    if (bad || ratio < 1e-13) atomicMin(st.breakdown_front, f);
-  }
-}
-
 // Deferred inertia count: one CTA per (saved panel block, batch member).
 template <typename T>
-__global__ void __launch_bounds__(kDiagThreads) k_bk_count_all(const int32_t* __restrict__ slots, DevFronts fr, int b,
+__global__ void __launch_bounds__(256) k_bk_count_all(const int32_t* __restrict__ slots, DevFronts fr, int b,
                                                                DevStatus st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* Bm = reinterpret_cast<T*>(smem_raw);  // bb x bb, row stride b
@@ -1316,56 +1443,33 @@ void launch_extend_add(T* F, const DevFronts& fr, const int32_t* children, int n
   k_extend_add<T><<<grid, block, 0, st>>>(F, fr, children, nchild, pref);
 }
 
-// One cluster of C CTAs per block inverse (complex poles, which need no
-// inertia count).
-template <typename T, bool GEN, int C>
-void launch_diag_inv_cluster_c(T* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int p0, int b,
-                               const BatchShifts& sh, DevStatus status, cudaStream_t st) {
-  constexpr int kDiagCluster = C;
+template <typename T, bool GEN>
+void launch_diag_inv_any(T* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int p0, int b,
+                         const BatchShifts& sh, DevStatus status, cudaStream_t st) {
+  if (nfronts <= 0) return;
+  if (nfronts * sh.nb > kDiagClusterMost) {
+    k_diag_inv_one<T, GEN><<<dim3(nfronts, sh.nb), 256, sizeof(T) * size_t(b) * (b + 1), st>>>(F, fr, fronts, p0, b, status);
+    return;
+  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(nfronts * kDiagCluster), unsigned(sh.nb), 1);
+  cfg.gridDim = dim3(unsigned(nfronts * kDiagCtas), unsigned(sh.nb), 1);
   cfg.blockDim = dim3(kDiagThreads, 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = diag_smem<T>();
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kDiagCluster;
+  attr[0].val.clusterDim.x = kDiagCtas;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_diag_inv_cluster<T, GEN, C>, F, fr, fronts, p0, b, status);
-}
-
-// The cluster size: wide enough to spread the launch's inversions over the
-// SMs, 1 (the single-CTA kernel) once they already fill them.
-int diag_cluster_size(int inversions) {
-  return inversions >= 152 ? 1 : inversions >= 76 ? 2 : inversions >= 38 ? 4 : 8;
-}
-
-template <typename T, bool GEN>
-bool launch_diag_inv_cluster(T* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int p0, int b,
-                             const BatchShifts& sh, DevStatus status, cudaStream_t st) {
-  switch (diag_cluster_size(nfronts * sh.nb)) {
-    case 8: launch_diag_inv_cluster_c<T, GEN, 8>(F, fr, fronts, nfronts, p0, b, sh, status, st); return true;
-    case 4: launch_diag_inv_cluster_c<T, GEN, 4>(F, fr, fronts, nfronts, p0, b, sh, status, st); return true;
-    case 2: launch_diag_inv_cluster_c<T, GEN, 2>(F, fr, fronts, nfronts, p0, b, sh, status, st); return true;
-    default: return false;
-  }
+  cudaLaunchKernelEx(&cfg, k_diag_inv_cluster<T, GEN>, F, fr, fronts, p0, b, status);
 }
 
 template <typename T>
 void launch_diag_inv(T* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int p0, int b,
-                     const BatchShifts& sh, DevStatus status, bool count_inertia, cudaStream_t st) {
-  if (nfronts <= 0) return;
-  // the cluster kernel: complex poles, and inertia shifts whose blocks are
-  // saved for the deferred count
-  if ((!count_inertia || status.dsave) && b <= 64 &&
-      launch_diag_inv_cluster<T, false>(F, fr, fronts, nfronts, p0, b, sh, status, st))
-    return;
-  size_t smem = sizeof(T) * size_t(b) * (b + 1) + (count_inertia ? sizeof(double) * b * b : 0);
-  dim3 grid(nfronts, sh.nb);
-  k_diag_inv<T><<<grid, kDiagThreads, smem, st>>>(F, fr, fronts, p0, b, status, count_inertia ? 1 : 0);
+                     const BatchShifts& sh, DevStatus status, cudaStream_t st) {
+  launch_diag_inv_any<T, false>(F, fr, fronts, nfronts, p0, b, sh, status, st);
 }
 
 template <typename T>
@@ -1443,18 +1547,21 @@ void launch_traces(const double* dm, const double* edm, const double* fdm, const
 }
 
 cudaError_t configure_kernels(int b) {
-  size_t need_c = sizeof(double2) * size_t(b) * (b + 1);
-  size_t need_r = sizeof(double) * size_t(b) * (b + 1) + sizeof(double) * b * b;
-  cudaError_t e = cudaFuncSetAttribute(k_diag_inv<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(need_c));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_diag_inv<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(need_r));
-  if (e != cudaSuccess) return e;
+  const std::pair<const void*, size_t> inv[] = {
+      {(const void*)k_diag_inv_one<double2, false>, sizeof(double2) * b * (b + 1)},
+      {(const void*)k_diag_inv_one<double2, true>, sizeof(double2) * b * (b + 1)},
+      {(const void*)k_diag_inv_one<double, false>, sizeof(double) * b * (b + 1)},
+      {(const void*)k_diag_inv_cluster<double2, false>, diag_smem<double2>()},
+      {(const void*)k_diag_inv_cluster<double2, true>, diag_smem<double2>()},
+      {(const void*)k_diag_inv_cluster<double, false>, diag_smem<double>()}};
+  cudaError_t e;
+  for (const auto& fn : inv) {
+    e = cudaFuncSetAttribute(fn.first, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fn.second));
+    if (e != cudaSuccess) return e;
+  }
   // LDU fronts: the Hermitian inertia count keeps a complex copy of the block
   e = cudaFuncSetAttribute(k_bk_count_all<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            int(sizeof(double2) * b * b));
-  if (e != cudaSuccess) return e;
-  const size_t need_g = sizeof(double2) * size_t(b) * (b + 1) + sizeof(double2) * b * b;
-  e = cudaFuncSetAttribute(k_diag_inv<double2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(need_g));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_selinv_diag_reduce<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            int(sizeof(double2) * b * b));
@@ -1489,14 +1596,8 @@ void launch_extend_add_full(double2* F, const DevFronts& fr, const int32_t* chil
 }
 
 void launch_diag_inv_gen(double2* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int p0, int b,
-                         const BatchShifts& sh, DevStatus status, bool count_inertia, cudaStream_t st) {
-  if (nfronts <= 0) return;
-  if ((!count_inertia || status.dsave) && b <= 64 &&
-      launch_diag_inv_cluster<double2, true>(F, fr, fronts, nfronts, p0, b, sh, status, st))
-    return;
-  size_t smem = sizeof(double2) * size_t(b) * (b + 1) + (count_inertia ? sizeof(double2) * b * b : 0);
-  dim3 grid(nfronts, sh.nb);
-  k_diag_inv<double2, true><<<grid, kDiagThreads, smem, st>>>(F, fr, fronts, p0, b, status, count_inertia ? 1 : 0);
+                         const BatchShifts& sh, DevStatus status, cudaStream_t st) {
+  launch_diag_inv_any<double2, true>(F, fr, fronts, nfronts, p0, b, sh, status, st);
 }
 
 void launch_panel_solve_gen(double2* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int max_row_tiles,
@@ -1548,7 +1649,7 @@ template <typename T>
 void launch_bk_count_all(const int32_t* slots, int nslots, const DevFronts& fr, int b, int nb, DevStatus status,
                          cudaStream_t st) {
   if (nslots <= 0 || nb <= 0) return;
-  k_bk_count_all<T><<<dim3(nslots, nb), kDiagThreads, sizeof(T) * b * b, st>>>(slots, fr, b, status);
+  k_bk_count_all<T><<<dim3(nslots, nb), 256, sizeof(T) * b * b, st>>>(slots, fr, b, status);
 }
 template void launch_bk_count_all<double>(const int32_t*, int, const DevFronts&, int, int, DevStatus, cudaStream_t);
 template void launch_bk_count_all<double2>(const int32_t*, int, const DevFronts&, int, int, DevStatus, cudaStream_t);
@@ -1559,7 +1660,7 @@ template void launch_bk_count_all<double2>(const int32_t*, int, const DevFronts&
   template void launch_extend_add<T>(T*, const DevFronts&, const int32_t*, int, const int32_t*, int64_t,        \
                                      const BatchShifts&, cudaStream_t);                                           \
   template void launch_diag_inv<T>(T*, const DevFronts&, const int32_t*, int, int, int, const BatchShifts&,      \
-                                   DevStatus, bool, cudaStream_t);                                                \
+                                   DevStatus, cudaStream_t);                                                      \
   template void launch_panel_solve<T>(T*, const DevFronts&, const int32_t*, int, int, int, int,                  \
                                       const BatchShifts&, cudaStream_t);                                          \
   template void launch_trailing<T>(T*, const DevFronts&, const int32_t*, int, int, int, int, const BatchShifts&, \

@@ -87,7 +87,7 @@ void launch_extend_add(T* F, const DevFronts& fr, const int32_t* children, int n
 
 template <typename T>
 void launch_diag_inv(T* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int p0, int b,
-                     const BatchShifts& sh, DevStatus status, bool count_inertia, cudaStream_t st);
+                     const BatchShifts& sh, DevStatus status, cudaStream_t st);
 
 template <typename T>
 void launch_panel_solve(T* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int max_row_tiles, int p0,
@@ -188,9 +188,8 @@ void launch_assemble_gen(double2* F, const double2* H, const double2* S, const i
                          int64_t pool, const BatchShifts& sh, cudaStream_t st);
 void launch_extend_add_full(double2* F, const DevFronts& fr, const int32_t* children, int nchild, const int32_t* pref,
                             int64_t total_tiles, const BatchShifts& sh, cudaStream_t st);
-// count_inertia (real shifts of Hermitian H, S): Hermitian Bunch-Kaufman count of each D block
 void launch_diag_inv_gen(double2* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int p0, int b,
-                         const BatchShifts& sh, DevStatus status, bool count_inertia, cudaStream_t st);
+                         const BatchShifts& sh, DevStatus status, cudaStream_t st);
 // upper = false: L[S,P] = A[S,P] D^-1 (A[P,S] stays); upper = true: U[P,S] = D^-1 A[P,S]
 void launch_panel_solve_gen(double2* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int max_row_tiles,
                             int p0, int b, const BatchShifts& sh, cudaStream_t st, bool upper);

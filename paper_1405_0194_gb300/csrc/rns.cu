@@ -1065,7 +1065,7 @@ void rns_factor_block(const RnsScratch& sc, T* F, T* Y, const DevFronts& fr, con
     int n = 0;
     while (n < nact && s[n] > p0 + pc) ++n;
     cudaEvent_t a = pf.begin(st);
-    launch_diag_inv<T>(F, fr, dfr, n, p0 + pc, b, sh, status, count, st);
+    launch_diag_inv<T>(F, fr, dfr, n, p0 + pc, b, sh, status, st);
     pf.end(a, P_DIAG, st, 0.0, 0.0);
     if (bw <= b) continue;
     a = pf.begin(st);

@@ -120,3 +120,24 @@ def test_budget_without_room_for_the_scratch():
     assert np.abs(small - ref).max() <= 1e-10 * np.abs(ref).max()
     assert np.abs(big - ref).max() <= 1e-10 * np.abs(ref).max()
     assert not np.array_equal(big, small)  # two different kernels ran
+
+
+@pytest.mark.parametrize("n", [5, 31, 48, 64])
+def test_both_block_inverses_give_the_same_bits(n):
+    """Launches of up to 99 block inverses run one on a cluster of CTAs, larger ones one per CTA, with the same
+    operations on every entry: a system gives the same bits alone and among 110 others."""
+    pats = [_full(n, 100 + k) for k in range(110)]
+    host = [px.pexsi_setup(n, p[0], p[1], opts=px.pexsi_opts_default(device=-1)) for p in pats]
+    group = px.pexsi_group_create(host, px.pexsi_opts_default(max_batch=1))
+    H = [p[2].T.ravel().copy() for p in pats]
+    S = [p[3].T.ravel().copy() for p in pats]
+    k = len(pats)
+    dm, edm, fdm, _ = px.pexsi_group_dm(group, H, S, [0.1] * k, [50.0] * k, 2, [4.0] * k)
+    px.pexsi_group_destroy(group)
+    plan = px.pexsi_setup(n, pats[0][0], pats[0][1], opts=px.pexsi_opts_default(max_batch=1))
+    for q in (0, 57, 109):
+        a, b, c, _ = px.pexsi_dm(plan, H[q], S[q], 0.1, 50.0, 2, 4.0)
+        assert np.array_equal(a, dm[q]) and np.array_equal(b, edm[q]) and np.array_equal(c, fdm[q])
+    px.pexsi_plan_destroy(plan)
+    for p in host:
+        px.pexsi_plan_destroy(p)
