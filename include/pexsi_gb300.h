@@ -252,7 +252,8 @@ int pexsi_plan_get_supernodes(const pexsi_plan* plan, int32_t* first, int64_t* r
  * selected inversion runs the two-sided Takahashi recursion Y[S,P] =
  * -Y[S,S] L[S,P], Y[P,S] = -U[P,S] Y[S,S], Y[P,P] = D^-1 - U[P,S] Y[S,P]
  * (Sec. II.B steps 3-4 with U in place of L^T). These calls run the FP64
- * kernels whatever the plan's split_slices.
+ * products (residues on the tensor cores, as split_slices = 0) on FP64 plans, and
+ * FP64 multiply-adds on plans with split_slices > 0.
  * Layout: H, S, DM, EDM, FDM and ainv hold nnz complex values as interleaved
  * (re, im) doubles (2 nnz doubles) in the plan's CSC order; H[(r,c)] must be
  * conj(H[(c,r)]) (likewise S), S positive definite. S == NULL means S = I.

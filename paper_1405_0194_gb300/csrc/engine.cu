@@ -750,6 +750,16 @@ void factor_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
                              lv.ea_total_full[k], sh, st);
       pf.end(a, P_EXTEND, st, 0.0, nb * lv.ea_elems_full[k] * 16.0);
     }
+    if (ws.rns.planes) {
+      RnsScratch sc = ws.rns;
+      sc.fail = ws.ozfail + (count ? 1 : 0);
+      for (int p0 = 0; p0 < lv.max_s; p0 += rns_block(b)) {
+        int nact = 0;
+        while (nact < int(lv.s.size()) && lv.s[nact] > p0) ++nact;
+        rns_factor_block_gen(sc, ws.F, ws.Y, fr, dfr, lv.s.data(), lv.m.data(), nact, p0, b, sh, status, pf, st);
+      }
+      continue;
+    }
     for (int p0 = 0; p0 < lv.max_s; p0 += b) {
       PanelGeom g = panel_geom(lv, p0, b);
       PanelWork w = pf.on ? panel_work(lv, p0, b, 16.0, 8.0) : PanelWork();
@@ -783,6 +793,16 @@ void selinv_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
     cudaEvent_t a = pf.begin(st);
     launch_gather(ws.Y, fr, dfr, int(lv.fronts.size()), p->d_tile_pref + lv.gather_pref_off, lv.gather_total, sh, st);
     pf.end(a, P_GATHER, st, 0.0, nb * lv.gather_bytes);
+    if (ws.rns.planes) {
+      RnsScratch sc = ws.rns;
+      sc.fail = ws.ozfail;
+      for (int p0 = (lv.max_s - 1) / rns_block(b) * rns_block(b); p0 >= 0; p0 -= rns_block(b)) {
+        int nact = 0;
+        while (nact < int(lv.s.size()) && lv.s[nact] > p0) ++nact;
+        rns_selinv_block_gen(sc, ws.Y, ws.F, fr, dfr, lv.s.data(), lv.m.data(), nact, p0, b, sh.nb, pf, st);
+      }
+      continue;
+    }
     const int last = ((lv.max_s - 1) / b) * b;
     for (int p0 = last; p0 >= 0; p0 -= b) {
       PanelGeom g = panel_geom(lv, p0, b);
@@ -807,7 +827,7 @@ void run_gen_batch(const pexsi_plan* p, Workspace& ws, const double2* dH, const 
   const int64_t pool = p->sym.front_elems;
   ck(cudaMemsetAsync(ws.F, 0, sizeof(double2) * size_t(pool) * sh.nb, ws.stream), "memset(F)");
   cudaEvent_t a = pf.begin(ws.stream);
-  launch_assemble_gen(ws.F, dH, dS, p->d_pos_full, p->sym.nnz, pool, sh, ws.stream);
+  launch_assemble_gen(ws.F, dH, dS, p->d_pos_full, p->sym.nnz, pool, sh, ws.gs, ws.stream);
   pf.end(a, P_ASSEMBLE, ws.stream, 0.0, double(p->sym.nnz) * (32.0 + 16.0 * sh.nb));
   factor_batch_gen(p, ws, sh, count, pf);
   if (selinv) selinv_batch_gen(p, ws, sh, pf);
@@ -829,6 +849,7 @@ int dm_range_herm(const pexsi_plan* p, Workspace& ws, Profiler* prof, const doub
   double2* d_ddm = p->d_hout + 3 * nnz;
   if (info) ck(cudaEventRecord(ws.ev0, st), "event");
   if (!accumulate) reset_status(ws, 0);
+  set_scales(p, ws, reinterpret_cast<const double*>(dH), reinterpret_cast<const double*>(S), 2);
   bool first = true;
   for (int b0 = begin; b0 < end; b0 += ws.batch) {
     const int nb = std::min(ws.batch, end - b0);
@@ -841,7 +862,7 @@ int dm_range_herm(const pexsi_plan* p, Workspace& ws, Profiler* prof, const doub
     const int overwrite = (first && !accumulate) ? 1 : 0;
     cudaEvent_t a = pf.begin(st);
     launch_pole_sum_herm(ws.Y, p->sym.front_elems, p->d_pos_full, p->d_pos_t, nnz, sh, overwrite, d_dm, d_edm, d_fdm,
-                         d_ddm, st);
+                         d_ddm, ws.gs, st);
     pf.end(a, P_POLESUM, st, 4.0 * 12.0 * nb * double(nnz), double(nnz) * (16.0 + 32.0 * nb + 64.0 * (overwrite ? 1 : 2)));
     first = false;
   }
@@ -874,6 +895,7 @@ int dm_range_herm(const pexsi_plan* p, Workspace& ws, Profiler* prof, const doub
   info->gemm_flops = (2.0 * p->flops.factor_gemm + 2.0 * p->flops.selinv_gemm) * (end - begin);
   info->n_poles = end - begin;
   info->breakdown_front = brk == INT_MAX ? -1 : brk;
+  if (split_failed(ws, 0, err, "tensor-core GEMM")) return PEXSI_ERR_TIMEOUT;
   if (brk != INT_MAX) {
     *err = "zero or tiny pivot in front " + std::to_string(brk);
     return PEXSI_ERR_BREAKDOWN;
@@ -891,6 +913,7 @@ int inertia_range_herm(const pexsi_plan* p, Workspace& ws, const double2* dH, co
   std::vector<std::complex<double>> z(n_shifts);
   for (int t = 0; t < n_shifts; ++t) z[t] = {shifts[t], 0.0};
   int brk_all = INT_MAX;
+  set_scales(p, ws, reinterpret_cast<const double*>(dH), reinterpret_cast<const double*>(S), 2);
   for (int b0 = 0; b0 < n_shifts; b0 += ws.batch) {
     const int nb = std::min(ws.batch, n_shifts - b0);
     BatchShifts sh = make_shifts(z, nullptr, nullptr, nullptr, b0, nb);
@@ -904,6 +927,7 @@ int inertia_range_herm(const pexsi_plan* p, Workspace& ws, const double2* dH, co
     ck(cudaStreamSynchronize(st), "sync");
     for (int t = 0; t < nb; ++t) counts[b0 + t] = neg[t];
     brk_all = std::min(brk_all, brk);
+    if (split_failed(ws, 1, err, "tensor-core GEMM (inertia)")) return PEXSI_ERR_TIMEOUT;
   }
   if (brk_all != INT_MAX) {
     *err = "zero or tiny pivot in front " + std::to_string(brk_all);
@@ -917,12 +941,14 @@ int selinv_one_herm(const pexsi_plan* p, Workspace& ws, const double2* dH, const
   std::vector<std::complex<double>> z{{z_re, z_im}};
   BatchShifts sh = make_shifts(z, nullptr, nullptr, nullptr, 0, 1);
   reset_status(ws, 0);
+  set_scales(p, ws, reinterpret_cast<const double*>(dH), reinterpret_cast<const double*>(dS ? dS : p->d_ident_c), 2);
   run_gen_batch(p, ws, dH, dS ? dS : p->d_ident_c, sh, false, true, g_off);
-  launch_extract(ws.Y, p->d_pos_full, p->sym.nnz, d_ainv, nullptr, ws.stream);
+  launch_extract(ws.Y, p->d_pos_full, p->sym.nnz, d_ainv, ws.gs, ws.stream);
   ck(cudaGetLastError(), "extract");
   int brk = INT_MAX;
   ck(cudaMemcpyAsync(&brk, ws.brk, sizeof(int), cudaMemcpyDeviceToHost, ws.stream), "status");
   ck(cudaStreamSynchronize(ws.stream), "sync");
+  if (split_failed(ws, 0, err, "tensor-core GEMM")) return PEXSI_ERR_TIMEOUT;
   if (brk != INT_MAX) {
     *err = "zero or tiny pivot in front " + std::to_string(brk);
     return PEXSI_ERR_BREAKDOWN;

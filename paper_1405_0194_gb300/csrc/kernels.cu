@@ -1338,10 +1338,12 @@ __global__ void k_pole_sum(const double2* __restrict__ Y, int64_t pool, const in
 // Assembly of an LDU front from complex H and S (interleaved, nnz each):
 // every CSC entry at its own position (both triangles), A = H - z S.
 __global__ void k_assemble_gen(double2* __restrict__ F, const double2* __restrict__ H, const double2* __restrict__ S,
-                               const int64_t* __restrict__ pos, int64_t nnz, int64_t pool, BatchShifts sh) {
+                               const int64_t* __restrict__ pos, int64_t nnz, int64_t pool, BatchShifts sh,
+                               const int16_t* __restrict__ gs) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t p = pos[e];
-    const double2 h = H[e], v = S[e];
+    const double sc = entry_scale(gs, e);
+    const double2 h = scalev(H[e], sc), v = scalev(S[e], sc);
     for (int b = 0; b < sh.nb; ++b)  // (hr + i hi) - (zr + i zi)(sr + i si)
       F[b * pool + p] = make_double2(h.x - fma(sh.re[b], v.x, -sh.im[b] * v.y), h.y - fma(sh.re[b], v.y, sh.im[b] * v.x));
   }
@@ -1354,7 +1356,7 @@ __global__ void k_assemble_gen(double2* __restrict__ F, const double2* __restric
 __global__ void k_pole_sum_herm(const double2* __restrict__ Y, int64_t pool, const int64_t* __restrict__ pos,
                                 const int64_t* __restrict__ pos_t, int64_t nnz, BatchShifts sh, int overwrite,
                                 double2* __restrict__ dm, double2* __restrict__ edm, double2* __restrict__ fdm,
-                                double2* __restrict__ ddm) {
+                                double2* __restrict__ ddm, const int16_t* __restrict__ gs) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t p = pos[e], q = pos_t[e];
     double2 o[4] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
@@ -1370,10 +1372,11 @@ __global__ void k_pole_sum_herm(const double2* __restrict__ Y, int64_t pool, con
         o[k].y += 0.5 * (t.x - a.x);
       }
     }
+    const double sc = entry_scale(gs, e);
     double2* outs[4] = {dm, edm, fdm, ddm};
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      if (outs[k]) outs[k][e] = overwrite ? o[k] : addv(outs[k][e], o[k]);
+      if (outs[k]) outs[k][e] = overwrite ? scalev(o[k], sc) : addv(outs[k][e], scalev(o[k], sc));
   }
 }
 
@@ -1584,8 +1587,8 @@ cudaError_t configure_kernels(int b) {
 
 // ---- LDU fronts of complex Hermitian H and S (general complex shifted matrices)
 void launch_assemble_gen(double2* F, const double2* H, const double2* S, const int64_t* pos, int64_t nnz,
-                         int64_t pool, const BatchShifts& sh, cudaStream_t st) {
-  k_assemble_gen<<<grid_for(nnz, 256), 256, 0, st>>>(F, H, S, pos, nnz, pool, sh);
+                         int64_t pool, const BatchShifts& sh, const int16_t* gs, cudaStream_t st) {
+  k_assemble_gen<<<grid_for(nnz, 256), 256, 0, st>>>(F, H, S, pos, nnz, pool, sh, gs);
 }
 
 void launch_extend_add_full(double2* F, const DevFronts& fr, const int32_t* children, int nchild, const int32_t* pref,
@@ -1641,8 +1644,8 @@ void launch_selinv_diag_reduce_gen(double2* Y, const double2* F, const double2* 
 
 void launch_pole_sum_herm(const double2* Y, int64_t pool, const int64_t* pos, const int64_t* pos_t, int64_t nnz,
                           const BatchShifts& sh, int overwrite, double2* dm, double2* edm, double2* fdm, double2* ddm,
-                          cudaStream_t st) {
-  k_pole_sum_herm<<<grid_for(nnz, 256), 256, 0, st>>>(Y, pool, pos, pos_t, nnz, sh, overwrite, dm, edm, fdm, ddm);
+                          const int16_t* gs, cudaStream_t st) {
+  k_pole_sum_herm<<<grid_for(nnz, 256), 256, 0, st>>>(Y, pool, pos, pos_t, nnz, sh, overwrite, dm, edm, fdm, ddm, gs);
 }
 
 template <typename T>

@@ -185,7 +185,7 @@ cudaError_t oz_configure(int S);
 // trailing square, and selected inversion computes Y[S,P] = -Y[S,S] L[S,P]
 // and Y[P,S] = -U[P,S] Y[S,S] separately, with Y[P,P] = D^-1 - U[P,S] Y[S,P].
 void launch_assemble_gen(double2* F, const double2* H, const double2* S, const int64_t* pos, int64_t nnz,
-                         int64_t pool, const BatchShifts& sh, cudaStream_t st);
+                         int64_t pool, const BatchShifts& sh, const int16_t* gs, cudaStream_t st);
 void launch_extend_add_full(double2* F, const DevFronts& fr, const int32_t* children, int nchild, const int32_t* pref,
                             int64_t total_tiles, const BatchShifts& sh, cudaStream_t st);
 void launch_diag_inv_gen(double2* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int p0, int b,
@@ -206,7 +206,7 @@ void launch_selinv_diag_reduce_gen(double2* Y, const double2* F, const double2* 
 // (w G - conj(w) G^H) / 2i at each CSC entry: pos = its own position, pos_t = that of its transpose
 void launch_pole_sum_herm(const double2* Y, int64_t pool, const int64_t* pos, const int64_t* pos_t, int64_t nnz,
                           const BatchShifts& sh, int overwrite, double2* dm, double2* edm, double2* fdm, double2* ddm,
-                          cudaStream_t st);
+                          const int16_t* gs, cudaStream_t st);
 
 // Inertia counts of all saved panel blocks (slots: (front, p0) pairs, nslots
 // of them) for nb batch members: one CTA per block and member, a Bunch-Kaufman

@@ -214,6 +214,12 @@ template <typename T>
 void rns_factor_block(const RnsScratch& sc, T* F, T* Y, const DevFronts& fr, const int32_t* dfr, const int32_t* s,
                       const int32_t* m, int nact, int p0, int b, const BatchShifts& sh, DevStatus status, bool count,
                       Profiler& pf, cudaStream_t st);
+void rns_factor_block_gen(const RnsScratch& sc, double2* F, double2* Y, const DevFronts& fr, const int32_t* dfr,
+                          const int32_t* s, const int32_t* m, int nact, int p0, int b, const BatchShifts& sh,
+                          DevStatus status, Profiler& pf, cudaStream_t st);
+void rns_selinv_block_gen(const RnsScratch& sc, double2* Y, double2* F, const DevFronts& fr, const int32_t* dfr,
+                          const int32_t* s, const int32_t* m, int nact, int p0, int b, int nb, Profiler& pf,
+                          cudaStream_t st);
 void rns_selinv_block(const RnsScratch& sc, double2* Y, double2* F, const DevFronts& fr, const int32_t* dfr,
                       const int32_t* s, const int32_t* m, int nact, int p0, int b, int nb, Profiler& pf,
                       cudaStream_t st);

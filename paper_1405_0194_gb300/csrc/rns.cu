@@ -106,15 +106,25 @@ enum Mode {
   kPanel,   // L[S,B] = W[S,B] B^-1
   kSchur,   // F[S,S] -= L W^T (lower triangle)
   kTak,     // Y[S,B] = -Y[S,S] L[S,B] and its mirror
-  kDiag     // Y[B,B] = B^-1 - L[S,B]^T Y[S,B]
+  kDiag,    // Y[B,B] = B^-1 - L[S,B]^T Y[S,B]
+  // LDU fronts (gen): whole squares, no mirrors, the block's plain inverse in place of its negative
+  // during the sweeps, and the row panels
+  kSweepDU, // B[p,R] = D^-1 U, U = B[p,R]
+  kPanelU,  // U[B,S] = B^-1 A[B,S]
+  kTakU     // Y[B,S] = -U[B,S] Y[S,S]
 };
 // Operands of k_rns_conv.
-enum Operand { kOpV, kOpD, kOpT, kOpR, kOpW, kOpB, kOpL, kOpLt, kOpY, kOpYt };
+enum Operand {
+  kOpV, kOpD, kOpT, kOpR, kOpW, kOpB, kOpL, kOpLt, kOpY, kOpYt,
+  // LDU fronts: rows of D^-1, B, B^-1, Y[S,S] and U[B,S]; columns of U, R, A[B,S], Y[S,S] and Y[S,B]
+  kOpDr, kOpBr, kOpXr, kOpYr, kOpUr, kOpU, kOpRc, kOpA, kOpYc, kOpYtc
+};
 
 struct Job {
-  int mode, nf, np, pole0;   // nf fronts of the level's list, poles pole0 .. pole0 + np - 1
+  int mode, gen;             // gen: LDU fronts
+  int nf, np, pole0;         // nf fronts of the level's list, poles pole0 .. pole0 + np - 1
   int p0, pc, b;             // block start, panel start inside the block (sweeps), panel width
-  int rt0;                   // first row tile of N (a front whose row tiles are taken in pieces)
+  int rt0, mt0;              // first tile of N or M (a front whose row tiles are taken in pieces)
   int o0, on;                // output tiles of this launch
   int kt;                    // K tiles of a slot
   int64_t slot, n_base, m_base;
@@ -147,13 +157,24 @@ __host__ __device__ __forceinline__ void product_dims(int mode, const Dims& d, i
     case kResid: case kRefine: rn = rm = d.bw > b ? d.bw : 0; k = d.bw; break;
     case kPanel: rn = d.mp; rm = d.mp > 0 ? d.bw : 0; k = d.bw; break;
     case kSchur: rn = rm = d.mp; k = d.bw; break;
+    case kSweepDU: rm = d.bw > b && d.pb > 0 ? d.bw : 0; rn = rm ? d.pb : 0; k = d.pb; break;
+    case kPanelU: rn = d.mp > 0 ? d.bw : 0; rm = d.mp; k = d.bw; break;
+    case kTakU: rn = d.mp > 0 ? d.bw : 0; rm = d.mp; k = d.mp; break;
     case kTak: rn = d.mp; rm = d.mp > 0 ? d.bw : 0; k = d.mp; break;
     default: rn = rm = d.bw; k = d.mp; break;
   }
 }
 
-__host__ __device__ __forceinline__ bool triangular(int mode) {
-  return mode == kSweepU || mode == kRefine || mode == kSchur || mode == kDiag;
+__host__ __device__ __forceinline__ bool triangular(int mode, int gen) {
+  return !gen && (mode == kSweepU || mode == kRefine || mode == kSchur || mode == kDiag);
+}
+
+// whether an operand is the M one of its products, and whether the cofactors' inverses go into its residues
+__host__ __device__ __forceinline__ bool m_side(int op) {
+  return op == kOpD || op == kOpB || op == kOpLt || op >= kOpU;
+}
+__host__ __device__ __forceinline__ bool scaled_op(int op) {
+  return op == kOpD || op == kOpT || op == kOpB || op == kOpL || op == kOpLt || op == kOpDr || op == kOpXr || op == kOpUr;
 }
 
 // largest f with pref[f] <= t
@@ -178,14 +199,16 @@ __device__ __forceinline__ OutTile out_tile(const Job& j, int o) {
   const int x = o - t.pole * per;
   t.f = owner(j.pref_o, j.nf, x);
   const int y = x - j.pref_o[t.f];
-  if (triangular(j.mode)) {
+  if (triangular(j.mode, j.gen)) {
     int i = int((sqrtf(8.0f * float(y) + 1.0f) - 1.0f) * 0.5f);
     while (i * (i + 1) / 2 > y) --i;
     while ((i + 1) * (i + 2) / 2 <= y) ++i;
     t.nt = i;
     t.mt = y - i * (i + 1) / 2;
   } else {
-    const int mtn = j.pref_m[t.f + 1] - j.pref_m[t.f];
+    // Y[B,B] of a front without rows below it has no operands, and one tile or two by two
+    int mtn = j.pref_m[t.f + 1] - j.pref_m[t.f];
+    if (mtn == 0) mtn = j.pref_o[t.f + 1] - j.pref_o[t.f] > 1 ? 2 : 1;
     t.nt = y / mtn;
     t.mt = y - t.nt * mtn;
   }
@@ -281,8 +304,8 @@ __global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, co
   const bool second = int(blockIdx.x) >= nblk_a;
   const int op = second ? op_b : op_a;
   const int blk = second ? int(blockIdx.x) - nblk_a : int(blockIdx.x);
-  const bool m_side = op == kOpD || op == kOpB || op == kOpLt;
-  const int* pref = m_side ? j.pref_m : j.pref_n;
+  const bool ms = m_side(op);
+  const int* pref = ms ? j.pref_m : j.pref_n;
   const int per = pref[j.nf];
   const int sub = threadIdx.x / (8 * OC);
   const int grp = blk * G + sub;             // 8-row group in the launch
@@ -300,19 +323,26 @@ __global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, co
     const int pole = flat / per, x = flat - pole * per, fi = owner(pref, j.nf, x);
     const int f = fronts[fi];
     d = dims_of(fr.s[f], fr.m[f], j.p0, j.pc, j.b);
-    const int rt = x - pref[fi] + (m_side ? 0 : j.rt0);
+    const int rt = x - pref[fi] + (ms ? j.mt0 : j.rt0);
     row = rt * kRnsTile + (grp & 15) * 8 + r;
     const int64_t base = int64_t(j.pole0 + pole) * fr.pool + fr.off[f], m = d.m;
     int64_t si = 1;
     switch (op) {
       case kOpV: case kOpT: src = F + base + j.p0 + m * (j.p0 + j.pc); rows = d.bw; K = d.pb; sk = m; break;
       case kOpD: src = F + base + (j.p0 + j.pc) + m * (j.p0 + j.pc); rows = K = d.pb; si = m; sk = 1; break;
-      case kOpR: src = Y + base + j.p0 + m * j.p0; rows = K = d.bw; si = m; sk = 1; break;
+      case kOpR: case kOpRc: src = Y + base + j.p0 + m * j.p0; rows = K = d.bw; si = m; sk = 1; break;
       case kOpW: case kOpL: src = F + base + d.q0 + m * j.p0; rows = d.mp; K = d.bw; sk = m; break;
       case kOpB: src = F + base + j.p0 + m * j.p0; rows = K = d.bw; si = m; sk = 1; break;
       case kOpLt: src = F + base + d.q0 + m * j.p0; rows = d.bw; K = d.mp; si = m; sk = 1; break;
-      case kOpY: src = Y + base + d.q0 + m * d.q0; rows = K = d.mp; si = m; sk = 1; break;
-      default: src = Y + base + d.q0 + m * j.p0; rows = d.bw; K = d.mp; si = m; sk = 1; break;  // kOpYt
+      case kOpY: case kOpYc: src = Y + base + d.q0 + m * d.q0; rows = K = d.mp; si = m; sk = 1; break;
+      case kOpDr: src = F + base + (j.p0 + j.pc) + m * (j.p0 + j.pc); rows = K = d.pb; sk = m; break;
+      case kOpBr: src = Y + base + j.p0 + m * j.p0; rows = K = d.bw; sk = m; break;
+      case kOpXr: src = F + base + j.p0 + m * j.p0; rows = K = d.bw; sk = m; break;
+      case kOpYr: src = Y + base + d.q0 + m * d.q0; rows = K = d.mp; sk = m; break;
+      case kOpUr: src = F + base + j.p0 + m * d.q0; rows = d.bw; K = d.mp; sk = m; break;
+      case kOpU: src = F + base + (j.p0 + j.pc) + m * j.p0; rows = d.bw; K = d.pb; si = m; sk = 1; break;
+      case kOpA: src = F + base + j.p0 + m * d.q0; rows = d.mp; K = d.bw; si = m; sk = 1; break;
+      default: src = Y + base + d.q0 + m * j.p0; rows = d.bw; K = d.mp; si = m; sk = 1; break;  // kOpYt, kOpYtc
     }
     src += si * row;
   }
@@ -372,9 +402,9 @@ __global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, co
     mx = max(mx, s_max[w0 + w][r]);
   }
   const int e = row_exponent(mx, sum, CPLX ? 2 * K : K);
-  uint8_t* slot = planes + (m_side ? j.m_base : j.n_base) + int64_t(flat) * j.slot;
+  uint8_t* slot = planes + (ms ? j.m_base : j.n_base) + int64_t(flat) * j.slot;
   if (o0 == 0) reinterpret_cast<int*>(slot + j.slot - kRnsTile * sizeof(int))[row & (kRnsTile - 1)] = e;
-  const bool scaled = op == kOpD || op == kOpT || op == kOpB || op == kOpL || op == kOpLt;
+  const bool scaled = scaled_op(op);
   const int ex = e == kNanRow ? 4000 : e;  // a row with Inf or NaN gives zeros here and NaN in the results
   const int64_t step = int64_t(j.kt) * (CPLX ? 2 : 1) * kPlane;
   const bool again = no > OC;
@@ -589,7 +619,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(DevFronts fr, const in
       const uint32_t a = tmem + lanes + uint32_t((u & 1) * 256) + col0,
                      a2 = tmem + lanes + uint32_t(((u & 1) ^ 1) * 256) + col0;
       const int nn = min(kRnsTile, rn - (j.rt0 + t.nt) * kRnsTile);  // rows of N in the tile
-      const bool m_in = t.mt * kRnsTile + mrow < rm;
+      const bool m_in = (j.mt0 + t.mt) * kRnsTile + mrow < rm;
       // (re, im) x 128 rows of M x 128 rows of N, one byte each
       uint8_t* o = out + (int64_t(it - l * j.on) * kRnsModuli + l) * (C * kRnsTile * kRnsTile) +
                    (CPLX ? h * kRnsTile * kRnsTile : 0) + mrow * kRnsTile + (CPLX ? 0 : h * NC);
@@ -725,9 +755,9 @@ __global__ void __launch_bounds__(256) k_rns_recon(T* __restrict__ F, T* __restr
   const bool last = j.pc + d.pb == d.bw;
 #pragma unroll 1
   for (int x = 0; x < 2; ++x) {
-    const int mr = int(blockIdx.y) * 16 + warp * 2 + x, c = t.mt * kRnsTile + mr;
+    const int mr = int(blockIdx.y) * 16 + warp * 2 + x, c = (j.mt0 + t.mt) * kRnsTile + mr;
     if (c >= rm || n0 >= rn) continue;
-    if (triangular(j.mode) && n0 + 3 < c) continue;
+    if (triangular(j.mode, j.gen) && n0 + 3 < c) continue;
     T v[4];
     if (K > 0) {
       const int eb = em[mr];
@@ -762,6 +792,31 @@ __global__ void __launch_bounds__(256) k_rns_recon(T* __restrict__ F, T* __restr
     for (int i = 0; i < 4; ++i) {
       const int r = n0 + i;
       if (r >= rn) break;
+      if (j.gen) {
+        const bool in_r = r >= j.pc && r < j.pc + d.pb, in_c = c >= j.pc && c < j.pc + d.pb;
+        const T minus = neg(v[i]);
+        T* fb = F + base + m * j.p0 + j.p0;  // the diagonal block
+        T* yb = Y + base + m * j.p0 + j.p0;
+        switch (j.mode) {
+          case kSweepT: if (!in_r) fb[m * (j.pc + c) + r] = minus; break;
+          case kSweepDU: if (!in_c) fb[m * c + j.pc + r] = v[i]; break;
+          // T is stored negated
+          case kSweepU: if (!in_r && !in_c) fb[m * c + r] = sub(fb[m * c + r], minus); break;
+          case kResid: yb[m * c + r] = r == c ? sub(one_of(minus), v[i]) : minus; break;
+          case kRefine: fb[m * c + r] = sub(fb[m * c + r], minus); break;
+          case kPanel: F[base + m * (j.p0 + c) + d.q0 + r] = v[i]; break;
+          case kPanelU: F[base + m * (d.q0 + c) + j.p0 + r] = v[i]; break;
+          case kSchur: {
+            T* e = F + base + m * (d.q0 + c) + d.q0 + r;
+            *e = sub(*e, v[i]);
+            break;
+          }
+          case kTak: Y[base + m * (j.p0 + c) + d.q0 + r] = minus; break;
+          case kTakU: Y[base + m * (d.q0 + c) + j.p0 + r] = minus; break;
+          default: yb[m * c + r] = sub(fb[m * c + r], v[i]); break;  // kDiag
+        }
+        continue;
+      }
       switch (j.mode) {
         case kSweepT: {  // column c of the panel; the block holds minus the inverse until the last panel's sweep
           T* col = F + base + m * (j.p0 + j.pc + c) + j.p0;
@@ -824,18 +879,18 @@ __global__ void __launch_bounds__(256) k_rns_recon(T* __restrict__ F, T* __restr
 }
 
 // Diagonal blocks of more than one panel before their inversion, both
-// triangles, into Y (free during the factorisation). One block of threads per
+// triangles (symmetric fronts hold the lower one), into Y (free during the factorisation). One block of threads per
 // 16 columns, front and pole.
 template <typename T>
 __global__ void __launch_bounds__(256) k_rns_save(const T* __restrict__ F, T* __restrict__ Y, DevFronts fr,
-                                                  const int32_t* __restrict__ fronts, int p0, int b) {
+                                                  const int32_t* __restrict__ fronts, int p0, int b, int gen) {
   const int f = fronts[blockIdx.y];
   const Dims d = dims_of(fr.s[f], fr.m[f], p0, 0, b);
   if (d.bw <= b) return;
   const int64_t base = int64_t(blockIdx.z) * fr.pool + fr.off[f] + p0 + int64_t(d.m) * p0;
   for (int c = blockIdx.x * 16; c < min(d.bw, int(blockIdx.x) * 16 + 16); ++c)
     for (int r = threadIdx.x; r < d.bw; r += 256) {
-      const int hi = max(r, c), lo = min(r, c);
+      const int hi = gen ? r : max(r, c), lo = gen ? c : min(r, c);
       Y[base + int64_t(d.m) * c + r] = F[base + int64_t(d.m) * lo + hi];
     }
 }
@@ -926,10 +981,12 @@ struct Runner {
   const int32_t *s, *m;   // the same on the host
   int b;
   cudaStream_t st;
+  int gen = 0;
 
   // Tile counts of a product over a piece; returns the output tiles.
   int job(Job& j, Mode mode, const Piece& q, int p0, int pc, int kt) const {
     j.mode = mode;
+    j.gen = gen;
     j.nf = q.nf;
     j.np = q.np;
     j.pole0 = q.pole0;
@@ -937,23 +994,22 @@ struct Runner {
     j.pc = pc;
     j.b = b;
     j.rt0 = mode == kTak ? q.rt0 : 0;
+    j.mt0 = mode == kTakU ? q.rt0 : 0;
     j.kt = kt;
     j.slot = rns_slot_bytes(32 * kt, CPLX);
     j.pref_n[0] = j.pref_m[0] = j.pref_o[0] = 0;
     for (int f = 0; f < q.nf; ++f) {
       int rn, rm, k;
       product_dims(mode, dims_of(s[q.f0 + f], m[q.f0 + f], p0, pc, b), b, rn, rm, k);
-      const int tn = q.rtn > 0 && mode == kTak ? q.rtn : tiles128(rn), tm = tiles128(rm);
+      const int tn = q.rtn > 0 && mode == kTak ? q.rtn : tiles128(rn), tm = q.rtn > 0 && mode == kTakU ? q.rtn : tiles128(rm);
       j.pref_n[f + 1] = j.pref_n[f] + (k > 0 ? tn : 0);  // K = 0 (Y[B,B] of a front without rows below): no operands
       j.pref_m[f + 1] = j.pref_m[f] + (k > 0 ? tm : 0);
-      j.pref_o[f + 1] = j.pref_o[f] + (triangular(mode) ? tn * (tn + 1) / 2 : tn * tm);
+      j.pref_o[f + 1] = j.pref_o[f] + (triangular(mode, gen) ? tn * (tn + 1) / 2 : tn * tm);
     }
     return j.pref_o[q.nf] * q.np;
   }
   int n_slots(const Job& j) const { return j.pref_n[j.nf] * j.np; }
   int m_slots(const Job& j) const { return j.pref_m[j.nf] * j.np; }
-
-  static bool m_side(Operand op) { return op == kOpD || op == kOpB || op == kOpLt; }
 
   void conv(const Job& j, const Piece& q, Operand a) const { conv2(j, q, a, a, false); }
   void conv(const Job& j, const Piece& q, Operand a, Operand c) const { conv2(j, q, a, c, true); }
@@ -979,7 +1035,6 @@ struct Runner {
   }
 };
 
-constexpr int kNewton = 1;  // Newton steps on the inverse of a diagonal block
 
 // Slots of the launch sequences of one front.
 Slots sweep_slots(const Dims& d, int b) {
@@ -987,6 +1042,12 @@ Slots sweep_slots(const Dims& d, int b) {
   return {2 * tiles128(d.bw) + 1, 0, b};
 }
 Slots refine_slots(const Dims& d, int b) { return {d.bw > b ? 3 * tiles128(d.bw) : 0, 0, d.bw}; }
+Slots gen_sweep_slots(const Dims& d, int b) {
+  if (d.bw <= b) return {0, 0, 32};
+  return {2 * tiles128(d.bw) + 2, 0, b};
+}
+Slots gen_refine_slots(const Dims& d, int b) { return {d.bw > b ? 2 * tiles128(d.bw) : 0, 0, d.bw}; }
+Slots gen_schur_slots(const Dims& d) { return {d.mp > 0 ? 2 * tiles128(d.mp) + tiles128(d.bw) : 0, 0, d.bw}; }
 Slots schur_slots(const Dims& d) { return {d.mp > 0 ? 2 * tiles128(d.mp) + tiles128(d.bw) : 0, 0, d.bw}; }
 Slots tak_slots(const Dims& d) {
   const int tm = tiles128(d.bw), tn = tiles128(d.mp);
@@ -1021,7 +1082,7 @@ void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& 
     for (size_t t = 0; t < lv.s.size(); ++t) {
       const Dims d = dims_of(lv.s[t], lv.m[t], 0, 0, p->b);
       const Slots a = sweep_slots(d, p->b), c = schur_slots(d), y = tak_slots(d), e = refine_slots(d, p->b);
-      const int64_t one = std::max({a.fixed * rns_slot_bytes(a.k, true), e.fixed * rns_slot_bytes(e.k, true), c.fixed * rns_slot_bytes(c.k, true),
+      const int64_t one = std::max({(a.fixed + 1) * rns_slot_bytes(a.k, true), e.fixed * rns_slot_bytes(e.k, true), c.fixed * rns_slot_bytes(c.k, true),
                                     2 * y.fixed * rns_slot_bytes(y.k, true)});
       least = std::max(least, one);
       sw += a.fixed;
@@ -1060,7 +1121,7 @@ void rns_factor_block(const RnsScratch& sc, T* F, T* Y, const DevFronts& fr, con
   Runner<T> r{sc, fr, F, Y, dfr, s, m, b, st};
   constexpr bool CPLX = sizeof(T) == 16;
   const int bw = std::min(rns_block(b), s[0] - p0);  // the widest front's block
-  if (bw > b) k_rns_save<T><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b);
+  if (bw > b) k_rns_save<T><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b, 0);
   for (int pc = 0; pc < bw; pc += b) {
     int n = 0;
     while (n < nact && s[n] > p0 + pc) ++n;
@@ -1105,14 +1166,11 @@ void rns_factor_block(const RnsScratch& sc, T* F, T* Y, const DevFronts& fr, con
       u.m_base = 2 * t.m_base;
       Job c = t;
       c.n_base = u.m_base;
-      for (int step = 0; step < kNewton; ++step) {
-        if (step == 0) r.conv(t, q, kOpR, kOpB);
-        else r.conv(t, q, kOpB);
-        r.product(t, q, to);
-        r.conv(c, q, kOpR);
-        r.product(u, q, uo);
-      }
-      kernels += 6 * kNewton;
+      r.conv(t, q, kOpR, kOpB);
+      r.product(t, q, to);
+      r.conv(c, q, kOpR);
+      r.product(u, q, uo);
+      kernels += 6;
     }
     pf.end(a, P_PANEL, st, 0.0, 0.0, kernels);
   }
@@ -1183,6 +1241,131 @@ void rns_selinv_block(const RnsScratch& sc, double2* Y, double2* F, const DevFro
     if (last) {
       cudaEvent_t a = pf.begin(st);
       if (to > 0) r.conv(g, q, kOpYt);
+      r.product(g, q, go);
+      pf.end(a, P_DPART, st, 0.0, 0.0, 3);
+    }
+  }
+}
+
+// The same for LDU fronts: B, X and the panels are not symmetric.
+void rns_factor_block_gen(const RnsScratch& sc, double2* F, double2* Y, const DevFronts& fr, const int32_t* dfr,
+                          const int32_t* s, const int32_t* m, int nact, int p0, int b, const BatchShifts& sh,
+                          DevStatus status, Profiler& pf, cudaStream_t st) {
+  Runner<double2> r{sc, fr, F, Y, dfr, s, m, b, st, 1};
+  const int bw = std::min(rns_block(b), s[0] - p0);
+  const int kb = (b + kK - 1) / kK;
+  if (bw > b) k_rns_save<double2><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b, 1);
+  for (int pc = 0; pc < bw; pc += b) {
+    int n = 0;
+    while (n < nact && s[n] > p0 + pc) ++n;
+    cudaEvent_t a = pf.begin(st);
+    launch_diag_inv_gen(F, fr, dfr, n, p0 + pc, b, sh, status, st);
+    pf.end(a, P_DIAG, st, 0.0, 0.0);
+    if (bw <= b) continue;
+    a = pf.begin(st);
+    int kernels = 0;
+    auto slots = [&](int f) { return gen_sweep_slots(dims_of(s[f], m[f], p0, pc, b), b); };
+    for (const Piece& q : pieces_of(n, sh.nb, sc.plane_bytes, true, slots)) {
+      Job t, x, u;
+      const int to = r.job(t, kSweepT, q, p0, pc, kb), xo = r.job(x, kSweepDU, q, p0, pc, kb),
+                uo = r.job(u, kSweepU, q, p0, pc, kb);
+      if (to == 0) continue;
+      const int64_t rows = int64_t(r.n_slots(t)) * t.slot, pan = int64_t(r.m_slots(t)) * t.slot;
+      t.n_base = 0;                      // V, T
+      u.n_base = 0;
+      x.m_base = u.m_base = rows;        // U
+      t.m_base = 2 * rows;               // columns of D^-1
+      x.n_base = 2 * rows + pan;         // rows of D^-1
+      r.conv(t, q, kOpV, kOpD);
+      r.conv(x, q, kOpDr, kOpU);
+      r.product(t, q, to);
+      r.product(x, q, xo);
+      r.conv(u, q, kOpT);
+      r.product(u, q, uo);
+      kernels += 9;
+    }
+    pf.end(a, P_PANEL, st, 0.0, 0.0, kernels);
+  }
+  if (bw > b) {
+    cudaEvent_t a = pf.begin(st);
+    int kernels = 0;
+    auto slots = [&](int f) { return gen_refine_slots(dims_of(s[f], m[f], p0, 0, b), b); };
+    for (const Piece& q : pieces_of(nact, sh.nb, sc.plane_bytes, true, slots)) {
+      const int kt = (std::min(rns_block(b), s[q.f0] - p0) + kK - 1) / kK;
+      Job t, u;
+      const int to = r.job(t, kResid, q, p0, 0, kt), uo = r.job(u, kRefine, q, p0, 0, kt);
+      if (to == 0) continue;
+      t.n_base = u.n_base = 0;  // rows of B, then of X
+      t.m_base = u.m_base = int64_t(r.n_slots(t)) * t.slot;  // columns of X, then of R
+      r.conv(t, q, kOpBr, kOpB);
+      r.product(t, q, to);
+      r.conv(u, q, kOpXr, kOpRc);
+      r.product(u, q, uo);
+      kernels += 6;
+    }
+    pf.end(a, P_PANEL, st, 0.0, 0.0, kernels);
+  }
+  auto slots = [&](int f) { return gen_schur_slots(dims_of(s[f], m[f], p0, 0, b)); };
+  for (const Piece& q : pieces_of(nact, sh.nb, sc.plane_bytes, true, slots)) {
+    const int kt = (std::min(rns_block(b), s[q.f0] - p0) + kK - 1) / kK;
+    Job l, u, x;
+    const int lo = r.job(l, kPanel, q, p0, 0, kt), uo = r.job(u, kSchur, q, p0, 0, kt), xo = r.job(x, kPanelU, q, p0, 0, kt);
+    if (lo == 0) continue;
+    const int64_t rows = int64_t(r.n_slots(l)) * l.slot;
+    l.n_base = u.n_base = 0;       // W, then L
+    u.m_base = x.m_base = rows;    // A[B,S]
+    l.m_base = x.n_base = 2 * rows;  // columns, then rows of B^-1
+    double fl = 0, sfl = 0;
+    if (pf.on)
+      for (int f = q.f0; f < q.f0 + q.nf; ++f) {
+        const Dims d = dims_of(s[f], m[f], p0, 0, b);
+        fl += 16.0 * q.np * d.mp * double(d.bw) * d.bw;
+        sfl += 8.0 * q.np * double(d.mp) * d.mp * d.bw;
+      }
+    cudaEvent_t a = pf.begin(st);
+    r.conv(l, q, kOpW, kOpB);
+    r.product(l, q, lo);
+    r.conv(u, q, kOpL, kOpA);
+    r.conv(x, q, kOpXr);
+    r.product(x, q, xo);
+    pf.end(a, P_PANEL, st, fl, 0.0, 7, fl * kRnsModuli);
+    a = pf.begin(st);
+    r.product(u, q, uo);
+    pf.end(a, P_SCHUR, st, sfl, 0.0, 2, sfl * kRnsModuli);
+  }
+}
+
+void rns_selinv_block_gen(const RnsScratch& sc, double2* Y, double2* F, const DevFronts& fr, const int32_t* dfr,
+                          const int32_t* s, const int32_t* m, int nact, int p0, int b, int nb, Profiler& pf,
+                          cudaStream_t st) {
+  Runner<double2> r{sc, fr, F, Y, dfr, s, m, b, st, 1};
+  auto slots = [&](int f) { return tak_slots(dims_of(s[f], m[f], p0, 0, b)); };
+  for (const Piece& q : pieces_of(nact, nb, sc.plane_bytes, true, slots)) {
+    int k = 32;
+    double fl = 0;
+    for (int f = q.f0; f < q.f0 + q.nf; ++f) {
+      const Dims d = dims_of(s[f], m[f], p0, 0, b);
+      k = std::max(k, d.mp);
+      fl += 16.0 * q.np * double(d.bw) * d.mp * (q.rtn > 0 ? double(q.rtn) * kRnsTile : d.mp);
+    }
+    const int kt = (k + kK - 1) / kK;
+    Job t, u, g;
+    const int to = r.job(t, kTak, q, p0, 0, kt), uo = r.job(u, kTakU, q, p0, 0, kt), go = r.job(g, kDiag, q, p0, 0, kt);
+    const bool last = q.rtn == 0 || q.rt0 + q.rtn >= tiles128(dims_of(s[q.f0], m[q.f0], p0, 0, b).mp);
+    // the panel operand (columns of L, then rows of U), then the rows or columns of Y[S,S], then the columns of Y[S,B]
+    t.m_base = u.n_base = g.n_base = 0;
+    t.n_base = u.m_base = g.m_base = int64_t(r.m_slots(t)) * t.slot;
+    if (to > 0) {
+      cudaEvent_t a = pf.begin(st);
+      r.conv(t, q, kOpLt, kOpYr);
+      r.product(t, q, to);
+      r.conv(u, q, kOpUr, kOpYc);
+      r.product(u, q, uo);
+      pf.end(a, P_OFFDIAG, st, fl, 0.0, 6, fl * kRnsModuli);
+    }
+    if (last) {
+      cudaEvent_t a = pf.begin(st);
+      if (to > 0) r.conv(g, q, kOpYtc);
       r.product(g, q, go);
       pf.end(a, P_DPART, st, 0.0, 0.0, 3);
     }

@@ -141,3 +141,22 @@ def test_both_block_inverses_give_the_same_bits(n):
     px.pexsi_plan_destroy(plan)
     for p in host:
         px.pexsi_plan_destroy(p)
+
+
+@pytest.mark.parametrize("n", [1, 64, 65, 129, 256, 257, 321, 520])
+def test_one_hermitian_front(n):
+    """LDU fronts: rows and columns of every product are different operands."""
+    colptr, rowind, H, S = _full(n, 5 * n)
+    rng = np.random.default_rng(n)
+    A, B = rng.standard_normal((n, n)) / np.sqrt(n), 0.05 * rng.standard_normal((n, n)) / n
+    H, S = H + 1j * (A - A.T), S + 1j * (B - B.T)
+    z = 0.1 + 0.05j
+    plan = px.pexsi_setup(n, colptr, rowind, opts=px.pexsi_opts_default(max_batch=2))
+    got = px.pexsi_selinv_hermitian(plan, H.T.ravel(), S.T.ravel(), z).reshape(n, n).T
+    shifts = np.array([-0.4, 0.2, 0.9])
+    counts = px.pexsi_inertia_hermitian(plan, H.T.ravel(), S.T.ravel(), shifts)
+    px.pexsi_plan_destroy(plan)
+    ref = np.linalg.inv(H - z * S)
+    assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref).max()
+    ev = np.linalg.eigvalsh(np.linalg.solve(np.linalg.cholesky(S), np.linalg.solve(np.linalg.cholesky(S), H).conj().T))
+    assert np.array_equal(counts, [(ev < x).sum() for x in shifts])
