@@ -317,7 +317,7 @@ void factor_batch(const pexsi_plan* p, Workspace& ws, T* F, const BatchShifts& s
       for (int p0 = 0; p0 < lv.max_s; p0 += rns_block(b)) {
         int nact = 0;
         while (nact < int(lv.s.size()) && lv.s[nact] > p0) ++nact;
-        rns_factor_block<T>(sc, F, reinterpret_cast<T*>(ws.Y), fr, dfr, lv.s.data(), lv.m.data(), nact, p0, b, sh, status, count, pf, st);
+        rns_factor_block<T>(p, lv, sc, F, reinterpret_cast<T*>(ws.Y), nact, p0, sh, status, pf, st);
       }
       continue;
     }
@@ -440,7 +440,7 @@ void selinv_batch(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh, Pro
       for (int p0 = (lv.max_s - 1) / rns_block(b) * rns_block(b); p0 >= 0; p0 -= rns_block(b)) {
         int nact = 0;
         while (nact < int(lv.s.size()) && lv.s[nact] > p0) ++nact;
-        rns_selinv_block(sc, ws.Y, ws.F, fr, dfr, lv.s.data(), lv.m.data(), nact, p0, b, sh.nb, pf, st);
+        rns_selinv_block(p, lv, sc, ws.Y, ws.F, nact, p0, sh.nb, pf, st);
       }
       continue;
     }
@@ -756,7 +756,7 @@ void factor_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
       for (int p0 = 0; p0 < lv.max_s; p0 += rns_block(b)) {
         int nact = 0;
         while (nact < int(lv.s.size()) && lv.s[nact] > p0) ++nact;
-        rns_factor_block_gen(sc, ws.F, ws.Y, fr, dfr, lv.s.data(), lv.m.data(), nact, p0, b, sh, status, pf, st);
+        rns_factor_block_gen(p, lv, sc, ws.F, ws.Y, nact, p0, sh, status, pf, st);
       }
       continue;
     }
@@ -799,7 +799,7 @@ void selinv_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
       for (int p0 = (lv.max_s - 1) / rns_block(b) * rns_block(b); p0 >= 0; p0 -= rns_block(b)) {
         int nact = 0;
         while (nact < int(lv.s.size()) && lv.s[nact] > p0) ++nact;
-        rns_selinv_block_gen(sc, ws.Y, ws.F, fr, dfr, lv.s.data(), lv.m.data(), nact, p0, b, sh.nb, pf, st);
+        rns_selinv_block_gen(p, lv, sc, ws.Y, ws.F, nact, p0, sh.nb, pf, st);
       }
       continue;
     }
@@ -1156,6 +1156,7 @@ void build_levels(pexsi_plan* p, std::vector<int32_t>& level_fronts, std::vector
     for (int32_t K : fr) {
       lv.s.push_back(S.s(K));
       lv.m.push_back(S.m(K));
+      lv.off.push_back(S.front_off[K]);
       lv.max_s = std::max(lv.max_s, S.s(K));
       level_fronts.push_back(K);
       int64_t r = S.r(K);

@@ -46,6 +46,7 @@ inline void ck(cudaError_t e, const char* what) {
 struct Level {
   int64_t front_off = 0;  // into the device list of level fronts
   std::vector<int32_t> fronts, s, m;
+  std::vector<int64_t> off;      // the fronts' offsets in one pole's pool
   std::vector<int64_t> ea_off;   // extend-add groups: rank k = k-th child of each parent
   std::vector<int32_t> ea_count, ea_tiles;
   std::vector<double> ea_elems;  // elements moved by each extend-add launch
@@ -210,19 +211,18 @@ constexpr int64_t kRnsPlaneBytes = int64_t(2) << 30;  // default of `most`
 // residue scratch where that fits too (planes, out; 0 without); 0: none fits.
 int fit_batch(const pexsi_plan* p, int64_t budget, int most, int64_t& planes, int64_t& out);
 
+// One block of columns [p0, p0 + 256) of a level's first nact fronts (those
+// with s > p0) through the residue products: elimination, and selected
+// inversion; _gen: LDU fronts.
 template <typename T>
-void rns_factor_block(const RnsScratch& sc, T* F, T* Y, const DevFronts& fr, const int32_t* dfr, const int32_t* s,
-                      const int32_t* m, int nact, int p0, int b, const BatchShifts& sh, DevStatus status, bool count,
-                      Profiler& pf, cudaStream_t st);
-void rns_factor_block_gen(const RnsScratch& sc, double2* F, double2* Y, const DevFronts& fr, const int32_t* dfr,
-                          const int32_t* s, const int32_t* m, int nact, int p0, int b, const BatchShifts& sh,
-                          DevStatus status, Profiler& pf, cudaStream_t st);
-void rns_selinv_block_gen(const RnsScratch& sc, double2* Y, double2* F, const DevFronts& fr, const int32_t* dfr,
-                          const int32_t* s, const int32_t* m, int nact, int p0, int b, int nb, Profiler& pf,
-                          cudaStream_t st);
-void rns_selinv_block(const RnsScratch& sc, double2* Y, double2* F, const DevFronts& fr, const int32_t* dfr,
-                      const int32_t* s, const int32_t* m, int nact, int p0, int b, int nb, Profiler& pf,
-                      cudaStream_t st);
+void rns_factor_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, T* F, T* Y, int nact, int p0,
+                      const BatchShifts& sh, DevStatus status, Profiler& pf, cudaStream_t st);
+void rns_selinv_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, double2* Y, double2* F, int nact,
+                      int p0, int nb, Profiler& pf, cudaStream_t st);
+void rns_factor_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, double2* F, double2* Y, int nact,
+                          int p0, const BatchShifts& sh, DevStatus status, Profiler& pf, cudaStream_t st);
+void rns_selinv_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, double2* Y, double2* F, int nact,
+                          int p0, int nb, Profiler& pf, cudaStream_t st);
 
 // Allocates ws for `batch` poles on `stream` (cudaMallocAsync when async),
 // with residue scratch of the given sizes (0: none).

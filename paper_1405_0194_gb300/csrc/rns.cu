@@ -77,11 +77,13 @@ __host__ __device__ constexpr int piece_coef(int l, int j, bool scaled) {
 __host__ __device__ constexpr uint32_t limb(u128 v, int j) {
   return j == 0 ? uint32_t(v & 0xFFFFF) : j == 1 ? uint32_t(v >> 20) : j == 2 ? uint32_t(v >> 52) : uint32_t(v >> 84);
 }
-// The residues are stored as r + 128: minus 128 times the sum of the cofactors' limbs.
-__host__ __device__ constexpr long long limb_bias(int j) {
-  long long s = 0;
-  for (int l = 0; l < kRnsModuli; ++l) s += limb(cofactor(l), j);
-  return -128 * s;
+// The residues are stored as r + 128, so the sum of the bytes times the cofactors
+// exceeds the integer by 128 times the sum of the cofactors and a multiple of P:
+// limbs of what is added to it to leave the integer plus a non-negative multiple.
+__host__ __device__ constexpr u128 byte_bias() {
+  u128 s = 0;
+  for (int l = 0; l < kRnsModuli; ++l) s = (s + 128 * (cofactor(l) % mod_product())) % mod_product();
+  return 2 * mod_product() - s;
 }
 
 constexpr int kBeta = 58;       // bits of the scaled integers
@@ -129,7 +131,12 @@ struct Job {
   int kt;                    // K tiles of a slot
   int64_t slot, n_base, m_base;
   int pref_n[kRnsFronts + 1], pref_m[kRnsFronts + 1], pref_o[kRnsFronts + 1];
+  // the fronts' sizes and places: as kernel arguments they cost no chain of global loads per item or block
+  int s[kRnsFronts], m[kRnsFronts];
+  int64_t off[kRnsFronts], pool;
 };
+
+static_assert(sizeof(Job) <= 3968, "kernel arguments hold 4 KiB");
 
 struct Dims {
   int s, m, bw, q0, mp, pb;
@@ -296,8 +303,8 @@ __device__ __forceinline__ int row_exponent(uint32_t mx, float sum, int count) {
 // r = tid % 8, octet o of OC) reads entries 8 o .. 8 o + 7 of its row, twice
 // when K > 8 OC (norm, then residues).
 template <typename T, int OC>
-__global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, const T* __restrict__ Y, DevFronts fr,
-                                                     const int32_t* __restrict__ fronts, const __grid_constant__ Job j,
+__global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, const T* __restrict__ Y,
+                                                     const __grid_constant__ Job j,
                                                      uint8_t* __restrict__ planes, int op_a, int nblk_a, int op_b) {
   constexpr bool CPLX = sizeof(T) == 16;
   constexpr int G = 32 / OC;  // row groups per block
@@ -321,11 +328,10 @@ __global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, co
   int64_t sk = 0;
   if (in) {
     const int pole = flat / per, x = flat - pole * per, fi = owner(pref, j.nf, x);
-    const int f = fronts[fi];
-    d = dims_of(fr.s[f], fr.m[f], j.p0, j.pc, j.b);
+    d = dims_of(j.s[fi], j.m[fi], j.p0, j.pc, j.b);
     const int rt = x - pref[fi] + (ms ? j.mt0 : j.rt0);
     row = rt * kRnsTile + (grp & 15) * 8 + r;
-    const int64_t base = int64_t(j.pole0 + pole) * fr.pool + fr.off[f], m = d.m;
+    const int64_t base = int64_t(j.pole0 + pole) * j.pool + j.off[fi], m = d.m;
     int64_t si = 1;
     switch (op) {
       case kOpV: case kOpT: src = F + base + j.p0 + m * (j.p0 + j.pc); rows = d.bw; K = d.pb; sk = m; break;
@@ -438,8 +444,7 @@ __constant__ float c_mod[kRnsModuli] = {256, 253, 251, 247, 241, 239, 233, 229, 
 // chunk's accumulator is reduced in place while the other one fills, and
 // carries its residue on.
 template <bool CPLX>
-__global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(DevFronts fr, const int32_t* __restrict__ fronts,
-                                                          const __grid_constant__ Job j,
+__global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant__ Job j,
                                                           const uint8_t* __restrict__ planes, uint8_t* __restrict__ out,
                                                           int* __restrict__ gfail, uint64_t wait_ns) {
   constexpr int C = CPLX ? 2 : 1;
@@ -481,8 +486,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(DevFronts fr, const in
   auto decode = [&](int it, int& l, OutTile& t, int& rn, int& rm) -> int {
     l = it / j.on;
     t = out_tile(j, j.o0 + it - l * j.on);
-    const int f = fronts[t.f];
-    const Dims d = dims_of(fr.s[f], fr.m[f], j.p0, j.pc, j.b);
+    const Dims d = dims_of(j.s[t.f], j.m[t.f], j.p0, j.pc, j.b);
     int k;
     product_dims(j.mode, d, j.b, rn, rm, k);
     return k <= 0 ? 0 : (k + kK - 1) / kK;
@@ -499,6 +503,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(DevFronts fr, const in
         const int64_t lo = int64_t(l) * j.kt * kOp;
         const uint8_t* gn = planes + j.n_base + (int64_t(t.pole) * j.pref_n[j.nf] + j.pref_n[t.f] + t.nt) * j.slot + lo;
         const uint8_t* gm = planes + j.m_base + (int64_t(t.pole) * j.pref_m[j.nf] + j.pref_m[t.f] + t.mt) * j.slot + lo;
+        // bytes of the 8-row groups that the tiles have, of each plane (a whole tile: both planes in one copy)
+        const uint32_t bn = uint32_t(min(kRnsTile, rn - (j.rt0 + t.nt) * kRnsTile) + 7) / 8 * 512,
+                       bm = uint32_t(min(kRnsTile, rm - (j.mt0 + t.mt) * kRnsTile) + 7) / 8 * 512;
         for (int kt = 0; kt < nkt; ++kt, ++n) {
           const int st = n % kStages, u = n / kStages;
           if (u > 0 && !bar_wait(smem_u32(&empty[st]), (u - 1) & 1, fail, wait_ns)) {
@@ -506,9 +513,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(DevFronts fr, const in
             ok = false;
             break;
           }
-          bar_expect(smem_u32(&full[st]), 2 * kOp);
-          bulk_load(smem_u32(sm + st * 2 * kOp), gm + int64_t(kt) * kOp, kOp, smem_u32(&full[st]));
-          bulk_load(smem_u32(sm + st * 2 * kOp + kOp), gn + int64_t(kt) * kOp, kOp, smem_u32(&full[st]));
+          bar_expect(smem_u32(&full[st]), C * (bm + bn));
+          const uint32_t dst = smem_u32(sm + st * 2 * kOp), bar = smem_u32(&full[st]);
+          const uint8_t *pm = gm + int64_t(kt) * kOp, *pn = gn + int64_t(kt) * kOp;
+          bulk_load(dst, pm, bm == kPlane ? kOp : bm, bar);
+          if (CPLX && bm != kPlane) bulk_load(dst + kPlane, pm + kPlane, bm, bar);
+          bulk_load(dst + kOp, pn, bn == kPlane ? kOp : bn, bar);
+          if (CPLX && bn != kPlane) bulk_load(dst + kOp + kPlane, pn + kPlane, bn, bar);
         }
       }
       // every copy issued has landed before the CTA leaves (bounded)
@@ -624,29 +635,37 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(DevFronts fr, const in
       uint8_t* o = out + (int64_t(it - l * j.on) * kRnsModuli + l) * (C * kRnsTile * kRnsTile) +
                    (CPLX ? h * kRnsTile * kRnsTile : 0) + mrow * kRnsTile + (CPLX ? 0 : h * NC);
 #pragma unroll 1
-      for (int x = 0; x < NC; x += 16) {
+      for (int x = 0; x < NC; x += 32) {
         if ((CPLX ? 0 : h * NC) + x >= nn) break;
-        uint32_t v[16], w[16];
-        tmem_ld16_nw(a + x, v);
-        if (two) tmem_ld16_nw(a2 + x, w);
-        tmem_wait_ld();
+        uint32_t v[32];
+        tmem_ld32(a + x, v);
+        if (two) {
+          uint32_t w[32];
+          tmem_ld32(a2 + x, w);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float f = __uint_as_float(v[i]);
-          if (two) {
+          for (int i = 0; i < 32; ++i) {
             const float g = __uint_as_float(w[i]);
-            f += fmaf(fmaf(g, inv, 12582912.0f) - 12582912.0f, -p, g);
+            v[i] = __float_as_uint(__uint_as_float(v[i]) + fmaf(fmaf(g, inv, 12582912.0f) - 12582912.0f, -p, g));
           }
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
           // r + 128 in the low byte (r = 128 of p = 256 wraps to its other representative)
+          const float f = __uint_as_float(v[i]);
           v[i] = __float_as_uint(fmaf(fmaf(f, inv, 12582912.0f) - 12582912.0f, -p, f) + 12583040.0f);
         }
-        uint4 b;
-        uint32_t* bw = &b.x;
+        if (m_in) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          bw[i] = __byte_perm(__byte_perm(v[4 * i], v[4 * i + 1], 0x0040), __byte_perm(v[4 * i + 2], v[4 * i + 3], 0x0040),
-                              0x5410);
-        if (m_in) *reinterpret_cast<uint4*>(o + x) = b;
+          for (int y = 0; y < 2; ++y) {
+            uint32_t bw[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const uint32_t* z = v + 16 * y + 4 * i;
+              bw[i] = __byte_perm(__byte_perm(z[0], z[1], 0x0040), __byte_perm(z[2], z[3], 0x0040), 0x5410);
+            }
+            *reinterpret_cast<uint4*>(o + x + 16 * y) = make_uint4(bw[0], bw[1], bw[2], bw[3]);
+          }
+        }
       }
       if (two) release(u - 1);
       release(u);
@@ -663,216 +682,179 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(DevFronts fr, const in
 }
 
 // ------------------------------------------------------------ reconstruction
-// v 2^sc of a 128-bit integer, from its 64 leading bits, rounded to nearest.
-__device__ __forceinline__ double i128_scaled(i128 v, int sc) {
-  if (v == 0) return 0.0;
-  const unsigned long long sign = v < 0 ? (1ull << 63) : 0ull;
-  const u128 a = v < 0 ? u128(-v) : u128(v);
-  unsigned long long hi = static_cast<unsigned long long>(a >> 64), lo = static_cast<unsigned long long>(a);
-  int lz;
-  if (hi == 0) {
-    lz = 64 + __clzll(static_cast<long long>(lo));
-    hi = lo;
-    lo = 0;
-  } else {
-    lz = __clzll(static_cast<long long>(hi));
-  }
-  const int s = lz & 63;
-  const unsigned long long top = s ? (hi << s) | (lo >> (64 - s)) : hi;
-  unsigned long long mant = top >> 11;
-  const unsigned long long rest = top & 0x7FFull;
-  if (rest > 0x400ull || (rest == 0x400ull && (mant & 1ull))) ++mant;
-  int E = 127 - lz + sc + 1023;
-  if (mant >> 53) {
-    mant >>= 1;
-    ++E;
-  }
-  if (E <= 0 || E >= 2047) return ldexp(sign ? -static_cast<double>(mant) : static_cast<double>(mant), E - 1075);
-  return __longlong_as_double(static_cast<long long>(sign | (static_cast<unsigned long long>(E) << 52) | (mant & 0xFFFFFFFFFFFFFull)));
-}
-
-// The integer of magnitude below P / 2 whose residues (plus 128) are byte
-// `b` of w: sum of u_l P / p_l less a multiple of P, exactly, in limbs.
+// X 2^sc, X the integer of magnitude below 2^116 whose residues (plus 128) are
+// byte `b` of w: the sum of u_l P / p_l less a multiple of P, exactly, in limbs of
+// 20, 32, 32 and 34 bits, rounded to the nearest double from its 64 leading bits.
 __device__ __forceinline__ double from_residues(const uint32_t (&w)[kRnsModuli], int b, int sc) {
+  constexpr u128 P = mod_product(), B = byte_bias();
   uint32_t a0 = 0;
-  unsigned long long a1 = 0, a2 = 0, a3 = 0;
+  unsigned long long a1 = limb(B, 1), a2 = limb(B, 2), a3 = static_cast<unsigned long long>(B >> 84);
   each_modulus([&](auto LC) {
     constexpr int l = decltype(LC)::value;
     constexpr uint32_t l0 = limb(cofactor(l), 0), l1 = limb(cofactor(l), 1), l2 = limb(cofactor(l), 2),
                        l3 = limb(cofactor(l), 3);
-    const uint32_t u = (w[l] >> (8 * b)) & 255u;
+    const uint32_t u = __byte_perm(w[l], 0u, 0x4440 + b);
     a0 += u * l0;
     a1 += static_cast<unsigned long long>(u) * l1;
     a2 += static_cast<unsigned long long>(u) * l2;
     a3 += static_cast<unsigned long long>(u) * l3;
   });
-  constexpr u128 P = mod_product();
-  constexpr long long b0 = limb_bias(0), b1 = limb_bias(1), b2 = limb_bias(2), b3 = limb_bias(3);
-  const long long s0 = static_cast<long long>(a0) + b0, s1 = static_cast<long long>(a1) + b1,
-                  s2 = static_cast<long long>(a2) + b2, s3 = static_cast<long long>(a3) + b3;
-  // the multiple of P, from the leading limb alone: |value| <= 2^116 against P / 2 > 2^116.3, and what the
-  // lower limbs and the float rounding leave out is below 2^-9 of P
-  constexpr float pinv = float(1.0 / (double(P >> 60) * double(1ull << 60)) * 19342813113834066795298816.0);  // 2^84 / P
-  const int k = __float2int_rn(__int2float_rn(static_cast<int>(s3 >> 8)) * (256.0f * pinv));
-  const i128 v = i128(s0) + (i128(s1) << 20) + (i128(s2) << 52) + (i128(s3) << 84) - i128(k) * i128(P);
-  return i128_scaled(v, sc);
+  // The multiple of P, from the leading limb alone: |X| <= 2^116 against P / 2 > 2^116.3, and what the lower limbs
+  // and the float rounding leave out is below 2^-9 of P. It lies between 0 and 22.
+  constexpr float pinv = float(19342813113834066795298816.0 / (double(P >> 60) * double(1ull << 60)));  // 2^84 / P
+  const uint32_t k = uint32_t(__float2int_rn(__uint2float_rn(uint32_t(a3 >> 8)) * (256.0f * pinv)));
+  constexpr uint32_t p0 = limb(P, 0), p1 = limb(P, 1), p2 = limb(P, 2);
+  constexpr unsigned long long p3 = static_cast<unsigned long long>(P >> 84);
+  const long long s0 = static_cast<long long>(a0) + static_cast<long long>(limb(B, 0)) - static_cast<long long>(k * p0);
+  const long long s1 = static_cast<long long>(a1 - static_cast<unsigned long long>(k) * p1) + (s0 >> 20);
+  const long long s2 = static_cast<long long>(a2 - static_cast<unsigned long long>(k) * p2) + (s1 >> 32);
+  const long long s3 = static_cast<long long>(a3 - k * p3) + (s2 >> 32);
+  // magnitude m3 2^84 + m2 2^52 + low (m3 < 2^32, low < 2^52)
+  const bool neg = s3 < 0;
+  const uint32_t flip = neg ? 0xFFFFFFFFu : 0u;
+  const unsigned long long flip52 = neg ? 0xFFFFFFFFFFFFFull : 0ull;
+  unsigned long long low = (static_cast<unsigned long long>(uint32_t(s1)) << 20) | (static_cast<uint32_t>(s0) & 0xFFFFFu);
+  low = (low ^ flip52) + (neg ? 1u : 0u);
+  const unsigned long long mid = static_cast<unsigned long long>(uint32_t(s2) ^ flip) + (low >> 52);
+  uint32_t A = (uint32_t(static_cast<unsigned long long>(s3)) ^ flip) + uint32_t(mid >> 32), Bw = uint32_t(mid),
+           Cw = uint32_t(low >> 20), Dw = uint32_t(low) << 12;
+  int E = 1023 + 84 + 31 + sc;  // biased exponent of bit 31 of A
+#pragma unroll
+  for (int t = 0; t < 3; ++t)
+    if (A == 0) {
+      A = Bw;
+      Bw = Cw;
+      Cw = Dw;
+      Dw = 0;
+      E -= 32;
+    }
+  if (A == 0) return 0.0;
+  const int lz = __clz(A);
+  const uint32_t hi = __funnelshift_l(Bw, A, lz), lo = __funnelshift_l(Cw, Bw, lz);
+  unsigned long long mant = ((static_cast<unsigned long long>(hi) << 32) | lo) >> 11;  // 53 bits
+  const uint32_t rest = lo & 0x7FFu;
+  mant += rest > 0x400u || (rest == 0x400u && (mant & 1ull)) ? 1u : 0u;
+  E -= lz;
+  if (E <= 0 || E >= 2046) {
+    const double v = ldexp(static_cast<double>(mant), E - 1023 - 52);
+    return neg ? -v : v;
+  }
+  // the leading bit adds 1 to the exponent field, and so does a carry out of the mantissa
+  return __longlong_as_double(static_cast<long long>((neg ? 1ull << 63 : 0ull) +
+                                                     (static_cast<unsigned long long>(E - 1) << 52) + mant));
 }
 
-__device__ __forceinline__ double nan_of() { return __longlong_as_double(0x7FF8000000000000LL); }
-__device__ __forceinline__ double sub(double a, double b) { return a - b; }
-__device__ __forceinline__ double2 sub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ double neg(double a) { return -a; }
-__device__ __forceinline__ double2 neg(double2 a) { return make_double2(-a.x, -a.y); }
-__device__ __forceinline__ double one_of(double) { return 1.0; }
-__device__ __forceinline__ double2 one_of(double2) { return make_double2(1.0, 0.0); }
-__device__ __forceinline__ double half_sum(double a, double b) { return 0.5 * (a + b); }
-__device__ __forceinline__ double2 half_sum(double2 a, double2 b) {
-  return make_double2(0.5 * (a.x + b.x), 0.5 * (a.y + b.y));
-}
+// One thread per part (re, im) of 4 consecutive front rows of a front column,
+// over the rows and columns that the output tile really has (small fronts fill
+// a few of its 128 x 128 entries): front columns are rows of M, front rows
+// (contiguous in memory) rows of N. Everything a product does to F or Y acts on
+// the parts alone. One thread's integers are a serial chain of some 600
+// instructions, so the small products of the diagonal blocks want many threads:
+// two units of both parts per thread took 17 us for a 256 x 256 block.
+constexpr int kReconThreads = 128;
 
-// One block per output tile and 16 of its rows of M (front columns): a warp
-// takes 2 of them, a lane 4 consecutive rows of N (front rows, contiguous in
-// memory).
 template <typename T>
-__global__ void __launch_bounds__(256) k_rns_recon(T* __restrict__ F, T* __restrict__ Y, DevFronts fr,
-                                                   const int32_t* __restrict__ fronts, const __grid_constant__ Job j,
-                                                   const uint8_t* __restrict__ planes, const uint8_t* __restrict__ out) {
-  constexpr bool CPLX = sizeof(T) == 16;
-  constexpr int C = CPLX ? 2 : 1;
+__global__ void __launch_bounds__(kReconThreads) k_rns_recon(double* __restrict__ F, double* __restrict__ Y,
+                                                             const __grid_constant__ Job j,
+                                                             const uint8_t* __restrict__ planes,
+                                                             const uint8_t* __restrict__ out) {
+  constexpr int C = sizeof(T) / sizeof(double);
   const OutTile t = out_tile(j, j.o0 + int(blockIdx.x));
-  const int f = fronts[t.f];
-  const Dims d = dims_of(fr.s[f], fr.m[f], j.p0, j.pc, j.b);
+  const Dims d = dims_of(j.s[t.f], j.m[t.f], j.p0, j.pc, j.b);
   int rn, rm, K;
   product_dims(j.mode, d, j.b, rn, rm, K);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = (j.rt0 + t.nt) * kRnsTile + lane * 4;
-  const int64_t base = int64_t(j.pole0 + t.pole) * fr.pool + fr.off[f], m = d.m;
-  const int tail = kRnsTile * int(sizeof(int));
-  const int* en = reinterpret_cast<const int*>(planes + j.n_base +
-                                               (int64_t(t.pole) * j.pref_n[j.nf] + j.pref_n[t.f] + t.nt + 1) * j.slot - tail);
-  const int* em = reinterpret_cast<const int*>(planes + j.m_base +
-                                               (int64_t(t.pole) * j.pref_m[j.nf] + j.pref_m[t.f] + t.mt + 1) * j.slot - tail);
-  const bool last = j.pc + d.pb == d.bw;
-#pragma unroll 1
-  for (int x = 0; x < 2; ++x) {
-    const int mr = int(blockIdx.y) * 16 + warp * 2 + x, c = (j.mt0 + t.mt) * kRnsTile + mr;
-    if (c >= rm || n0 >= rn) continue;
-    if (triangular(j.mode, j.gen) && n0 + 3 < c) continue;
-    T v[4];
-    if (K > 0) {
-      const int eb = em[mr];
-      int ea[4];
+  const int row0 = (j.rt0 + t.nt) * kRnsTile, col0 = (j.mt0 + t.mt) * kRnsTile;
+  const int quads = (min(kRnsTile, rn - row0) + 3) / 4, units = C * quads * min(kRnsTile, rm - col0);
+  const int unit = int(blockIdx.y) * kReconThreads + threadIdx.x;
+  if (unit >= units) return;
+  const int part = unit % C, x = unit / C, mr = x / quads, q = x - mr * quads, c = col0 + mr, n0 = row0 + q * 4;
+  const bool tri = triangular(j.mode, j.gen);
+  if (tri && n0 + 3 < c) return;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  if (K > 0) {
+    const int tail = kRnsTile * int(sizeof(int));
+    const int* en = reinterpret_cast<const int*>(planes + j.n_base +
+                                                 (int64_t(t.pole) * j.pref_n[j.nf] + j.pref_n[t.f] + t.nt + 1) * j.slot - tail);
+    const int* em = reinterpret_cast<const int*>(planes + j.m_base +
+                                                 (int64_t(t.pole) * j.pref_m[j.nf] + j.pref_m[t.f] + t.mt + 1) * j.slot - tail);
+    uint32_t w[kRnsModuli];
+    const uint8_t* src = out + int64_t(blockIdx.x) * kRnsModuli * (C * kRnsTile * kRnsTile) + part * kRnsTile * kRnsTile +
+                         mr * kRnsTile + q * 4;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) ea[i] = n0 + i < rn ? en[lane * 4 + i] : 0;
+    for (int l = 0; l < kRnsModuli; ++l)
+      w[l] = *reinterpret_cast<const uint32_t*>(src + int64_t(l) * (C * kRnsTile * kRnsTile));
+    const int eb = em[mr];
+    int ea[4];
 #pragma unroll
-      for (int part = 0; part < C; ++part) {
-        uint32_t w[kRnsModuli];
-        const uint8_t* src = out + int64_t(blockIdx.x) * kRnsModuli * (C * kRnsTile * kRnsTile) +
-                             part * kRnsTile * kRnsTile + mr * kRnsTile + lane * 4;
-#pragma unroll
-        for (int l = 0; l < kRnsModuli; ++l)
-          w[l] = *reinterpret_cast<const uint32_t*>(src + int64_t(l) * (C * kRnsTile * kRnsTile));
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          double r = from_residues(w, i, ea[i] + eb - 2 * kBeta);
-          if (ea[i] == kNanRow || eb == kNanRow) r = nan_of();
-          if constexpr (CPLX) {
-            if (part) v[i].y = r;
-            else v[i].x = r;
-          } else {
-            v[i] = r;
-          }
-        }
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] = T{};
-    }
+    for (int i = 0; i < 4; ++i) ea[i] = n0 + i < rn ? en[q * 4 + i] : 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int r = n0 + i;
-      if (r >= rn) break;
-      if (j.gen) {
-        const bool in_r = r >= j.pc && r < j.pc + d.pb, in_c = c >= j.pc && c < j.pc + d.pb;
-        const T minus = neg(v[i]);
-        T* fb = F + base + m * j.p0 + j.p0;  // the diagonal block
-        T* yb = Y + base + m * j.p0 + j.p0;
-        switch (j.mode) {
-          case kSweepT: if (!in_r) fb[m * (j.pc + c) + r] = minus; break;
-          case kSweepDU: if (!in_c) fb[m * c + j.pc + r] = v[i]; break;
-          // T is stored negated
-          case kSweepU: if (!in_r && !in_c) fb[m * c + r] = sub(fb[m * c + r], minus); break;
-          case kResid: yb[m * c + r] = r == c ? sub(one_of(minus), v[i]) : minus; break;
-          case kRefine: fb[m * c + r] = sub(fb[m * c + r], minus); break;
-          case kPanel: F[base + m * (j.p0 + c) + d.q0 + r] = v[i]; break;
-          case kPanelU: F[base + m * (d.q0 + c) + j.p0 + r] = v[i]; break;
-          case kSchur: {
-            T* e = F + base + m * (d.q0 + c) + d.q0 + r;
-            *e = sub(*e, v[i]);
-            break;
-          }
-          case kTak: Y[base + m * (j.p0 + c) + d.q0 + r] = minus; break;
-          case kTakU: Y[base + m * (d.q0 + c) + j.p0 + r] = minus; break;
-          default: yb[m * c + r] = sub(fb[m * c + r], v[i]); break;  // kDiag
+      v[i] = from_residues(w, i, ea[i] + eb - 2 * kBeta);
+      if (ea[i] == kNanRow || eb == kNanRow) v[i] = __longlong_as_double(0x7FF8000000000000LL);
+    }
+  }
+  // this part of the front, of its diagonal block and of the same places in Y; the columns' stride
+  const int64_t m = int64_t(C) * d.m, base = C * (int64_t(j.pole0 + t.pole) * j.pool + j.off[t.f]) + part;
+  double *fb = F + base + m * j.p0 + C * j.p0, *yb = Y + base + m * j.p0 + C * j.p0;
+  const int below = C * d.bw;  // from the diagonal block's rows to the rows below it
+  const bool in_c = c >= j.pc && c < j.pc + d.pb, last = j.pc + d.pb == d.bw;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = n0 + i;
+    if (r >= rn || (tri && r < c)) continue;
+    const bool in_r = r >= j.pc && r < j.pc + d.pb;
+    double* at = fb + m * c + C * r;   // entry (r, c) of the diagonal block
+    double* to = fb + m * r + C * c;   // and (c, r)
+    switch (j.mode) {
+      case kSweepT: {  // column c of the panel; a symmetric block holds minus the inverse until the last panel's sweep
+        double* e = fb + m * (j.pc + c) + C * r;
+        if (j.gen) {
+          if (!in_r) *e = -v[i];
+        } else if (in_r) {
+          if (!last) *e = -*e;
+        } else {
+          const double val = last ? -v[i] : v[i];
+          *e = val;
+          fb[m * r + C * (j.pc + c)] = val;
         }
-        continue;
+        break;
       }
-      switch (j.mode) {
-        case kSweepT: {  // column c of the panel; the block holds minus the inverse until the last panel's sweep
-          T* col = F + base + m * (j.p0 + j.pc + c) + j.p0;
-          if (r >= j.pc && r < j.pc + d.pb) {
-            if (!last) col[r] = neg(col[r]);
-          } else {
-            const T val = last ? neg(v[i]) : v[i];
-            col[r] = val;
-            F[base + m * (j.p0 + r) + j.p0 + j.pc + c] = val;
-          }
-          break;
+      case kSweepDU: if (!in_c) fb[m * c + C * (j.pc + r)] = v[i]; break;
+      case kSweepU: {
+        if (in_r || in_c) break;
+        if (j.gen) {  // T is stored negated
+          *at = *at + v[i];
+        } else {      // the last sweep's T is already negated, and so is its result
+          const double val = last ? -(*at + v[i]) : *at - v[i];
+          *at = val;
+          *to = val;
         }
-        case kSweepU: {
-          if (r < c || (r >= j.pc && r < j.pc + d.pb) || (c >= j.pc && c < j.pc + d.pb)) break;
-          T* e = F + base + m * (j.p0 + c) + j.p0 + r;
-          // the last sweep's T is already negated, and so is its result
-          const T val = last ? neg(sub(*e, neg(v[i]))) : sub(*e, v[i]);
-          *e = val;
-          F[base + m * (j.p0 + r) + j.p0 + c] = val;
-          break;
-        }
-        case kResid: {
-          T x = neg(v[i]);
-          if (r == c) x = sub(one_of(x), v[i]);
-          Y[base + m * (j.p0 + c) + j.p0 + r] = x;
-          break;
-        }
-        case kRefine: {
-          if (r < c) break;
-          T* e = F + base + m * (j.p0 + c) + j.p0 + r;
-          const T val = sub(*e, neg(v[i]));
-          *e = val;
-          F[base + m * (j.p0 + r) + j.p0 + c] = val;
-          break;
-        }
-        case kPanel: F[base + m * (j.p0 + c) + d.q0 + r] = v[i]; break;
-        case kSchur:
-          if (r >= c) {
-            T* e = F + base + m * (d.q0 + c) + d.q0 + r;
-            *e = sub(*e, v[i]);
-          }
-          break;
-        case kTak: {
-          const T val = neg(v[i]);
-          Y[base + m * (j.p0 + c) + d.q0 + r] = val;
-          Y[base + m * (d.q0 + r) + j.p0 + c] = val;
-          break;
-        }
-        default: {  // kDiag
-          if (r < c) break;
-          const T a = F[base + m * (j.p0 + c) + j.p0 + r], b = F[base + m * (j.p0 + r) + j.p0 + c];
-          const T val = sub(half_sum(a, b), v[i]);
-          Y[base + m * (j.p0 + c) + j.p0 + r] = val;
-          Y[base + m * (j.p0 + r) + j.p0 + c] = val;
-          break;
-        }
+        break;
+      }
+      case kResid: yb[m * c + C * r] = (r == c && part == 0 ? 1.0 : 0.0) - v[i]; break;
+      case kRefine: {
+        const double val = *at + v[i];
+        *at = val;
+        if (!j.gen) *to = val;
+        break;
+      }
+      case kPanel: fb[m * c + below + C * r] = v[i]; break;
+      case kPanelU: fb[m * (d.bw + c) + C * r] = v[i]; break;
+      case kSchur: {
+        double* e = fb + m * (d.bw + c) + below + C * r;
+        *e = *e - v[i];
+        break;
+      }
+      case kTak:
+        yb[m * c + below + C * r] = -v[i];
+        if (!j.gen) yb[m * (d.bw + r) + C * c] = -v[i];
+        break;
+      case kTakU: yb[m * (d.bw + c) + C * r] = -v[i]; break;
+      default: {  // kDiag
+        const double val = (j.gen ? *at : 0.5 * (*at + *to)) - v[i];
+        yb[m * c + C * r] = val;
+        if (!j.gen) yb[m * r + C * c] = val;
+        break;
       }
     }
   }
@@ -975,10 +957,10 @@ template <typename T>
 struct Runner {
   static constexpr bool CPLX = sizeof(T) == 16;
   const RnsScratch& sc;
-  DevFronts fr;
   T *F, *Y;
-  const int32_t* fronts;  // device list of the level
-  const int32_t *s, *m;   // the same on the host
+  const int32_t *s, *m;  // sizes of the level's fronts
+  const int64_t* off;    // and their places in a pole's pool
+  int64_t pool;
   int b;
   cudaStream_t st;
   int gen = 0;
@@ -997,8 +979,12 @@ struct Runner {
     j.mt0 = mode == kTakU ? q.rt0 : 0;
     j.kt = kt;
     j.slot = rns_slot_bytes(32 * kt, CPLX);
+    j.pool = pool;
     j.pref_n[0] = j.pref_m[0] = j.pref_o[0] = 0;
     for (int f = 0; f < q.nf; ++f) {
+      j.s[f] = s[q.f0 + f];
+      j.m[f] = m[q.f0 + f];
+      j.off[f] = off[q.f0 + f];
       int rn, rm, k;
       product_dims(mode, dims_of(s[q.f0 + f], m[q.f0 + f], p0, pc, b), b, rn, rm, k);
       const int tn = q.rtn > 0 && mode == kTak ? q.rtn : tiles128(rn), tm = q.rtn > 0 && mode == kTakU ? q.rtn : tiles128(rm);
@@ -1018,8 +1004,8 @@ struct Runner {
     auto blocks = [&](Operand op) { return ((m_side(op) ? m_slots(j) : n_slots(j)) * 16 + g - 1) / g; };
     const int na = blocks(a), n = na + (both ? blocks(c) : 0);
     if (n <= 0) return;
-    if (oc == 8) k_rns_conv<T, 8><<<n, 256, 0, st>>>(F, Y, fr, fronts + q.f0, j, sc.planes, a, na, c);
-    else k_rns_conv<T, 32><<<n, 256, 0, st>>>(F, Y, fr, fronts + q.f0, j, sc.planes, a, na, c);
+    if (oc == 8) k_rns_conv<T, 8><<<n, 256, 0, st>>>(F, Y, j, sc.planes, a, na, c);
+    else k_rns_conv<T, 32><<<n, 256, 0, st>>>(F, Y, j, sc.planes, a, na, c);
   }
 
   // The product and its reconstruction, in pieces of the output scratch.
@@ -1029,8 +1015,9 @@ struct Runner {
       j.o0 = o;
       j.on = std::min(cap, tiles - o);
       k_rns_gemm<CPLX><<<std::min(sms(), j.on * kRnsModuli), kThreads, kStages * 2 * (CPLX ? 2 : 1) * kPlane, st>>>(
-          fr, fronts + q.f0, j, sc.planes, sc.out, sc.fail, sc.wait_ns);
-      k_rns_recon<T><<<dim3(j.on, kRnsTile / 16), 256, 0, st>>>(F, Y, fr, fronts + q.f0, j, sc.planes, sc.out);
+          j, sc.planes, sc.out, sc.fail, sc.wait_ns);
+      k_rns_recon<T><<<dim3(j.on, (CPLX ? 2 : 1) * kRnsTile * kRnsTile / 4 / kReconThreads), kReconThreads, 0, st>>>(
+          reinterpret_cast<double*>(F), reinterpret_cast<double*>(Y), j, sc.planes, sc.out);
     }
   }
 };
@@ -1115,10 +1102,12 @@ int64_t rns_out_bytes(const pexsi_plan* p, int batch) {
 // first nact, those with s > p0): inverts the diagonal block, L[S,B] and the
 // update of F[S,S].
 template <typename T>
-void rns_factor_block(const RnsScratch& sc, T* F, T* Y, const DevFronts& fr, const int32_t* dfr, const int32_t* s,
-                      const int32_t* m, int nact, int p0, int b, const BatchShifts& sh, DevStatus status, bool count,
-                      Profiler& pf, cudaStream_t st) {
-  Runner<T> r{sc, fr, F, Y, dfr, s, m, b, st};
+void rns_factor_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, T* F, T* Y, int nact, int p0,
+                      const BatchShifts& sh, DevStatus status, Profiler& pf, cudaStream_t st) {
+  const int b = p->b, *s = lv.s.data(), *m = lv.m.data();
+  const DevFronts fr = p->fronts();
+  const int32_t* dfr = p->d_level_fronts + lv.front_off;
+  Runner<T> r{sc, F, Y, s, m, lv.off.data(), fr.pool, b, st};
   constexpr bool CPLX = sizeof(T) == 16;
   const int bw = std::min(rns_block(b), s[0] - p0);  // the widest front's block
   if (bw > b) k_rns_save<T><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b, 0);
@@ -1208,10 +1197,10 @@ void rns_factor_block(const RnsScratch& sc, T* F, T* Y, const DevFronts& fr, con
 }
 
 // Y[S,B], its mirror and Y[B,B] of the block at p0 of the level's first nact fronts.
-void rns_selinv_block(const RnsScratch& sc, double2* Y, double2* F, const DevFronts& fr, const int32_t* dfr,
-                      const int32_t* s, const int32_t* m, int nact, int p0, int b, int nb, Profiler& pf,
-                      cudaStream_t st) {
-  Runner<double2> r{sc, fr, F, Y, dfr, s, m, b, st};
+void rns_selinv_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, double2* Y, double2* F, int nact,
+                      int p0, int nb, Profiler& pf, cudaStream_t st) {
+  const int b = p->b, *s = lv.s.data(), *m = lv.m.data();
+  Runner<double2> r{sc, F, Y, s, m, lv.off.data(), p->sym.front_elems, b, st};
   auto slots = [&](int f) { return tak_slots(dims_of(s[f], m[f], p0, 0, b)); };
   for (const Piece& q : pieces_of(nact, nb, sc.plane_bytes, true, slots)) {
     int k = 32;
@@ -1248,10 +1237,12 @@ void rns_selinv_block(const RnsScratch& sc, double2* Y, double2* F, const DevFro
 }
 
 // The same for LDU fronts: B, X and the panels are not symmetric.
-void rns_factor_block_gen(const RnsScratch& sc, double2* F, double2* Y, const DevFronts& fr, const int32_t* dfr,
-                          const int32_t* s, const int32_t* m, int nact, int p0, int b, const BatchShifts& sh,
-                          DevStatus status, Profiler& pf, cudaStream_t st) {
-  Runner<double2> r{sc, fr, F, Y, dfr, s, m, b, st, 1};
+void rns_factor_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, double2* F, double2* Y, int nact,
+                          int p0, const BatchShifts& sh, DevStatus status, Profiler& pf, cudaStream_t st) {
+  const int b = p->b, *s = lv.s.data(), *m = lv.m.data();
+  const DevFronts fr = p->fronts();
+  const int32_t* dfr = p->d_level_fronts + lv.front_off;
+  Runner<double2> r{sc, F, Y, s, m, lv.off.data(), fr.pool, b, st, 1};
   const int bw = std::min(rns_block(b), s[0] - p0);
   const int kb = (b + kK - 1) / kK;
   if (bw > b) k_rns_save<double2><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b, 1);
@@ -1335,10 +1326,10 @@ void rns_factor_block_gen(const RnsScratch& sc, double2* F, double2* Y, const De
   }
 }
 
-void rns_selinv_block_gen(const RnsScratch& sc, double2* Y, double2* F, const DevFronts& fr, const int32_t* dfr,
-                          const int32_t* s, const int32_t* m, int nact, int p0, int b, int nb, Profiler& pf,
-                          cudaStream_t st) {
-  Runner<double2> r{sc, fr, F, Y, dfr, s, m, b, st, 1};
+void rns_selinv_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, double2* Y, double2* F, int nact,
+                          int p0, int nb, Profiler& pf, cudaStream_t st) {
+  const int b = p->b, *s = lv.s.data(), *m = lv.m.data();
+  Runner<double2> r{sc, F, Y, s, m, lv.off.data(), p->sym.front_elems, b, st, 1};
   auto slots = [&](int f) { return tak_slots(dims_of(s[f], m[f], p0, 0, b)); };
   for (const Piece& q : pieces_of(nact, nb, sc.plane_bytes, true, slots)) {
     int k = 32;
@@ -1372,11 +1363,9 @@ void rns_selinv_block_gen(const RnsScratch& sc, double2* Y, double2* F, const De
   }
 }
 
-template void rns_factor_block<double>(const RnsScratch&, double*, double*, const DevFronts&, const int32_t*, const int32_t*,
-                                       const int32_t*, int, int, int, const BatchShifts&, DevStatus, bool, Profiler&,
-                                       cudaStream_t);
-template void rns_factor_block<double2>(const RnsScratch&, double2*, double2*, const DevFronts&, const int32_t*, const int32_t*,
-                                        const int32_t*, int, int, int, const BatchShifts&, DevStatus, bool, Profiler&,
-                                        cudaStream_t);
+template void rns_factor_block<double>(const pexsi_plan*, const Level&, const RnsScratch&, double*, double*, int, int,
+                                       const BatchShifts&, DevStatus, Profiler&, cudaStream_t);
+template void rns_factor_block<double2>(const pexsi_plan*, const Level&, const RnsScratch&, double2*, double2*, int, int,
+                                        const BatchShifts&, DevStatus, Profiler&, cudaStream_t);
 
 }  // namespace pexsi

@@ -86,20 +86,35 @@ def limbs(v):
 
 def test_reconstruction_from_bytes():
     w = [limbs(P // p) for p in MODULI]
-    bias = [-128 * sum(x[j] for x in w) for j in range(4)]
+    bias = limbs(2 * P - 128 * sum(P // p for p in MODULI) % P)
+    pl = limbs(P)
     assert 255 * sum(x[0] for x in w) < 2 ** 32  # the lowest limb's sum stays in 32 bits
-    assert all(255 * sum(x[j] for x in w) < 2 ** 63 for j in range(4))
+    assert all(255 * sum(x[j] for x in w) + 2 ** 36 < 2 ** 63 for j in range(4))
     pinv = np.float32(np.float32(2.0 ** 84 / P) * np.float32(256.0))
     rng = random.Random(3)
     top = 2 ** (2 * BETA)
-    xs = [0, 1, -1, top, -top] + [rng.randint(-top, top) >> rng.randint(0, 116) for _ in range(2000)]
+    xs = [0, 1, -1, top - 1, 1 - top, 2 ** 84, -2 ** 84, 2 ** 52, -2 ** 52, 2 ** 20, -2 ** 20]
+    xs += [rng.randint(1 - top, top - 1) >> rng.randint(0, 116) for _ in range(2000)]
     for x in xs:
         u = []
         for p in MODULI:
             c = x * pow(P // p % p, -1, p) % p
             r = c - p if c > p // 2 else c
             u.append((r + 128) & 0xFF)
-        s = [sum(a * x_[j] for a, x_ in zip(u, w)) + bias[j] for j in range(4)]
-        assert -2 ** 38 < s[3] < 2 ** 38  # its 31 leading bits fit an int
-        k = int(np.rint(np.float32(s[3] >> 8) * pinv))
-        assert s[0] + (s[1] << 20) + (s[2] << 52) + (s[3] << 84) - k * P == x
+        a = [sum(q * x_[j] for q, x_ in zip(u, w)) + bias[j] for j in range(4)]
+        assert a[3] >> 8 < 2 ** 32
+        k = int(np.rint(np.float32(a[3] >> 8) * pinv))
+        assert 0 <= k <= 22 and k * pl[0] < 2 ** 32
+        s0 = a[0] - k * pl[0]
+        s1 = a[1] - k * pl[1] + (s0 >> 20)
+        s2 = a[2] - k * pl[2] + (s1 >> 32)
+        s3 = a[3] - k * pl[3] + (s2 >> 32)
+        assert (s3 << 84) + ((s2 & 0xFFFFFFFF) << 52) + ((s1 & 0xFFFFFFFF) << 20) + (s0 & 0xFFFFF) == x
+        # the magnitude by inverting the words, with carries
+        neg = s3 < 0
+        low = ((s1 & 0xFFFFFFFF) << 20) | (s0 & 0xFFFFF)
+        low = (low ^ (2 ** 52 - 1 if neg else 0)) + neg
+        mid = ((s2 & 0xFFFFFFFF) ^ (0xFFFFFFFF if neg else 0)) + (low >> 52)
+        A = (((s3 & 0xFFFFFFFF) ^ (0xFFFFFFFF if neg else 0)) + (mid >> 32)) & 0xFFFFFFFF
+        low &= 2 ** 52 - 1
+        assert (A << 84) + ((mid & 0xFFFFFFFF) << 52) + low == abs(x)
