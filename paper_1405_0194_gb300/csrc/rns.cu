@@ -94,6 +94,8 @@ constexpr int kChunkTiles = 15;            // 480 of K: 2 x 480 x 2^14 + 2^7 < 2
 constexpr int kStages = 6;
 constexpr int kEpi = 8;                    // epilogue warps: 4 lane quarters x (re, im)
 constexpr int kThreads = (kEpi + 2) * 32;
+constexpr int kItems = 128;                // most items of a CTA (a table in shared memory); a multiple of 32
+constexpr int gemm_smem(bool cplx) { return kStages * 2 * (cplx ? 2 : 1) * kPlane; }
 static_assert(mod_product() >> 117 == 1, "the bound on the integer products needs 2^117 <= P < 2^118");
 static_assert(2 * kChunkTiles * kK * 128 * 128 + 128 < (1 << 24), "the FP32 accumulators stay exact");
 
@@ -106,7 +108,7 @@ enum Mode {
   kResid,   // R = I - B X, X = the swept inverse, B = the block as it was (kept in Y, which takes R)
   kRefine,  // X += X R
   kPanel,   // L[S,B] = W[S,B] B^-1
-  kSchur,   // F[S,S] -= L W^T (lower triangle)
+  kSchur,   // F[S,C] -= L W^T (lower triangle; C and the columns of L and W: Update)
   kTak,     // Y[S,B] = -Y[S,S] L[S,B] and its mirror
   kDiag,    // Y[B,B] = B^-1 - L[S,B]^T Y[S,B]
   // LDU fronts (gen): whole squares, no mirrors, the block's plain inverse in place of its negative
@@ -119,7 +121,9 @@ enum Mode {
 enum Operand {
   kOpV, kOpD, kOpT, kOpR, kOpW, kOpB, kOpL, kOpLt, kOpY, kOpYt,
   // LDU fronts: rows of D^-1, B, B^-1, Y[S,S] and U[B,S]; columns of U, R, A[B,S], Y[S,S] and Y[S,B]
-  kOpDr, kOpBr, kOpXr, kOpYr, kOpUr, kOpU, kOpRc, kOpA, kOpYc, kOpYtc
+  kOpDr, kOpBr, kOpXr, kOpYr, kOpUr, kOpU, kOpRc, kOpA, kOpYc, kOpYtc,
+  // W[C,.] and A[.,S] of several blocks, kept in Y
+  kOpWs, kOpAs
 };
 
 struct Job {
@@ -128,7 +132,8 @@ struct Job {
   int p0, pc, b;             // block start, panel start inside the block (sweeps), panel width
   int rt0, mt0;              // first tile of N or M (a front whose row tiles are taken in pieces)
   int o0, on;                // output tiles of this launch
-  int kt;                    // K tiles of a slot
+  int kt, nkt;               // K tiles of a slot, of every item (0: they differ)
+  int g0, k0, width;         // kSchur: first column of the block's group, of its update, columns updated (0: all)
   int64_t slot, n_base, m_base;
   int pref_n[kRnsFronts + 1], pref_m[kRnsFronts + 1], pref_o[kRnsFronts + 1];
   // the fronts' sizes and places: as kernel arguments they cost no chain of global loads per item or block
@@ -154,16 +159,43 @@ __host__ __device__ __forceinline__ Dims dims_of(int s, int m, int p0, int pc, i
   return d;
 }
 
+// The update after the block at p0: which columns it reaches (the first `cols`
+// of S, and for LDU fronts the rows alike) and which eliminated ones it applies
+// (K of them from k0 on). Blocks come in groups of up to kRnsGroup. After the
+// i-th block of a group the last b = i & -i blocks are applied to the next b
+// blocks' columns; after the group's last block, or the front's, the group is
+// applied to all of S. Each column so gets each block once, and most of the
+// front is read, updated and written once per group instead of once per block.
+struct Update {
+  int k0, k, cols;
+};
+
+__host__ __device__ __forceinline__ Update update_of(const Dims& d, int g0, int k0, int width) {
+  Update u;
+  const bool all = width == 0 || d.q0 == d.s;
+  u.k0 = all ? g0 : k0;
+  u.k = d.q0 - u.k0;
+  u.cols = all ? d.mp : (d.s - d.q0 < width ? d.s - d.q0 : width);
+  return u;
+}
+
 __host__ __device__ __forceinline__ int tiles128(int n) { return n <= 0 ? 0 : (n + kRnsTile - 1) / kRnsTile; }
 
 // rows of N, rows of M, K of a product; sweeps skip blocks of one panel
-__host__ __device__ __forceinline__ void product_dims(int mode, const Dims& d, int b, int& rn, int& rm, int& k) {
-  switch (mode) {
+__host__ __device__ __forceinline__ void product_dims(const Job& j, const Dims& d, int& rn, int& rm, int& k) {
+  const int b = j.b;
+  switch (j.mode) {
     case kSweepT: rn = d.bw > b && d.pb > 0 ? d.bw : 0; rm = rn ? d.pb : 0; k = d.pb; break;
     case kSweepU: rn = rm = d.bw > b && d.pb > 0 ? d.bw : 0; k = d.pb; break;
     case kResid: case kRefine: rn = rm = d.bw > b ? d.bw : 0; k = d.bw; break;
     case kPanel: rn = d.mp; rm = d.mp > 0 ? d.bw : 0; k = d.bw; break;
-    case kSchur: rn = rm = d.mp; k = d.bw; break;
+    case kSchur: {
+      const Update u = update_of(d, j.g0, j.k0, j.width);
+      rn = d.mp;
+      rm = j.gen ? d.mp : u.cols;
+      k = u.k;
+      break;
+    }
     case kSweepDU: rm = d.bw > b && d.pb > 0 ? d.bw : 0; rn = rm ? d.pb : 0; k = d.pb; break;
     case kPanelU: rn = d.mp > 0 ? d.bw : 0; rm = d.mp; k = d.bw; break;
     case kTakU: rn = d.mp > 0 ? d.bw : 0; rm = d.mp; k = d.mp; break;
@@ -185,7 +217,7 @@ __host__ __device__ __forceinline__ bool scaled_op(int op) {
 }
 
 // largest f with pref[f] <= t
-__device__ __forceinline__ int owner(const int* pref, int n, int t) {
+__host__ __device__ __forceinline__ int owner(const int* pref, int n, int t) {
   int lo = 0, hi = n;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -199,19 +231,36 @@ struct OutTile {
   int pole, f, nt, mt;  // pole and front list index of the job, tile of N, tile of M
 };
 
-__device__ __forceinline__ OutTile out_tile(const Job& j, int o) {
+__host__ __device__ __forceinline__ OutTile out_tile(const Job& j, int o) {
   OutTile t;
   const int per = j.pref_o[j.nf];
   t.pole = o / per;
   const int x = o - t.pole * per;
   t.f = owner(j.pref_o, j.nf, x);
   const int y = x - j.pref_o[t.f];
-  if (triangular(j.mode, j.gen)) {
+  // the tiles of M that an update reaches: a trapezoid, for LDU fronts the rows beyond them alike
+  int tm = j.pref_m[t.f + 1] - j.pref_m[t.f];
+  if (j.mode == kSchur) tm = tiles128(update_of(dims_of(j.s[t.f], j.m[t.f], j.p0, j.pc, j.b), j.g0, j.k0, j.width).cols);
+  const int tri = tm * (tm + 1) / 2;
+  if (triangular(j.mode, j.gen) && (j.mode != kSchur || y < tri)) {
     int i = int((sqrtf(8.0f * float(y) + 1.0f) - 1.0f) * 0.5f);
     while (i * (i + 1) / 2 > y) --i;
     while ((i + 1) * (i + 2) / 2 <= y) ++i;
     t.nt = i;
     t.mt = y - i * (i + 1) / 2;
+  } else if (j.mode == kSchur) {
+    const int tn = j.pref_n[t.f + 1] - j.pref_n[t.f], z = j.gen ? y : y - tri;
+    if (!j.gen) {
+      t.nt = tm + z / tm;
+      t.mt = z - (t.nt - tm) * tm;
+    } else if (z < tn * tm) {
+      t.nt = z / tm;
+      t.mt = z - t.nt * tm;
+    } else {
+      const int w = z - tn * tm, side = tn - tm;
+      t.nt = w / side;
+      t.mt = tm + w - t.nt * side;
+    }
   } else {
     // Y[B,B] of a front without rows below it has no operands, and one tile or two by two
     int mtn = j.pref_m[t.f + 1] - j.pref_m[t.f];
@@ -333,11 +382,15 @@ __global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, co
     row = rt * kRnsTile + (grp & 15) * 8 + r;
     const int64_t base = int64_t(j.pole0 + pole) * j.pool + j.off[fi], m = d.m;
     int64_t si = 1;
+    const Update up = update_of(d, j.g0, j.k0, j.width);
     switch (op) {
       case kOpV: case kOpT: src = F + base + j.p0 + m * (j.p0 + j.pc); rows = d.bw; K = d.pb; sk = m; break;
       case kOpD: src = F + base + (j.p0 + j.pc) + m * (j.p0 + j.pc); rows = K = d.pb; si = m; sk = 1; break;
       case kOpR: case kOpRc: src = Y + base + j.p0 + m * j.p0; rows = K = d.bw; si = m; sk = 1; break;
-      case kOpW: case kOpL: src = F + base + d.q0 + m * j.p0; rows = d.mp; K = d.bw; sk = m; break;
+      case kOpW: src = F + base + d.q0 + m * j.p0; rows = d.mp; K = d.bw; sk = m; break;
+      case kOpL: src = F + base + d.q0 + m * up.k0; rows = d.mp; K = up.k; sk = m; break;
+      case kOpWs: src = Y + base + d.q0 + m * up.k0; rows = up.cols; K = up.k; sk = m; break;
+      case kOpAs: src = Y + base + up.k0 + m * d.q0; rows = d.mp; K = up.k; si = m; sk = 1; break;
       case kOpB: src = F + base + j.p0 + m * j.p0; rows = K = d.bw; si = m; sk = 1; break;
       case kOpLt: src = F + base + d.q0 + m * j.p0; rows = d.bw; K = d.mp; si = m; sk = 1; break;
       case kOpY: case kOpYc: src = Y + base + d.q0 + m * d.q0; rows = K = d.mp; si = m; sk = 1; break;
@@ -443,6 +496,10 @@ __constant__ float c_mod[kRnsModuli] = {256, 253, 251, 247, 241, 239, 233, 229, 
 // next one's MMAs. Items with K > 480 alternate them between chunks of 480: a
 // chunk's accumulator is reduced in place while the other one fills, and
 // carries its residue on.
+// Items are decoded 32 at a time, a lane each (the producer's into a table, the
+// epilogue's into registers): the integer divisions and searches of one item
+// after the other let the ring of stages run dry (820 tiles at K = 256: complex
+// 1341 -> 1419 TFLOP/s, real 450 -> 498).
 template <bool CPLX>
 __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant__ Job j,
                                                           const uint8_t* __restrict__ planes, uint8_t* __restrict__ out,
@@ -452,6 +509,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant_
   extern __shared__ __align__(128) uint8_t sm[];
   __shared__ __align__(8) uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], mma_done;
   __shared__ uint32_t tmem_slot;
+  __shared__ int4 s_item[kItems];
   __shared__ int s_fail, s_skip;
   if (threadIdx.x == 0) s_skip = *static_cast<volatile int*>(gfail);
   __syncthreads();
@@ -486,26 +544,46 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant_
   auto decode = [&](int it, int& l, OutTile& t, int& rn, int& rm) -> int {
     l = it / j.on;
     t = out_tile(j, j.o0 + it - l * j.on);
-    const Dims d = dims_of(j.s[t.f], j.m[t.f], j.p0, j.pc, j.b);
     int k;
-    product_dims(j.mode, d, j.b, rn, rm, k);
+    product_dims(j, dims_of(j.s[t.f], j.m[t.f], j.p0, j.pc, j.b), rn, rm, k);
     return k <= 0 ? 0 : (k + kK - 1) / kK;
+  };
+  // Lane i decodes the CTA's i-th item from `it` on: slots of its operands, K tiles and modulus, rows of N and M.
+  auto ahead = [&](int it, int& sn, int& sm_, uint32_t& kl, uint32_t& nm) {
+    it += lane * int(gridDim.x);
+    if (it < items) {
+      int l, rn, rm;
+      OutTile t;
+      const int nkt = decode(it, l, t, rn, rm);
+      sn = t.pole * j.pref_n[j.nf] + j.pref_n[t.f] + t.nt;
+      sm_ = t.pole * j.pref_m[j.nf] + j.pref_m[t.f] + t.mt;
+      kl = uint32_t(nkt) | uint32_t(l) << 24;
+      nm = uint32_t(min(kRnsTile, rn - (j.rt0 + t.nt) * kRnsTile)) |
+           uint32_t(min(kRnsTile, rm - (j.mt0 + t.mt) * kRnsTile)) << 16;
+    }
+    __syncwarp();
   };
 
   if (warp == kEpi) {
+    // the CTA's items, decoded by all lanes
+    for (int x = 0; x * int(gridDim.x) + int(blockIdx.x) < items; x += 32) {
+      int sn = 0, sm_ = 0;
+      uint32_t kl = 0, nm = 0;
+      ahead(int(blockIdx.x) + x * int(gridDim.x), sn, sm_, kl, nm);
+      s_item[x + lane] = make_int4(sn, sm_, int(kl), int(nm));
+    }
+    __syncwarp();
     if (lane == 0) {  // ---- producer
       int n = 0;
       bool ok = true;
-      for (int it = blockIdx.x; it < items && ok && !*fail; it += gridDim.x) {
-        int l, rn, rm;
-        OutTile t;
-        const int nkt = decode(it, l, t, rn, rm);
+      for (int it = blockIdx.x, x = 0; it < items && ok && !*fail; it += gridDim.x, ++x) {
+        const int4 t = s_item[x];
+        const int l = int(uint32_t(t.z) >> 24), nkt = t.z & 0xFFFFFF;
         const int64_t lo = int64_t(l) * j.kt * kOp;
-        const uint8_t* gn = planes + j.n_base + (int64_t(t.pole) * j.pref_n[j.nf] + j.pref_n[t.f] + t.nt) * j.slot + lo;
-        const uint8_t* gm = planes + j.m_base + (int64_t(t.pole) * j.pref_m[j.nf] + j.pref_m[t.f] + t.mt) * j.slot + lo;
+        const uint8_t* gn = planes + j.n_base + int64_t(t.x) * j.slot + lo;
+        const uint8_t* gm = planes + j.m_base + int64_t(t.y) * j.slot + lo;
         // bytes of the 8-row groups that the tiles have, of each plane (a whole tile: both planes in one copy)
-        const uint32_t bn = uint32_t(min(kRnsTile, rn - (j.rt0 + t.nt) * kRnsTile) + 7) / 8 * 512,
-                       bm = uint32_t(min(kRnsTile, rm - (j.mt0 + t.mt) * kRnsTile) + 7) / 8 * 512;
+        const uint32_t bn = uint32_t((t.w & 0xFFFF) + 7) / 8 * 512, bm = uint32_t((t.w >> 16) + 7) / 8 * 512;
         for (int kt = 0; kt < nkt; ++kt, ++n) {
           const int st = n % kStages, u = n / kStages;
           if (u > 0 && !bar_wait(smem_u32(&empty[st]), (u - 1) & 1, fail, wait_ns)) {
@@ -533,7 +611,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant_
       for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
         int l, rn, rm;
         OutTile t;
-        const int nkt = decode(it, l, t, rn, rm);
+        const int nkt = j.nkt > 0 ? j.nkt : decode(it, l, t, rn, rm);
         for (int k0 = 0; k0 < nkt && ok; k0 += kChunkTiles, ++u) {
           const int buf = u & 1;
           if (u > 1 && !bar_wait(smem_u32(&acc_empty[buf]), ((u >> 1) - 1) & 1, fail, wait_ns)) {
@@ -596,10 +674,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant_
       __syncwarp();
       if (lane == 0) bar_arrive(smem_u32(&acc_empty[use & 1]));
     };
-    for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-      int l, rn, rm;
-      OutTile t;
-      const int nkt = decode(it, l, t, rn, rm), nch = (nkt + kChunkTiles - 1) / kChunkTiles;
+    int sn = 0, sm_ = 0;
+    uint32_t kl = 0, nm = 0;
+    for (int it = blockIdx.x, y = 0; it < items && ok; it += gridDim.x, ++y) {
+      if ((y & 31) == 0) ahead(it, sn, sm_, kl, nm);
+      const uint32_t k = __shfl_sync(0xFFFFFFFFu, kl, y & 31), rows = __shfl_sync(0xFFFFFFFFu, nm, y & 31);
+      const int l = int(k >> 24), nch = (int(k & 0xFFFFFF) + kChunkTiles - 1) / kChunkTiles;
       if (nch == 0) continue;
       const float p = c_mod[l], inv = 1.0f / p;
       for (int c = 0; c + 2 < nch && ok; ++c, ++u) {  // chunks whose accumulator carries on: reduced in place
@@ -629,8 +709,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant_
       if (!(ok = wait_full(u))) break;
       const uint32_t a = tmem + lanes + uint32_t((u & 1) * 256) + col0,
                      a2 = tmem + lanes + uint32_t(((u & 1) ^ 1) * 256) + col0;
-      const int nn = min(kRnsTile, rn - (j.rt0 + t.nt) * kRnsTile);  // rows of N in the tile
-      const bool m_in = (j.mt0 + t.mt) * kRnsTile + mrow < rm;
+      const int nn = int(rows & 0xFFFF);  // rows of N in the tile
+      const bool m_in = mrow < int(rows >> 16);
       // (re, im) x 128 rows of M x 128 rows of N, one byte each
       uint8_t* o = out + (int64_t(it - l * j.on) * kRnsModuli + l) * (C * kRnsTile * kRnsTile) +
                    (CPLX ? h * kRnsTile * kRnsTile : 0) + mrow * kRnsTile + (CPLX ? 0 : h * NC);
@@ -762,7 +842,7 @@ __global__ void __launch_bounds__(kReconThreads) k_rns_recon(double* __restrict_
   const OutTile t = out_tile(j, j.o0 + int(blockIdx.x));
   const Dims d = dims_of(j.s[t.f], j.m[t.f], j.p0, j.pc, j.b);
   int rn, rm, K;
-  product_dims(j.mode, d, j.b, rn, rm, K);
+  product_dims(j, d, rn, rm, K);
   const int row0 = (j.rt0 + t.nt) * kRnsTile, col0 = (j.mt0 + t.mt) * kRnsTile;
   const int quads = (min(kRnsTile, rn - row0) + 3) / 4, units = C * quads * min(kRnsTile, rm - col0);
   const int unit = int(blockIdx.y) * kReconThreads + threadIdx.x;
@@ -770,6 +850,8 @@ __global__ void __launch_bounds__(kReconThreads) k_rns_recon(double* __restrict_
   const int part = unit % C, x = unit / C, mr = x / quads, q = x - mr * quads, c = col0 + mr, n0 = row0 + q * 4;
   const bool tri = triangular(j.mode, j.gen);
   if (tri && n0 + 3 < c) return;
+  // an LDU front's update reaches the rows or the columns below `cols`
+  const int cols = j.mode == kSchur && j.gen ? update_of(d, j.g0, j.k0, j.width).cols : 1 << 30;
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   if (K > 0) {
     const int tail = kRnsTile * int(sizeof(int));
@@ -801,7 +883,7 @@ __global__ void __launch_bounds__(kReconThreads) k_rns_recon(double* __restrict_
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = n0 + i;
-    if (r >= rn || (tri && r < c)) continue;
+    if (r >= rn || (tri && r < c) || (r >= cols && c >= cols)) continue;
     const bool in_r = r >= j.pc && r < j.pc + d.pb;
     double* at = fb + m * c + C * r;   // entry (r, c) of the diagonal block
     double* to = fb + m * r + C * c;   // and (c, r)
@@ -875,6 +957,27 @@ __global__ void __launch_bounds__(256) k_rns_save(const T* __restrict__ F, T* __
       const int hi = gen ? r : max(r, c), lo = gen ? c : min(r, c);
       Y[base + int64_t(d.m) * c + r] = F[base + int64_t(d.m) * lo + hi];
     }
+}
+
+// W = F[S,B] (and A[B,S] of LDU fronts: ROWS) of the fronts whose groups have
+// more than one block, into the same places of Y, for the group's updates. A
+// block of threads takes 16 columns of 256 rows.
+template <typename T, bool ROWS>
+__global__ void __launch_bounds__(256) k_rns_keep(const T* __restrict__ F, T* __restrict__ Y, DevFronts fr,
+                                                  const int32_t* __restrict__ fronts, int p0, int b, int g0) {
+  const int f = fronts[blockIdx.y];
+  const Dims d = dims_of(fr.s[f], fr.m[f], p0, 0, b);
+  if (d.s <= g0 + rns_block(b)) return;
+  const int across = ROWS ? 1 : (rns_block(b) + 15) / 16;
+  const int r = int(blockIdx.x) / across * 256 * (ROWS ? 0 : 1) + threadIdx.x;
+  const int c0 = (ROWS ? int(blockIdx.x) : int(blockIdx.x) % across) * 16;
+  const int nr = ROWS ? d.bw : d.mp, nc = ROWS ? d.mp : d.bw;
+  if (r >= nr) return;
+  const int64_t at = int64_t(blockIdx.z) * fr.pool + fr.off[f] + (ROWS ? p0 : d.q0) + r +
+                     int64_t(d.m) * ((ROWS ? d.q0 : p0) + c0);
+#pragma unroll
+  for (int c = 0; c < 16; ++c)
+    if (c0 + c < nc) Y[at + int64_t(d.m) * c] = F[at + int64_t(d.m) * c];
 }
 
 // ------------------------------------------------------------ scaling
@@ -953,6 +1056,8 @@ std::vector<Piece> pieces_of(int nact, int nb, int64_t cap, bool cplx, Fn slots)
   return out;
 }
 
+Slots update_slots(const Dims& d, const Update& u) { return {2 * tiles128(d.mp), 0, u.k}; }
+
 template <typename T>
 struct Runner {
   static constexpr bool CPLX = sizeof(T) == 16;
@@ -964,6 +1069,74 @@ struct Runner {
   int b;
   cudaStream_t st;
   int gen = 0;
+  int group = 1;  // blocks of a group
+
+  // The update after the block at p0 (Update).
+  void update(Job& j, int p0) const {
+    const int blk = rns_block(b), i = p0 / blk + 1, low = i & -i;
+    j.g0 = (i - 1) / group * group * blk;
+    j.k0 = p0 + blk - low * blk;
+    j.width = i % group == 0 ? 0 : low * blk;
+  }
+
+  // W (and A of LDU fronts) of the block at p0 into Y, where the group's updates read it again.
+  void keep(const DevFronts& fr, const int32_t* dfr, int nact, int p0, int np) const {
+    Job j;
+    update(j, p0);
+    int n = 0, rows = 0;
+    for (; n < nact && s[n] > j.g0 + rns_block(b); ++n) rows = std::max(rows, dims_of(s[n], m[n], p0, 0, b).mp);
+    if (group == 1 || rows == 0) return;
+    const int across = (rns_block(b) + 15) / 16;
+    k_rns_keep<T, false><<<dim3((rows + 255) / 256 * across, n, np), 256, 0, st>>>(F, Y, fr, dfr, p0, b, j.g0);
+    if (gen) k_rns_keep<T, true><<<dim3((rows + 15) / 16, n, np), 256, 0, st>>>(F, Y, fr, dfr, p0, b, j.g0);
+  }
+  // The widest update of the block's fronts; one of more than a block applies columns kept in Y.
+  int update_k(int nact, int p0) const {
+    Job j;
+    update(j, p0);
+    int k = 0;
+    for (int f = 0; f < nact; ++f) {
+      const Dims d = dims_of(s[f], m[f], p0, 0, b);
+      if (d.mp > 0) k = std::max(k, update_of(d, j.g0, j.k0, j.width).k);
+    }
+    return k;
+  }
+  // That update, apart from the block's panel products.
+  void apart(int nact, int p0, int nb, Profiler& pf) const {
+    Job w;
+    update(w, p0);
+    auto up = [&](int f) { return update_of(dims_of(s[f], m[f], p0, 0, b), w.g0, w.k0, w.width); };
+    auto slots = [&](int f) { return update_slots(dims_of(s[f], m[f], p0, 0, b), up(f)); };
+    for (const Piece& q : pieces_of(nact, nb, sc.plane_bytes, CPLX, slots)) {
+      int k = 32;
+      for (int f = q.f0; f < q.f0 + q.nf; ++f) k = std::max(k, up(f).k);
+      Job u;
+      const int uo = job(u, kSchur, q, p0, 0, (k + kK - 1) / kK);
+      if (uo == 0) continue;
+      u.n_base = 0;
+      u.m_base = int64_t(n_slots(u)) * u.slot;
+      cudaEvent_t a = pf.begin(st);
+      conv(u, q, kOpL, gen ? kOpAs : kOpWs);
+      pf.end(a, P_SLICE, st, 0.0, 0.0);
+      a = pf.begin(st);
+      product(u, q, uo);
+      const double fl = pf.on ? update_flops(q, p0) : 0.0;
+      pf.end(a, P_SCHUR, st, fl, 0.0, 2, fl * kRnsModuli);
+    }
+  }
+  double update_flops(const Piece& q, int p0) const {
+    Job w;
+    update(w, p0);
+    double fl = 0;
+    for (int f = q.f0; f < q.f0 + q.nf; ++f) {
+      const Dims d = dims_of(s[f], m[f], p0, 0, b);
+      const Update u = update_of(d, w.g0, w.k0, w.width);
+      const double rest = d.mp - u.cols, cols = u.cols;
+      fl += (CPLX ? 8.0 : 2.0) * q.np * u.k *
+            (gen ? double(d.mp) * d.mp - rest * rest : cols * (cols + 1) / 2 + rest * cols);
+    }
+    return fl;
+  }
 
   // Tile counts of a product over a piece; returns the output tiles.
   int job(Job& j, Mode mode, const Piece& q, int p0, int pc, int kt) const {
@@ -975,6 +1148,7 @@ struct Runner {
     j.p0 = p0;
     j.pc = pc;
     j.b = b;
+    update(j, p0);
     j.rt0 = mode == kTak ? q.rt0 : 0;
     j.mt0 = mode == kTakU ? q.rt0 : 0;
     j.kt = kt;
@@ -986,11 +1160,17 @@ struct Runner {
       j.m[f] = m[q.f0 + f];
       j.off[f] = off[q.f0 + f];
       int rn, rm, k;
-      product_dims(mode, dims_of(s[q.f0 + f], m[q.f0 + f], p0, pc, b), b, rn, rm, k);
+      const Dims d = dims_of(s[q.f0 + f], m[q.f0 + f], p0, pc, b);
+      product_dims(j, d, rn, rm, k);
+      if (mode == kSchur) rm = rn;  // slots as the rows have them
       const int tn = q.rtn > 0 && mode == kTak ? q.rtn : tiles128(rn), tm = q.rtn > 0 && mode == kTakU ? q.rtn : tiles128(rm);
+      const int nkt = k <= 0 ? 0 : (k + kK - 1) / kK;
+      j.nkt = f == 0 || nkt == j.nkt ? nkt : 0;
       j.pref_n[f + 1] = j.pref_n[f] + (k > 0 ? tn : 0);  // K = 0 (Y[B,B] of a front without rows below): no operands
       j.pref_m[f + 1] = j.pref_m[f] + (k > 0 ? tm : 0);
-      j.pref_o[f + 1] = j.pref_o[f] + (triangular(mode, gen) ? tn * (tn + 1) / 2 : tn * tm);
+      const int out = mode == kSchur ? tiles128(update_of(d, j.g0, j.k0, j.width).cols) : 0, rest = tn - out;
+      j.pref_o[f + 1] = j.pref_o[f] + (mode == kSchur ? (gen ? tn * tn - rest * rest : out * (out + 1) / 2 + rest * out)
+                                       : triangular(mode, gen) ? tn * (tn + 1) / 2 : tn * tm);
     }
     return j.pref_o[q.nf] * q.np;
   }
@@ -1010,11 +1190,11 @@ struct Runner {
 
   // The product and its reconstruction, in pieces of the output scratch.
   void product(Job& j, const Piece& q, int tiles) const {
-    const int cap = int(std::min<int64_t>(sc.out_bytes / (int64_t(kRnsOutTile) * (CPLX ? 2 : 1)), 1 << 20));
+    const int cap = int(std::min<int64_t>(sc.out_bytes / (int64_t(kRnsOutTile) * (CPLX ? 2 : 1)), kItems * sms() / kRnsModuli));
     for (int o = 0; o < tiles; o += cap) {
       j.o0 = o;
       j.on = std::min(cap, tiles - o);
-      k_rns_gemm<CPLX><<<std::min(sms(), j.on * kRnsModuli), kThreads, kStages * 2 * (CPLX ? 2 : 1) * kPlane, st>>>(
+      k_rns_gemm<CPLX><<<std::min(sms(), j.on * kRnsModuli), kThreads, gemm_smem(CPLX), st>>>(
           j, sc.planes, sc.out, sc.fail, sc.wait_ns);
       k_rns_recon<T><<<dim3(j.on, (CPLX ? 2 : 1) * kRnsTile * kRnsTile / 4 / kReconThreads), kReconThreads, 0, st>>>(
           reinterpret_cast<double*>(F), reinterpret_cast<double*>(Y), j, sc.planes, sc.out);
@@ -1022,6 +1202,21 @@ struct Runner {
   }
 };
 
+
+// Blocks of a group on a level: as many as the scratch has room for the operands
+// of. Each block alone, the rest of a front is read, reconstructed and written
+// once per 256 columns and the products' K is 256; in groups the operands of a
+// group are converted again. Groups of 1, 2 and 4 blocks: 55.4, 52.7 and 51.3 ms
+// for the inertia counts of 256 atoms in a fluid, 60.8, 58.9 and 58.1 ms for the
+// density matrix of 512, 53.0, 51.7 and 51.4 ms for a sheet of 14 x 14; fronts of
+// a few hundred columns do not care.
+int group_of(const int* s, const int* m, int nact, int b, int64_t cap, bool cplx) {
+  int rows = 0;
+  for (int f = 0; f < nact && s[f] > rns_block(b); ++f) rows = std::max(rows, m[f]);
+  int g = kRnsGroup;
+  while (g > 1 && 2 * tiles128(rows) * rns_slot_bytes(std::min(s[0], g * rns_block(b)), cplx) > cap) g /= 2;
+  return g;
+}
 
 // Slots of the launch sequences of one front.
 Slots sweep_slots(const Dims& d, int b) {
@@ -1052,9 +1247,9 @@ void launch_rns_scales(const double* H, const double* S, int wide, const int64_t
 }
 
 cudaError_t rns_configure() {
-  cudaError_t e = cudaFuncSetAttribute(k_rns_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStages * 4 * kPlane);
+  cudaError_t e = cudaFuncSetAttribute(k_rns_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(true));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_rns_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStages * 2 * kPlane);
+    e = cudaFuncSetAttribute(k_rns_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(false));
   return e;
 }
 
@@ -1075,7 +1270,7 @@ void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& 
       sw += a.fixed;
       lw += c.fixed;
       tw += y.fixed + y.n;
-      ks = std::max(ks, c.k);
+      ks = std::max({ks, c.k, std::min<int>(lv.s[t], kRnsGroup * rns_block(p->b))});
       kt = std::max(kt, y.k);
     }
     want = std::max({want, sw * batch * rns_slot_bytes(p->b, true), lw * batch * rns_slot_bytes(ks, true),
@@ -1109,7 +1304,9 @@ void rns_factor_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc
   const int32_t* dfr = p->d_level_fronts + lv.front_off;
   Runner<T> r{sc, F, Y, s, m, lv.off.data(), fr.pool, b, st};
   constexpr bool CPLX = sizeof(T) == 16;
+  r.group = group_of(s, m, int(lv.s.size()), b, sc.plane_bytes, CPLX);
   const int bw = std::min(rns_block(b), s[0] - p0);  // the widest front's block
+  r.keep(fr, dfr, nact, p0, sh.nb);
   if (bw > b) k_rns_save<T><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b, 0);
   for (int pc = 0; pc < bw; pc += b) {
     int n = 0;
@@ -1163,6 +1360,7 @@ void rns_factor_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc
     }
     pf.end(a, P_PANEL, st, 0.0, 0.0, kernels);
   }
+  const bool joint = r.update_k(nact, p0) <= rns_block(b);  // the update's W is the panel product's operand
   auto slots = [&](int f) { return schur_slots(dims_of(s[f], m[f], p0, 0, b)); };
   for (const Piece& q : pieces_of(nact, sh.nb, sc.plane_bytes, CPLX, slots)) {
     const int kt = (std::min(rns_block(b), s[q.f0] - p0) + kK - 1) / kK;
@@ -1173,13 +1371,11 @@ void rns_factor_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc
     u.n_base = int64_t(r.n_slots(l)) * l.slot;
     l.m_base = 2 * u.n_base;  // W, L, B^-1
     u.m_base = 0;
-    double fl = 0, sfl = 0;
+    double fl = 0;
     if (pf.on)
       for (int f = q.f0; f < q.f0 + q.nf; ++f) {
         const Dims d = dims_of(s[f], m[f], p0, 0, b);
-        const double fma_fl = CPLX ? 8.0 : 2.0;
-        fl += fma_fl * q.np * d.mp * double(d.bw) * d.bw;
-        sfl += fma_fl * q.np * (double(d.mp) * (d.mp + 1) / 2) * d.bw;
+        fl += (CPLX ? 8.0 : 2.0) * q.np * d.mp * double(d.bw) * d.bw;
       }
     cudaEvent_t a = pf.begin(st);
     r.conv(l, q, kOpW, kOpB);
@@ -1187,13 +1383,16 @@ void rns_factor_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc
     a = pf.begin(st);
     r.product(l, q, lo);
     pf.end(a, P_PANEL, st, fl, 0.0, 2, fl * kRnsModuli);
+    if (!joint) continue;
     a = pf.begin(st);
     r.conv(u, q, kOpL);
     pf.end(a, P_SLICE, st, 0.0, 0.0);
     a = pf.begin(st);
     r.product(u, q, uo);
+    const double sfl = pf.on ? r.update_flops(q, p0) : 0.0;
     pf.end(a, P_SCHUR, st, sfl, 0.0, 2, sfl * kRnsModuli);
   }
+  if (!joint) r.apart(nact, p0, sh.nb, pf);
 }
 
 // Y[S,B], its mirror and Y[B,B] of the block at p0 of the level's first nact fronts.
@@ -1243,8 +1442,10 @@ void rns_factor_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch
   const DevFronts fr = p->fronts();
   const int32_t* dfr = p->d_level_fronts + lv.front_off;
   Runner<double2> r{sc, F, Y, s, m, lv.off.data(), fr.pool, b, st, 1};
+  r.group = group_of(s, m, int(lv.s.size()), b, sc.plane_bytes, true);
   const int bw = std::min(rns_block(b), s[0] - p0);
   const int kb = (b + kK - 1) / kK;
+  r.keep(fr, dfr, nact, p0, sh.nb);
   if (bw > b) k_rns_save<double2><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b, 1);
   for (int pc = 0; pc < bw; pc += b) {
     int n = 0;
@@ -1296,6 +1497,7 @@ void rns_factor_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch
     }
     pf.end(a, P_PANEL, st, 0.0, 0.0, kernels);
   }
+  const bool joint = r.update_k(nact, p0) <= rns_block(b);
   auto slots = [&](int f) { return gen_schur_slots(dims_of(s[f], m[f], p0, 0, b)); };
   for (const Piece& q : pieces_of(nact, sh.nb, sc.plane_bytes, true, slots)) {
     const int kt = (std::min(rns_block(b), s[q.f0] - p0) + kK - 1) / kK;
@@ -1306,24 +1508,27 @@ void rns_factor_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch
     l.n_base = u.n_base = 0;       // W, then L
     u.m_base = x.m_base = rows;    // A[B,S]
     l.m_base = x.n_base = 2 * rows;  // columns, then rows of B^-1
-    double fl = 0, sfl = 0;
+    double fl = 0;
     if (pf.on)
       for (int f = q.f0; f < q.f0 + q.nf; ++f) {
         const Dims d = dims_of(s[f], m[f], p0, 0, b);
         fl += 16.0 * q.np * d.mp * double(d.bw) * d.bw;
-        sfl += 8.0 * q.np * double(d.mp) * d.mp * d.bw;
       }
     cudaEvent_t a = pf.begin(st);
     r.conv(l, q, kOpW, kOpB);
     r.product(l, q, lo);
-    r.conv(u, q, kOpL, kOpA);
+    if (joint) r.conv(u, q, kOpL, kOpA);
+    else r.conv(x, q, kOpA);
     r.conv(x, q, kOpXr);
     r.product(x, q, xo);
     pf.end(a, P_PANEL, st, fl, 0.0, 7, fl * kRnsModuli);
+    if (!joint) continue;
     a = pf.begin(st);
     r.product(u, q, uo);
+    const double sfl = pf.on ? r.update_flops(q, p0) : 0.0;
     pf.end(a, P_SCHUR, st, sfl, 0.0, 2, sfl * kRnsModuli);
   }
+  if (!joint) r.apart(nact, p0, sh.nb, pf);
 }
 
 void rns_selinv_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, double2* Y, double2* F, int nact,

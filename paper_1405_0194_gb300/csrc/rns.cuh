@@ -12,6 +12,7 @@ namespace pexsi {
 constexpr int kRnsModuli = 15;   // product of the moduli 2^117.8
 constexpr int kRnsBlock = 256;   // most columns eliminated together (a block of panels)
 constexpr int kRnsFronts = 128;  // fronts per launch (tile prefix sums travel as kernel arguments)
+constexpr int kRnsGroup = 4;     // most blocks whose updates are applied together (a power of two)
 constexpr int kRnsTile = 128;    // rows of an operand tile, edge of an output tile
 constexpr int kRnsOutTile = kRnsTile * kRnsTile * kRnsModuli;  // residue bytes of a real output tile
 

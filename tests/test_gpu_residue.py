@@ -160,3 +160,53 @@ def test_one_hermitian_front(n):
     assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref).max()
     ev = np.linalg.eigvalsh(np.linalg.solve(np.linalg.cholesky(S), np.linalg.solve(np.linalg.cholesky(S), H).conj().T))
     assert np.array_equal(counts, [(ev < x).sum() for x in shifts])
+
+
+# Blocks of 256 columns go into the rest of a front in groups of up to 4: fronts of one block to more than a
+# group, whole and ragged, alone and with rows below them, in each kind of factorisation. Bounds as above.
+@pytest.mark.parametrize("n", [514, 1024, 1025, 1100, 1281])
+def test_grouped_updates_of_one_front(n):
+    colptr, rowind, H, S = _full(n, n + 1)
+    h, s, z = H.T.ravel(), S.T.ravel(), 0.1 + 0.05j
+    got = _selinv(n, colptr, rowind, h, s, z).reshape(n, n).T
+    ref = np.linalg.inv(H - z * S)
+    assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref).max()
+    shifts = np.array([-0.7, 0.3])
+    plan = px.pexsi_setup(n, colptr, rowind, opts=px.pexsi_opts_default(max_batch=2))
+    counts = px.pexsi_inertia(plan, h, s, shifts)
+    A = np.random.default_rng(n).standard_normal((n, n)) / np.sqrt(n)
+    Hc = H + 1j * (A - A.T)
+    herm = px.pexsi_selinv_hermitian(plan, Hc.T.ravel(), S.T.ravel().astype(complex), z).reshape(n, n).T
+    px.pexsi_plan_destroy(plan)
+    assert np.array_equal(counts, dense.inertia_counts(n, colptr, rowind, h, s, shifts))
+    ref = np.linalg.inv(Hc - z * S)
+    assert np.abs(herm - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("norb,leaf", [(290, 600), (270, 1100), (128, 512)])
+def test_grouped_updates_with_rows_below(norb, leaf):
+    s = ns.make_chain(natoms=6, seed=norb, norb=norb)
+    z = 0.2 + 0.05j
+    ref = dense.selected_inverse(s.n, s.colptr, s.rowind, s.H, s.S, z)
+    got = _selinv(s.n, s.colptr, s.rowind, s.H, s.S, z, leaf_cols=leaf, amalgamate=0)
+    assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+def test_grouped_updates_in_little_scratch():
+    """From the least memory that a plan accepts upwards: without the residue scratch, with the least of it, in
+    smaller groups and in whole ones, all give the same inverse to rounding."""
+    n = 1100
+    colptr, rowind, H, S = _full(n, 13)
+    h, s, z = H.T.ravel(), S.T.ravel(), 0.1 + 0.05j
+    ref = np.linalg.inv(H - z * S).T.ravel()
+    budget, seen = 40 << 20, []
+    while budget < 1 << 30:
+        try:
+            got = _selinv(n, colptr, rowind, h, s, z, hbm_budget=int(budget))
+            assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref).max()
+            if not any(np.array_equal(got, x) for x in seen):
+                seen.append(got)
+        except px.PexsiError as e:
+            assert e.code == -3 and not seen
+        budget *= 1.12
+    assert len(seen) >= 3
