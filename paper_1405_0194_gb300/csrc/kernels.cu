@@ -1454,6 +1454,8 @@ void launch_diag_inv_any(T* F, const DevFronts& fr, const int32_t* fronts, int n
     k_diag_inv_one<T, GEN><<<dim3(nfronts, sh.nb), 256, sizeof(T) * size_t(b) * (b + 1), st>>>(F, fr, fronts, p0, b, status);
     return;
   }
+  // not chained itself: clusters placed while the kernel before still holds SMs share the ones it has left, and
+  // two on one SM take turns at its FP64 unit (96 inversions a launch: 17.3 -> 19.4 ms for 96 atoms in a fluid)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(nfronts * kDiagCtas), unsigned(sh.nb), 1);
   cfg.blockDim = dim3(kDiagThreads, 1, 1);

@@ -22,6 +22,40 @@ struct BatchShifts {
   double wd_re[kMaxBatch], wd_im[kMaxBatch];  // w^d (mu-derivative of the Fermi function)
 };
 
+// Kernels launched in a chain (programmatic stream serialisation): a kernel is
+// set up once every block of the one before has called chain_next or ended, and
+// waits in chain_begin, which all its threads pass before they touch memory
+// that others write, or end. It returns when the kernel before has ended, which
+// has passed its own first, so all earlier work is done and visible. The
+// pointers go through the wait, so that no load through them moves ahead of it.
+// The short kernels call chain_next at once. Those that fill the SMs' shared
+// memory or FP64 units do not: blocks that start beside them wait with little
+// L1 (a GEMM's neighbours) or slow them down. Chained, the counts of 256 atoms in
+// a fluid take 49.3 instead of 51.6 ms, a Hermitian density matrix of 64 atoms
+// 10.5 instead of 11.3 ms, a selected inverse of 24 atoms 1.66 instead of 1.70 ms.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+template <typename... P>
+__device__ __forceinline__ void chain_begin(P&... p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  (..., [](auto& q) { asm volatile("" : "+l"(q)::"memory"); }(p));
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Front geometry on the device.
 struct DevFronts {
   const int64_t* off;   // element offset of each front in one pole's pool

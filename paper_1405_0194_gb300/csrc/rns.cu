@@ -405,6 +405,8 @@ __global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, co
     }
     src += si * row;
   }
+  chain_next();
+  chain_begin(src);
   const bool row_in = in && row < rows;
   auto load = [&](int o, double (&re)[8], double (&im)[8]) {
 #pragma unroll
@@ -511,6 +513,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant_
   __shared__ uint32_t tmem_slot;
   __shared__ int4 s_item[kItems];
   __shared__ int s_fail, s_skip;
+  chain_begin();
   if (threadIdx.x == 0) s_skip = *static_cast<volatile int*>(gfail);
   __syncthreads();
   if (s_skip) return;  // an earlier CTA gave up: leave together
@@ -846,6 +849,8 @@ __global__ void __launch_bounds__(kReconThreads) k_rns_recon(double* __restrict_
   const int row0 = (j.rt0 + t.nt) * kRnsTile, col0 = (j.mt0 + t.mt) * kRnsTile;
   const int quads = (min(kRnsTile, rn - row0) + 3) / 4, units = C * quads * min(kRnsTile, rm - col0);
   const int unit = int(blockIdx.y) * kReconThreads + threadIdx.x;
+  chain_next();
+  chain_begin(F, Y, planes, out);
   if (unit >= units) return;
   const int part = unit % C, x = unit / C, mr = x / quads, q = x - mr * quads, c = col0 + mr, n0 = row0 + q * 4;
   const bool tri = triangular(j.mode, j.gen);
@@ -949,6 +954,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_rns_save(const T* __restrict__ F, T* __restrict__ Y, DevFronts fr,
                                                   const int32_t* __restrict__ fronts, int p0, int b, int gen) {
   const int f = fronts[blockIdx.y];
+  chain_next();
+  chain_begin(F, Y);
   const Dims d = dims_of(fr.s[f], fr.m[f], p0, 0, b);
   if (d.bw <= b) return;
   const int64_t base = int64_t(blockIdx.z) * fr.pool + fr.off[f] + p0 + int64_t(d.m) * p0;
@@ -966,6 +973,8 @@ template <typename T, bool ROWS>
 __global__ void __launch_bounds__(256) k_rns_keep(const T* __restrict__ F, T* __restrict__ Y, DevFronts fr,
                                                   const int32_t* __restrict__ fronts, int p0, int b, int g0) {
   const int f = fronts[blockIdx.y];
+  chain_next();
+  chain_begin(F, Y);
   const Dims d = dims_of(fr.s[f], fr.m[f], p0, 0, b);
   if (d.s <= g0 + rns_block(b)) return;
   const int across = ROWS ? 1 : (rns_block(b) + 15) / 16;
@@ -1087,8 +1096,8 @@ struct Runner {
     for (; n < nact && s[n] > j.g0 + rns_block(b); ++n) rows = std::max(rows, dims_of(s[n], m[n], p0, 0, b).mp);
     if (group == 1 || rows == 0) return;
     const int across = (rns_block(b) + 15) / 16;
-    k_rns_keep<T, false><<<dim3((rows + 255) / 256 * across, n, np), 256, 0, st>>>(F, Y, fr, dfr, p0, b, j.g0);
-    if (gen) k_rns_keep<T, true><<<dim3((rows + 15) / 16, n, np), 256, 0, st>>>(F, Y, fr, dfr, p0, b, j.g0);
+    launch_chained(k_rns_keep<T, false>, dim3((rows + 255) / 256 * across, n, np), 256, 0, st, F, Y, fr, dfr, p0, b, j.g0);
+    if (gen) launch_chained(k_rns_keep<T, true>, dim3((rows + 15) / 16, n, np), 256, 0, st, F, Y, fr, dfr, p0, b, j.g0);
   }
   // The widest update of the block's fronts; one of more than a block applies columns kept in Y.
   int update_k(int nact, int p0) const {
@@ -1184,8 +1193,8 @@ struct Runner {
     auto blocks = [&](Operand op) { return ((m_side(op) ? m_slots(j) : n_slots(j)) * 16 + g - 1) / g; };
     const int na = blocks(a), n = na + (both ? blocks(c) : 0);
     if (n <= 0) return;
-    if (oc == 8) k_rns_conv<T, 8><<<n, 256, 0, st>>>(F, Y, j, sc.planes, a, na, c);
-    else k_rns_conv<T, 32><<<n, 256, 0, st>>>(F, Y, j, sc.planes, a, na, c);
+    if (oc == 8) launch_chained(k_rns_conv<T, 8>, n, 256, 0, st, F, Y, j, sc.planes, a, na, c);
+    else launch_chained(k_rns_conv<T, 32>, n, 256, 0, st, F, Y, j, sc.planes, a, na, c);
   }
 
   // The product and its reconstruction, in pieces of the output scratch.
@@ -1194,10 +1203,10 @@ struct Runner {
     for (int o = 0; o < tiles; o += cap) {
       j.o0 = o;
       j.on = std::min(cap, tiles - o);
-      k_rns_gemm<CPLX><<<std::min(sms(), j.on * kRnsModuli), kThreads, gemm_smem(CPLX), st>>>(
-          j, sc.planes, sc.out, sc.fail, sc.wait_ns);
-      k_rns_recon<T><<<dim3(j.on, (CPLX ? 2 : 1) * kRnsTile * kRnsTile / 4 / kReconThreads), kReconThreads, 0, st>>>(
-          reinterpret_cast<double*>(F), reinterpret_cast<double*>(Y), j, sc.planes, sc.out);
+      launch_chained(k_rns_gemm<CPLX>, std::min(sms(), j.on * kRnsModuli), kThreads, gemm_smem(CPLX), st, j, sc.planes,
+                     sc.out, sc.fail, sc.wait_ns);
+      launch_chained(k_rns_recon<T>, dim3(j.on, (CPLX ? 2 : 1) * kRnsTile * kRnsTile / 4 / kReconThreads), kReconThreads, 0,
+                     st, reinterpret_cast<double*>(F), reinterpret_cast<double*>(Y), j, sc.planes, sc.out);
     }
   }
 };
@@ -1307,7 +1316,7 @@ void rns_factor_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc
   r.group = group_of(s, m, int(lv.s.size()), b, sc.plane_bytes, CPLX);
   const int bw = std::min(rns_block(b), s[0] - p0);  // the widest front's block
   r.keep(fr, dfr, nact, p0, sh.nb);
-  if (bw > b) k_rns_save<T><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b, 0);
+  if (bw > b) launch_chained(k_rns_save<T>, dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st, F, Y, fr, dfr, p0, b, 0);
   for (int pc = 0; pc < bw; pc += b) {
     int n = 0;
     while (n < nact && s[n] > p0 + pc) ++n;
@@ -1446,7 +1455,7 @@ void rns_factor_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch
   const int bw = std::min(rns_block(b), s[0] - p0);
   const int kb = (b + kK - 1) / kK;
   r.keep(fr, dfr, nact, p0, sh.nb);
-  if (bw > b) k_rns_save<double2><<<dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st>>>(F, Y, fr, dfr, p0, b, 1);
+  if (bw > b) launch_chained(k_rns_save<double2>, dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st, F, Y, fr, dfr, p0, b, 1);
   for (int pc = 0; pc < bw; pc += b) {
     int n = 0;
     while (n < nact && s[n] > p0 + pc) ++n;
