@@ -94,7 +94,7 @@ void rns_scratch(const pexsi_plan* p, int batch, int64_t most, int64_t& planes, 
   int64_t least, want;
   rns_scratch_range(p, batch, least, want);
   planes = std::max(least, std::min(want, most));
-  out = rns_out_bytes(p, batch);
+  out = rns_out_bytes(p, batch, most > 0 ? kRnsOutTiles : kRnsOutTilesLeast);
 }
 
 int fit_batch(const pexsi_plan* p, int64_t budget, int most, int64_t& planes, int64_t& out) {

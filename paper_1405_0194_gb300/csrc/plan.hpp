@@ -204,7 +204,7 @@ int64_t bytes_fixed(const pexsi_plan* p);
 // 0 for split-precision plans.
 void rns_scratch(const pexsi_plan* p, int batch, int64_t most, int64_t& planes, int64_t& out);
 void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& want);
-int64_t rns_out_bytes(const pexsi_plan* p, int batch);
+int64_t rns_out_bytes(const pexsi_plan* p, int batch, int most);
 constexpr int64_t kRnsPlaneBytes = int64_t(2) << 30;  // default of `most`
 
 // The largest batch (at most `most`) whose workspace fits the budget, with

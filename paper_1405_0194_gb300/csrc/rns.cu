@@ -1289,7 +1289,7 @@ void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& 
   want = std::max(want, least);
 }
 
-int64_t rns_out_bytes(const pexsi_plan* p, int batch) {
+int64_t rns_out_bytes(const pexsi_plan* p, int batch, int most) {
   int64_t tiles = 1;
   for (const Level& lv : p->levels) {
     int64_t t = 0;
@@ -1299,7 +1299,7 @@ int64_t rns_out_bytes(const pexsi_plan* p, int batch) {
     }
     tiles = std::max(tiles, t * batch);
   }
-  return std::min<int64_t>(tiles, kRnsOutTiles) * kRnsOutTile * 2;
+  return std::min<int64_t>(tiles, most) * kRnsOutTile * 2;
 }
 
 // Eliminates the block of columns [p0, p0 + 256) of the level's fronts (the
