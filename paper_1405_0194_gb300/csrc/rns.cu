@@ -303,29 +303,46 @@ __device__ __forceinline__ uint32_t bf16x2(float a, float b) {
   return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
 }
 
+// Coefficients of the four pieces, plain and scaled, the modulus and its reciprocal.
+struct PieceTable {
+  float c[2][kRnsModuli][6];
+};
+constexpr PieceTable piece_table() {
+  PieceTable t = {};
+  for (int s = 0; s < 2; ++s)
+    for (int l = 0; l < kRnsModuli; ++l) {
+      for (int k = 0; k < 4; ++k) t.c[s][l][k] = float(piece_coef(l, k, s != 0));
+      t.c[s][l][4] = float(modulus(l));
+      t.c[s][l][5] = 1.0f / float(modulus(l));
+    }
+  return t;
+}
+__constant__ PieceTable c_piece = piece_table();
+
 // Residues of 8 consecutive k of one row: one 16-byte word per modulus. The
 // sum of pieces times coefficients is an exact integer below 2^24 in FP32, its
-// quotient by p is rounded by the add of 1.5 2^23, and the residue is exact.
-template <bool SCALED>
-__device__ __forceinline__ void store_residues(const float (&p)[8][4], uint8_t* dst, int64_t step) {
-  each_modulus([&](auto LC) {
-    constexpr int l = decltype(LC)::value;
-    constexpr float c0 = float(piece_coef(l, 0, SCALED)), c1 = float(piece_coef(l, 1, SCALED)),
-                    c2 = float(piece_coef(l, 2, SCALED)), c3 = float(piece_coef(l, 3, SCALED)), pm = float(modulus(l)),
-                    inv = 1.0f / float(modulus(l));
+// quotient by p is rounded by the add of 1.5 2^23, and the residue is exact. A
+// loop over the moduli, since all of them in line, for both kinds and parts, were
+// 70 KB of instructions that the warps waited for.
+__device__ __forceinline__ void store_residues(const float (&p)[8][4], bool scaled, uint8_t* dst, int64_t step) {
+  const float(*tab)[6] = c_piece.c[scaled ? 1 : 0];
+#pragma unroll 5
+  for (int l = 0; l < kRnsModuli; ++l) {
+    const float c0 = tab[l][0], c1 = tab[l][1], c2 = tab[l][2], c3 = tab[l][3], pm = tab[l][4], inv = tab[l][5];
     float r[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      float t = SCALED ? p[u][0] * c0 : p[u][0];
+      float t = p[u][0] * c0;
       t = fmaf(p[u][1], c1, t);
       t = fmaf(p[u][2], c2, t);
       t = fmaf(p[u][3], c3, t);
       const float q = fmaf(t, inv, 12582912.0f) - 12582912.0f;
       r[u] = fmaf(q, -pm, t);
     }
-    *reinterpret_cast<uint4*>(dst + l * step) =
+    *reinterpret_cast<uint4*>(dst) =
         make_uint4(bf16x2(r[0], r[1]), bf16x2(r[2], r[3]), bf16x2(r[4], r[5]), bf16x2(r[6], r[7]));
-  });
+    dst += step;
+  }
 }
 
 // |x| as a float, rounded down; 0 below the float range, garbage above it
@@ -351,8 +368,12 @@ __device__ __forceinline__ int row_exponent(uint32_t mx, float sum, int count) {
 // its slots. A block of 256 threads takes 32 / OC groups of 8 rows: thread (row
 // r = tid % 8, octet o of OC) reads entries 8 o .. 8 o + 7 of its row, twice
 // when K > 8 OC (norm, then residues).
+// Three blocks to an SM where their registers
+// fit without spilling (real values, and short rows with the parts in turn:
+// a 500-atom chain 6.35 -> 6.23 ms, inertia 48.1 -> 47.4 ms); complex long rows
+// keep two (three: 57.5 -> 58.8 ms for 512 atoms).
 template <typename T, int OC>
-__global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, const T* __restrict__ Y,
+__global__ void __launch_bounds__(256, (sizeof(T) == 16 && OC == 32) ? 2 : 3) k_rns_conv(const T* __restrict__ F, const T* __restrict__ Y,
                                                      const __grid_constant__ Job j,
                                                      uint8_t* __restrict__ planes, int op_a, int nblk_a, int op_b) {
   constexpr bool CPLX = sizeof(T) == 16;
@@ -473,13 +494,12 @@ __global__ void __launch_bounds__(256, 2) k_rns_conv(const T* __restrict__ F, co
     if (again) load(o, re, im);
     uint8_t* dst = slot + int64_t(o >> 2) * ((CPLX ? 2 : 1) * kPlane) + ((row & (kRnsTile - 1)) >> 3) * 512 +
                    (o & 3) * 128 + r * 16;
-#pragma unroll
+#pragma unroll (CPLX && OC == 8 ? 1 : 2)
     for (int c = 0; c < (CPLX ? 2 : 1); ++c) {
       float p[8][4];
 #pragma unroll
       for (int u = 0; u < 8; ++u) pieces(c ? im[u] : re[u], ex, p[u]);
-      if (scaled) store_residues<true>(p, dst + c * kPlane, step);
-      else store_residues<false>(p, dst + c * kPlane, step);
+      store_residues(p, scaled, dst + c * kPlane, step);
     }
   }
 }
