@@ -137,7 +137,7 @@ class ClockSampler:
 
 def roofline_of(dom: dict, total_kernel_ms: float, peaks: dict, split: int) -> dict:
     """Roofline entry of the dominant launch class. A class that runs on the
-    tensor cores (the split-precision GEMMs) is measured by the bf16 flops its
+    tensor cores (residue products, split-precision GEMMs) is measured by the bf16 flops its
     MMAs execute against the measured sustained bf16 peak (the class is timed
     inside a seconds-long step); an FP64 class by its algorithmic flops against
     the FP64 DFMA peak (no measured FP64 peak exists)."""
@@ -150,7 +150,8 @@ def roofline_of(dom: dict, total_kernel_ms: float, peaks: dict, split: int) -> d
         r.update({"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                   "peak_source": "bf16_tflops_sustained of MEASURED_PEAKS.json (of measured)",
                   "fp64_equivalent_tflops": dom["flops"] / secs / 1e12,
-                  "note": f"achieved = bf16 flops the tcgen05 MMAs execute: {split * (split + 1) // 2} slice pairs "
+                  "note": "achieved = bf16 flops the tcgen05 MMAs execute: "
+                          f"{f'{split * (split + 1) // 2} slice pairs' if split else '15 residues'} "
                           "x 4 real products x 2 flops per complex multiply-add; fp64_equivalent_tflops counts "
                           "8 flops per complex multiply-add of the FP64 product it replaces"})
     else:
@@ -426,7 +427,7 @@ def run_ours(args):
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": ("f64 in/out; supernode GEMMs as bf16x%d slices on tcgen05 (exact fp32 / int64 accumulation)"
-                  % args.split) if args.split else "f64",
+                  % args.split) if args.split else "f64 (supernode products of 58-bit integers in 15 bf16 residues on tcgen05, exact)",
         "data": "synthetic",
         "config": {"workload": WORKLOADS[args.workload]["desc"], "poles_per_step": B, "split_slices": args.split,
                    "inertia_shifts": f"{per60} per {P} poles, spread over the steps", "seed": args.seed,
