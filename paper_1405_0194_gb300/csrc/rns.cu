@@ -26,9 +26,10 @@
 //
 // The fronts are eliminated in blocks of kRnsBlock = 256 columns (against the
 // panels of the DFMA path): the 256 x 256 diagonal block B is inverted by
-// symmetric sweeps over its panels (k_diag_inv per panel, the rest as residue
-// products), L[S,B] = W[S,B] B^-1 and F[S,S] -= L W^T are one product of K = 256
-// each, and Y[S,B] = -Y[S,S] L[S,B] converts Y[S,S] once per 256 columns.
+// symmetric sweeps over its panels (launch_diag_inv per panel, the rest as
+// residue products), L[S,B] = W[S,B] B^-1 is one product, F[S,S] -= L W^T goes in
+// groups of blocks (Update), and Y[S,B] = -Y[S,S] L[S,B] converts Y[S,S] once
+// per 256 columns.
 #include <algorithm>
 #include <cstdint>
 #include <utility>
