@@ -137,9 +137,10 @@ class ClockSampler:
 
 def roofline_of(dom: dict, total_kernel_ms: float, peaks: dict, split: int) -> dict:
     """Roofline entry of the dominant launch class. A class that runs on the
-    tensor cores (residue products, split-precision GEMMs) is measured by the bf16 flops its
-    MMAs execute against the measured sustained bf16 peak (the class is timed
-    inside a seconds-long step); an FP64 class by its algorithmic flops against
+    tensor cores (residue products, split-precision GEMMs) is measured by the
+    bf16 flops its MMAs execute against the measured sustained bf16 peak (the
+    class is timed inside a seconds-long step); a class without flops by its
+    bytes against the copy rate; an FP64 class by its algorithmic flops against
     the FP64 DFMA peak (no measured FP64 peak exists)."""
     secs = dom["ms"] / 1e3
     r = {"kernel": dom["name"], "launches": dom["launches"], "avg_launch_ms": dom["ms"] / max(1, dom["launches"]),
@@ -154,6 +155,11 @@ def roofline_of(dom: dict, total_kernel_ms: float, peaks: dict, split: int) -> d
                           f"{f'{split * (split + 1) // 2} slice pairs' if split else '15 residues'} "
                           "x 4 real products x 2 flops per complex multiply-add; fp64_equivalent_tflops counts "
                           "8 flops per complex multiply-add of the FP64 product it replaces"})
+    elif dom["flops"] == 0 and dom.get("bytes", 0) > 0 and secs > 0:
+        peak, ach = float(peaks["hbm_gbs"]), dom["bytes"] / secs / 1e9
+        r.update({"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
+                  "peak_source": "hbm_gbs of MEASURED_PEAKS.json (of measured)",
+                  "note": "bytes read and written by the launches, operand slots in whole"})
     else:
         ach = dom["flops"] / secs / 1e12 if secs > 0 else 0.0
         r.update({"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",

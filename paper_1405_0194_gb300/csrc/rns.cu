@@ -1147,7 +1147,7 @@ struct Runner {
       u.m_base = int64_t(n_slots(u)) * u.slot;
       cudaEvent_t a = pf.begin(st);
       conv(u, q, kOpL, gen ? kOpAs : kOpWs);
-      pf.end(a, P_SLICE, st, 0.0, 0.0);
+      pf.end(a, P_SLICE, st, 0.0, slot_bytes(u, kOpL) + slot_bytes(u, kOpWs));
       a = pf.begin(st);
       product(u, q, uo);
       const double fl = pf.on ? update_flops(q, p0) : 0.0;
@@ -1207,6 +1207,10 @@ struct Runner {
   int n_slots(const Job& j) const { return j.pref_n[j.nf] * j.np; }
   int m_slots(const Job& j) const { return j.pref_m[j.nf] * j.np; }
 
+  // Bytes that the conversion of an operand reads and writes, in whole slots.
+  double slot_bytes(const Job& j, Operand a) const {
+    return double(m_side(a) ? m_slots(j) : n_slots(j)) * double(j.slot) * (1.0 + 8.0 / 30.0);
+  }
   void conv(const Job& j, const Piece& q, Operand a) const { conv2(j, q, a, a, false); }
   void conv(const Job& j, const Piece& q, Operand a, Operand c) const { conv2(j, q, a, c, true); }
   void conv2(const Job& j, const Piece& q, Operand a, Operand c, bool both) const {
@@ -1409,14 +1413,14 @@ void rns_factor_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc
       }
     cudaEvent_t a = pf.begin(st);
     r.conv(l, q, kOpW, kOpB);
-    pf.end(a, P_SLICE, st, 0.0, 0.0);
+    pf.end(a, P_SLICE, st, 0.0, r.slot_bytes(l, kOpW) + r.slot_bytes(l, kOpB));
     a = pf.begin(st);
     r.product(l, q, lo);
     pf.end(a, P_PANEL, st, fl, 0.0, 2, fl * kRnsModuli);
     if (!joint) continue;
     a = pf.begin(st);
     r.conv(u, q, kOpL);
-    pf.end(a, P_SLICE, st, 0.0, 0.0);
+    pf.end(a, P_SLICE, st, 0.0, r.slot_bytes(u, kOpL));
     a = pf.begin(st);
     r.product(u, q, uo);
     const double sfl = pf.on ? r.update_flops(q, p0) : 0.0;
@@ -1451,7 +1455,7 @@ void rns_selinv_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc
       cudaEvent_t a = pf.begin(st);
       if (first) r.conv(t, q, kOpLt, kOpY);
       else r.conv(t, q, kOpY);
-      pf.end(a, P_SLICE, st, 0.0, 0.0);
+      pf.end(a, P_SLICE, st, 0.0, r.slot_bytes(t, kOpY) + (first ? r.slot_bytes(t, kOpLt) : 0.0));
       a = pf.begin(st);
       r.product(t, q, to);
       pf.end(a, P_OFFDIAG, st, fl, 0.0, 2, fl * kRnsModuli);
