@@ -51,8 +51,9 @@ enum {
   PEXSI_ERR_BREAKDOWN = -5,     /* zero / non-finite pivot in a diagonal block */
   PEXSI_ERR_INTERNAL = -6,      /* violated internal invariant (a bug)         */
   PEXSI_ERR_CANCELLED = -7,     /* server request cancelled before completion  */
-  PEXSI_ERR_TIMEOUT = -8,       /* a bounded device-side wait ran out (split-
-                                   precision kernels; pexsi_opts.wait_ns)      */
+  PEXSI_ERR_TIMEOUT = -8,       /* a bounded device-side wait ran out (tensor-
+                                   core kernels, block inverses on a cluster;
+                                   pexsi_opts.wait_ns)                         */
   PEXSI_PENDING = 1             /* server request not finished yet (poll)      */
 };
 
@@ -85,16 +86,18 @@ typedef struct pexsi_opts {
   int64_t hbm_budget;      /* bytes of device workspace the batch may use, 0 = auto  */
   int64_t wait_ns;         /* bound, in ns of wall time, of every wait of one role of
                               a tensor-core kernel on another (an mbarrier phase
-                              of a copy, of the MMAs, of a TMEM drain); 0 = 1 s. A
-                              wait that runs out stops the launch cleanly (every
-                              role returns, TMEM is freed, later launches of the
-                              call return at once) and the call returns
+                              of a copy, of the MMAs, of a TMEM drain) and of one
+                              CTA of a block inverse on the others of its cluster;
+                              0 = 1 s. A wait that runs out stops the launch cleanly
+                              (every role returns, TMEM is freed, later GEMM launches
+                              of the call return at once) and the call returns
                               PEXSI_ERR_TIMEOUT. No other kernel waits.           */
   int32_t inject;          /* fault injection for tests of the error paths, 0 = off
                               (default). 1: CTA 0 of every short-K split GEMM launch
                               issues no operand copy, so that its MMA issuer's wait
-                              runs out after wait_ns (PEXSI_ERR_TIMEOUT; split_slices
-                              > 0 only). 2: a breakdown of front 0 is recorded from
+                              runs out after wait_ns (PEXSI_ERR_TIMEOUT); on plans
+                              with split_slices = 0 the first column of every
+                              block inverse on a cluster comes late instead. 2: a breakdown of front 0 is recorded from
                               the host after the first pole batch of every call with
                               accumulate = 0 (PEXSI_ERR_BREAKDOWN at the end of the
                               chain).                                             */
@@ -182,7 +185,7 @@ int pexsi_pole_table(double beta, double delta_e, int32_t n_poles, double mu,
  * output may be NULL. S == NULL means S = I (H's diagonal positions). The
  * call is synchronous. On error the outputs are undefined.
  * Errors: INVALID_ARG, NOMEM, CUDA, BREAKDOWN (info->breakdown_front),
- * TIMEOUT (a bounded device-side wait of a tensor-core kernel ran out). */
+ * TIMEOUT (a bounded device-side wait ran out). */
 int pexsi_dm(pexsi_plan* plan, const double* H, const double* S, double mu, double beta,
              int32_t n_poles, double delta_e, double* dm, double* edm, double* fdm,
              pexsi_dm_info* info);

@@ -118,7 +118,7 @@ const unsigned long long kInfBits = 0x7FF0000000000000ull;
 
 // Clears the status words of one chain (0 = poles, 1 = inertia shifts): the
 // first breakdown front, the smallest pivot ratio and the failure flag of
-// the split-precision waits.
+// the bounded waits.
 void reset_status(Workspace& ws, int which) {
   ck(cudaMemcpyAsync(ws.brk + which, &kBig, sizeof(int), cudaMemcpyHostToDevice, ws.stream), "status");
   ck(cudaMemcpyAsync(ws.minpiv + which, &kInfBits, sizeof(kInfBits), cudaMemcpyHostToDevice, ws.stream), "status");
@@ -299,7 +299,8 @@ void factor_batch(const pexsi_plan* p, Workspace& ws, T* F, const BatchShifts& s
   // the inertia shifts (count) keep their own status words; their panel blocks
   // are saved and counted after the factorisation
   DevStatus status{ws.brk + (count ? 1 : 0), ws.minpiv + (count ? 1 : 0), ws.neg, count ? ws.dsave : nullptr,
-                   p->d_col0, p->sym.n * int64_t(p->b)};
+                   p->d_col0, p->sym.n * int64_t(p->b), ws.ozfail + (count ? 1 : 0), p->wait_ns,
+                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0};
   const int b = p->b;
   const double es = double(sizeof(T)), fl = sizeof(T) == 16 ? 8.0 : 2.0, nb = sh.nb;
   for (size_t L = 0; L < p->levels.size(); ++L) {
@@ -508,15 +509,15 @@ BatchShifts make_shifts(const std::vector<std::complex<double>>& z, const std::v
   return sh;
 }
 
-// A bounded wait inside the split-precision kernels ran out: the site it
-// gave up at, read from the status word of the chain (0 = poles, 1 = inertia).
+// A bounded wait inside a kernel ran out: the site it gave up at, read from the
+// status word of the chain (0 = poles, 1 = inertia).
 int split_failed(Workspace& ws, int which, std::string* err, const char* what) {
   if (!ws.ozfail) return 0;
   int f = 0;
   ck(cudaMemcpyAsync(&f, ws.ozfail + which, sizeof(int), cudaMemcpyDeviceToHost, ws.stream), "status");
   ck(cudaStreamSynchronize(ws.stream), "sync");
   if (f && err)
-    *err = std::string(what) + ": a bounded device-side wait ran out (mode " + std::to_string((f >> 28) & 3) +
+    *err = std::string(((f >> 20) & 15) == 13 ? "block inverse" : what) + ": a bounded device-side wait ran out (mode " + std::to_string((f >> 28) & 3) +
            ", wait " + std::to_string(((f >> 20) & 255) & 15) + ", K tile " + std::to_string(((f >> 20) & 255) >> 4) +
            ", CTA " + std::to_string((f - 1) & ((1 << 20) - 1)) + ")";
   return f;
@@ -738,7 +739,8 @@ void factor_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
   cudaStream_t st = ws.stream;
   DevFronts fr = p->fronts();
   DevStatus status{ws.brk + (count ? 1 : 0), ws.minpiv + (count ? 1 : 0), ws.neg, count ? ws.dsave : nullptr,
-                   p->d_col0, p->sym.n * int64_t(p->b)};
+                   p->d_col0, p->sym.n * int64_t(p->b), ws.ozfail + (count ? 1 : 0), p->wait_ns,
+                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0};
   const int b = p->b;
   const double nb = sh.nb;
   for (size_t L = 0; L < p->levels.size(); ++L) {

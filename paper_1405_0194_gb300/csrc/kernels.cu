@@ -641,7 +641,8 @@ constexpr int kDiagCtas = 8;
 constexpr int kDiagUpdate = 192;
 constexpr int kDiagThreads = 256;
 constexpr int kDiagClusterMost = 99;
-constexpr unsigned long long kDiagWaitNs = 1000000000ull;
+constexpr unsigned long long kDiagDrainNs = 1000000000ull;
+constexpr int kDiagSite = 13;  // among the wait sites of record_fail (tensor_core.cuh)
 
 template <typename T>
 struct DiagStep {  // what a pivot step needs besides the column, sent by the column's owner
@@ -658,9 +659,19 @@ constexpr size_t diag_smem() {
          4 * (64 / kDiagCtas + 1) * sizeof(T);
 }
 
-// Bounded wait for phase 0 of a barrier; false after a second (the block is
-// then reported as broken down, and the kernel runs on without waiting).
-__device__ __forceinline__ bool diag_wait(uint32_t bar) {
+__device__ __forceinline__ unsigned long long diag_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// Wait for phase 0 of a barrier, bounded: `lost` after wait_ns. A thread that is
+// lost waits no more and writes nothing back, but sends what it would have sent,
+// so that no other wait runs out because of it and every barrier still gets its
+// bytes; the CTA drains its barriers before it leaves, since a late send into a
+// CTA that has gone would be an invalid access. A wait that ends does not look at
+// the flag: a test of it around every wait cost 2 us an inverse.
+__device__ __forceinline__ void diag_wait(uint32_t bar, unsigned long long wait_ns, bool& lost) {
   unsigned long long t0 = 0;
   for (uint32_t it = 0;; ++it) {
     uint32_t ok;
@@ -670,12 +681,11 @@ __device__ __forceinline__ bool diag_wait(uint32_t bar) {
         : "=r"(ok)
         : "r"(bar)
         : "memory");
-    if (ok) return true;
+    if (ok || lost) return;
     if ((it & 63u) == 63u) {
-      unsigned long long t;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      const unsigned long long t = diag_ns();
       if (t0 == 0) t0 = t;
-      else if (t - t0 > kDiagWaitNs) return false;
+      else if (t - t0 > wait_ns) lost = true;
     }
   }
 }
@@ -771,7 +781,8 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
   __syncthreads();
   cg::this_cluster().sync();  // every CTA runs and its barriers are set before any remote access
   if (tid == 0) *cg::this_cluster().map_shared_rank(&s_maxes[r], 0) = s_lmax;  // block max, gathered in CTA 0
-  bool lost = false;  // a wait ran out
+  bool lost = false;  // a wait of this thread ran out
+  auto wait = [&](uint32_t bar) { diag_wait(bar, st.wait_ns, lost); };
   // the holder of row i of column k hands it on: to its search warp and to every CTA
   auto hand_on = [&](int k, T v) {
     s_stage[i] = v;
@@ -780,11 +791,15 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
     for (int q = 0; q < C; ++q)
       send(cluster_addr(col0 + uint32_t((k * 64 + i) * sizeof(T)), q), v, cluster_addr(full0 + 8 * k, q));
   };
-  if (r == 0 && holds && g == 0) hand_on(0, a[0]);
+  if (r == 0 && holds && g == 0) {
+    if (st.hold)
+      for (const unsigned long long t0 = diag_ns(); diag_ns() - t0 < 4 * st.wait_ns;) __nanosleep(10000);
+    hand_on(0, a[0]);
+  }
 
   if (searcher) {
     for (int k = c0; k < c0 + nc; ++k) {
-      if (!diag_wait(ready0 + 8 * k)) lost = true;
+      wait(ready0 + 8 * k);
       // the first row from k on of the largest magnitude, as a serial scan finds it; NaN counts as below all
       const T v0 = lane >= k && lane < bb ? s_stage[lane] : zero_of(T());
       const T v1 = lane + 32 >= k && lane + 32 < bb ? s_stage[lane + 32] : zero_of(T());
@@ -805,7 +820,7 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
       const T piv = s_stage[row];
       const T rec = recip_piv(piv);
       const double best = mag1(piv);
-      if (k > 0 && !diag_wait(inv0 + 8 * (k - 1))) lost = true;  // long here: column k was updated with it
+      if (k > 0) wait(inv0 + 8 * (k - 1));  // long here: column k was updated with it
       const bool bad = (k > 0 && s_step[k - 1].bad) || !(best > 0.0) || !isfinite(best);
       if (lane < C) {
         const uint32_t d = cluster_addr(step0 + uint32_t(k * sizeof(DiagStep<T>)), lane), bar = cluster_addr(inv0 + 8 * k, lane);
@@ -816,7 +831,7 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
     }
   } else if (updater) {
     for (int k = 0; k < bb; ++k) {
-      if (!diag_wait(full0 + 8 * k)) lost = true;
+      wait(full0 + 8 * k);
       const int row = int(s_step[k].row), par = (k & 1) * (64 / C + 1);
       const T fac = s_col[k * 64 + (i == row ? k : i)];
       if (holds && (i == row || i == k)) {
@@ -830,7 +845,7 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
         }
       }
       asm volatile("bar.sync 1, %0;" ::"n"(NU) : "memory");
-      if (!diag_wait(inv0 + 8 * k)) lost = true;
+      wait(inv0 + 8 * k);
       const T inv = s_step[k].inv;
       // row k is scaled by the reciprocal; column k keeps the multipliers' negatives over the pivot
       auto update = [&](T old, int jl, T rk) {
@@ -859,11 +874,12 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
       }
     }
     // write back: the row interchanges are column interchanges of the inverse,
-    // undone in reverse order, applied to each column's destination index
+    // undone in reverse order, applied to each column's destination index (a
+    // thread whose waits all ended has every step's pivot row)
 #pragma unroll
     for (int q = 0; q < E; ++q) {
       const int jl = g + ng * q;
-      if (holds && jl < nc) {
+      if (holds && jl < nc && !lost) {
         int pos = c0 + jl;
         for (int k = bb - 1; k >= 0; --k) {
           const int x = int(s_step[k].row);
@@ -874,9 +890,16 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
       }
     }
   }
-  if (lost) atomicMin(st.breakdown_front, f);
+  const bool gave_up = __syncthreads_or(lost);
+  if (gave_up && tid < bb) {  // what is still on its way here
+    bool late = false;
+    diag_wait(full0 + 8 * tid, kDiagDrainNs, late);
+    diag_wait(inv0 + 8 * tid, kDiagDrainNs, late);
+  }
   cg::this_cluster().sync();  // every remote write of the cluster is done before any CTA leaves
-  if (r == 0 && tid == 0) {
+  if (gave_up) {
+    if (tid == 0) atomicMax(st.fail, 1 + (kDiagSite << 20) + min(int(blockIdx.x), (1 << 20) - 1));
+  } else if (r == 0 && tid == 0) {
     double mx = 0.0, pmin = DBL_MAX;
     for (int q = 0; q < C; ++q) mx = fmax(mx, s_maxes[q]);
     for (int k = 0; k < bb; ++k) pmin = fmin(pmin, s_step[k].best);

@@ -78,6 +78,9 @@ struct DevStatus {
   void* dsave;
   const int32_t* col0;               // first column of each front
   int64_t dsave_stride;
+  int* fail;                         // atomicMax of where a wait of a cluster block inverse ran out (0 = none)
+  uint64_t wait_ns;                  // bound of these waits (wall time)
+  int hold;                          // fault injection: the first column of each cluster comes after 4 wait_ns
 };
 
 // Scratch of the split-precision GEMM: bf16 slice tiles of A = Y[S,S] and

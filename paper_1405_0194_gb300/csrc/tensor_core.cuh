@@ -153,9 +153,12 @@ __device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;");
 }
 
-// Where a wait ran out: site (1..8) + 16 * (K tile mod 16), below 256; the
+// Where a wait ran out: site (1..12) + 16 * (K tile mod 16), below 256; the
 // launch reports 1 + (mode << 28) + (this << 20) + CTA index, mode 1-3 for the
-// short-K GEMM (its MODE), 0 for the Takahashi / Y[P,P] kernel.
+// short-K GEMM of the split path (its MODE), 0 for its Takahashi / Y[P,P] kernel
+// and for the residue GEMM. The residue GEMM's sites: 9 its producer, 10 and 11
+// the MMA issuer (accumulator, operands), 12 the reduction, 3 and 7 the copies
+// and MMAs in flight. 13 is the cluster block inverse (kernels.cu).
 __device__ __forceinline__ void record_fail(int* s_fail, int site, int kt) {
   atomicCAS(s_fail, 0, site + 16 * (kt & 15));
 }

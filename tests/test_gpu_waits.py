@@ -1,0 +1,67 @@
+"""Waits of the FP64 path that run out, made to happen without faulting the GPU
+(pexsi_opts.inject = 1, wait_ns = 2 ms): the launch ends cleanly, the call
+returns PEXSI_ERR_TIMEOUT and names the wait, and the context stays usable.
+
+A front of up to 64 columns without rows below it runs the block inverse and no
+GEMM, so its timeout is the block inverse's: the first column of the cluster
+comes 8 ms late.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_1405_0194_gb300 as px  # noqa: E402
+
+WAIT_NS = 2_000_000
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_1405_0194_gb300 import build
+    build.build()
+
+
+def _full(n, seed):
+    """A dense symmetric pair on the full pattern (one front of n columns)."""
+    rng = np.random.default_rng(seed)
+    H = rng.standard_normal((n, n)) / np.sqrt(n)
+    H = H + H.T
+    S = np.eye(n)
+    return np.arange(0, n * n + 1, n, dtype=np.int64), np.tile(np.arange(n, dtype=np.int32), n), H, S
+
+
+def _times_out(call, what):
+    with pytest.raises(px.PexsiError) as e:
+        call()
+    assert e.value.code == px.capi.PEXSI_ERR_TIMEOUT
+    assert what in str(e.value) and "wait ran out" in str(e.value)
+
+
+def _works(n, colptr, rowind, H, S):
+    torch.cuda.synchronize()  # no sticky error: the launches returned normally
+    plan = px.pexsi_setup(n, colptr, rowind, opts=px.pexsi_opts_default(max_batch=2, wait_ns=500_000_000))
+    got = px.pexsi_selinv(plan, H.ravel(), S.ravel(), 0.1 + 0.05j).reshape(n, n)
+    px.pexsi_plan_destroy(plan)
+    ref = np.linalg.inv(H - (0.1 + 0.05j) * S)
+    assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [1, 13, 48, 64])
+def test_block_inverse(n):
+    colptr, rowind, H, S = _full(n, n)
+    plan = px.pexsi_setup(n, colptr, rowind, opts=px.pexsi_opts_default(max_batch=2, inject=1, wait_ns=WAIT_NS))
+    try:
+        _times_out(lambda: px.pexsi_selinv(plan, H.ravel(), S.ravel(), 0.1 + 0.05j), "block inverse")
+        _times_out(lambda: px.pexsi_dm(plan, H.ravel(), S.ravel(), 0.1, 50.0, 2, 4.0), "block inverse")
+        _times_out(lambda: px.pexsi_inertia(plan, H.ravel(), S.ravel(), [0.1, 0.2]), "block inverse")
+        Hc = H.ravel().astype(complex)
+        _times_out(lambda: px.pexsi_selinv_hermitian(plan, Hc, S.ravel().astype(complex), 0.1 + 0.05j), "block inverse")
+        _times_out(lambda: px.pexsi_inertia_hermitian(plan, Hc, S.ravel().astype(complex), [0.1]), "block inverse")
+    finally:
+        px.pexsi_plan_destroy(plan)
+    _works(n, colptr, rowind, H, S)
