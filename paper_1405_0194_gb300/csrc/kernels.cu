@@ -818,6 +818,7 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
         send(cluster_addr(step0 + uint32_t(k * sizeof(DiagStep<T>) + offsetof(DiagStep<T>, row)), lane),
              __longlong_as_double(row), cluster_addr(full0 + 8 * k, lane));
       const T piv = s_stage[row];
+      __syncwarp();  // every lane has read the column before a lane's reciprocal lets the update threads stage the next
       const T rec = recip_piv(piv);
       const double best = mag1(piv);
       if (k > 0) wait(inv0 + 8 * (k - 1));  // long here: column k was updated with it

@@ -65,3 +65,18 @@ def test_block_inverse(n):
     finally:
         px.pexsi_plan_destroy(plan)
     _works(n, colptr, rowind, H, S)
+
+
+@pytest.mark.parametrize("n", [33, 64])
+def test_cluster_inverses_repeat_their_bits(n):
+    """The staged pivot column is read by every lane of the search warp before the next one replaces it: the inverses of
+    many launches, with row interchanges in nearly every step, are the same bits each time."""
+    colptr, rowind, H, S = _full(n, 7 * n)
+    Hc = (H + 1j * (np.triu(H, 1) - np.tril(H, -1))).T.ravel()
+    plan = px.pexsi_setup(n, colptr, rowind, opts=px.pexsi_opts_default(max_batch=2))
+    first = px.pexsi_selinv(plan, H.ravel(), S.ravel(), 0.1 + 0.05j)
+    herm = px.pexsi_selinv_hermitian(plan, Hc, S.ravel().astype(complex), 0.1 + 0.05j)
+    for _ in range(60):
+        assert np.array_equal(first, px.pexsi_selinv(plan, H.ravel(), S.ravel(), 0.1 + 0.05j))
+        assert np.array_equal(herm, px.pexsi_selinv_hermitian(plan, Hc, S.ravel().astype(complex), 0.1 + 0.05j))
+    px.pexsi_plan_destroy(plan)
