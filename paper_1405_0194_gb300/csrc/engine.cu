@@ -300,7 +300,7 @@ void factor_batch(const pexsi_plan* p, Workspace& ws, T* F, const BatchShifts& s
   // are saved and counted after the factorisation
   DevStatus status{ws.brk + (count ? 1 : 0), ws.minpiv + (count ? 1 : 0), ws.neg, count ? ws.dsave : nullptr,
                    p->d_col0, p->sym.n * int64_t(p->b), ws.ozfail + (count ? 1 : 0), p->wait_ns,
-                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0};
+                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g};
   const int b = p->b;
   const double es = double(sizeof(T)), fl = sizeof(T) == 16 ? 8.0 : 2.0, nb = sh.nb;
   for (size_t L = 0; L < p->levels.size(); ++L) {
@@ -740,7 +740,7 @@ void factor_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
   DevFronts fr = p->fronts();
   DevStatus status{ws.brk + (count ? 1 : 0), ws.minpiv + (count ? 1 : 0), ws.neg, count ? ws.dsave : nullptr,
                    p->d_col0, p->sym.n * int64_t(p->b), ws.ozfail + (count ? 1 : 0), p->wait_ns,
-                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0};
+                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g};
   const int b = p->b;
   const double nb = sh.nb;
   for (size_t L = 0; L < p->levels.size(); ++L) {
@@ -1383,10 +1383,17 @@ int upload_plan(pexsi_plan* p) {
   }
   if (p->sys_col_off.empty()) p->sys_col_off = {0, S.n};
   if (p->oz_slices == 0) {
-    std::vector<int32_t> col(S.nnz);
-    for (int64_t c = 0; c < S.n; ++c) std::fill(col.begin() + p->col_start[c], col.begin() + p->col_start[c + 1], int32_t(c));
-    p->d_diag = dev_upload(p->diag_entries);
-    p->d_row = dev_upload(p->entry_row);
+    std::vector<int32_t> row(S.nnz), col(S.nnz);
+    std::vector<int64_t> diag(S.n);
+    for (int64_t c = 0; c < S.n; ++c) {
+      diag[S.iperm[c]] = p->diag_entries[c];
+      for (int64_t e = p->col_start[c]; e < p->col_start[c + 1]; ++e) {
+        row[e] = S.iperm[p->entry_row[e]];
+        col[e] = S.iperm[c];
+      }
+    }
+    p->d_diag = dev_upload(diag);
+    p->d_row = dev_upload(row);
     p->d_col = dev_upload(col);
   }
   ck(cudaStreamCreateWithFlags(&p->ws.stream, cudaStreamNonBlocking), "cudaStreamCreate");

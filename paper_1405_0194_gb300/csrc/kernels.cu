@@ -322,11 +322,14 @@ __device__ __forceinline__ void zero_acc(T (&acc)[4][4]) {
     for (int j = 0; j < 4; ++j) acc[i][j] = zero_of(T());
 }
 
+// 2^e, |e| <= 1022
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
 // ------------------------------------------------------------ assembly
 // 2^-g of entry e of a plan whose rows and columns are scaled (gs: sum of the
 // two exponents per CSC entry; NULL: no scaling), |g| <= 1022.
 __device__ __forceinline__ double entry_scale(const int16_t* __restrict__ gs, int64_t e) {
-  return gs ? __hiloint2double((1023 - int(gs[e])) << 20, 0) : 1.0;
+  return gs ? pow2(-int(gs[e])) : 1.0;
 }
 
 template <typename T>
@@ -725,6 +728,7 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
   uint64_t* s_ready = s_inv + 64;                                            // [64]: the next column is staged
   __shared__ double s_lmax, s_maxes[C];
   __shared__ T s_scaled[64 / C];
+  __shared__ int s_ex[64];  // scaling exponents of the block's rows and columns
   const int f = fronts[blockIdx.x / C];
   const int r = int(cg::this_cluster().block_rank());
   const int pb = blockIdx.y;
@@ -748,6 +752,7 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
   const uint32_t col0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_col));
   const uint32_t step0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_step));
   if (tid < 64) {
+    s_ex[tid] = st.g && tid < bb ? st.g[st.col0[f] + p0 + tid] : 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8 * tid));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(inv0 + 8 * tid));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(ready0 + 8 * tid), "r"(bb));
@@ -772,7 +777,7 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
     a[q] = zero_of(T());
     if (holds && jl < nc) {
       a[q] = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
-      lmax = fmax(lmax, mag1(a[q]));
+      lmax = fmax(lmax, mag1(a[q]) * pow2(s_ex[i] + s_ex[j]));
       if (save) save[i * b + j] = a[q];
     }
   }
@@ -900,13 +905,25 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
   cg::this_cluster().sync();  // every remote write of the cluster is done before any CTA leaves
   if (gave_up) {
     if (tid == 0) atomicMax(st.fail, 1 + (kDiagSite << 20) + min(int(blockIdx.x), (1 << 20) - 1));
-  } else if (r == 0 && tid == 0) {
-    double mx = 0.0, pmin = DBL_MAX;
-    for (int q = 0; q < C; ++q) mx = fmax(mx, s_maxes[q]);
-    for (int k = 0; k < bb; ++k) pmin = fmin(pmin, s_step[k].best);
-    const double ratio = mx > 0 ? pmin / mx : 0.0;
-    atomicMin(st.min_pivot, (unsigned long long)__double_as_longlong(ratio));
-    if (s_step[bb - 1].bad || ratio < 1e-13) atomicMin(st.breakdown_front, f);
+  } else if (r == 0 && tid < (bb + 31) / 32 * 32) {  // a step per thread, one warp or two
+    double pmin = DBL_MAX;
+    if (tid < bb) {
+      int row = int(s_step[tid].row);  // the pivot's row before the interchanges
+      if (st.g)
+        for (int k = tid - 1; k >= 0; --k) {
+          const int x = int(s_step[k].row);
+          row = row == k ? x : row == x ? k : row;
+        }
+      pmin = fmin(pmin, s_step[tid].best * pow2(s_ex[row] + s_ex[tid]));
+    }
+    for (int o = 16; o > 0; o >>= 1) pmin = fmin(pmin, __shfl_xor_sync(0xffffffffu, pmin, o));
+    if (lane == 0) {
+      double mx = 0.0;
+      for (int q = 0; q < C; ++q) mx = fmax(mx, s_maxes[q]);
+      const double ratio = mx > 0 ? pmin / mx : 0.0;
+      atomicMin(st.min_pivot, (unsigned long long)__double_as_longlong(ratio));
+      if (s_step[bb - 1].bad || ratio < 1e-13) atomicMin(st.breakdown_front, f);
+    }
   }
 }
 
@@ -929,6 +946,9 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
   __shared__ T s_fac[64];
   __shared__ T s_inv;
   __shared__ int s_perm[64];
+  __shared__ int s_ex[2][64];  // scaling exponents of the columns, and of the rows as they are interchanged
+  if (threadIdx.x < 64) s_ex[0][threadIdx.x] = s_ex[1][threadIdx.x] =
+      st.g && int(threadIdx.x) < bb ? st.g[st.col0[f] + p0 + threadIdx.x] : 0;
   if (threadIdx.x == 0) { s_max = 0.0; s_pmin = DBL_MAX; s_bad = false; }
   __syncthreads();
   double lmax = 0.0;
@@ -937,7 +957,7 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
     // symmetric fronts hold the lower triangle; LDU fronts (GEN) both
     T v = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
     Aug[i * ld + j] = v;
-    lmax = fmax(lmax, mag1(v));
+    lmax = fmax(lmax, mag1(v) * pow2(s_ex[0][i] + s_ex[0][j]));
   }
   // block max |entry| for the pivot ratio
   for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
@@ -969,7 +989,8 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
       if (threadIdx.x == 0) {
         const double best = mag1(Aug[bi * ld + k]);
         s_piv = bi;
-        s_pmin = fmin(s_pmin, best);
+        s_pmin = fmin(s_pmin, best * pow2(s_ex[1][bi] + s_ex[0][k]));
+        s_ex[1][bi] = s_ex[1][k];
         if (!(best > 0.0) || !isfinite(best)) s_bad = true;
       }
     }

@@ -81,6 +81,9 @@ struct DevStatus {
   int* fail;                         // atomicMax of where a wait of a cluster block inverse ran out (0 = none)
   uint64_t wait_ns;                  // bound of these waits (wall time)
   int hold;                          // fault injection: the first column of each cluster comes after 4 wait_ns
+  // fronts of a scaled matrix (launch_rns_scales; NULL: unscaled): exponent per column in elimination order. The
+  // pivot ratio is that of the matrix as the caller gave it.
+  const int32_t* g;
 };
 
 // Scratch of the split-precision GEMM: bf16 slice tiles of A = Y[S,S] and

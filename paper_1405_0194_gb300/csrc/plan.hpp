@@ -107,7 +107,7 @@ struct Workspace {
   int *exA = nullptr, *exB = nullptr, *ozfail = nullptr;
   uint32_t* ymax = nullptr;  // split path: row maxima of Y per pole
   RnsScratch rns;            // FP64 path: scratch of the residue products (no planes: DFMA kernels)
-  int32_t* g = nullptr;      // its power-of-two scaling: exponent per row, and per CSC entry of the current H and S
+  int32_t* g = nullptr;      // its power-of-two scaling: exponent per column, and per CSC entry of the current H and S
   int16_t* gs = nullptr;
   cudaStream_t stream = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -170,7 +170,8 @@ struct pexsi_plan {
   std::vector<int64_t> diag_entries;  // CSC entries on the diagonal
   std::vector<int32_t> entry_row;     // row of every CSC entry, and the column bounds, both of this plan's matrix
   std::vector<int64_t> col_start;
-  int64_t* d_diag = nullptr;          // FP64 plans: the diagonal entry of every column, the row and column of every entry
+  // FP64 plans: the diagonal entry of every column, the row and column of every entry; columns in elimination order
+  int64_t* d_diag = nullptr;
   int32_t *d_row = nullptr, *d_col = nullptr;
   // A plan that merges several systems (pexsi_group): the first CSC entry of
   // each system among the concatenated entries (nsys + 1), and each system's
