@@ -647,6 +647,23 @@ constexpr int kDiagClusterMost = 99;
 constexpr unsigned long long kDiagDrainNs = 1000000000ull;
 constexpr int kDiagSite = 13;  // among the wait sites of record_fail (tensor_core.cuh)
 
+// *at = min(*at, v) of non-negative values in shared memory (NaN does not count)
+__device__ __forceinline__ void least(double* at, double v) {
+  atomicMin(reinterpret_cast<unsigned long long*>(at), (unsigned long long)__double_as_longlong(v));
+}
+
+// Smallest pivot and largest entry of a block: of the matrix as the caller gave
+// it (pmin, mx), which is what the call reports, and of the scaled one (gmin,
+// gx). It breaks down where the ratio is below the limit in both: in the first
+// alone a graded matrix would, in the second alone a level near a shift beside
+// orbitals of small diagonal.
+__device__ __forceinline__ void report_pivots(const DevStatus& st, int f, bool bad, double pmin, double mx, double gmin,
+                                              double gx) {
+  const double ratio = mx > 0 ? pmin / mx : 0.0, scaled = gx > 0 ? gmin / gx : 0.0;
+  atomicMin(st.min_pivot, (unsigned long long)__double_as_longlong(ratio));
+  if (bad || (ratio < 1e-13 && scaled < 1e-13)) atomicMin(st.breakdown_front, f);
+}
+
 template <typename T>
 struct DiagStep {  // what a pivot step needs besides the column, sent by the column's owner
   T inv;           // reciprocal of the pivot (0 once a pivot was zero or not finite)
@@ -710,8 +727,10 @@ __device__ __forceinline__ void send(uint32_t a, double2 v, uint32_t bar) {
                : "memory");
 }
 
+// Three CTAs to an SM (real: four): at 88 registers and two of them the clusters
+// of 40 inversions a launch took turns (a 64-atom chain 0.858 -> 0.949 ms).
 template <typename T, bool GEN>
-__global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restrict__ F, DevFronts fr,
+__global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_inv_cluster(T* __restrict__ F, DevFronts fr,
                                                                       const int32_t* __restrict__ fronts, int p0, int b,
                                                                       DevStatus st) {
   namespace cg = cooperative_groups;
@@ -726,7 +745,9 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
   uint64_t* s_full = reinterpret_cast<uint64_t*>(s_row + 2 * (64 / C + 1));  // [64]: column and pivot row are here
   uint64_t* s_inv = s_full + 64;                                             // [64]: the reciprocal is here
   uint64_t* s_ready = s_inv + 64;                                            // [64]: the next column is staged
-  __shared__ double s_lmax, s_maxes[C];
+  // smallest pivot and largest entry of this CTA's columns, as the caller gave the matrix and as it is scaled, and of
+  // every CTA's, gathered in CTA 0
+  __shared__ double s_ext[4], s_exts[4][C];
   __shared__ T s_scaled[64 / C];
   __shared__ int s_ex[64];  // scaling exponents of the block's rows and columns
   const int f = fronts[blockIdx.x / C];
@@ -764,11 +785,11 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(inv0 + 8 * tid), "r"(int(sizeof(T)) + 16)
                  : "memory");
   }
-  if (tid == 0) s_lmax = 0.0;
+  if (tid < 4) s_ext[tid] = tid & 1 ? 0.0 : DBL_MAX;
   __syncthreads();
   // symmetric fronts hold the lower triangle; LDU fronts (GEN) both
   T a[E];
-  double lmax = 0.0;
+  double lmax = 0.0, gmax = 0.0;  // largest entry as the caller gave the matrix, and as it is scaled
   T* save = st.dsave ? reinterpret_cast<T*>(st.dsave) + int64_t(pb) * st.dsave_stride + int64_t(st.col0[f] + p0) * b
                      : nullptr;  // inertia shifts: the block before inversion, counted later
 #pragma unroll
@@ -777,15 +798,19 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
     a[q] = zero_of(T());
     if (holds && jl < nc) {
       a[q] = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
+      gmax = fmax(gmax, mag1(a[q]));
       lmax = fmax(lmax, mag1(a[q]) * pow2(s_ex[i] + s_ex[j]));
       if (save) save[i * b + j] = a[q];
     }
   }
-  for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-  if (lane == 0) atomicMax(reinterpret_cast<unsigned long long*>(&s_lmax), __double_as_longlong(lmax));
+  for (int o = 16; o > 0; o >>= 1) {
+    lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+    gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+  }
+  if (lane < 2)
+    atomicMax(reinterpret_cast<unsigned long long*>(&s_ext[2 * lane + 1]), __double_as_longlong(lane == 0 ? lmax : gmax));
   __syncthreads();
   cg::this_cluster().sync();  // every CTA runs and its barriers are set before any remote access
-  if (tid == 0) *cg::this_cluster().map_shared_rank(&s_maxes[r], 0) = s_lmax;  // block max, gathered in CTA 0
   bool lost = false;  // a wait of this thread ran out
   auto wait = [&](uint32_t bar) { diag_wait(bar, st.wait_ns, lost); };
   // the holder of row i of column k hands it on: to its search warp and to every CTA
@@ -893,6 +918,11 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
           else if (pos == x) pos = k;
         }
         Fd[i + int64_t(m) * pos] = a[q];
+        if (i == 0) {  // pos: the row of this column's pivot before the interchanges
+          const double best = s_step[c0 + jl].best;
+          least(&s_ext[0], best * pow2(s_ex[pos] + s_ex[c0 + jl]));
+          least(&s_ext[2], best);
+        }
       }
     }
   }
@@ -902,28 +932,15 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_inv_cluster(T* __restr
     diag_wait(full0 + 8 * tid, kDiagDrainNs, late);
     diag_wait(inv0 + 8 * tid, kDiagDrainNs, late);
   }
+  if (tid < 4) *cg::this_cluster().map_shared_rank(&s_exts[tid][r], 0) = s_ext[tid];
   cg::this_cluster().sync();  // every remote write of the cluster is done before any CTA leaves
   if (gave_up) {
     if (tid == 0) atomicMax(st.fail, 1 + (kDiagSite << 20) + min(int(blockIdx.x), (1 << 20) - 1));
-  } else if (r == 0 && tid < (bb + 31) / 32 * 32) {  // a step per thread, one warp or two
-    double pmin = DBL_MAX;
-    if (tid < bb) {
-      int row = int(s_step[tid].row);  // the pivot's row before the interchanges
-      if (st.g)
-        for (int k = tid - 1; k >= 0; --k) {
-          const int x = int(s_step[k].row);
-          row = row == k ? x : row == x ? k : row;
-        }
-      pmin = fmin(pmin, s_step[tid].best * pow2(s_ex[row] + s_ex[tid]));
-    }
-    for (int o = 16; o > 0; o >>= 1) pmin = fmin(pmin, __shfl_xor_sync(0xffffffffu, pmin, o));
-    if (lane == 0) {
-      double mx = 0.0;
-      for (int q = 0; q < C; ++q) mx = fmax(mx, s_maxes[q]);
-      const double ratio = mx > 0 ? pmin / mx : 0.0;
-      atomicMin(st.min_pivot, (unsigned long long)__double_as_longlong(ratio));
-      if (s_step[bb - 1].bad || ratio < 1e-13) atomicMin(st.breakdown_front, f);
-    }
+  } else if (r == 0 && tid == 0) {
+    double ext[4] = {DBL_MAX, 0.0, DBL_MAX, 0.0};
+    for (int q = 0; q < C; ++q)
+      for (int x = 0; x < 4; ++x) ext[x] = x & 1 ? fmax(ext[x], s_exts[x][q]) : fmin(ext[x], s_exts[x][q]);
+    report_pivots(st, f, s_step[bb - 1].bad, ext[0], ext[1], ext[2], ext[3]);
   }
 }
 
@@ -939,29 +956,36 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
   const int bb = min(b, s - p0);
   const int ld = b + 1;
   T* Fd = F + int64_t(pb) * fr.pool + fr.off[f] + p0 + int64_t(m) * p0;
-  __shared__ double s_max;
+  __shared__ double s_max[2];  // largest entry and smallest pivot: as the caller gave the matrix, and scaled
   __shared__ int s_piv;
-  __shared__ double s_pmin;
+  __shared__ double s_pmin[2];
   __shared__ bool s_bad;
   __shared__ T s_fac[64];
   __shared__ T s_inv;
   __shared__ int s_perm[64];
   __shared__ int s_ex[2][64];  // scaling exponents of the columns, and of the rows as they are interchanged
+  __shared__ double s_best[64];
   if (threadIdx.x < 64) s_ex[0][threadIdx.x] = s_ex[1][threadIdx.x] =
       st.g && int(threadIdx.x) < bb ? st.g[st.col0[f] + p0 + threadIdx.x] : 0;
-  if (threadIdx.x == 0) { s_max = 0.0; s_pmin = DBL_MAX; s_bad = false; }
+  if (threadIdx.x < 2) { s_max[threadIdx.x] = 0.0; s_pmin[threadIdx.x] = DBL_MAX; s_bad = false; }
   __syncthreads();
-  double lmax = 0.0;
+  double lmax = 0.0, gmax = 0.0;
   for (int idx = threadIdx.x; idx < bb * bb; idx += 256) {
     int i = idx % bb, j = idx / bb;
     // symmetric fronts hold the lower triangle; LDU fronts (GEN) both
     T v = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
     Aug[i * ld + j] = v;
+    gmax = fmax(gmax, mag1(v));
     lmax = fmax(lmax, mag1(v) * pow2(s_ex[0][i] + s_ex[0][j]));
   }
   // block max |entry| for the pivot ratio
-  for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned long long*>(&s_max), __double_as_longlong(lmax));
+  for (int o = 16; o > 0; o >>= 1) {
+    lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+    gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+  }
+  if ((threadIdx.x & 31) < 2)
+    atomicMax(reinterpret_cast<unsigned long long*>(&s_max[threadIdx.x & 31]),
+              __double_as_longlong((threadIdx.x & 31) == 0 ? lmax : gmax));
   __syncthreads();
 
   if (st.dsave) {
@@ -989,8 +1013,10 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
       if (threadIdx.x == 0) {
         const double best = mag1(Aug[bi * ld + k]);
         s_piv = bi;
-        s_pmin = fmin(s_pmin, best * pow2(s_ex[1][bi] + s_ex[0][k]));
+        s_best[k] = best;
+        const int ex = s_ex[1][bi];
         s_ex[1][bi] = s_ex[1][k];
+        s_ex[1][k] = ex;
         if (!(best > 0.0) || !isfinite(best)) s_bad = true;
       }
     }
@@ -1018,6 +1044,10 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
     }
     __syncthreads();
   }
+  if (int(threadIdx.x) < bb) {
+    least(&s_pmin[0], s_best[threadIdx.x] * pow2(s_ex[1][threadIdx.x] + s_ex[0][threadIdx.x]));
+    least(&s_pmin[1], s_best[threadIdx.x]);
+  }
   // the row interchanges become column interchanges of the inverse, undone in reverse order
   for (int k = bb - 1; k >= 0; --k) {
     const int pr = s_perm[k];
@@ -1031,11 +1061,7 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
     int i = idx % bb, j = idx / bb;
     Fd[i + int64_t(m) * j] = Aug[i * ld + j];
   }
-  if (threadIdx.x == 0) {
-    double ratio = s_max > 0 ? s_pmin / s_max : 0.0;
-    atomicMin(st.min_pivot, (unsigned long long)__double_as_longlong(ratio));
-    if (s_bad || ratio < 1e-13) atomicMin(st.breakdown_front, f);
-  }
+  if (threadIdx.x == 0) report_pivots(st, f, s_bad, s_pmin[0], s_max[0], s_pmin[1], s_max[1]);
 }
 
 // Deferred inertia count: one CTA per (saved panel block, batch member).

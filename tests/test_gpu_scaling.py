@@ -54,12 +54,13 @@ def test_pivot_ratio_is_the_callers(n, blocks):
 @pytest.mark.parametrize("others,refused", [(1e-3, False), (1.0, True)])
 def test_what_is_refused(others, refused):
     """A level 2^-46 from the shift: a pivot ratio of 1e-11 beside orbitals of 1e-3, of 1e-14 (below the limit of 1e-13)
-    beside orbitals of order one, whatever the size of the level's own H and S."""
+    beside orbitals of order one. A graded pencil is not refused."""
     n = 60
     colptr, rowind = _pattern(n)
     h, s = np.full(n, 2.0 * others), np.full(n, others)
     h[17], s[17] = 1.0, 1.0
     shift = 1.0 - 2.0 ** -46
+    d = 2.0 ** -np.random.default_rng(4).integers(0, 31, n)
     plan = px.pexsi_setup(n, colptr, rowind, opts=px.pexsi_opts_default(max_batch=1))
     try:
         for call, dt in ((px.pexsi_inertia, float), (px.pexsi_inertia_hermitian, complex)):
@@ -70,5 +71,6 @@ def test_what_is_refused(others, refused):
                 assert e.value.code == px.capi.PEXSI_ERR_BREAKDOWN
             else:
                 assert call(plan, H, S, [shift]).tolist() == [0]
+            assert call(plan, np.diag(d * d).ravel().astype(dt), np.diag(d * d).ravel().astype(dt), [0.5]).tolist() == [0]
     finally:
         px.pexsi_plan_destroy(plan)
