@@ -78,6 +78,7 @@ int64_t kpart_stride(const pexsi_plan* p) {
 
 int64_t bytes_per_pole(const pexsi_plan* p, bool rns) {
   return (2 * p->sym.front_elems + p->part_stride + (rns ? 0 : kpart_stride(p))) * int64_t(sizeof(double2)) +
+         (rns ? 2 * p->sym.n * scale_stride(1) * int64_t(sizeof(int16_t)) : 0) +
          2 * p->sym.n * int64_t(p->b) * int64_t(sizeof(double)) +
          std::max(p->ozA_stride, 2 * p->ozA_stride_r) + std::max(p->ozB_stride, 2 * p->ozB_stride_r) +
          8 * (p->exA_stride + p->exB_stride) + 4 * p->ymax_stride;
@@ -85,7 +86,7 @@ int64_t bytes_per_pole(const pexsi_plan* p, bool rns) {
 
 int64_t bytes_fixed(const pexsi_plan* p) {
   return 9 * p->sym.nnz * int64_t(sizeof(double)) + 4 * p->trace_blocks * 8 + 4096 +
-         (p->oz_slices > 0 ? 0 : 2 * p->sym.nnz + 4 * p->sym.n);
+         (p->oz_slices > 0 ? 0 : 2 * p->sym.n);
 }
 
 void rns_scratch(const pexsi_plan* p, int batch, int64_t most, int64_t& planes, int64_t& out) {
@@ -162,8 +163,10 @@ void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, int64_t rns_
   if (rns_planes > 0) {
     wsalloc(&ws.rns.planes, size_t(rns_planes), ws, "alloc(residue planes)");
     wsalloc(&ws.rns.out, size_t(rns_out), ws, "alloc(residue tiles)");
-    wsalloc(&ws.g, sizeof(int32_t) * size_t(p->sym.n), ws, "alloc(scaling)");
-    wsalloc(&ws.gs, sizeof(int16_t) * nnz, ws, "alloc(scaling)");
+    // for `batch` poles, or twice as many inertia shifts
+    wsalloc(&ws.g, sizeof(int16_t) * size_t(p->sym.n * scale_stride(batch)), ws, "alloc(scaling)");
+    wsalloc(&ws.g0, sizeof(int16_t) * size_t(p->sym.n * scale_stride(batch)), ws, "alloc(scaling)");
+    wsalloc(&ws.h, sizeof(int16_t) * size_t(p->sym.n), ws, "alloc(scaling)");
     ws.rns.plane_bytes = rns_planes;
     ws.rns.out_bytes = rns_out;
     ws.rns.wait_ns = p->wait_ns;
@@ -185,7 +188,7 @@ void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, int64_t rns_
 void workspace_free(Workspace& ws) {
   void* ptrs[] = {ws.F,  ws.Y,        ws.part,  ws.H,    ws.S,   ws.out, ws.brk, ws.minpiv, ws.neg,
                   ws.partials, ws.trace3, ws.ainv, ws.ozA, ws.ozB, ws.exA, ws.exB, ws.ozfail, ws.ymax, ws.kpart,
-                  ws.dsave, ws.rns.planes, ws.rns.out, ws.g, ws.gs};
+                  ws.dsave, ws.rns.planes, ws.rns.out, ws.g, ws.g0, ws.h};
   for (void* q : ptrs) {
     if (!q) continue;
     if (ws.async) cudaFreeAsync(q, ws.stream);
@@ -300,7 +303,7 @@ void factor_batch(const pexsi_plan* p, Workspace& ws, T* F, const BatchShifts& s
   // are saved and counted after the factorisation
   DevStatus status{ws.brk + (count ? 1 : 0), ws.minpiv + (count ? 1 : 0), ws.neg, count ? ws.dsave : nullptr,
                    p->d_col0, p->sym.n * int64_t(p->b), ws.ozfail + (count ? 1 : 0), p->wait_ns,
-                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g};
+                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g, ws.h, scale_stride(ws.batch)};
   const int b = p->b;
   const double es = double(sizeof(T)), fl = sizeof(T) == 16 ? 8.0 : 2.0, nb = sh.nb;
   for (size_t L = 0; L < p->levels.size(); ++L) {
@@ -571,21 +574,23 @@ void factor_selinv(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh, Pr
   ck(cudaGraphLaunch(g.exec, ws.stream), "cudaGraphLaunch");
 }
 
-// The scaling exponents of the values H and S (plans and workspaces with
-// residue products; wide: 1 real, 2 complex values).
-void set_scales(const pexsi_plan* p, Workspace& ws, const double* dH, const double* dS, int wide = 1, size_t q = 0) {
-  if (!ws.gs) return;
-  const int64_t e0 = p->sys_entry_off[q], ne = p->sys_entry_off[q + 1] - e0;
-  launch_rns_scales(dH, dS, wide, p->d_diag, p->sys_col_off[q], p->sys_col_off[q + 1] - p->sys_col_off[q], p->d_row,
-                    p->d_col, e0, ne, ws.g, ws.gs, ws.stream);
+// The scaling exponents of A = H - z S for the shifts of a batch (workspaces with
+// residue products; wide: 1 real, 2 complex values; q: system of a group).
+void set_scales(const pexsi_plan* p, Workspace& ws, const double* dH, const double* dS, const BatchShifts& sh,
+                int wide = 1, size_t q = 0) {
+  if (!ws.g) return;
+  const int64_t c0 = p->sys_col_off[q], n = p->sys_col_off[q + 1] - c0;
+  launch_rns_scales(dH, dS, wide, sh, p->d_colptr + c0, p->d_diag + c0, n, c0, p->sys_entry_off[q], p->d_row, p->d_col,
+                    ws.h, ws.g0, ws.g, scale_stride(ws.batch), ws.stream);
 }
 
 void run_complex_batch(const pexsi_plan* p, Workspace& ws, const double* dH, const double* dS, const BatchShifts& sh,
                        Profiler& pf) {
   const int64_t pool = p->sym.front_elems;
+  set_scales(p, ws, dH, dS, sh);
   ck(cudaMemsetAsync(ws.F, 0, sizeof(double2) * size_t(pool) * sh.nb, ws.stream), "memset(F)");
   cudaEvent_t a = pf.begin(ws.stream);
-  launch_assemble<double2>(ws.F, dH, dS, p->d_asm_src, p->d_asm_pos, p->nlow, pool, sh, ws.gs, ws.stream);
+  launch_assemble<double2>(ws.F, dH, dS, p->d_asm_src, p->d_asm_pos, p->nlow, pool, sh, entry_scale_of(p, ws), ws.stream);
   pf.end(a, P_ASSEMBLE, ws.stream, 0.0, double(p->nlow) * (32.0 + 16.0 * sh.nb));
   factor_selinv(p, ws, sh, pf);
 }
@@ -609,7 +614,6 @@ int dm_range(const pexsi_plan* p, Workspace& ws, Profiler* prof, const double* d
   // them (info != NULL) reports a breakdown or a timed-out wait of any batch
   // of the chain.
   if (!accumulate) reset_status(ws, 0);
-  set_scales(p, ws, dH, S);
   bool first = true;
   for (int b0 = begin; b0 < end; b0 += ws.batch) {
     int nb = std::min(ws.batch, end - b0);
@@ -624,7 +628,7 @@ int dm_range(const pexsi_plan* p, Workspace& ws, Profiler* prof, const double* d
     int overwrite = (first && !accumulate) ? 1 : 0;
     cudaEvent_t a = pf.begin(st);
     launch_pole_sum(ws.Y, p->sym.front_elems, p->d_entry_pos, p->sym.nnz, sh, overwrite, d_dm, d_edm, d_fdm, d_ddm,
-                    ws.gs, st);
+                    entry_scale_of(p, ws), st);
     int nout = 1 + (d_dm ? 1 : 0) + (d_edm ? 1 : 0) + (d_fdm ? 1 : 0);
     pf.end(a, P_POLESUM, st, 6.0 * nout * nb * double(p->sym.nnz),
            double(p->sym.nnz) * (8.0 + 16.0 * nb + 8.0 * nout * (overwrite ? 1 : 2)));
@@ -676,15 +680,15 @@ int inertia_range(const pexsi_plan* p, Workspace& ws, Profiler* prof, const doub
   std::vector<std::complex<double>> z(n_shifts);
   for (int t = 0; t < n_shifts; ++t) z[t] = {shifts[t], 0.0};
   int brk_all = INT_MAX;
-  set_scales(p, ws, dH, S);  // a congruence: the counts are the same
   for (int b0 = 0; b0 < n_shifts; b0 += cap) {
     int nb = std::min(cap, n_shifts - b0);
     BatchShifts sh = make_shifts(z, nullptr, nullptr, nullptr, b0, nb);
     reset_status(ws, 1);
+    set_scales(p, ws, dH, S, sh);  // a congruence: the counts are the same
     ck(cudaMemsetAsync(ws.neg, 0, sizeof(int) * kMaxBatch, st), "status");
     ck(cudaMemsetAsync(F, 0, sizeof(double) * size_t(pool) * nb, st), "memset(F)");
     cudaEvent_t a = pf.begin(st);
-    launch_assemble<double>(F, dH, S, p->d_asm_src, p->d_asm_pos, p->nlow, pool, sh, ws.gs, st);
+    launch_assemble<double>(F, dH, S, p->d_asm_src, p->d_asm_pos, p->nlow, pool, sh, entry_scale_of(p, ws), st);
     pf.end(a, P_ASSEMBLE, st, 0.0, double(p->nlow) * (32.0 + 8.0 * nb));
     factor_batch<double>(p, ws, F, sh, true, pf);
     int neg[kMaxBatch];
@@ -708,9 +712,8 @@ int selinv_one(const pexsi_plan* p, Workspace& ws, const double* dH, const doubl
   std::vector<std::complex<double>> z{{z_re, z_im}};
   BatchShifts sh = make_shifts(z, nullptr, nullptr, nullptr, 0, 1);
   reset_status(ws, 0);
-  set_scales(p, ws, dH, dS ? dS : p->d_ident);
   run_complex_batch(p, ws, dH, dS ? dS : p->d_ident, sh, g_off);
-  launch_extract(ws.Y, p->d_entry_pos, p->sym.nnz, d_ainv, ws.gs, ws.stream);
+  launch_extract(ws.Y, p->d_entry_pos, p->sym.nnz, d_ainv, entry_scale_of(p, ws), ws.stream);
   ck(cudaGetLastError(), "extract");
   int brk = INT_MAX;
   ck(cudaMemcpyAsync(&brk, ws.brk, sizeof(int), cudaMemcpyDeviceToHost, ws.stream), "status");
@@ -740,7 +743,7 @@ void factor_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
   DevFronts fr = p->fronts();
   DevStatus status{ws.brk + (count ? 1 : 0), ws.minpiv + (count ? 1 : 0), ws.neg, count ? ws.dsave : nullptr,
                    p->d_col0, p->sym.n * int64_t(p->b), ws.ozfail + (count ? 1 : 0), p->wait_ns,
-                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g};
+                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g, ws.h, scale_stride(ws.batch)};
   const int b = p->b;
   const double nb = sh.nb;
   for (size_t L = 0; L < p->levels.size(); ++L) {
@@ -827,9 +830,10 @@ void selinv_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
 void run_gen_batch(const pexsi_plan* p, Workspace& ws, const double2* dH, const double2* dS, const BatchShifts& sh,
                    bool count, bool selinv, Profiler& pf) {
   const int64_t pool = p->sym.front_elems;
+  set_scales(p, ws, reinterpret_cast<const double*>(dH), reinterpret_cast<const double*>(dS), sh, 2);
   ck(cudaMemsetAsync(ws.F, 0, sizeof(double2) * size_t(pool) * sh.nb, ws.stream), "memset(F)");
   cudaEvent_t a = pf.begin(ws.stream);
-  launch_assemble_gen(ws.F, dH, dS, p->d_pos_full, p->sym.nnz, pool, sh, ws.gs, ws.stream);
+  launch_assemble_gen(ws.F, dH, dS, p->d_pos_full, p->sym.nnz, pool, sh, entry_scale_of(p, ws), ws.stream);
   pf.end(a, P_ASSEMBLE, ws.stream, 0.0, double(p->sym.nnz) * (32.0 + 16.0 * sh.nb));
   factor_batch_gen(p, ws, sh, count, pf);
   if (selinv) selinv_batch_gen(p, ws, sh, pf);
@@ -851,7 +855,6 @@ int dm_range_herm(const pexsi_plan* p, Workspace& ws, Profiler* prof, const doub
   double2* d_ddm = p->d_hout + 3 * nnz;
   if (info) ck(cudaEventRecord(ws.ev0, st), "event");
   if (!accumulate) reset_status(ws, 0);
-  set_scales(p, ws, reinterpret_cast<const double*>(dH), reinterpret_cast<const double*>(S), 2);
   bool first = true;
   for (int b0 = begin; b0 < end; b0 += ws.batch) {
     const int nb = std::min(ws.batch, end - b0);
@@ -864,7 +867,7 @@ int dm_range_herm(const pexsi_plan* p, Workspace& ws, Profiler* prof, const doub
     const int overwrite = (first && !accumulate) ? 1 : 0;
     cudaEvent_t a = pf.begin(st);
     launch_pole_sum_herm(ws.Y, p->sym.front_elems, p->d_pos_full, p->d_pos_t, nnz, sh, overwrite, d_dm, d_edm, d_fdm,
-                         d_ddm, ws.gs, st);
+                         d_ddm, entry_scale_of(p, ws), st);
     pf.end(a, P_POLESUM, st, 4.0 * 12.0 * nb * double(nnz), double(nnz) * (16.0 + 32.0 * nb + 64.0 * (overwrite ? 1 : 2)));
     first = false;
   }
@@ -915,7 +918,6 @@ int inertia_range_herm(const pexsi_plan* p, Workspace& ws, const double2* dH, co
   std::vector<std::complex<double>> z(n_shifts);
   for (int t = 0; t < n_shifts; ++t) z[t] = {shifts[t], 0.0};
   int brk_all = INT_MAX;
-  set_scales(p, ws, reinterpret_cast<const double*>(dH), reinterpret_cast<const double*>(S), 2);
   for (int b0 = 0; b0 < n_shifts; b0 += ws.batch) {
     const int nb = std::min(ws.batch, n_shifts - b0);
     BatchShifts sh = make_shifts(z, nullptr, nullptr, nullptr, b0, nb);
@@ -943,9 +945,8 @@ int selinv_one_herm(const pexsi_plan* p, Workspace& ws, const double2* dH, const
   std::vector<std::complex<double>> z{{z_re, z_im}};
   BatchShifts sh = make_shifts(z, nullptr, nullptr, nullptr, 0, 1);
   reset_status(ws, 0);
-  set_scales(p, ws, reinterpret_cast<const double*>(dH), reinterpret_cast<const double*>(dS ? dS : p->d_ident_c), 2);
   run_gen_batch(p, ws, dH, dS ? dS : p->d_ident_c, sh, false, true, g_off);
-  launch_extract(ws.Y, p->d_pos_full, p->sym.nnz, d_ainv, ws.gs, ws.stream);
+  launch_extract(ws.Y, p->d_pos_full, p->sym.nnz, d_ainv, entry_scale_of(p, ws), ws.stream);
   ck(cudaGetLastError(), "extract");
   int brk = INT_MAX;
   ck(cudaMemcpyAsync(&brk, ws.brk, sizeof(int), cudaMemcpyDeviceToHost, ws.stream), "status");
@@ -1035,7 +1036,6 @@ int dm_range_group(const pexsi_plan* p, Workspace& ws, Profiler* prof, int wave,
   wave = std::max(1, std::min(wave > 0 ? wave : ws.batch, ws.batch));
   if (info) ck(cudaEventRecord(ws.ev0, st), "event");
   if (!accumulate) reset_status(ws, 0);
-  for (int q = 0; q < nsys; ++q) set_scales(p, ws, dH[q], dS[q] ? dS[q] : p->d_ident + p->sys_entry_off[q], 1, q);
   bool first = true;
   for (int b0 = begin; b0 < end; b0 += wave) {
     const int nb = std::min(wave, end - b0);
@@ -1045,9 +1045,10 @@ int dm_range_group(const pexsi_plan* p, Workspace& ws, Profiler* prof, int wave,
       sh[q] = make_shifts(z[q], &wr[q], &we[q], &wf[q], b0, nb, &wd[q]);
       const int64_t a0 = p->sys_asm_off[q], na = p->sys_asm_off[q + 1] - a0;
       const double* S = dS[q] ? dS[q] : p->d_ident + p->sys_entry_off[q];
+      set_scales(p, ws, dH[q], S, sh[q], 1, q);
       cudaEvent_t a = pf.begin(st);
       launch_assemble<double2>(ws.F, dH[q], S, p->d_asm_src + a0, p->d_asm_pos + a0, na, pool, sh[q],
-                               ws.gs ? ws.gs + p->sys_entry_off[q] : nullptr, st);
+                               entry_scale_of(p, ws, q), st);
       pf.end(a, P_ASSEMBLE, st, 0.0, double(na) * (32.0 + 16.0 * nb));
     }
     factor_selinv(p, ws, sh[0], pf);
@@ -1056,7 +1057,7 @@ int dm_range_group(const pexsi_plan* p, Workspace& ws, Profiler* prof, int wave,
       const int64_t e0 = p->sys_entry_off[q], ne = p->sys_entry_off[q + 1] - e0;
       cudaEvent_t a = pf.begin(st);
       launch_pole_sum(ws.Y, pool, p->d_entry_pos + e0, ne, sh[q], overwrite, d_dm[q], d_edm[q], d_fdm[q],
-                      ws.out + 3 * nnz_all + e0, ws.gs ? ws.gs + e0 : nullptr, st);
+                      ws.out + 3 * nnz_all + e0, entry_scale_of(p, ws, q), st);
       pf.end(a, P_POLESUM, st, 24.0 * nb * double(ne), double(ne) * (8.0 + 16.0 * nb + 32.0 * (overwrite ? 1 : 2)));
     }
     first = false;
@@ -1108,7 +1109,7 @@ void free_plan_device(pexsi_plan* p) {
                   p->d_entry_pos, p->d_level_fronts, p->d_ea, p->d_tile_pref, p->d_part_off, p->d_ident,
                   p->d_ozA_off, p->d_ozB_off, p->d_exA_off, p->d_exB_off, p->d_ozA_off_r, p->d_ozB_off_r,
                   p->d_ymax_off, p->d_pos_full, p->d_pos_t, p->d_ident_c, p->d_hH, p->d_hS, p->d_hout,
-                  p->d_col0, p->d_bk_slots, p->d_diag, p->d_row, p->d_col};
+                  p->d_col0, p->d_bk_slots, p->d_diag, p->d_row, p->d_col, p->d_colptr};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   cudaStream_t st = p->ws.stream;
@@ -1395,6 +1396,7 @@ int upload_plan(pexsi_plan* p) {
     p->d_diag = dev_upload(diag);
     p->d_row = dev_upload(row);
     p->d_col = dev_upload(col);
+    p->d_colptr = dev_upload(p->col_start);
   }
   ck(cudaStreamCreateWithFlags(&p->ws.stream, cudaStreamNonBlocking), "cudaStreamCreate");
   return PEXSI_OK;

@@ -322,25 +322,37 @@ __device__ __forceinline__ void zero_acc(T (&acc)[4][4]) {
     for (int j = 0; j < 4; ++j) acc[i][j] = zero_of(T());
 }
 
-// 2^e, |e| <= 1022
-__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// 2^e, |e| <= 1000 (beyond: 2^+-1000)
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + max(-1000, min(1000, e))) << 20, 0); }
 
 // ------------------------------------------------------------ assembly
-// 2^-g of entry e of a plan whose rows and columns are scaled (gs: sum of the
-// two exponents per CSC entry; NULL: no scaling), |g| <= 1022.
-__device__ __forceinline__ double entry_scale(const int16_t* __restrict__ gs, int64_t e) {
-  return gs ? pow2(-int(gs[e])) : 1.0;
+// v 2^e, |e| <= 1000, by the exponent field: an FP64 multiply takes ten times as long.
+__device__ __forceinline__ double scale2(double v, int e) {
+  const int hi = __double2hiint(v), E = (hi >> 20) & 0x7FF;
+  if (E == 0 || E == 0x7FF || unsigned(E + e - 1) >= 0x7FEu) return v * pow2(e);
+  return __hiloint2double(hi + e * (1 << 20), __double2loint(v));
+}
+__device__ __forceinline__ double2 scale2(double2 v, int e) { return make_double2(scale2(v.x, e), scale2(v.y, e)); }
+
+// The scale of entries between two columns in batch member b, gr and gc their
+// exponents (EntryScale::of): 2^-(g_r + g_c), |g| <= 500.
+__device__ __forceinline__ int entry_exp(const int16_t* gr, const int16_t* gc, int b) {
+  return -(int(__ldg(gr + b)) + int(__ldg(gc + b)));
 }
 
 template <typename T>
 __global__ void k_assemble(T* __restrict__ F, const double* __restrict__ H, const double* __restrict__ S,
                            const int64_t* __restrict__ src, const int64_t* __restrict__ pos, int64_t nlow,
-                           int64_t pool, BatchShifts sh, const int16_t* __restrict__ gs) {
+                           int64_t pool, BatchShifts sh, EntryScale sc) {
   for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < nlow; t += int64_t(gridDim.x) * blockDim.x) {
     int64_t e = src[t], p = pos[t];
-    const double sc = entry_scale(gs, e);
-    double h = H[e] * sc, s = S[e] * sc;
-    for (int b = 0; b < sh.nb; ++b) F[b * pool + p] = make_shift<T>(h, s, sh, b);
+    const double h = H[e], s = S[e];
+    const int16_t *gr = sc.of_row(e), *gc = sc.of_col(e);
+#pragma unroll 4
+    for (int b = 0; b < sh.nb; ++b) {
+      const T a = make_shift<T>(h, s, sh, b);
+      F[b * pool + p] = gr ? scale2(a, entry_exp(gr, gc, b)) : a;
+    }
   }
 }
 
@@ -634,8 +646,9 @@ __device__ void bk_count<double>(double* Bm, int n, int ld, int* out_neg, bool* 
 // one after the other on blocks in shared memory.
 //
 // Warps: 6 update warps on three of the four SM partitions (warps 0-2, 4-6), the
-// search warp alone on the fourth (warp 3; warp 7 only takes part in the CTA
-// barriers), whose chain of steps the updates would hold up: 118 us against 124.
+// search warp alone on the fourth (warp 3), whose chain of steps the updates would
+// hold up: 118 us against 124. Warp 7 there only follows the pivots of the block
+// for the pivot ratio, in CTA 0, whose own searches come first.
 //
 // Clusters up to 99 inversions of a launch, one CTA each from 100 (48 x 48
 // complex, us): 40: 116 against 217; 80: 209 / 216; 160: 389 / 295. Clusters of 2
@@ -652,16 +665,29 @@ __device__ __forceinline__ void least(double* at, double v) {
   atomicMin(reinterpret_cast<unsigned long long*>(at), (unsigned long long)__double_as_longlong(v));
 }
 
-// Smallest pivot and largest entry of a block: of the matrix as the caller gave
-// it (pmin, mx), which is what the call reports, and of the scaled one (gmin,
-// gx). It breaks down where the ratio is below the limit in both: in the first
-// alone a graded matrix would, in the second alone a level near a shift beside
-// orbitals of small diagonal.
+// Units of a block's entries: exponents of column `col` in member pb that bring
+// the scaled matrix back to the caller's (low half) and to rows of which each is
+// scaled by its own H and S before they cancel (high half).
+__device__ __forceinline__ int units_of(const DevStatus& st, int pb, int col) {
+  if (!st.g) return 0;
+  const int g = st.g[col * st.g_stride + pb], h = st.h[col];
+  return (g & 0xFFFF) | (g - h) << 16;
+}
+template <int U>
+__device__ __forceinline__ double in_units(double v, int row, int col) {
+  return scale2(v, max(-1000, min(1000, U == 0 ? int(int16_t(row)) + int(int16_t(col)) : (row >> 16) + (col >> 16))));
+}
+
+// Smallest pivot and largest entry of a block in the caller's units (pmin, mx),
+// whose ratio the call reports, and in those of the rows (gmin, gx). It breaks
+// down where the ratio is below the limit in both: in the first alone a graded
+// matrix would, in the second alone a level near a shift beside orbitals of small
+// diagonal.
 __device__ __forceinline__ void report_pivots(const DevStatus& st, int f, bool bad, double pmin, double mx, double gmin,
                                               double gx) {
-  const double ratio = mx > 0 ? pmin / mx : 0.0, scaled = gx > 0 ? gmin / gx : 0.0;
+  const double ratio = mx > 0 ? pmin / mx : 0.0, own = gx > 0 ? gmin / gx : 0.0;
   atomicMin(st.min_pivot, (unsigned long long)__double_as_longlong(ratio));
-  if (bad || (ratio < 1e-13 && scaled < 1e-13)) atomicMin(st.breakdown_front, f);
+  if (bad || (ratio < 1e-13 && own < 1e-13)) atomicMin(st.breakdown_front, f);
 }
 
 template <typename T>
@@ -688,8 +714,8 @@ __device__ __forceinline__ unsigned long long diag_ns() {
 // Wait for phase 0 of a barrier, bounded: `lost` after wait_ns. A thread that is
 // lost waits no more and writes nothing back, but sends what it would have sent,
 // so that no other wait runs out because of it and every barrier still gets its
-// bytes; the CTA drains its barriers before it leaves, since a late send into a
-// CTA that has gone would be an invalid access. A wait that ends does not look at
+// bytes; it waits for those before its CTA leaves, since a late send into a CTA
+// that has gone would be an invalid access. A wait that ends does not look at
 // the flag: a test of it around every wait cost 2 us an inverse.
 __device__ __forceinline__ void diag_wait(uint32_t bar, unsigned long long wait_ns, bool& lost) {
   unsigned long long t0 = 0;
@@ -745,11 +771,9 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
   uint64_t* s_full = reinterpret_cast<uint64_t*>(s_row + 2 * (64 / C + 1));  // [64]: column and pivot row are here
   uint64_t* s_inv = s_full + 64;                                             // [64]: the reciprocal is here
   uint64_t* s_ready = s_inv + 64;                                            // [64]: the next column is staged
-  // smallest pivot and largest entry of this CTA's columns, as the caller gave the matrix and as it is scaled, and of
-  // every CTA's, gathered in CTA 0
-  __shared__ double s_ext[4], s_exts[4][C];
+  __shared__ double s_lmax[2], s_maxes[2][C];  // largest entry in both units, of this CTA and (in CTA 0) of every one
   __shared__ T s_scaled[64 / C];
-  __shared__ int s_ex[64];  // scaling exponents of the block's rows and columns
+  __shared__ int s_ex[64];  // units of the block's rows and columns
   const int f = fronts[blockIdx.x / C];
   const int r = int(cg::this_cluster().block_rank());
   const int pb = blockIdx.y;
@@ -772,8 +796,16 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
   const uint32_t ready0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_ready));
   const uint32_t col0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_col));
   const uint32_t step0 = static_cast<uint32_t>(__cvta_generic_to_shared(s_step));
+  // symmetric fronts hold the lower triangle; LDU fronts (GEN) both
+  T a[E];
+#pragma unroll
+  for (int q = 0; q < E; ++q) {
+    const int jl = g + ng * q, j = c0 + jl;
+    a[q] = zero_of(T());
+    if (holds && jl < nc) a[q] = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
+  }
   if (tid < 64) {
-    s_ex[tid] = st.g && tid < bb ? st.g[st.col0[f] + p0 + tid] : 0;
+    s_ex[tid] = tid < bb ? units_of(st, pb, st.col0[f] + p0 + tid) : 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8 * tid));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(inv0 + 8 * tid));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(ready0 + 8 * tid), "r"(bb));
@@ -785,21 +817,17 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(inv0 + 8 * tid), "r"(int(sizeof(T)) + 16)
                  : "memory");
   }
-  if (tid < 4) s_ext[tid] = tid & 1 ? 0.0 : DBL_MAX;
+  if (tid < 2) s_lmax[tid] = 0.0;
   __syncthreads();
-  // symmetric fronts hold the lower triangle; LDU fronts (GEN) both
-  T a[E];
-  double lmax = 0.0, gmax = 0.0;  // largest entry as the caller gave the matrix, and as it is scaled
+  double lmax = 0.0, gmax = 0.0;
   T* save = st.dsave ? reinterpret_cast<T*>(st.dsave) + int64_t(pb) * st.dsave_stride + int64_t(st.col0[f] + p0) * b
                      : nullptr;  // inertia shifts: the block before inversion, counted later
 #pragma unroll
   for (int q = 0; q < E; ++q) {
     const int jl = g + ng * q, j = c0 + jl;
-    a[q] = zero_of(T());
     if (holds && jl < nc) {
-      a[q] = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
-      gmax = fmax(gmax, mag1(a[q]));
-      lmax = fmax(lmax, mag1(a[q]) * pow2(s_ex[i] + s_ex[j]));
+      lmax = fmax(lmax, in_units<0>(mag1(a[q]), s_ex[i], s_ex[j]));
+      gmax = fmax(gmax, in_units<1>(mag1(a[q]), s_ex[i], s_ex[j]));
       if (save) save[i * b + j] = a[q];
     }
   }
@@ -808,9 +836,11 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
     gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
   }
   if (lane < 2)
-    atomicMax(reinterpret_cast<unsigned long long*>(&s_ext[2 * lane + 1]), __double_as_longlong(lane == 0 ? lmax : gmax));
+    atomicMax(reinterpret_cast<unsigned long long*>(&s_lmax[lane]), __double_as_longlong(lane == 0 ? lmax : gmax));
   __syncthreads();
   cg::this_cluster().sync();  // every CTA runs and its barriers are set before any remote access
+  if (tid < 2) *cg::this_cluster().map_shared_rank(&s_maxes[tid][r], 0) = s_lmax[tid];
+  double pmin = DBL_MAX, gmin = DBL_MAX;
   bool lost = false;  // a wait of this thread ran out
   auto wait = [&](uint32_t bar) { diag_wait(bar, st.wait_ns, lost); };
   // the holder of row i of column k hands it on: to its search warp and to every CTA
@@ -918,29 +948,39 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
           else if (pos == x) pos = k;
         }
         Fd[i + int64_t(m) * pos] = a[q];
-        if (i == 0) {  // pos: the row of this column's pivot before the interchanges
-          const double best = s_step[c0 + jl].best;
-          least(&s_ext[0], best * pow2(s_ex[pos] + s_ex[c0 + jl]));
-          least(&s_ext[2], best);
-        }
       }
     }
+  } else if (r == 0) {  // warp 7: the pivots in both units, each in the row that the interchanges brought to its place
+    int at0 = lane, at1 = lane + 32;
+    for (int k = 0; k < bb; ++k) {
+      wait(full0 + 8 * k);
+      wait(inv0 + 8 * k);
+      const int row = int(s_step[k].row);
+      const int from_k = __shfl_sync(0xffffffffu, k < 32 ? at0 : at1, k & 31);
+      const int from = __shfl_sync(0xffffffffu, row < 32 ? at0 : at1, row & 31);
+      if (lane == (row & 31)) (row < 32 ? at0 : at1) = from_k;
+      if (lane == (k & 31)) (k < 32 ? at0 : at1) = from;
+      const double best = s_step[k].best;
+      pmin = fmin(pmin, in_units<0>(best, s_ex[from], s_ex[k]));
+      gmin = fmin(gmin, in_units<1>(best, s_ex[from], s_ex[k]));
+    }
   }
-  const bool gave_up = __syncthreads_or(lost);
-  if (gave_up && tid < bb) {  // what is still on its way here
+  if (lost) {  // what is still on its way here
     bool late = false;
-    diag_wait(full0 + 8 * tid, kDiagDrainNs, late);
-    diag_wait(inv0 + 8 * tid, kDiagDrainNs, late);
+    for (int k = 0; k < bb; ++k) {
+      diag_wait(full0 + 8 * k, kDiagDrainNs, late);
+      diag_wait(inv0 + 8 * k, kDiagDrainNs, late);
+    }
+    atomicMax(st.fail, 1 + (kDiagSite << 20) + min(int(blockIdx.x), (1 << 20) - 1));
   }
-  if (tid < 4) *cg::this_cluster().map_shared_rank(&s_exts[tid][r], 0) = s_ext[tid];
   cg::this_cluster().sync();  // every remote write of the cluster is done before any CTA leaves
-  if (gave_up) {
-    if (tid == 0) atomicMax(st.fail, 1 + (kDiagSite << 20) + min(int(blockIdx.x), (1 << 20) - 1));
-  } else if (r == 0 && tid == 0) {
-    double ext[4] = {DBL_MAX, 0.0, DBL_MAX, 0.0};
-    for (int q = 0; q < C; ++q)
-      for (int x = 0; x < 4; ++x) ext[x] = x & 1 ? fmax(ext[x], s_exts[x][q]) : fmin(ext[x], s_exts[x][q]);
-    report_pivots(st, f, s_step[bb - 1].bad, ext[0], ext[1], ext[2], ext[3]);
+  if (r == 0 && tid == kDiagThreads - 32 && !lost) {
+    double mx = 0.0, gx = 0.0;
+    for (int q = 0; q < C; ++q) {
+      mx = fmax(mx, s_maxes[0][q]);
+      gx = fmax(gx, s_maxes[1][q]);
+    }
+    report_pivots(st, f, s_step[bb - 1].bad, pmin, mx, gmin, gx);
   }
 }
 
@@ -956,17 +996,17 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
   const int bb = min(b, s - p0);
   const int ld = b + 1;
   T* Fd = F + int64_t(pb) * fr.pool + fr.off[f] + p0 + int64_t(m) * p0;
-  __shared__ double s_max[2];  // largest entry and smallest pivot: as the caller gave the matrix, and scaled
+  __shared__ double s_max[2];  // largest entry and smallest pivot, in both units
   __shared__ int s_piv;
   __shared__ double s_pmin[2];
   __shared__ bool s_bad;
   __shared__ T s_fac[64];
   __shared__ T s_inv;
   __shared__ int s_perm[64];
-  __shared__ int s_ex[2][64];  // scaling exponents of the columns, and of the rows as they are interchanged
+  __shared__ int s_ex[2][64];  // units of the columns, and of the rows as they are interchanged
   __shared__ double s_best[64];
   if (threadIdx.x < 64) s_ex[0][threadIdx.x] = s_ex[1][threadIdx.x] =
-      st.g && int(threadIdx.x) < bb ? st.g[st.col0[f] + p0 + threadIdx.x] : 0;
+      int(threadIdx.x) < bb ? units_of(st, pb, st.col0[f] + p0 + int(threadIdx.x)) : 0;
   if (threadIdx.x < 2) { s_max[threadIdx.x] = 0.0; s_pmin[threadIdx.x] = DBL_MAX; s_bad = false; }
   __syncthreads();
   double lmax = 0.0, gmax = 0.0;
@@ -975,8 +1015,8 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
     // symmetric fronts hold the lower triangle; LDU fronts (GEN) both
     T v = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
     Aug[i * ld + j] = v;
-    gmax = fmax(gmax, mag1(v));
-    lmax = fmax(lmax, mag1(v) * pow2(s_ex[0][i] + s_ex[0][j]));
+    lmax = fmax(lmax, in_units<0>(mag1(v), s_ex[0][i], s_ex[0][j]));
+    gmax = fmax(gmax, in_units<1>(mag1(v), s_ex[0][i], s_ex[0][j]));
   }
   // block max |entry| for the pivot ratio
   for (int o = 16; o > 0; o >>= 1) {
@@ -1045,8 +1085,8 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
     __syncthreads();
   }
   if (int(threadIdx.x) < bb) {
-    least(&s_pmin[0], s_best[threadIdx.x] * pow2(s_ex[1][threadIdx.x] + s_ex[0][threadIdx.x]));
-    least(&s_pmin[1], s_best[threadIdx.x]);
+    least(&s_pmin[0], in_units<0>(s_best[threadIdx.x], s_ex[1][threadIdx.x], s_ex[0][threadIdx.x]));
+    least(&s_pmin[1], in_units<1>(s_best[threadIdx.x], s_ex[1][threadIdx.x], s_ex[0][threadIdx.x]));
   }
   // the row interchanges become column interchanges of the inverse, undone in reverse order
   for (int k = bb - 1; k >= 0; --k) {
@@ -1382,23 +1422,32 @@ __global__ void k_selinv_diag_reduce(double2* __restrict__ Y, const double2* __r
 __global__ void k_pole_sum(const double2* __restrict__ Y, int64_t pool, const int64_t* __restrict__ entry_pos,
                            int64_t nnz, BatchShifts sh, int overwrite, double* __restrict__ dm,
                            double* __restrict__ edm, double* __restrict__ fdm, double* __restrict__ ddm,
-                           const int16_t* __restrict__ gs) {
+                           EntryScale sc) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t p = entry_pos[e];
     double a = 0.0, ae = 0.0, af = 0.0, ad = 0.0;
-    for (int b = 0; b < sh.nb; ++b) {
-      double2 v = Y[b * pool + p];
-      // Im(w v) = w.re v.im + w.im v.re
-      a = fma(sh.wr_re[b], v.y, fma(sh.wr_im[b], v.x, a));
-      ae = fma(sh.we_re[b], v.y, fma(sh.we_im[b], v.x, ae));
-      af = fma(sh.wf_re[b], v.y, fma(sh.wf_im[b], v.x, af));
-      ad = fma(sh.wd_re[b], v.y, fma(sh.wd_im[b], v.x, ad));
+    const int16_t *gr = sc.of_row(e), *gc = sc.of_col(e);
+    for (int b0 = 0; b0 < sh.nb; b0 += 4) {  // the loads of four members in flight
+      double2 v[4];
+      int x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int b = min(b0 + u, sh.nb - 1);
+        v[u] = Y[b * pool + p];
+        x[u] = gr ? entry_exp(gr, gc, b) : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int b = b0 + u;
+        if (b >= sh.nb) break;
+        const double2 w = gr ? scale2(v[u], x[u]) : v[u];
+        // Im(w v) = w.re v.im + w.im v.re
+        a = fma(sh.wr_re[b], w.y, fma(sh.wr_im[b], w.x, a));
+        ae = fma(sh.we_re[b], w.y, fma(sh.we_im[b], w.x, ae));
+        af = fma(sh.wf_re[b], w.y, fma(sh.wf_im[b], w.x, af));
+        ad = fma(sh.wd_re[b], w.y, fma(sh.wd_im[b], w.x, ad));
+      }
     }
-    const double sc = entry_scale(gs, e);
-    a *= sc;
-    ae *= sc;
-    af *= sc;
-    ad *= sc;
     if (dm) dm[e] = overwrite ? a : dm[e] + a;
     if (edm) edm[e] = overwrite ? ae : edm[e] + ae;
     if (fdm) fdm[e] = overwrite ? af : fdm[e] + af;
@@ -1410,13 +1459,15 @@ __global__ void k_pole_sum(const double2* __restrict__ Y, int64_t pool, const in
 // every CSC entry at its own position (both triangles), A = H - z S.
 __global__ void k_assemble_gen(double2* __restrict__ F, const double2* __restrict__ H, const double2* __restrict__ S,
                                const int64_t* __restrict__ pos, int64_t nnz, int64_t pool, BatchShifts sh,
-                               const int16_t* __restrict__ gs) {
+                               EntryScale sc) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t p = pos[e];
-    const double sc = entry_scale(gs, e);
-    const double2 h = scalev(H[e], sc), v = scalev(S[e], sc);
-    for (int b = 0; b < sh.nb; ++b)  // (hr + i hi) - (zr + i zi)(sr + i si)
-      F[b * pool + p] = make_double2(h.x - fma(sh.re[b], v.x, -sh.im[b] * v.y), h.y - fma(sh.re[b], v.y, sh.im[b] * v.x));
+    const double2 h = H[e], v = S[e];
+    const int16_t *gr = sc.of_row(e), *gc = sc.of_col(e);
+    for (int b = 0; b < sh.nb; ++b) {  // (hr + i hi) - (zr + i zi)(sr + i si)
+      const double2 a = make_double2(h.x - fma(sh.re[b], v.x, -sh.im[b] * v.y), h.y - fma(sh.re[b], v.y, sh.im[b] * v.x));
+      F[b * pool + p] = gr ? scale2(a, entry_exp(gr, gc, b)) : a;
+    }
   }
 }
 
@@ -1427,12 +1478,18 @@ __global__ void k_assemble_gen(double2* __restrict__ F, const double2* __restric
 __global__ void k_pole_sum_herm(const double2* __restrict__ Y, int64_t pool, const int64_t* __restrict__ pos,
                                 const int64_t* __restrict__ pos_t, int64_t nnz, BatchShifts sh, int overwrite,
                                 double2* __restrict__ dm, double2* __restrict__ edm, double2* __restrict__ fdm,
-                                double2* __restrict__ ddm, const int16_t* __restrict__ gs) {
+                                double2* __restrict__ ddm, EntryScale sc) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t p = pos[e], q = pos_t[e];
     double2 o[4] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
+    const int16_t *gr = sc.of_row(e), *gc = sc.of_col(e);
     for (int b = 0; b < sh.nb; ++b) {
-      const double2 g = Y[b * pool + p], gt = Y[b * pool + q];
+      double2 g = Y[b * pool + p], gt = Y[b * pool + q];
+      if (gr) {
+        const int x = entry_exp(gr, gc, b);
+        g = scale2(g, x);
+        gt = scale2(gt, x);
+      }
       const double wr[4] = {sh.wr_re[b], sh.we_re[b], sh.wf_re[b], sh.wd_re[b]};
       const double wi[4] = {sh.wr_im[b], sh.we_im[b], sh.wf_im[b], sh.wd_im[b]};
 #pragma unroll
@@ -1443,24 +1500,23 @@ __global__ void k_pole_sum_herm(const double2* __restrict__ Y, int64_t pool, con
         o[k].y += 0.5 * (t.x - a.x);
       }
     }
-    const double sc = entry_scale(gs, e);
     double2* outs[4] = {dm, edm, fdm, ddm};
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      if (outs[k]) outs[k][e] = overwrite ? scalev(o[k], sc) : addv(outs[k][e], scalev(o[k], sc));
+      if (outs[k]) outs[k][e] = overwrite ? o[k] : addv(outs[k][e], o[k]);
   }
 }
 
 __global__ void k_extract(const double2* __restrict__ Y, const int64_t* __restrict__ entry_pos, int64_t nnz,
-                          double2* __restrict__ out, const int16_t* __restrict__ gs) {
+                          double2* __restrict__ out, EntryScale sc) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x)
-    out[e] = scalev(Y[entry_pos[e]], entry_scale(gs, e));
+    out[e] = sc.g ? scale2(Y[entry_pos[e]], entry_exp(sc.of_row(e), sc.of_col(e), 0)) : Y[entry_pos[e]];
 }
 
 __global__ void k_scaled_imag(const double2* __restrict__ Y, const int64_t* __restrict__ entry_pos, int64_t nnz,
-                              double scale, double* __restrict__ out, const int16_t* __restrict__ gs) {
+                              double scale, double* __restrict__ out, EntryScale sc) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x)
-    out[e] = scale * (Y[entry_pos[e]].y * entry_scale(gs, e));
+    out[e] = scale * (sc.g ? scale2(Y[entry_pos[e]].y, entry_exp(sc.of_row(e), sc.of_col(e), 0)) : Y[entry_pos[e]].y);
 }
 
 __global__ void k_trace_partial(const double* dm, const double* edm, const double* fdm, const double* ddm,
@@ -1505,8 +1561,8 @@ inline int grid_for(int64_t n, int threads) {
 // ------------------------------------------------------------ launchers
 template <typename T>
 void launch_assemble(T* F, const double* H, const double* S, const int64_t* src, const int64_t* pos, int64_t nlow,
-                     int64_t pool, const BatchShifts& sh, const int16_t* gs, cudaStream_t st) {
-  k_assemble<T><<<grid_for(nlow, 256), 256, 0, st>>>(F, H, S, src, pos, nlow, pool, sh, gs);
+                     int64_t pool, const BatchShifts& sh, const EntryScale& sc, cudaStream_t st) {
+  k_assemble<T><<<grid_for(nlow, 256), 256, 0, st>>>(F, H, S, src, pos, nlow, pool, sh, sc);
 }
 
 template <typename T>
@@ -1601,19 +1657,19 @@ void launch_selinv_diag_reduce(double2* Y, const double2* F, const double2* part
 }
 
 void launch_pole_sum(const double2* Y, int64_t pool, const int64_t* entry_pos, int64_t nnz, const BatchShifts& sh,
-                     int overwrite, double* dm, double* edm, double* fdm, double* ddm, const int16_t* gs,
+                     int overwrite, double* dm, double* edm, double* fdm, double* ddm, const EntryScale& sc,
                      cudaStream_t st) {
-  k_pole_sum<<<grid_for(nnz, 256), 256, 0, st>>>(Y, pool, entry_pos, nnz, sh, overwrite, dm, edm, fdm, ddm, gs);
+  k_pole_sum<<<grid_for(nnz, 256), 256, 0, st>>>(Y, pool, entry_pos, nnz, sh, overwrite, dm, edm, fdm, ddm, sc);
 }
 
-void launch_extract(const double2* Y, const int64_t* entry_pos, int64_t nnz, double2* out, const int16_t* gs,
+void launch_extract(const double2* Y, const int64_t* entry_pos, int64_t nnz, double2* out, const EntryScale& sc,
                     cudaStream_t st) {
-  k_extract<<<grid_for(nnz, 256), 256, 0, st>>>(Y, entry_pos, nnz, out, gs);
+  k_extract<<<grid_for(nnz, 256), 256, 0, st>>>(Y, entry_pos, nnz, out, sc);
 }
 
 void launch_scaled_imag(const double2* Y, const int64_t* entry_pos, int64_t nnz, double scale, double* out,
-                        const int16_t* gs, cudaStream_t st) {
-  k_scaled_imag<<<grid_for(nnz, 256), 256, 0, st>>>(Y, entry_pos, nnz, scale, out, gs);
+                        const EntryScale& sc, cudaStream_t st) {
+  k_scaled_imag<<<grid_for(nnz, 256), 256, 0, st>>>(Y, entry_pos, nnz, scale, out, sc);
 }
 
 void launch_traces(const double* dm, const double* edm, const double* fdm, const double* ddm, const double* S,
@@ -1660,8 +1716,8 @@ cudaError_t configure_kernels(int b) {
 
 // ---- LDU fronts of complex Hermitian H and S (general complex shifted matrices)
 void launch_assemble_gen(double2* F, const double2* H, const double2* S, const int64_t* pos, int64_t nnz,
-                         int64_t pool, const BatchShifts& sh, const int16_t* gs, cudaStream_t st) {
-  k_assemble_gen<<<grid_for(nnz, 256), 256, 0, st>>>(F, H, S, pos, nnz, pool, sh, gs);
+                         int64_t pool, const BatchShifts& sh, const EntryScale& sc, cudaStream_t st) {
+  k_assemble_gen<<<grid_for(nnz, 256), 256, 0, st>>>(F, H, S, pos, nnz, pool, sh, sc);
 }
 
 void launch_extend_add_full(double2* F, const DevFronts& fr, const int32_t* children, int nchild, const int32_t* pref,
@@ -1717,8 +1773,8 @@ void launch_selinv_diag_reduce_gen(double2* Y, const double2* F, const double2* 
 
 void launch_pole_sum_herm(const double2* Y, int64_t pool, const int64_t* pos, const int64_t* pos_t, int64_t nnz,
                           const BatchShifts& sh, int overwrite, double2* dm, double2* edm, double2* fdm, double2* ddm,
-                          const int16_t* gs, cudaStream_t st) {
-  k_pole_sum_herm<<<grid_for(nnz, 256), 256, 0, st>>>(Y, pool, pos, pos_t, nnz, sh, overwrite, dm, edm, fdm, ddm, gs);
+                          const EntryScale& sc, cudaStream_t st) {
+  k_pole_sum_herm<<<grid_for(nnz, 256), 256, 0, st>>>(Y, pool, pos, pos_t, nnz, sh, overwrite, dm, edm, fdm, ddm, sc);
 }
 
 template <typename T>
@@ -1732,7 +1788,7 @@ template void launch_bk_count_all<double2>(const int32_t*, int, const DevFronts&
 
 #define PEXSI_INSTANTIATE(T)                                                                                        \
   template void launch_assemble<T>(T*, const double*, const double*, const int64_t*, const int64_t*, int64_t,    \
-                                   int64_t, const BatchShifts&, const int16_t*, cudaStream_t);                   \
+                                   int64_t, const BatchShifts&, const EntryScale&, cudaStream_t);                   \
   template void launch_extend_add<T>(T*, const DevFronts&, const int32_t*, int, const int32_t*, int64_t,        \
                                      const BatchShifts&, cudaStream_t);                                           \
   template void launch_diag_inv<T>(T*, const DevFronts&, const int32_t*, int, int, int, const BatchShifts&,      \

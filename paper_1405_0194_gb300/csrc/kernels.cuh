@@ -81,9 +81,21 @@ struct DevStatus {
   int* fail;                         // atomicMax of where a wait of a cluster block inverse ran out (0 = none)
   uint64_t wait_ns;                  // bound of these waits (wall time)
   int hold;                          // fault injection: the first column of each cluster comes after 4 wait_ns
-  // fronts of a scaled matrix (launch_rns_scales; NULL: unscaled): exponent per column in elimination order. The
-  // pivot ratio is that of the matrix as the caller gave it.
-  const int32_t* g;
+  // fronts of a scaled matrix (launch_rns_scales; NULL: unscaled): exponents of the members for the c-th column in
+  // elimination order from g + c * g_stride on, and of the columns' own H and S at h (k_diag_inv_*: the pivot ratios)
+  const int16_t *g, *h;
+  int64_t g_stride;
+};
+
+// The scaling of a batch (launch_rns_scales; g NULL: none) and the row and column
+// of every CSC entry, in elimination order.
+struct EntryScale {
+  const int16_t* g;
+  int64_t stride;
+  const int32_t *row, *col;
+  // the members' exponents of entry e's row and column
+  __device__ __forceinline__ const int16_t* of_row(int64_t e) const { return g ? g + row[e] * stride : nullptr; }
+  __device__ __forceinline__ const int16_t* of_col(int64_t e) const { return g ? g + col[e] * stride : nullptr; }
 };
 
 // Scratch of the split-precision GEMM: bf16 slice tiles of A = Y[S,S] and
@@ -115,11 +127,10 @@ struct OzScratch {
 };
 
 // ---- launchers (T = double for real inertia, double2 for complex poles) ----
-// gs (per CSC entry, NULL: none): A is assembled as D A D with D = 2^-g per row,
-// and Y is read out as D Y D, 2^-gs[e] per entry (see launch_rns_scales).
+// sc: A is assembled as D A D with D = 2^-g per row, and Y is read out as D Y D.
 template <typename T>
 void launch_assemble(T* F, const double* H, const double* S, const int64_t* src, const int64_t* pos, int64_t nlow,
-                     int64_t pool, const BatchShifts& sh, const int16_t* gs, cudaStream_t st);
+                     int64_t pool, const BatchShifts& sh, const EntryScale& sc, cudaStream_t st);
 
 template <typename T>
 void launch_extend_add(T* F, const DevFronts& fr, const int32_t* children, int nchild, const int32_t* pref,
@@ -155,15 +166,15 @@ void launch_selinv_diag_reduce(double2* Y, const double2* F, const double2* part
                                int b, const BatchShifts& sh, cudaStream_t st);
 
 void launch_pole_sum(const double2* Y, int64_t pool, const int64_t* entry_pos, int64_t nnz, const BatchShifts& sh,
-                     int overwrite, double* dm, double* edm, double* fdm, double* ddm, const int16_t* gs,
+                     int overwrite, double* dm, double* edm, double* fdm, double* ddm, const EntryScale& sc,
                      cudaStream_t st);
 
-void launch_extract(const double2* Y, const int64_t* entry_pos, int64_t nnz, double2* out, const int16_t* gs,
+void launch_extract(const double2* Y, const int64_t* entry_pos, int64_t nnz, double2* out, const EntryScale& sc,
                     cudaStream_t st);
 
 // out[e] = scale * Im Y[entry_pos[e]] (the LDOS matrix from one selected inverse).
 void launch_scaled_imag(const double2* Y, const int64_t* entry_pos, int64_t nnz, double scale, double* out,
-                        const int16_t* gs, cudaStream_t st);
+                        const EntryScale& sc, cudaStream_t st);
 
 // Split-precision Takahashi step Y[S,P] = -Y[S,S] L[S,P] and its mirror, with
 // A = Y[S,S] sliced on the fly inside the GEMM: prep = true computes the row
@@ -225,7 +236,7 @@ cudaError_t oz_configure(int S);
 // trailing square, and selected inversion computes Y[S,P] = -Y[S,S] L[S,P]
 // and Y[P,S] = -U[P,S] Y[S,S] separately, with Y[P,P] = D^-1 - U[P,S] Y[S,P].
 void launch_assemble_gen(double2* F, const double2* H, const double2* S, const int64_t* pos, int64_t nnz,
-                         int64_t pool, const BatchShifts& sh, const int16_t* gs, cudaStream_t st);
+                         int64_t pool, const BatchShifts& sh, const EntryScale& sc, cudaStream_t st);
 void launch_extend_add_full(double2* F, const DevFronts& fr, const int32_t* children, int nchild, const int32_t* pref,
                             int64_t total_tiles, const BatchShifts& sh, cudaStream_t st);
 void launch_diag_inv_gen(double2* F, const DevFronts& fr, const int32_t* fronts, int nfronts, int p0, int b,
@@ -246,7 +257,7 @@ void launch_selinv_diag_reduce_gen(double2* Y, const double2* F, const double2* 
 // (w G - conj(w) G^H) / 2i at each CSC entry: pos = its own position, pos_t = that of its transpose
 void launch_pole_sum_herm(const double2* Y, int64_t pool, const int64_t* pos, const int64_t* pos_t, int64_t nnz,
                           const BatchShifts& sh, int overwrite, double2* dm, double2* edm, double2* fdm, double2* ddm,
-                          const int16_t* gs, cudaStream_t st);
+                          const EntryScale& sc, cudaStream_t st);
 
 // Inertia counts of all saved panel blocks (slots: (front, p0) pairs, nslots
 // of them) for nb batch members: one CTA per block and member, a Bunch-Kaufman

@@ -107,8 +107,8 @@ struct Workspace {
   int *exA = nullptr, *exB = nullptr, *ozfail = nullptr;
   uint32_t* ymax = nullptr;  // split path: row maxima of Y per pole
   RnsScratch rns;            // FP64 path: scratch of the residue products (no planes: DFMA kernels)
-  int32_t* g = nullptr;      // its power-of-two scaling: exponent per column, and per CSC entry of the current H and S
-  int16_t* gs = nullptr;
+  // its power-of-two scaling: exponents of the batch's columns, a first guess, and those of the columns' own H and S
+  int16_t *g = nullptr, *g0 = nullptr, *h = nullptr;
   cudaStream_t stream = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // captured level schedules (factorisation + selected inversion of nb
@@ -170,8 +170,9 @@ struct pexsi_plan {
   std::vector<int64_t> diag_entries;  // CSC entries on the diagonal
   std::vector<int32_t> entry_row;     // row of every CSC entry, and the column bounds, both of this plan's matrix
   std::vector<int64_t> col_start;
-  // FP64 plans: the diagonal entry of every column, the row and column of every entry; columns in elimination order
-  int64_t* d_diag = nullptr;
+  // FP64 plans: the columns' bounds in the entries; in elimination order, the diagonal entry of every column, and the
+  // row and column of every entry
+  int64_t *d_colptr = nullptr, *d_diag = nullptr;
   int32_t *d_row = nullptr, *d_col = nullptr;
   // A plan that merges several systems (pexsi_group): the first CSC entry of
   // each system among the concatenated entries (nsys + 1), and each system's
@@ -224,6 +225,17 @@ void rns_factor_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch
                           int p0, const BatchShifts& sh, DevStatus status, Profiler& pf, cudaStream_t st);
 void rns_selinv_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch& sc, double2* Y, double2* F, int nact,
                           int p0, int nb, Profiler& pf, cudaStream_t st);
+
+// Scaling exponents kept per column: of `batch` poles, or twice as many inertia
+// shifts, in whole 16-byte words.
+inline int64_t scale_stride(int batch) { return (2 * batch + 7) / 8 * 8; }
+
+// The scaling of a workspace's current batch for the entries of system q.
+inline EntryScale entry_scale_of(const pexsi_plan* p, const Workspace& ws, size_t q = 0) {
+  if (!ws.g) return EntryScale{};
+  const int64_t e0 = p->sys_entry_off[q];
+  return EntryScale{ws.g, scale_stride(ws.batch), p->d_row + e0, p->d_col + e0};
+}
 
 // Allocates ws for `batch` poles on `stream` (cudaMallocAsync when async),
 // with residue scratch of the given sizes (0: none).

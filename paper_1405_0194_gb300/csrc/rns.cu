@@ -1011,23 +1011,98 @@ __global__ void __launch_bounds__(256) k_rns_keep(const T* __restrict__ F, T* __
 }
 
 // ------------------------------------------------------------ scaling
-__global__ void k_rns_row_scale(const double* __restrict__ H, const double* __restrict__ S, int wide,
-                                const int64_t* __restrict__ diag, int64_t c0, int64_t n, int64_t e0,
-                                int32_t* __restrict__ g) {
+constexpr int kNoExp = -20000;  // of zero, subnormal and non-finite values, which do not count
+
+__device__ __forceinline__ uint32_t high_word(double x) { return uint32_t(__double2hiint(x)) & 0x7FFFFFFFu; }
+// floor(log2) of a value by its high word
+__device__ __forceinline__ int exponent(uint32_t high) {
+  const int E = int(high >> 20);
+  return E == 0 || E == 0x7FF ? kNoExp : E - 1023;
+}
+
+// First guess: half the exponent of the diagonal entry of H - z S. h: of max(|H_cc|, |S_cc|).
+template <int W>
+__global__ void k_rns_diag_scale(const double* __restrict__ H, const double* __restrict__ S,
+                                 const int64_t* __restrict__ diag, int64_t n, int64_t c0, int64_t e0,
+                                 const __grid_constant__ BatchShifts sh, int64_t stride, int16_t* __restrict__ h,
+                                 int16_t* __restrict__ g0) {
+  const int b = blockIdx.y;
   for (int64_t c = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; c < n; c += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t e = (diag[c0 + c] - e0) * wide;
-    const double a = fmax(fabs(H[e]), fabs(S[e]));
-    const int E = int((__double2hiint(a) >> 20) & 0x7FF);
-    // zero, subnormal and non-finite diagonals stay unscaled
-    g[c0 + c] = E == 0 || E == 0x7FF ? 0 : max(-500, min(500, (E - 1023) >> 1));
+    const int64_t e = (diag[c] - e0) * W;
+    const double Hc = H[e], Sc = S[e];  // of Hermitian H and S: real
+    if (b == 0) {
+      const int E = exponent(max(high_word(Hc), high_word(Sc)));
+      h[c0 + c] = int16_t(E == kNoExp ? 0 : max(-500, min(500, E >> 1)));
+    }
+    const int E = exponent(max(high_word(fma(-sh.re[b], Sc, Hc)), high_word(sh.im[b] * Sc)));
+    g0[(c0 + c) * stride + b] = int16_t(E == kNoExp ? kNoExp : (E + 1) >> 1);
   }
 }
 
-__global__ void k_rns_entry_scale(const int32_t* __restrict__ row, const int32_t* __restrict__ col, int64_t e0,
-                                  int64_t nnz, const int32_t* __restrict__ g, int16_t* __restrict__ gs) {
-  for (int64_t e = e0 + blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < e0 + nnz;
-       e += int64_t(gridDim.x) * blockDim.x)
-    gs[e] = int16_t(g[row[e]] + g[col[e]]);
+// Then raised until no entry of the column is above 1: against a row of a larger
+// guess by what is missing, against one of a smaller guess by half of the
+// entry's exponent, which that row takes the other half of. The exponents alone
+// tell an upper bound of |H - z S|, without an FP64 operation. A warp per column
+// and 8 members, whose exponents are one 16-byte word.
+template <int W>
+__global__ void __launch_bounds__(256) k_rns_scale(const double* __restrict__ H, const double* __restrict__ S,
+                                                   const int64_t* __restrict__ colptr, const int32_t* __restrict__ row,
+                                                   const int32_t* __restrict__ col, int64_t n, int64_t e0,
+                                                   const __grid_constant__ BatchShifts sh, int64_t stride,
+                                                   const int16_t* __restrict__ h, const int16_t* __restrict__ g0,
+                                                   int16_t* __restrict__ g) {
+  union Word {
+    uint4 u;
+    int16_t x[8];
+  };
+  const int lane = threadIdx.x & 31, b0 = blockIdx.y * 8;
+  int ez[8];  // |z| < 2^(ez + 1)
+#pragma unroll
+  for (int b = 0; b < 8; ++b) ez[b] = b0 + b < sh.nb ? exponent(max(high_word(sh.re[b0 + b]), high_word(sh.im[b0 + b]))) : 0;
+  for (int64_t j = blockIdx.x * 8 + (threadIdx.x >> 5); j < n; j += int64_t(gridDim.x) * 8) {
+    const int64_t lo = colptr[j], hi = colptr[j + 1];
+    const int c = col[lo], hc = h[c];
+    Word top;
+    top.u = *reinterpret_cast<const uint4*>(g0 + c * stride + b0);
+    int t[8];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) t[b] = top.x[b];
+    for (int64_t ea = lo + lane; ea < hi; ea += 32 * 4) {  // four entries in flight
+      int r[4], eh[4], es[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t e = min(ea + 32 * u, hi - 1);
+        r[u] = row[e];
+        if constexpr (W == 1) {
+          eh[u] = exponent(high_word(H[e - e0]));
+          es[u] = exponent(high_word(S[e - e0]));
+        } else {
+          const double2 a = reinterpret_cast<const double2*>(H)[e - e0], s = reinterpret_cast<const double2*>(S)[e - e0];
+          eh[u] = exponent(max(high_word(a.x), high_word(a.y)));
+          es[u] = exponent(max(high_word(s.x), high_word(s.y)));
+        }
+      }
+      Word gr[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) gr[u].u = *reinterpret_cast<const uint4*>(g0 + r[u] * stride + b0);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (r[u] == c) continue;
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+          const int E = max(eh[u], es[u] + ez[b] + 1);
+          if (E > kNoExp / 2) t[b] = max(t[b], min(E - int(gr[u].x[b]), (E + 1) >> 1));
+        }
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const int m = __reduce_max_sync(0xFFFFFFFFu, t[b]);
+      const int x = m == kNoExp ? 0 : max(-500, min(500, m));
+      top.x[b] = int16_t(abs(x - hc) <= kRnsNear ? hc : x);
+    }
+    if (lane == 0) *reinterpret_cast<uint4*>(g + c * stride + b0) = top.u;
+  }
 }
 
 // ------------------------------------------------------------ host schedule
@@ -1272,12 +1347,17 @@ Slots tak_slots(const Dims& d) {
 
 }  // namespace
 
-void launch_rns_scales(const double* H, const double* S, int wide, const int64_t* diag, int64_t c0, int64_t n,
-                       const int32_t* row, const int32_t* col, int64_t e0, int64_t nnz, int32_t* g, int16_t* gs,
-                       cudaStream_t st) {
-  auto grid = [](int64_t k) { return int(std::min<int64_t>((k + 255) / 256, 152 * 8)); };
-  k_rns_row_scale<<<grid(n), 256, 0, st>>>(H, S, wide, diag, c0, n, e0, g);
-  k_rns_entry_scale<<<grid(nnz), 256, 0, st>>>(row, col, e0, nnz, g, gs);
+void launch_rns_scales(const double* H, const double* S, int wide, const BatchShifts& sh, const int64_t* colptr,
+                       const int64_t* diag, int64_t n, int64_t c0, int64_t e0, const int32_t* row, const int32_t* col,
+                       int16_t* h, int16_t* g0, int16_t* g, int64_t stride, cudaStream_t st) {
+  auto grid = [](int64_t k) { return int(std::min<int64_t>(k, 152 * 8)); };
+  auto run = [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    k_rns_diag_scale<W><<<dim3(grid((n + 255) / 256), sh.nb), 256, 0, st>>>(H, S, diag, n, c0, e0, sh, stride, h, g0);
+    k_rns_scale<W><<<dim3(grid((n + 7) / 8), (sh.nb + 7) / 8), 256, 0, st>>>(H, S, colptr, row, col, n, e0, sh, stride, h, g0, g);
+  };
+  if (wide == 1) run(std::integral_constant<int, 1>{});
+  else run(std::integral_constant<int, 2>{});
 }
 
 cudaError_t rns_configure() {

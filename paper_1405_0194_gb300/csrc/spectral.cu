@@ -65,7 +65,7 @@ extern "C" int pexsi_ldos(pexsi_plan* p, const double* H, const double* S, doubl
     if (!ws.ainv) ck(cudaMalloc(&ws.ainv, sizeof(double2) * nnz), "cudaMalloc(ainv)");
     rc = pexsi::selinv_one(p, ws, ws.H, dS, eps, eta, ws.ainv, &err);
     if (rc) { p->last_error = err; return rc; }
-    pexsi::launch_scaled_imag(ws.Y, p->d_entry_pos, p->sym.nnz, 2.0 / kPi, ws.out, ws.gs, ws.stream);
+    pexsi::launch_scaled_imag(ws.Y, p->d_entry_pos, p->sym.nnz, 2.0 / kPi, ws.out, entry_scale_of(p, ws), ws.stream);
     ck(cudaGetLastError(), "ldos");
     ck(cudaMemcpyAsync(ldos, ws.out, sizeof(double) * nnz, cudaMemcpyDeviceToHost, ws.stream), "D2H(ldos)");
     ck(cudaStreamSynchronize(ws.stream), "sync");
