@@ -92,9 +92,9 @@ int64_t bytes_fixed(const pexsi_plan* p) {
 void rns_scratch(const pexsi_plan* p, int batch, int64_t most, int64_t& planes, int64_t& out) {
   planes = out = 0;
   if (p->oz_slices > 0) return;
-  int64_t least, want;
-  rns_scratch_range(p, batch, least, want);
-  planes = std::max(least, std::min(want, most));
+  int64_t least, whole, want;
+  rns_scratch_range(p, batch, least, whole, want);
+  planes = most > 0 ? std::max(whole, std::min(want, most)) : least;
   out = rns_out_bytes(p, batch, most > 0 ? kRnsOutTiles : kRnsOutTilesLeast);
 }
 

@@ -202,10 +202,10 @@ int64_t bytes_per_pole(const pexsi_plan* p, bool rns);
 int64_t bytes_fixed(const pexsi_plan* p);
 
 // Residue scratch of FP64 plans (rns.cu): planes for `batch` poles, at most
-// `most` bytes unless the largest front needs more, and the output tiles; both
-// 0 for split-precision plans.
+// `most` bytes unless whole groups of the largest front need more (most = 0: the
+// least that works), and the output tiles; both 0 for split-precision plans.
 void rns_scratch(const pexsi_plan* p, int batch, int64_t most, int64_t& planes, int64_t& out);
-void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& want);
+void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& whole, int64_t& want);
 int64_t rns_out_bytes(const pexsi_plan* p, int batch, int most);
 constexpr int64_t kRnsPlaneBytes = int64_t(2) << 30;  // default of `most`
 

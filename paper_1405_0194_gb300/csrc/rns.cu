@@ -1129,7 +1129,7 @@ struct Slots {
 };
 
 // The pieces of a launch sequence that fit the scratch, in order. A front whose
-// fixed slots alone do not fit cannot occur (rns_min_bytes).
+// fixed slots alone do not fit cannot occur (rns_scratch_range).
 template <typename Fn>
 std::vector<Piece> pieces_of(int nact, int nb, int64_t cap, bool cplx, Fn slots) {
   std::vector<Piece> out;
@@ -1312,18 +1312,29 @@ struct Runner {
 };
 
 
-// Blocks of a group on a level: as many as the scratch has room for the operands
-// of. Each block alone, the rest of a front is read, reconstructed and written
+// Scratch for the operands of a front's update by a group of g blocks (complex,
+// also for real fronts): the most over the plan's fronts of more than a block.
+int64_t group_bytes(const pexsi_plan* p, int g) {
+  int64_t most = 0;
+  const int blk = rns_block(p->b);
+  for (const Level& lv : p->levels)
+    for (size_t f = 0; f < lv.s.size() && lv.s[f] > blk; ++f)
+      most = std::max(most, 2 * tiles128(lv.m[f]) * rns_slot_bytes(std::min(lv.s[f], g * blk), true));
+  return most;
+}
+
+// Blocks of a group: as many as the scratch has room for the operands of, by the
+// plan's largest fronts and not by a level's or a batch's, so that a front's sums
+// are grouped alike whatever runs beside it (rns_scratch_range reserves the room
+// for whole groups; only the least scratch has smaller ones). Each block alone, the rest of a front is read, reconstructed and written
 // once per 256 columns and the products' K is 256; in groups the operands of a
 // group are converted again. Groups of 1, 2 and 4 blocks: 55.4, 52.7 and 51.3 ms
 // for the inertia counts of 256 atoms in a fluid, 60.8, 58.9 and 58.1 ms for the
 // density matrix of 512, 53.0, 51.7 and 51.4 ms for a sheet of 14 x 14; fronts of
 // a few hundred columns do not care.
-int group_of(const int* s, const int* m, int nact, int b, int64_t cap, bool cplx) {
-  int rows = 0;
-  for (int f = 0; f < nact && s[f] > rns_block(b); ++f) rows = std::max(rows, m[f]);
+int group_of(const pexsi_plan* p, int64_t cap) {
   int g = kRnsGroup;
-  while (g > 1 && 2 * tiles128(rows) * rns_slot_bytes(std::min(s[0], g * rns_block(b)), cplx) > cap) g /= 2;
+  while (g > 1 && group_bytes(p, g) > cap) g /= 2;
   return g;
 }
 
@@ -1368,9 +1379,9 @@ cudaError_t rns_configure() {
 }
 
 // Scratch bytes below which some front's operands do not fit (a front's Y[S,S]
-// is taken in pieces of at least its panel operand's tiles), and what lets
-// every level run in one piece; both with room for the output tiles.
-void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& want) {
+// is taken in pieces of at least its panel operand's tiles), what whole groups of
+// blocks need (group_of), and what lets every level run in one piece.
+void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& whole, int64_t& want) {
   least = want = 0;
   for (const Level& lv : p->levels) {
     int64_t lw = 0, tw = 0, sw = 0;
@@ -1391,7 +1402,8 @@ void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& 
                      tw * batch * rns_slot_bytes(kt, true)});
   }
   least += rns_slot_bytes(32, true);
-  want = std::max(want, least);
+  whole = std::max(least, group_bytes(p, kRnsGroup));
+  want = std::max(want, whole);
 }
 
 int64_t rns_out_bytes(const pexsi_plan* p, int batch, int most) {
@@ -1418,7 +1430,7 @@ void rns_factor_block(const pexsi_plan* p, const Level& lv, const RnsScratch& sc
   const int32_t* dfr = p->d_level_fronts + lv.front_off;
   Runner<T> r{sc, F, Y, s, m, lv.off.data(), fr.pool, b, st};
   constexpr bool CPLX = sizeof(T) == 16;
-  r.group = group_of(s, m, int(lv.s.size()), b, sc.plane_bytes, CPLX);
+  r.group = group_of(p, sc.plane_bytes);
   const int bw = std::min(rns_block(b), s[0] - p0);  // the widest front's block
   r.keep(fr, dfr, nact, p0, sh.nb);
   if (bw > b) launch_chained(k_rns_save<T>, dim3((bw + 15) / 16, nact, sh.nb), 256, 0, st, F, Y, fr, dfr, p0, b, 0);
@@ -1556,7 +1568,7 @@ void rns_factor_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch
   const DevFronts fr = p->fronts();
   const int32_t* dfr = p->d_level_fronts + lv.front_off;
   Runner<double2> r{sc, F, Y, s, m, lv.off.data(), fr.pool, b, st, 1};
-  r.group = group_of(s, m, int(lv.s.size()), b, sc.plane_bytes, true);
+  r.group = group_of(p, sc.plane_bytes);
   const int bw = std::min(rns_block(b), s[0] - p0);
   const int kb = (b + kK - 1) / kK;
   r.keep(fr, dfr, nact, p0, sh.nb);
