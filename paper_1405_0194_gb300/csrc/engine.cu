@@ -89,23 +89,36 @@ int64_t bytes_fixed(const pexsi_plan* p) {
          (p->oz_slices > 0 ? 0 : 2 * p->sym.n);
 }
 
-void rns_scratch(const pexsi_plan* p, int batch, int64_t most, int64_t& planes, int64_t& out) {
-  planes = out = 0;
-  if (p->oz_slices > 0) return;
-  int64_t least, whole, want;
-  rns_scratch_range(p, batch, least, whole, want);
-  planes = most > 0 ? std::max(whole, std::min(want, most)) : least;
-  out = rns_out_bytes(p, batch, most > 0 ? kRnsOutTiles : kRnsOutTilesLeast);
-}
-
+// The batch and scratch of a budget. With scratch for whole groups of blocks: as
+// much as lets every level of that batch run in one piece, 2 GB of planes and 640
+// output tiles at most; if that leaves one pole or none, half and half again of
+// the planes where more poles fit for it (poles of a batch share the chain of the
+// diagonal blocks, smaller scratch only cuts launches in pieces). Else with the
+// least that works, else with none (DFMA kernels).
 int fit_batch(const pexsi_plan* p, int64_t budget, int most, int64_t& planes, int64_t& out) {
   const int64_t room = budget - bytes_fixed(p);
+  int best = 0;
   if (p->oz_slices == 0) {
-    rns_scratch(p, most, kRnsPlaneBytes, planes, out);
-    const int64_t nb = (room - planes - out) / bytes_per_pole(p, true);
-    if (nb >= 1) return int(std::min<int64_t>(nb, most));
-    rns_scratch(p, 1, 0, planes, out);
-    if (room - planes - out >= bytes_per_pole(p, true)) return 1;
+    const int64_t pole = bytes_per_pole(p, true);
+    int64_t least = 0, whole = 0, want = 0;
+    auto take = [&](int64_t cap, int tiles) {
+      for (int nb = most; nb > best; --nb) {
+        rns_scratch_range(p, nb, least, whole, want);
+        const int64_t pl = cap > 0 ? std::max(whole, std::min(want, cap)) : least, o = rns_out_bytes(p, nb, tiles);
+        if (pl + o + nb * pole > room) continue;
+        best = nb;
+        planes = pl;
+        out = o;
+        return;
+      }
+    };
+    take(kRnsPlaneBytes, kRnsOutTiles);
+    for (int64_t cap = kRnsPlaneBytes / 2; best <= 1 && best < most; cap /= 2) {
+      take(cap, kRnsOutTilesLeast);
+      if (cap <= whole) break;
+    }
+    if (best == 0) take(0, kRnsOutTilesLeast);
+    if (best > 0) return best;
   }
   planes = out = 0;
   const int64_t nb = room / std::max<int64_t>(bytes_per_pole(p, false), 1);

@@ -201,13 +201,12 @@ int64_t bytes_per_pole(const pexsi_plan* p, bool rns);
 // Fixed bytes of a workspace (staging + status + trace scratch).
 int64_t bytes_fixed(const pexsi_plan* p);
 
-// Residue scratch of FP64 plans (rns.cu): planes for `batch` poles, at most
-// `most` bytes unless whole groups of the largest front need more (most = 0: the
-// least that works), and the output tiles; both 0 for split-precision plans.
-void rns_scratch(const pexsi_plan* p, int batch, int64_t most, int64_t& planes, int64_t& out);
+// Residue scratch of FP64 plans (rns.cu): operand planes (what works at all, what
+// whole groups of blocks need, what lets every level run in one piece), and the
+// bytes of up to `most` output tiles.
 void rns_scratch_range(const pexsi_plan* p, int batch, int64_t& least, int64_t& whole, int64_t& want);
 int64_t rns_out_bytes(const pexsi_plan* p, int batch, int most);
-constexpr int64_t kRnsPlaneBytes = int64_t(2) << 30;  // default of `most`
+constexpr int64_t kRnsPlaneBytes = int64_t(2) << 30;  // most planes
 
 // The largest batch (at most `most`) whose workspace fits the budget, with
 // residue scratch where that fits too (planes, out; 0 without); 0: none fits.

@@ -59,3 +59,34 @@ def test_bits_do_not_follow_the_neighbours():
     beside = _inverses(_blocks([1100, 700, 300], 1), 2)
     for a, b in zip(alone, beside):
         assert np.array_equal(a, b[1100 * 1100:1100 * 1100 + 700 * 700])
+
+
+@pytest.mark.parametrize("kind", ["chain", "sheet", "blocks"])
+def test_batch_under_a_budget(kind):
+    """A fifth more than the workspace that eight poles take with all the scratch they want (the budget also counts what
+    other calls allocate later) holds at least eight of an automatic batch, half of it at least three, and nothing exceeds
+    a budget."""
+    import nao_synth as ns
+    if kind == "blocks":
+        n, colptr, rowind, H, S = _blocks([300, 300, 200], 2)
+    else:
+        s = ns.make_chain(natoms=300) if kind == "chain" else ns.make_sheet(ncell=8)
+        n, colptr, rowind, H, S = s.n, s.colptr, s.rowind, s.H, s.S
+
+    def chosen(**opts):
+        plan = px.pexsi_setup(n, colptr, rowind, opts=px.pexsi_opts_default(**opts))
+        try:
+            px.pexsi_selinv(plan, H, S, 0.1 + 0.05j)
+            st = px.pexsi_plan_get_stats(plan)
+            return st["batch"], st["workspace_bytes"]
+        except px.PexsiError as e:
+            assert e.code == -3
+            return 0, 0
+        finally:
+            px.pexsi_plan_destroy(plan)
+
+    _, eight = chosen(max_batch=8)
+    for x in (0.02, 0.1, 0.2, 0.35, 0.6, 0.8, 1.2, 2.0, 4.0):
+        batch, used = chosen(hbm_budget=int(x * eight))
+        assert used <= int(x * eight)
+        assert batch >= (8 if x >= 1.2 else 3 if x >= 0.6 else 0)
