@@ -183,6 +183,7 @@ void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, int64_t rns_
     ws.rns.plane_bytes = rns_planes;
     ws.rns.out_bytes = rns_out;
     ws.rns.wait_ns = p->wait_ns;
+    ws.rns.sms = p->sms;
   }
   if (p->oz_slices > 0) {
     // complex poles use `batch` members, the real inertia shifts up to 2 batch
@@ -1319,6 +1320,7 @@ int init_opts(pexsi_plan* p, const pexsi_opts* opts) {
 int upload_plan(pexsi_plan* p) {
   ck(cudaSetDevice(p->opts.device), "cudaSetDevice");
   ck(configure_kernels(p->b), "cudaFuncSetAttribute");
+  ck(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->opts.device), "cudaDeviceGetAttribute");
   if (p->oz_slices > 0) ck(oz_configure(p->oz_slices), "cudaFuncSetAttribute(split)");
   else ck(rns_configure(), "cudaFuncSetAttribute(residues)");
   const Symbolic& S = p->sym;

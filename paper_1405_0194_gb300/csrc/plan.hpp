@@ -132,6 +132,7 @@ struct pexsi_plan {
   std::string last_error;
   int b = 64;
   uint64_t wait_ns = 1000000000ull;  // bound of the device-side waits (opts.wait_ns, 0 = 1 s)
+  int sms = 152;                     // multiprocessors of the device
   int64_t* d_front_off = nullptr;
   int32_t *d_s = nullptr, *d_m = nullptr, *d_parent = nullptr, *d_rel = nullptr;
   int64_t* d_rptr = nullptr;

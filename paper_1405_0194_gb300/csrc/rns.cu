@@ -1106,17 +1106,6 @@ __global__ void __launch_bounds__(256) k_rns_scale(const double* __restrict__ H,
 }
 
 // ------------------------------------------------------------ host schedule
-int sms() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    n = v > 0 ? v : 152;
-  }
-  return n;
-}
-
 // Fronts [f0, f0 + nf) of a level's list for the poles [pole0, pole0 + np), or
 // row tiles [rt0, rt0 + rtn) of the one front's N operand (rtn = 0: all).
 struct Piece {
@@ -1299,11 +1288,11 @@ struct Runner {
 
   // The product and its reconstruction, in pieces of the output scratch.
   void product(Job& j, const Piece& q, int tiles) const {
-    const int cap = int(std::min<int64_t>(sc.out_bytes / (int64_t(kRnsOutTile) * (CPLX ? 2 : 1)), kItems * sms() / kRnsModuli));
+    const int cap = int(std::min<int64_t>(sc.out_bytes / (int64_t(kRnsOutTile) * (CPLX ? 2 : 1)), kItems * sc.sms / kRnsModuli));
     for (int o = 0; o < tiles; o += cap) {
       j.o0 = o;
       j.on = std::min(cap, tiles - o);
-      launch_chained(k_rns_gemm<CPLX>, std::min(sms(), j.on * kRnsModuli), kThreads, gemm_smem(CPLX), st, j, sc.planes,
+      launch_chained(k_rns_gemm<CPLX>, std::min(sc.sms, j.on * kRnsModuli), kThreads, gemm_smem(CPLX), st, j, sc.planes,
                      sc.out, sc.fail, sc.wait_ns);
       launch_chained(k_rns_recon<T>, dim3(j.on, (CPLX ? 2 : 1) * kRnsTile * kRnsTile / 4 / kReconThreads), kReconThreads, 0,
                      st, reinterpret_cast<double*>(F), reinterpret_cast<double*>(Y), j, sc.planes, sc.out);

@@ -28,6 +28,7 @@ struct RnsScratch {
   int64_t out_bytes = 0;
   int* fail = nullptr;
   uint64_t wait_ns = 0;
+  int sms = 152;  // of the plan's device
 };
 
 // Bytes of one operand slot: 128 rows x K (rounded up to 32) bf16 residues of
