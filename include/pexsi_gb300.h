@@ -96,8 +96,9 @@ typedef struct pexsi_opts {
                               (default). 1: CTA 0 of every short-K split GEMM launch
                               issues no operand copy, so that its MMA issuer's wait
                               runs out after wait_ns (PEXSI_ERR_TIMEOUT); on plans
-                              with split_slices = 0 the first column of every
-                              block inverse on a cluster comes late instead. 2: a breakdown of front 0 is recorded from
+                              with split_slices = 0 CTA 0 of every residue GEMM, and
+                              the first column of every block inverse on a cluster
+                              comes late. 2: a breakdown of front 0 is recorded from
                               the host after the first pole batch of every call with
                               accumulate = 0 (PEXSI_ERR_BREAKDOWN at the end of the
                               chain).                                             */

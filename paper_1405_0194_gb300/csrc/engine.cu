@@ -184,6 +184,7 @@ void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, int64_t rns_
     ws.rns.out_bytes = rns_out;
     ws.rns.wait_ns = p->wait_ns;
     ws.rns.sms = p->sms;
+    ws.rns.hold = p->opts.inject == 1 ? 1 : 0;
   }
   if (p->oz_slices > 0) {
     // complex poles use `batch` members, the real inertia shifts up to 2 batch

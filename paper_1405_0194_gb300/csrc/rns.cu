@@ -526,7 +526,7 @@ __constant__ float c_mod[kRnsModuli] = {256, 253, 251, 247, 241, 239, 233, 229, 
 template <bool CPLX>
 __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant__ Job j,
                                                           const uint8_t* __restrict__ planes, uint8_t* __restrict__ out,
-                                                          int* __restrict__ gfail, uint64_t wait_ns) {
+                                                          int* __restrict__ gfail, uint64_t wait_ns, int hold) {
   constexpr int C = CPLX ? 2 : 1;
   constexpr int kOp = C * kPlane;  // bytes of one operand's K tile
   extern __shared__ __align__(128) uint8_t sm[];
@@ -600,7 +600,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_rns_gemm(const __grid_constant_
     if (lane == 0) {  // ---- producer
       int n = 0;
       bool ok = true;
-      for (int it = blockIdx.x, x = 0; it < items && ok && !*fail; it += gridDim.x, ++x) {
+      // hold (fault injection): CTA 0 copies nothing, and its MMA issuer's wait for operands runs out
+      for (int it = hold && blockIdx.x == 0 ? items : int(blockIdx.x), x = 0; it < items && ok && !*fail; it += gridDim.x, ++x) {
         const int4 t = s_item[x];
         const int l = int(uint32_t(t.z) >> 24), nkt = t.z & 0xFFFFFF;
         const int64_t lo = int64_t(l) * j.kt * kOp;
@@ -1293,7 +1294,7 @@ struct Runner {
       j.o0 = o;
       j.on = std::min(cap, tiles - o);
       launch_chained(k_rns_gemm<CPLX>, std::min(sc.sms, j.on * kRnsModuli), kThreads, gemm_smem(CPLX), st, j, sc.planes,
-                     sc.out, sc.fail, sc.wait_ns);
+                     sc.out, sc.fail, sc.wait_ns, sc.hold);
       launch_chained(k_rns_recon<T>, dim3(j.on, (CPLX ? 2 : 1) * kRnsTile * kRnsTile / 4 / kReconThreads), kReconThreads, 0,
                      st, reinterpret_cast<double*>(F), reinterpret_cast<double*>(Y), j, sc.planes, sc.out);
     }

@@ -29,6 +29,7 @@ struct RnsScratch {
   int* fail = nullptr;
   uint64_t wait_ns = 0;
   int sms = 152;  // of the plan's device
+  int hold = 0;   // fault injection: CTA 0 of every GEMM copies no operands
 };
 
 // Bytes of one operand slot: 128 rows x K (rounded up to 32) bf16 residues of

@@ -4,7 +4,8 @@ returns PEXSI_ERR_TIMEOUT and names the wait, and the context stays usable.
 
 A front of up to 64 columns without rows below it runs the block inverse and no
 GEMM, so its timeout is the block inverse's: the first column of the cluster
-comes 8 ms late.
+comes 8 ms late. Where the block inverses run one to a CTA, which does not wait,
+the timeout is the residue GEMM's: its CTA 0 copies no operands.
 """
 import numpy as np
 import pytest
@@ -65,6 +66,26 @@ def test_block_inverse(n):
     finally:
         px.pexsi_plan_destroy(plan)
     _works(n, colptr, rowind, H, S)
+
+
+def test_residue_gemm():
+    """Two fronts of 300 columns for 64 poles at once: more than 99 block inverses a launch, which run one to a CTA without
+    waits, so that the timeout is the GEMM's."""
+    n = 300
+    colptr, rowind, H, S = _full(n, n)
+    colptr = np.concatenate([colptr, colptr[-1] + colptr[1:]])
+    rowind = np.concatenate([rowind, rowind + n])
+    h, s = np.tile(H.ravel(), 2), np.tile(S.ravel(), 2)
+    plan = px.pexsi_setup(2 * n, colptr, rowind.astype(np.int32),
+                          opts=px.pexsi_opts_default(max_batch=64, inject=1, wait_ns=WAIT_NS))
+    try:
+        _times_out(lambda: px.pexsi_dm(plan, h, s, 0.1, 50.0, 64, 4.0), "tensor-core GEMM")
+        _times_out(lambda: px.pexsi_inertia(plan, h, s, np.linspace(0.1, 0.2, 64)), "tensor-core GEMM")
+        _times_out(lambda: px.pexsi_dm_hermitian(plan, h.astype(complex), s.astype(complex), 0.1, 50.0, 64, 4.0),
+                   "tensor-core GEMM")
+    finally:
+        px.pexsi_plan_destroy(plan)
+    _works(n, *_full(n, n))
 
 
 @pytest.mark.parametrize("n", [33, 64])
