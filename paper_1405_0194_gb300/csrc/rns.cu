@@ -1118,8 +1118,9 @@ struct Slots {
   int k;         // contraction length: the slot size
 };
 
-// The pieces of a launch sequence that fit the scratch, in order. A front whose
-// fixed slots alone do not fit cannot occur (rns_scratch_range).
+// The pieces of a launch sequence that fit the scratch, in order. Every front's
+// fixed slots and one row tile fit (rns_scratch_range); a front for which they did
+// not would be left out without a word, so that is an error.
 template <typename Fn>
 std::vector<Piece> pieces_of(int nact, int nb, int64_t cap, bool cplx, Fn slots) {
   std::vector<Piece> out;
@@ -1137,7 +1138,8 @@ std::vector<Piece> pieces_of(int nact, int nb, int64_t cap, bool cplx, Fn slots)
     const int64_t fit = cap / rns_slot_bytes(k, cplx);
     if (sum > fit) {  // one front, in pieces of its row tiles
       const Slots q = slots(f0);
-      const int step = int(std::max<int64_t>(1, fit - q.fixed));
+      const int step = int(fit - q.fixed);
+      if (q.n <= 0 || step <= 0) throw CudaError{cudaErrorInvalidValue, "residue scratch below a front's operands"};
       for (int pole = 0; pole < nb; ++pole)
         for (int r = 0; r < q.n; r += step) out.push_back({f0, 1, pole, 1, r, std::min(step, q.n - r)});
     } else if (sum > 0) {
@@ -1339,7 +1341,6 @@ Slots gen_sweep_slots(const Dims& d, int b) {
   return {2 * tiles128(d.bw) + 2, 0, b};
 }
 Slots gen_refine_slots(const Dims& d, int b) { return {d.bw > b ? 2 * tiles128(d.bw) : 0, 0, d.bw}; }
-Slots gen_schur_slots(const Dims& d) { return {d.mp > 0 ? 2 * tiles128(d.mp) + tiles128(d.bw) : 0, 0, d.bw}; }
 Slots schur_slots(const Dims& d) { return {d.mp > 0 ? 2 * tiles128(d.mp) + tiles128(d.bw) : 0, 0, d.bw}; }
 Slots tak_slots(const Dims& d) {
   const int tm = tiles128(d.bw), tn = tiles128(d.mp);
@@ -1614,7 +1615,7 @@ void rns_factor_block_gen(const pexsi_plan* p, const Level& lv, const RnsScratch
     pf.end(a, P_PANEL, st, 0.0, 0.0, kernels);
   }
   const bool joint = r.update_k(nact, p0) <= rns_block(b);
-  auto slots = [&](int f) { return gen_schur_slots(dims_of(s[f], m[f], p0, 0, b)); };
+  auto slots = [&](int f) { return schur_slots(dims_of(s[f], m[f], p0, 0, b)); };
   for (const Piece& q : pieces_of(nact, sh.nb, sc.plane_bytes, true, slots)) {
     const int kt = (std::min(rns_block(b), s[q.f0] - p0) + kK - 1) / kK;
     Job l, u, x;
