@@ -143,7 +143,9 @@ def roofline_of(dom: dict, total_kernel_ms: float, peaks: dict, split: int) -> d
     bytes against the copy rate; an FP64 class by its algorithmic flops against
     the FP64 DFMA peak (no measured FP64 peak exists)."""
     secs = dom["ms"] / 1e3
-    r = {"kernel": dom["name"], "launches": dom["launches"], "avg_launch_ms": dom["ms"] / max(1, dom["launches"]),
+    # one launch class cuts the operands of both paths
+    name = "residue_conversion" if dom["name"] == "split_slice" and not split else dom["name"]
+    r = {"kernel": name, "launches": dom["launches"], "avg_launch_ms": dom["ms"] / max(1, dom["launches"]),
          "time_share": dom["ms"] / total_kernel_ms if total_kernel_ms else None}
     if dom.get("tensor_flops", 0) > 0 and secs > 0:
         peak = float(peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops", 1700.0)))
