@@ -73,8 +73,14 @@ typedef struct pexsi_opts {
   int32_t split_slices;    /* 0: FP64 products (default): exact integer products of
                               58-bit operands in residues modulo 15 numbers on the
                               tcgen05 tensor cores, accurate to 2^-59 of the
-                              operands' row norms, or FP64 multiply-adds where the
-                              budget leaves no room for their scratch. 2..6: the supernode GEMMs
+                              operands' row norms (of a matrix equilibrated by
+                              powers of two), or FP64 multiply-adds where the
+                              budget leaves no room for their scratch. So an entry
+                              below 2^-5 of its row's norm has fewer bits than in a
+                              multiply-add: entries of an inverse that decays over
+                              many orders within one front are accurate against the
+                              largest ones, not each to its own size. 2..6: the
+                              supernode GEMMs
                               (panel solve L = W D^-1, Schur update F -= L W^T,
                               Takahashi step Y[S,P] = -Y[S,S] L[S,P] and Y[P,P] =
                               D^-1 - L[S,P]^T Y[S,P]; real ones of the inertia
@@ -133,7 +139,8 @@ typedef struct pexsi_dm_info {
   double trace_dm_s;       /* Tr[DM S] = N_e (Eq. Nmu); computed on the device   */
   double trace_edm_s;      /* Tr[EDM S]                                          */
   double trace_fdm_s;      /* Tr[FDM S] (grand potential)                        */
-  double min_pivot_ratio;  /* min over diagonal blocks of |pivot| / max |entry|, |z| = |Re z| + |Im z| */
+  double min_pivot_ratio;  /* min over diagonal blocks of |pivot| / max |entry|, |z| = |Re z| + |Im z|,
+                              in the units of H - z S as given                                      */
   double ms_total;         /* wall time of the call (device events)             */
   double gemm_flops;       /* algorithmic GEMM flops executed by the call       */
   int32_t n_poles;         /* poles evaluated by the call                       */
