@@ -180,6 +180,7 @@ void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, int64_t rns_
     wsalloc(&ws.g, sizeof(int16_t) * size_t(p->sym.n * scale_stride(batch)), ws, "alloc(scaling)");
     wsalloc(&ws.g0, sizeof(int16_t) * size_t(p->sym.n * scale_stride(batch)), ws, "alloc(scaling)");
     wsalloc(&ws.h, sizeof(int16_t) * size_t(p->sym.n), ws, "alloc(scaling)");
+    wsalloc(&ws.scaled, sizeof(int), ws, "alloc(scaling)");
     ws.rns.plane_bytes = rns_planes;
     ws.rns.out_bytes = rns_out;
     ws.rns.wait_ns = p->wait_ns;
@@ -203,7 +204,7 @@ void workspace_alloc(const pexsi_plan* p, Workspace& ws, int batch, int64_t rns_
 void workspace_free(Workspace& ws) {
   void* ptrs[] = {ws.F,  ws.Y,        ws.part,  ws.H,    ws.S,   ws.out, ws.brk, ws.minpiv, ws.neg,
                   ws.partials, ws.trace3, ws.ainv, ws.ozA, ws.ozB, ws.exA, ws.exB, ws.ozfail, ws.ymax, ws.kpart,
-                  ws.dsave, ws.rns.planes, ws.rns.out, ws.g, ws.g0, ws.h};
+                  ws.dsave, ws.rns.planes, ws.rns.out, ws.g, ws.g0, ws.h, ws.scaled};
   for (void* q : ptrs) {
     if (!q) continue;
     if (ws.async) cudaFreeAsync(q, ws.stream);
@@ -318,7 +319,7 @@ void factor_batch(const pexsi_plan* p, Workspace& ws, T* F, const BatchShifts& s
   // are saved and counted after the factorisation
   DevStatus status{ws.brk + (count ? 1 : 0), ws.minpiv + (count ? 1 : 0), ws.neg, count ? ws.dsave : nullptr,
                    p->d_col0, p->sym.n * int64_t(p->b), ws.ozfail + (count ? 1 : 0), p->wait_ns,
-                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g, ws.h, scale_stride(ws.batch)};
+                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g, ws.h, scale_stride(ws.batch), ws.scaled};
   const int b = p->b;
   const double es = double(sizeof(T)), fl = sizeof(T) == 16 ? 8.0 : 2.0, nb = sh.nb;
   for (size_t L = 0; L < p->levels.size(); ++L) {
@@ -596,7 +597,7 @@ void set_scales(const pexsi_plan* p, Workspace& ws, const double* dH, const doub
   if (!ws.g) return;
   const int64_t c0 = p->sys_col_off[q], n = p->sys_col_off[q + 1] - c0;
   launch_rns_scales(dH, dS, wide, sh, p->d_colptr + c0, p->d_diag + c0, n, c0, p->sys_entry_off[q], p->d_row, p->d_col,
-                    ws.h, ws.g0, ws.g, scale_stride(ws.batch), ws.stream);
+                    ws.h, ws.g0, ws.g, scale_stride(ws.batch), ws.scaled, q == 0, ws.stream);
 }
 
 void run_complex_batch(const pexsi_plan* p, Workspace& ws, const double* dH, const double* dS, const BatchShifts& sh,
@@ -758,7 +759,7 @@ void factor_batch_gen(const pexsi_plan* p, Workspace& ws, const BatchShifts& sh,
   DevFronts fr = p->fronts();
   DevStatus status{ws.brk + (count ? 1 : 0), ws.minpiv + (count ? 1 : 0), ws.neg, count ? ws.dsave : nullptr,
                    p->d_col0, p->sym.n * int64_t(p->b), ws.ozfail + (count ? 1 : 0), p->wait_ns,
-                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g, ws.h, scale_stride(ws.batch)};
+                   p->oz_slices == 0 && p->opts.inject == 1 ? 1 : 0, ws.g, ws.h, scale_stride(ws.batch), ws.scaled};
   const int b = p->b;
   const double nb = sh.nb;
   for (size_t L = 0; L < p->levels.size(); ++L) {

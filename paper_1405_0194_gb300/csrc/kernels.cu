@@ -344,10 +344,11 @@ template <typename T>
 __global__ void k_assemble(T* __restrict__ F, const double* __restrict__ H, const double* __restrict__ S,
                            const int64_t* __restrict__ src, const int64_t* __restrict__ pos, int64_t nlow,
                            int64_t pool, BatchShifts sh, EntryScale sc) {
+  const bool on = sc.on();
   for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < nlow; t += int64_t(gridDim.x) * blockDim.x) {
     int64_t e = src[t], p = pos[t];
     const double h = H[e], s = S[e];
-    const int16_t *gr = sc.of_row(e), *gc = sc.of_col(e);
+    const int16_t *gr = on ? sc.of_row(e) : nullptr, *gc = on ? sc.of_col(e) : nullptr;
 #pragma unroll 4
     for (int b = 0; b < sh.nb; ++b) {
       const T a = make_shift<T>(h, s, sh, b);
@@ -647,8 +648,10 @@ __device__ void bk_count<double>(double* Bm, int n, int ld, int* out_neg, bool* 
 //
 // Warps: 6 update warps on three of the four SM partitions (warps 0-2, 4-6), the
 // search warp alone on the fourth (warp 3), whose chain of steps the updates would
-// hold up: 118 us against 124. Warp 7 there only follows the pivots of the block
-// for the pivot ratio, in CTA 0, whose own searches come first.
+// hold up: 118 us against 124. Warp 7 there takes the pivot ratio: the largest
+// entries of the CTA's columns, and in CTA 0, whose own searches come first, the
+// pivots. The update threads finding the largest entries before the first step and
+// one thread the pivots after the last cost 4 us more.
 //
 // Clusters up to 99 inversions of a launch, one CTA each from 100 (48 x 48
 // complex, us): 40: 116 against 217; 80: 209 / 216; 160: 389 / 295. Clusters of 2
@@ -669,7 +672,6 @@ __device__ __forceinline__ void least(double* at, double v) {
 // the scaled matrix back to the caller's (low half) and to rows of which each is
 // scaled by its own H and S before they cancel (high half).
 __device__ __forceinline__ int units_of(const DevStatus& st, int pb, int col) {
-  if (!st.g) return 0;
   const int g = st.g[col * st.g_stride + pb], h = st.h[col];
   return (g & 0xFFFF) | (g - h) << 16;
 }
@@ -771,9 +773,8 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
   uint64_t* s_full = reinterpret_cast<uint64_t*>(s_row + 2 * (64 / C + 1));  // [64]: column and pivot row are here
   uint64_t* s_inv = s_full + 64;                                             // [64]: the reciprocal is here
   uint64_t* s_ready = s_inv + 64;                                            // [64]: the next column is staged
-  __shared__ double s_lmax[2], s_maxes[2][C];  // largest entry in both units, of this CTA and (in CTA 0) of every one
+  __shared__ double s_maxes[2][C];  // in CTA 0: largest entries of every CTA's columns, in both units
   __shared__ T s_scaled[64 / C];
-  __shared__ int s_ex[64];  // units of the block's rows and columns
   const int f = fronts[blockIdx.x / C];
   const int r = int(cg::this_cluster().block_rank());
   const int pb = blockIdx.y;
@@ -786,7 +787,7 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = tid >> 5;
   const bool searcher = warp == 3;
-  const bool updater = !searcher && warp != 7;
+  const bool updater = !searcher && warp != 7;  // warp 7: the pivot ratios
   const int ut = warp > 3 ? tid - 32 : tid;  // update thread
   const int g = ut / bb, i = ut - g * bb;
   const bool holds = updater && g < ng;
@@ -805,7 +806,6 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
     if (holds && jl < nc) a[q] = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
   }
   if (tid < 64) {
-    s_ex[tid] = tid < bb ? units_of(st, pb, st.col0[f] + p0 + tid) : 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8 * tid));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(inv0 + 8 * tid));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(ready0 + 8 * tid), "r"(bb));
@@ -817,29 +817,27 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(inv0 + 8 * tid), "r"(int(sizeof(T)) + 16)
                  : "memory");
   }
-  if (tid < 2) s_lmax[tid] = 0.0;
-  __syncthreads();
-  double lmax = 0.0, gmax = 0.0;
   T* save = st.dsave ? reinterpret_cast<T*>(st.dsave) + int64_t(pb) * st.dsave_stride + int64_t(st.col0[f] + p0) * b
                      : nullptr;  // inertia shifts: the block before inversion, counted later
+  if (save) {
 #pragma unroll
-  for (int q = 0; q < E; ++q) {
-    const int jl = g + ng * q, j = c0 + jl;
-    if (holds && jl < nc) {
-      lmax = fmax(lmax, in_units<0>(mag1(a[q]), s_ex[i], s_ex[j]));
-      gmax = fmax(gmax, in_units<1>(mag1(a[q]), s_ex[i], s_ex[j]));
-      if (save) save[i * b + j] = a[q];
+    for (int q = 0; q < E; ++q) {
+      const int jl = g + ng * q;
+      if (holds && jl < nc) save[i * b + c0 + jl] = a[q];
     }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-    gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+  // warp 7: magnitudes of the CTA's columns, rows `lane` and `lane` + 32 of each
+  double mag[2 * (64 / C)];
+  if (warp == 7) {
+#pragma unroll
+    for (int q = 0; q < 2 * (64 / C); ++q) {
+      const int row = lane + 32 * (q & 1), j = c0 + q / 2;
+      mag[q] = 0.0;
+      if (row < bb && q / 2 < nc) mag[q] = mag1((GEN || row >= j) ? Fd[row + int64_t(m) * j] : Fd[j + int64_t(m) * row]);
+    }
   }
-  if (lane < 2)
-    atomicMax(reinterpret_cast<unsigned long long*>(&s_lmax[lane]), __double_as_longlong(lane == 0 ? lmax : gmax));
   __syncthreads();
   cg::this_cluster().sync();  // every CTA runs and its barriers are set before any remote access
-  if (tid < 2) *cg::this_cluster().map_shared_rank(&s_maxes[tid][r], 0) = s_lmax[tid];
   double pmin = DBL_MAX, gmin = DBL_MAX;
   bool lost = false;  // a wait of this thread ran out
   auto wait = [&](uint32_t bar) { diag_wait(bar, st.wait_ns, lost); };
@@ -950,9 +948,28 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
         Fd[i + int64_t(m) * pos] = a[q];
       }
     }
-  } else if (r == 0) {  // warp 7: the pivots in both units, each in the row that the interchanges brought to its place
+  } else {  // the block's entries and pivots in both units, beside the updates
+    int ex0 = 0, ex1 = 0;  // units of rows and columns `lane` and `lane` + 32
+    if (st.g && *st.scaled) {
+      if (lane < bb) ex0 = units_of(st, pb, st.col0[f] + p0 + lane);
+      if (lane + 32 < bb) ex1 = units_of(st, pb, st.col0[f] + p0 + lane + 32);
+    }
+    auto units = [&](int x) { return __shfl_sync(0xffffffffu, x < 32 ? ex0 : ex1, x & 31); };
+    double lmax = 0.0, gmax = 0.0;
+#pragma unroll
+    for (int q = 0; q < 2 * (64 / C); ++q) {
+      const int row = q & 1 ? ex1 : ex0, col = units(c0 + q / 2 < 64 ? c0 + q / 2 : 0);
+      lmax = fmax(lmax, in_units<0>(mag[q], row, col));
+      gmax = fmax(gmax, in_units<1>(mag[q], row, col));
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+      gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+    }
+    if (lane < 2) *cg::this_cluster().map_shared_rank(&s_maxes[lane][r], 0) = lane == 0 ? lmax : gmax;
+    // the pivots, each in the row that the interchanges brought to its place: CTA 0, whose own searches come first
     int at0 = lane, at1 = lane + 32;
-    for (int k = 0; k < bb; ++k) {
+    for (int k = 0; k < (r == 0 ? bb : 0); ++k) {
       wait(full0 + 8 * k);
       wait(inv0 + 8 * k);
       const int row = int(s_step[k].row);
@@ -961,8 +978,9 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 16 ? 3 : 4) k_diag_
       if (lane == (row & 31)) (row < 32 ? at0 : at1) = from_k;
       if (lane == (k & 31)) (k < 32 ? at0 : at1) = from;
       const double best = s_step[k].best;
-      pmin = fmin(pmin, in_units<0>(best, s_ex[from], s_ex[k]));
-      gmin = fmin(gmin, in_units<1>(best, s_ex[from], s_ex[k]));
+      const int row_ex = units(from), col_ex = units(k);
+      pmin = fmin(pmin, in_units<0>(best, row_ex, col_ex));
+      gmin = fmin(gmin, in_units<1>(best, row_ex, col_ex));
     }
   }
   if (lost) {  // what is still on its way here
@@ -1005,8 +1023,9 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
   __shared__ int s_perm[64];
   __shared__ int s_ex[2][64];  // units of the columns, and of the rows as they are interchanged
   __shared__ double s_best[64];
-  if (threadIdx.x < 64) s_ex[0][threadIdx.x] = s_ex[1][threadIdx.x] =
-      int(threadIdx.x) < bb ? units_of(st, pb, st.col0[f] + p0 + int(threadIdx.x)) : 0;
+  const bool scaled = st.g && *st.scaled;  // else both units are those of the entries
+  if (scaled && int(threadIdx.x) < bb)
+    s_ex[0][threadIdx.x] = s_ex[1][threadIdx.x] = units_of(st, pb, st.col0[f] + p0 + int(threadIdx.x));
   if (threadIdx.x < 2) { s_max[threadIdx.x] = 0.0; s_pmin[threadIdx.x] = DBL_MAX; s_bad = false; }
   __syncthreads();
   double lmax = 0.0, gmax = 0.0;
@@ -1015,8 +1034,9 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
     // symmetric fronts hold the lower triangle; LDU fronts (GEN) both
     T v = (GEN || i >= j) ? Fd[i + int64_t(m) * j] : Fd[j + int64_t(m) * i];
     Aug[i * ld + j] = v;
-    lmax = fmax(lmax, in_units<0>(mag1(v), s_ex[0][i], s_ex[0][j]));
-    gmax = fmax(gmax, in_units<1>(mag1(v), s_ex[0][i], s_ex[0][j]));
+    const double mag = mag1(v);
+    lmax = fmax(lmax, scaled ? in_units<0>(mag, s_ex[0][i], s_ex[0][j]) : mag);
+    if (scaled) gmax = fmax(gmax, in_units<1>(mag, s_ex[0][i], s_ex[0][j]));
   }
   // block max |entry| for the pivot ratio
   for (int o = 16; o > 0; o >>= 1) {
@@ -1054,9 +1074,11 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
         const double best = mag1(Aug[bi * ld + k]);
         s_piv = bi;
         s_best[k] = best;
-        const int ex = s_ex[1][bi];
-        s_ex[1][bi] = s_ex[1][k];
-        s_ex[1][k] = ex;
+        if (scaled) {
+          const int ex = s_ex[1][bi];
+          s_ex[1][bi] = s_ex[1][k];
+          s_ex[1][k] = ex;
+        }
         if (!(best > 0.0) || !isfinite(best)) s_bad = true;
       }
     }
@@ -1085,8 +1107,9 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
     __syncthreads();
   }
   if (int(threadIdx.x) < bb) {
-    least(&s_pmin[0], in_units<0>(s_best[threadIdx.x], s_ex[1][threadIdx.x], s_ex[0][threadIdx.x]));
-    least(&s_pmin[1], in_units<1>(s_best[threadIdx.x], s_ex[1][threadIdx.x], s_ex[0][threadIdx.x]));
+    const double best = s_best[threadIdx.x];
+    least(&s_pmin[0], scaled ? in_units<0>(best, s_ex[1][threadIdx.x], s_ex[0][threadIdx.x]) : best);
+    if (scaled) least(&s_pmin[1], in_units<1>(best, s_ex[1][threadIdx.x], s_ex[0][threadIdx.x]));
   }
   // the row interchanges become column interchanges of the inverse, undone in reverse order
   for (int k = bb - 1; k >= 0; --k) {
@@ -1101,7 +1124,7 @@ __global__ void __launch_bounds__(256) k_diag_inv_one(T* __restrict__ F, DevFron
     int i = idx % bb, j = idx / bb;
     Fd[i + int64_t(m) * j] = Aug[i * ld + j];
   }
-  if (threadIdx.x == 0) report_pivots(st, f, s_bad, s_pmin[0], s_max[0], s_pmin[1], s_max[1]);
+  if (threadIdx.x == 0) report_pivots(st, f, s_bad, s_pmin[0], s_max[0], s_pmin[scaled], s_max[scaled]);
 }
 
 // Deferred inertia count: one CTA per (saved panel block, batch member).
@@ -1423,10 +1446,11 @@ __global__ void k_pole_sum(const double2* __restrict__ Y, int64_t pool, const in
                            int64_t nnz, BatchShifts sh, int overwrite, double* __restrict__ dm,
                            double* __restrict__ edm, double* __restrict__ fdm, double* __restrict__ ddm,
                            EntryScale sc) {
+  const bool on = sc.on();
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t p = entry_pos[e];
     double a = 0.0, ae = 0.0, af = 0.0, ad = 0.0;
-    const int16_t *gr = sc.of_row(e), *gc = sc.of_col(e);
+    const int16_t *gr = on ? sc.of_row(e) : nullptr, *gc = on ? sc.of_col(e) : nullptr;
     for (int b0 = 0; b0 < sh.nb; b0 += 4) {  // the loads of four members in flight
       double2 v[4];
       int x[4];
@@ -1460,10 +1484,11 @@ __global__ void k_pole_sum(const double2* __restrict__ Y, int64_t pool, const in
 __global__ void k_assemble_gen(double2* __restrict__ F, const double2* __restrict__ H, const double2* __restrict__ S,
                                const int64_t* __restrict__ pos, int64_t nnz, int64_t pool, BatchShifts sh,
                                EntryScale sc) {
+  const bool on = sc.on();
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t p = pos[e];
     const double2 h = H[e], v = S[e];
-    const int16_t *gr = sc.of_row(e), *gc = sc.of_col(e);
+    const int16_t *gr = on ? sc.of_row(e) : nullptr, *gc = on ? sc.of_col(e) : nullptr;
     for (int b = 0; b < sh.nb; ++b) {  // (hr + i hi) - (zr + i zi)(sr + i si)
       const double2 a = make_double2(h.x - fma(sh.re[b], v.x, -sh.im[b] * v.y), h.y - fma(sh.re[b], v.y, sh.im[b] * v.x));
       F[b * pool + p] = gr ? scale2(a, entry_exp(gr, gc, b)) : a;
@@ -1479,10 +1504,11 @@ __global__ void k_pole_sum_herm(const double2* __restrict__ Y, int64_t pool, con
                                 const int64_t* __restrict__ pos_t, int64_t nnz, BatchShifts sh, int overwrite,
                                 double2* __restrict__ dm, double2* __restrict__ edm, double2* __restrict__ fdm,
                                 double2* __restrict__ ddm, EntryScale sc) {
+  const bool on = sc.on();
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t p = pos[e], q = pos_t[e];
     double2 o[4] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
-    const int16_t *gr = sc.of_row(e), *gc = sc.of_col(e);
+    const int16_t *gr = on ? sc.of_row(e) : nullptr, *gc = on ? sc.of_col(e) : nullptr;
     for (int b = 0; b < sh.nb; ++b) {
       double2 g = Y[b * pool + p], gt = Y[b * pool + q];
       if (gr) {
@@ -1509,14 +1535,16 @@ __global__ void k_pole_sum_herm(const double2* __restrict__ Y, int64_t pool, con
 
 __global__ void k_extract(const double2* __restrict__ Y, const int64_t* __restrict__ entry_pos, int64_t nnz,
                           double2* __restrict__ out, EntryScale sc) {
+  const bool on = sc.on();
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x)
-    out[e] = sc.g ? scale2(Y[entry_pos[e]], entry_exp(sc.of_row(e), sc.of_col(e), 0)) : Y[entry_pos[e]];
+    out[e] = on ? scale2(Y[entry_pos[e]], entry_exp(sc.of_row(e), sc.of_col(e), 0)) : Y[entry_pos[e]];
 }
 
 __global__ void k_scaled_imag(const double2* __restrict__ Y, const int64_t* __restrict__ entry_pos, int64_t nnz,
                               double scale, double* __restrict__ out, EntryScale sc) {
+  const bool on = sc.on();
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < nnz; e += int64_t(gridDim.x) * blockDim.x)
-    out[e] = scale * (sc.g ? scale2(Y[entry_pos[e]].y, entry_exp(sc.of_row(e), sc.of_col(e), 0)) : Y[entry_pos[e]].y);
+    out[e] = scale * (on ? scale2(Y[entry_pos[e]].y, entry_exp(sc.of_row(e), sc.of_col(e), 0)) : Y[entry_pos[e]].y);
 }
 
 __global__ void k_trace_partial(const double* dm, const double* edm, const double* fdm, const double* ddm,

@@ -85,6 +85,7 @@ struct DevStatus {
   // elimination order from g + c * g_stride on, and of the columns' own H and S at h (k_diag_inv_*: the pivot ratios)
   const int16_t *g, *h;
   int64_t g_stride;
+  const int* scaled;                 // whether any exponent is not zero
 };
 
 // The scaling of a batch (launch_rns_scales; g NULL: none) and the row and column
@@ -93,9 +94,11 @@ struct EntryScale {
   const int16_t* g;
   int64_t stride;
   const int32_t *row, *col;
+  const int* scaled;  // whether any exponent is not zero
+  __device__ __forceinline__ bool on() const { return g && *scaled; }
   // the members' exponents of entry e's row and column
-  __device__ __forceinline__ const int16_t* of_row(int64_t e) const { return g ? g + row[e] * stride : nullptr; }
-  __device__ __forceinline__ const int16_t* of_col(int64_t e) const { return g ? g + col[e] * stride : nullptr; }
+  __device__ __forceinline__ const int16_t* of_row(int64_t e) const { return g + row[e] * stride; }
+  __device__ __forceinline__ const int16_t* of_col(int64_t e) const { return g + col[e] * stride; }
 };
 
 // Scratch of the split-precision GEMM: bf16 slice tiles of A = Y[S,S] and

@@ -109,6 +109,7 @@ struct Workspace {
   RnsScratch rns;            // FP64 path: scratch of the residue products (no planes: DFMA kernels)
   // its power-of-two scaling: exponents of the batch's columns, a first guess, and those of the columns' own H and S
   int16_t *g = nullptr, *g0 = nullptr, *h = nullptr;
+  int* scaled = nullptr;     // whether any of them is not zero
   cudaStream_t stream = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // captured level schedules (factorisation + selected inversion of nb
@@ -234,7 +235,7 @@ inline int64_t scale_stride(int batch) { return (2 * batch + 7) / 8 * 8; }
 inline EntryScale entry_scale_of(const pexsi_plan* p, const Workspace& ws, size_t q = 0) {
   if (!ws.g) return EntryScale{};
   const int64_t e0 = p->sys_entry_off[q];
-  return EntryScale{ws.g, scale_stride(ws.batch), p->d_row + e0, p->d_col + e0};
+  return EntryScale{ws.g, scale_stride(ws.batch), p->d_row + e0, p->d_col + e0, ws.scaled};
 }
 
 // Allocates ws for `batch` poles on `stream` (cudaMallocAsync when async),

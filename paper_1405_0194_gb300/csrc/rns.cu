@@ -1026,8 +1026,9 @@ template <int W>
 __global__ void k_rns_diag_scale(const double* __restrict__ H, const double* __restrict__ S,
                                  const int64_t* __restrict__ diag, int64_t n, int64_t c0, int64_t e0,
                                  const __grid_constant__ BatchShifts sh, int64_t stride, int16_t* __restrict__ h,
-                                 int16_t* __restrict__ g0) {
+                                 int16_t* __restrict__ g0, int* __restrict__ scaled, bool first) {
   const int b = blockIdx.y;
+  if (first && b == 0 && blockIdx.x == 0 && threadIdx.x == 0) *scaled = 0;
   for (int64_t c = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; c < n; c += int64_t(gridDim.x) * blockDim.x) {
     const int64_t e = (diag[c] - e0) * W;
     const double Hc = H[e], Sc = S[e];  // of Hermitian H and S: real
@@ -1051,7 +1052,7 @@ __global__ void __launch_bounds__(256) k_rns_scale(const double* __restrict__ H,
                                                    const int32_t* __restrict__ col, int64_t n, int64_t e0,
                                                    const __grid_constant__ BatchShifts sh, int64_t stride,
                                                    const int16_t* __restrict__ h, const int16_t* __restrict__ g0,
-                                                   int16_t* __restrict__ g) {
+                                                   int16_t* __restrict__ g, int* __restrict__ scaled) {
   union Word {
     uint4 u;
     int16_t x[8];
@@ -1063,6 +1064,7 @@ __global__ void __launch_bounds__(256) k_rns_scale(const double* __restrict__ H,
   for (int64_t j = blockIdx.x * 8 + (threadIdx.x >> 5); j < n; j += int64_t(gridDim.x) * 8) {
     const int64_t lo = colptr[j], hi = colptr[j + 1];
     const int c = col[lo], hc = h[c];
+    bool any = false;
     Word top;
     top.u = *reinterpret_cast<const uint4*>(g0 + c * stride + b0);
     int t[8];
@@ -1100,9 +1102,12 @@ __global__ void __launch_bounds__(256) k_rns_scale(const double* __restrict__ H,
     for (int b = 0; b < 8; ++b) {
       const int m = __reduce_max_sync(0xFFFFFFFFu, t[b]);
       const int x = m == kNoExp ? 0 : max(-500, min(500, m));
-      top.x[b] = int16_t(abs(x - hc) <= kRnsNear ? hc : x);
+      const int gc = abs(x - hc) <= kRnsNear ? hc : x;
+      top.x[b] = int16_t(gc);
+      if (b0 + b < sh.nb && (gc | hc)) any = true;
     }
     if (lane == 0) *reinterpret_cast<uint4*>(g + c * stride + b0) = top.u;
+    if (lane == 0 && any) *scaled = 1;
   }
 }
 
@@ -1351,12 +1356,12 @@ Slots tak_slots(const Dims& d) {
 
 void launch_rns_scales(const double* H, const double* S, int wide, const BatchShifts& sh, const int64_t* colptr,
                        const int64_t* diag, int64_t n, int64_t c0, int64_t e0, const int32_t* row, const int32_t* col,
-                       int16_t* h, int16_t* g0, int16_t* g, int64_t stride, cudaStream_t st) {
+                       int16_t* h, int16_t* g0, int16_t* g, int64_t stride, int* scaled, bool first, cudaStream_t st) {
   auto grid = [](int64_t k) { return int(std::min<int64_t>(k, 152 * 8)); };
   auto run = [&](auto w) {
     constexpr int W = decltype(w)::value;
-    k_rns_diag_scale<W><<<dim3(grid((n + 255) / 256), sh.nb), 256, 0, st>>>(H, S, diag, n, c0, e0, sh, stride, h, g0);
-    k_rns_scale<W><<<dim3(grid((n + 7) / 8), (sh.nb + 7) / 8), 256, 0, st>>>(H, S, colptr, row, col, n, e0, sh, stride, h, g0, g);
+    k_rns_diag_scale<W><<<dim3(grid((n + 255) / 256), sh.nb), 256, 0, st>>>(H, S, diag, n, c0, e0, sh, stride, h, g0, scaled, first);
+    k_rns_scale<W><<<dim3(grid((n + 7) / 8), (sh.nb + 7) / 8), 256, 0, st>>>(H, S, colptr, row, col, n, e0, sh, stride, h, g0, g, scaled);
   };
   if (wide == 1) run(std::integral_constant<int, 1>{});
   else run(std::integral_constant<int, 2>{});

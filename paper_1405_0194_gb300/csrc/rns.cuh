@@ -70,9 +70,10 @@ constexpr int kRnsNear = 5;
 // c0 on, e0 its first entry; row, col and the exponents (g0, g: the members' of
 // column c from c * stride on, a multiple of 8) of all systems in elimination
 // order. h: half the exponents of max(|H_cc|, |S_cc|), by which the breakdown
-// limit knows a row's own size before H and z S cancel.
+// limit knows a row's own size before H and z S cancel. scaled: whether any
+// exponent is not zero (of a group, set from its first system on).
 void launch_rns_scales(const double* H, const double* S, int wide, const BatchShifts& sh, const int64_t* colptr,
                        const int64_t* diag, int64_t n, int64_t c0, int64_t e0, const int32_t* row, const int32_t* col,
-                       int16_t* h, int16_t* g0, int16_t* g, int64_t stride, cudaStream_t st);
+                       int16_t* h, int16_t* g0, int16_t* g, int64_t stride, int* scaled, bool first, cudaStream_t st);
 
 }  // namespace pexsi
