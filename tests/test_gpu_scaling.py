@@ -150,3 +150,23 @@ def test_scaling_follows_each_shift():
     for p in (plan, one):
         px.pexsi_plan_destroy(p)
     assert np.abs(both - alone).max() <= 1e-13 * np.abs(alone).max()  # the same inverses, added up in another order
+
+
+# Entry by entry: rounding every operation of an elimination without growth leaves |dG| <= n eps |G| |A| |G|; as much again
+# for the reference.
+@pytest.mark.parametrize("kind", ["chain", "fluid", "sheet"])
+@pytest.mark.parametrize("overlap", [True, False])
+def test_entries_of_ordinary_systems(kind, overlap):
+    """The operands are rounded against their rows' norms; on the patterns of such systems every entry of the inverse is
+    still accurate to its own size."""
+    import nao_synth as ns
+    s = {"chain": ns.make_chain, "fluid": lambda: ns.make_fluid(nmol=24), "sheet": lambda: ns.make_sheet(ncell=6)}[kind]()
+    cols = np.repeat(np.arange(s.n), np.diff(s.colptr))
+    A, z = np.zeros((s.n, s.n), complex), 0.1 + 0.01j
+    A[s.rowind, cols] = s.H - z * (s.S if overlap else (s.rowind == cols))
+    plan = px.pexsi_setup(s.n, s.colptr, s.rowind, opts=px.pexsi_opts_default(max_batch=1))
+    got = px.pexsi_selinv(plan, s.H, s.S if overlap else None, z)
+    px.pexsi_plan_destroy(plan)
+    G = np.linalg.inv(A)
+    bound = 2 * s.n * np.finfo(float).eps * (np.abs(G) @ np.abs(A) @ np.abs(G))
+    assert (np.abs(got - G[s.rowind, cols]) <= bound[s.rowind, cols]).all()
